@@ -16,17 +16,18 @@ struct lks_batch {
     cudaStream_t st = nullptr;        // own stream: graphs need a capturable stream
     cudaEvent_t ev = nullptr;
     char* dmem = nullptr;
-    Inst* dinst = nullptr;
+    void* dinst = nullptr;
     int* dpre = nullptr;
     int* nbase = nullptr;
+    RunResult* result = nullptr;
     Plan plan;
     bool have_plan = false;
     std::vector<int> gens;
     GraphCache graphs;
     bool use_graphs = true;
-    int tile_req[2] = {-1, -1};       // requested tile shapes, -1 = autotune
+    int tile_req[2] = {-1, -1};       // requested strip heights, -1 = autotune
     int tile[2] = {-1, -1};           // in use
-    float tune_ms[2][kTileCfgs];
+    float tune_ms[2][kStripCfgs];
     long long launches = 0;
     std::string err;
 };
@@ -75,12 +76,12 @@ lks_status batch_prepare(lks_batch* b, int n_steps) {
     for (size_t i = 0; i < b->cs.size(); ++i) stale = stale || b->gens[i] != b->cs[i]->geo_gen;
     if (stale) {
         b->graphs.clear();
-        BCU(build_plan(b->cs, b->dinst, b->dpre, b->nbase, b->st, b->plan));
+        BCU(build_plan<float>(b->cs, b->dinst, b->dpre, b->nbase, b->st, b->plan));
         for (size_t i = 0; i < b->cs.size(); ++i) b->gens[i] = b->cs[i]->geo_gen;
         b->have_plan = true;
         b->tile[0] = b->tile[1] = -1;
     }
-    // autotune: time every tile shape of the fused step and adjoint kernels on this batch
+    // autotune: time every strip height of the fused step and adjoint kernels on this batch
     if (b->tile[0] < 0 || b->tile[1] < 0) {
         for (int w = 0; w < 2; ++w) {
             if (b->tile_req[w] >= 0) {
@@ -88,23 +89,24 @@ lks_status batch_prepare(lks_batch* b, int n_steps) {
                 continue;
             }
             BCU(launch_set_int(b->nbase, 0, b->st));
-            BCU(launch_t_design_pos(b->plan, 1, b->st));
-            BCU(launch_t_transfer2d(b->plan, 1, -1, false, b->st));
+            BCU(launch_t_transfer<float>(b->plan, 1, 1, -1, b->st));
             for (lks_ctx* c : b->cs) {
                 BCU(cudaMemsetAsync(c->lam[0], 0, c->snap_bytes, b->st));
                 BCU(cudaMemsetAsync(c->lam[1], 0, c->snap_bytes, b->st));
+                BCU(cudaMemcpyAsync(c->s[0], c->s0, c->snap_bytes, cudaMemcpyDeviceToDevice, b->st));
+                BCU(cudaMemcpyAsync(c->s[1], c->s0, c->snap_bytes, cudaMemcpyDeviceToDevice, b->st));
             }
             cudaEvent_t e0, e1;
             BCU(cudaEventCreate(&e0));
             BCU(cudaEventCreate(&e1));
             int best = 0;
-            const int ncfg = w == 0 ? kTileCfgs : kAdjCfgs;
-            for (int k = 0; k < kTileCfgs; ++k) b->tune_ms[w][k] = -1.f;
-            for (int k = 0; k < ncfg; ++k) {
+            for (int k = 0; k < kStripCfgs; ++k) {
+                // step 1 from the first working buffer into the second, and its adjoint step
+                const StripRun rf{1, 1, 0, 0, 0, kBoxBuffer, 0, 0};
+                const StripRun ra{1, 1, 1, 0, BUF_S0, kBoxBuffer, -1, 0};
                 auto run = [&]() -> cudaError_t {
-                    return w == 0 ? launch_t_step2d(b->plan, k, BUF_INIT, BUF_S1, -1, b->st)
-                                  : launch_t_adj2d(b->plan, k, 1, BUF_LAM0, BUF_LAM1, BUF_INIT,
-                                                   BUF_INIT, -1, b->st);
+                    return w == 0 ? launch_t_step<float>(b->plan, k, rf, b->st)
+                                  : launch_t_adj<float>(b->plan, k, ra, b->st);
                 };
                 cudaError_t e = cudaSuccess;
                 for (int r = 0; r < 2 && e == cudaSuccess; ++r) e = run();
@@ -140,6 +142,7 @@ Group batch_group(lks_batch* b) {
     G.table = true;
     G.plan = &b->plan;
     G.nbase = b->nbase;
+    G.result = b->result;
     G.tile_fwd = b->tile[0];
     G.tile_adj = b->tile[1];
     G.graphs = b->use_graphs ? &b->graphs : nullptr;
@@ -158,7 +161,7 @@ lks_status lks_batch_create(lks_ctx* const* ctxs, int n, lks_batch** out) {
     for (int i = 0; i < n; ++i) {
         lks_ctx* c = ctxs[i];
         if (!c) return LKS_ERR_ARG;
-        if (!c->fused2d) {
+        if (!c->fused2d || c->prec != LKS_FP32) {
             fprintf(stderr, "lks_batch_create: instance %d is not a D2Q9 FP32 context on the "
                             "fused kernels\n", i);
             return LKS_ERR_ARG;
@@ -179,25 +182,26 @@ lks_status lks_batch_create(lks_ctx* const* ctxs, int n, lks_batch** out) {
     b->cs.assign(ctxs, ctxs + n);
     b->gens.assign(n, -1);
     b->user_st = ctxs[0]->st;
-    const size_t inst_bytes = align256(sizeof(Inst) * n);
+    const size_t inst_bytes = align256(sizeof(Inst<float>) * n);
     const size_t pre_bytes = align256(sizeof(int) * U_COUNT * (n + 1));
     if (cudaStreamCreateWithFlags(&b->st, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess ||
-        dev_alloc((void**)&b->dmem, inst_bytes + pre_bytes + 256) != cudaSuccess) {
+        dev_alloc((void**)&b->dmem, inst_bytes + pre_bytes + 256 + sizeof(RunResult) * n) != cudaSuccess) {
         cudaGetLastError();
         lks_batch_destroy(b);
         return LKS_ERR_NOMEM;
     }
-    b->dinst = (Inst*)b->dmem;
+    b->dinst = b->dmem;
     b->dpre = (int*)(b->dmem + inst_bytes);
     b->nbase = (int*)(b->dmem + inst_bytes + pre_bytes);
+    b->result = (RunResult*)(b->dmem + inst_bytes + pre_bytes + 256);
     *out = b;
     return LKS_OK;
 }
 
 lks_status lks_batch_set_options(lks_batch* b, int use_graphs, int tile_fwd, int tile_adj) {
     if (!b) return LKS_ERR_ARG;
-    if (tile_fwd < -1 || tile_fwd >= kTileCfgs || tile_adj < -1 || tile_adj >= kAdjCfgs)
+    if (tile_fwd < -1 || tile_fwd >= kStripCfgs || tile_adj < -1 || tile_adj >= kStripCfgs)
         return bfail(b, LKS_ERR_ARG, "tile shape index out of range");
     b->use_graphs = use_graphs != 0;
     b->tile_req[0] = tile_fwd;
@@ -260,11 +264,11 @@ lks_status lks_batch_adjoint(lks_batch* b, double* const* dJdgamma, int on_devic
 
 int lks_batch_tile_shapes(int* txty, int cap) {
     if (cap < 0 || (!txty && cap > 0)) return -1;
-    for (int k = 0; k < kTileCfgs && k < cap; ++k) {
-        txty[2 * k] = tile_tx(k);
-        txty[2 * k + 1] = tile_ty(k);
+    for (int k = 0; k < kStripCfgs && k < cap; ++k) {
+        txty[2 * k] = kStripW;
+        txty[2 * k + 1] = strip_rows(k);
     }
-    return kTileCfgs;
+    return kStripCfgs;
 }
 
 lks_status lks_batch_tuning(const lks_batch* b, int* chosen2, float* ms) {
@@ -273,8 +277,8 @@ lks_status lks_batch_tuning(const lks_batch* b, int* chosen2, float* ms) {
     chosen2[1] = b->tile[1];
     if (ms)
         for (int w = 0; w < 2; ++w)
-            for (int k = 0; k < kTileCfgs; ++k)
-                ms[w * kTileCfgs + k] =
+            for (int k = 0; k < kStripCfgs; ++k)
+                ms[w * kStripCfgs + k] =
                     (b->tile_req[w] < 0 && b->tile[w] >= 0) ? b->tune_ms[w][k] : -1.f;
     return LKS_OK;
 }

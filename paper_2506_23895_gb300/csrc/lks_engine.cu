@@ -159,6 +159,7 @@ struct Layout {
     size_t off[96];
     size_t total;
     int ktape_slots;   // slots of the transfer tape (0: none)
+    int pos_slots;     // steps of design positions
     int pool_slots;
     size_t snap;
 };
@@ -166,13 +167,13 @@ struct Layout {
 enum {
     L_S0, L_S1, L_SINIT, L_L0, L_L1, L_F, L_MU, L_PHI, L_KUS, L_E, L_GAMMA, L_KREF, L_KPRIME,
     L_GACC, L_JSTEP, L_CBASE, L_CFRAC, L_ZTI, L_ZTW, L_TCNT, L_TIDX, L_TW, L_CM, L_DZB, L_DZF,
-    L_FLAGS, L_KREFT, L_K2, L_FACE, L_TGT, L_U3, L_MOTION, L_BUFS, L_INST, L_PRE, L_GBAR,
+    L_FLAGS, L_KREFT, L_K2, L_FACE, L_TGT, L_U3, L_MOTION, L_INST, L_PRE, L_GBAR,
     L_HP, L_FWS, L_GOUT, L_GTMP, L_SCAL, L_CSC, L_KS, L_SEND, L_LEND, L_GBASE, L_GFRAC,
     L_GCNT, L_GIDX,
     // the second transfer buffer set (3D): same sizes as L_KUS, L_K2, L_CBASE, ...
     L_KUS2, L_K22, L_CBASE2, L_CFRAC2, L_CSC2, L_ZTI2, L_ZTW2, L_TCNT2, L_TIDX2, L_TW2, L_CM2,
     L_DZB2, L_DZF2, L_GBASE2, L_GFRAC2, L_GCNT2, L_GIDX2, L_E2,
-    L_KTAPE, L_PB2, L_PSC2, L_POOL,
+    L_KTAPE, L_ETAPE, L_PB, L_PSC, L_JPART, L_POOL,
     L_COUNT
 };
 static_assert(L_COUNT <= 96, "Layout::off holds 96 regions");
@@ -227,8 +228,7 @@ Layout make_layout(const lks_config* cfg) {
     }
     sz[L_FLAGS] = 64;
     sz[L_MOTION] = (size_t)(cfg->max_steps + 1) * sizeof(Motion);
-    sz[L_BUFS] = (size_t)(BUF_POOL + P) * sizeof(void*);
-    sz[L_INST] = sizeof(Inst);
+    sz[L_INST] = std::max(sizeof(Inst<float>), sizeof(Inst<double>));
     sz[L_PRE] = (size_t)U_COUNT * 2 * sizeof(int);
     sz[L_GBAR] = sz[L_HP] = sz[L_FWS] = sz[L_GOUT] = sz[L_GTMP] = (size_t)std::max(nd, 1LL) * 8;
     sz[L_SCAL] = 64;
@@ -257,20 +257,23 @@ Layout make_layout(const lks_config* cfg) {
         for (int i = 0; i < 17; ++i) sz[L_KUS2 + i] = two ? sz[first[i]] : 0;
         sz[L_E2] = two ? sz[L_E] : 0;
     }
-    // FP32 2D contexts with a design keep the transfer (kappa, u_S on the footprint box) of each
-    // taped step, so that the adjoint of the step reads it instead of transferring again; a tape
-    // of up to max(ceil(sqrt(N)) + 2, 64) steps (the checkpointed schedules' tape length, and
-    // short full-history runs), each slot sized for the whole grid (the box is known only once
-    // the motion is set)
+    // 2D contexts on the table kernels form the transfers (kappa, u_S on the footprint box) of many
+    // steps in one launch and keep those of a taped segment for its adjoint: a tape of up to
+    // max(ceil(sqrt(N)) + 2, 64) steps (the checkpointed schedules' tape length, and short
+    // full-history runs), at least 16 where the pool is smaller, each slot sized for the whole grid
+    // (the box is known only once the motion is set); e of the same steps for the sensitivity
+    // gather, and the design positions of up to 32 steps
     {
-        const bool t2d = cfg->precision == LKS_FP32 && dim == 2 && nd > 0 &&
-                         !(cfg->flags & (LKS_FLAG_PLAIN_KERNELS | LKS_FLAG_PAPER_ALKS));
+        const bool table = dim == 2 && !(cfg->flags & (LKS_FLAG_PLAIN_KERNELS | LKS_FLAG_PAPER_ALKS));
+        const bool t2d = table && nd > 0;
         const long long kt = std::max((long long)std::ceil(std::sqrt((double)N)) + 2, 64LL);
-        L.ktape_slots = t2d ? (int)std::min(P, kt) : 0;
+        L.ktape_slots = t2d ? (int)std::min(N + 1, std::max(std::min(P, kt), 16LL)) : 0;
         sz[L_KTAPE] = (size_t)L.ktape_slots * state;
-        // design positions of the steps of odd parity (even: L_CBASE, L_CSC)
-        sz[L_PB2] = t2d ? (size_t)ncol * 8 : 0;
-        sz[L_PSC2] = t2d ? (size_t)ncol * 16 : 0;
+        sz[L_ETAPE] = (size_t)L.ktape_slots * (size_t)nodes * T;
+        L.pos_slots = std::min(L.ktape_slots, 32);
+        sz[L_PB] = (size_t)L.pos_slots * (size_t)ncol * 8;
+        sz[L_PSC] = (size_t)L.pos_slots * (size_t)ncol * 4 * T;
+        sz[L_JPART] = table ? (size_t)(cfg->max_steps + 2) * obj_parts(count_target(cfg)) * 8 : 0;
     }
     sz[L_POOL] = (size_t)P * state;
     size_t off = 0;
@@ -417,15 +420,16 @@ lks_status lks_create(const lks_config* cfg, void* workspace, size_t ws_bytes, l
     c->pool = w + L.off[L_POOL];
     c->pool_slots = L.pool_slots;
     c->snap_bytes = L.snap;
-    c->fused2d = (c->prec == LKS_FP32) && g.dim == 2 &&
-                 !(cfg->flags & (LKS_FLAG_PLAIN_KERNELS | LKS_FLAG_PAPER_ALKS));
+    c->fused2d = g.dim == 2 && !(cfg->flags & (LKS_FLAG_PLAIN_KERNELS | LKS_FLAG_PAPER_ALKS));
     c->ktape_slots = c->fused2d ? L.ktape_slots : 0;
     c->ktape = c->ktape_slots > 0 ? (void*)(w + L.off[L_KTAPE]) : nullptr;
-    c->pos2_b = w + L.off[L_PB2];
-    c->pos2_sc = (float4*)(w + L.off[L_PSC2]);
+    c->etape = w + L.off[L_ETAPE];
+    c->pos_b = w + L.off[L_PB];
+    c->pos_sc = w + L.off[L_PSC];
+    c->pos_slots = L.pos_slots;
+    c->jpart = (double*)(w + L.off[L_JPART]);
     c->dmotion = (Motion*)(w + L.off[L_MOTION]);
-    c->dbufs = (void**)(w + L.off[L_BUFS]);
-    c->dinst = (Inst*)(w + L.off[L_INST]);
+    c->dinst = w + L.off[L_INST];
     c->dpre = (int*)(w + L.off[L_PRE]);
     c->gbar = (double*)(w + L.off[L_GBAR]);
     c->hp = (double*)(w + L.off[L_HP]);
@@ -479,12 +483,11 @@ lks_status lks_create(const lks_config* cfg, void* workspace, size_t ws_bytes, l
     c->hbufs[BUF_INIT] = c->s0;
     c->hbufs[BUF_LAM0] = c->lam[0];
     c->hbufs[BUF_LAM1] = c->lam[1];
+    c->hbufs[BUF_SEND] = c->s_end;
+    c->hbufs[BUF_LEND] = c->l_end;
     for (int k = 0; k < c->pool_slots; ++k) c->hbufs[BUF_POOL + k] = slot_ptr(c, k);
     lks_status s = LKS_OK;
-    if (cudaMemcpy(c->dbufs, c->hbufs.data(), c->hbufs.size() * sizeof(void*),
-                   cudaMemcpyHostToDevice) != cudaSuccess)
-        s = LKS_ERR_CUDA;
-    if (s == LKS_OK && cudaMemsetAsync(c->flags, 0, 64, c->st) != cudaSuccess) s = LKS_ERR_CUDA;
+    if (cudaMemsetAsync(c->flags, 0, 64, c->st) != cudaSuccess) s = LKS_ERR_CUDA;
     if (s == LKS_OK) s = c->prec == LKS_FP64 ? reset_initial<double>(c) : reset_initial<float>(c);
     if (s != LKS_OK) {
         lks_destroy(c);
@@ -584,8 +587,8 @@ lks_status lks_set_static(lks_ctx* c, const double* kappa_s) {
         c->g.ks = c->ks;
     }
     if (c->fused2d && c->have_motion) {
-        std::vector<lks_ctx*> one(1, c);
-        CU(build_plan(one, c->dinst, c->dpre, c->nbase, c->st, c->plan));
+        const lks_status s = own_plan(c);
+        if (s != LKS_OK) return s;
     }
     ++c->geo_gen;
     return LKS_OK;
@@ -801,7 +804,7 @@ lks_status lks_transfer(lks_ctx* c, int step, double* kappa_out, double* us_out)
 }
 
 int lks_uses_fused(const lks_ctx* c) {
-    return !c ? 0 : ((c->fused3d && !c->g.ks) ? 1 : (c->fused2d ? 2 : 0));
+    return !c ? 0 : ((c->fused3d && !c->g.ks) ? 1 : (c->fused2d && c->prec == LKS_FP32 ? 2 : 0));
 }
 
 lks_status lks_step_variant(lks_ctx* c, int request, int* chosen) {

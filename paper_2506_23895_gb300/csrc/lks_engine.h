@@ -78,10 +78,15 @@ struct lks_ctx {
     char* pool;
     int pool_slots;
     size_t snap_bytes;
-    void* ktape = nullptr;       // transfer tape of the 2D table path (ktape_slots box records)
+    // 2D table path: kappa, u_S on the footprint box and e for ktape_slots steps, design
+    // positions (base, sin/cos table) for pos_slots steps, partial objective sums
+    void* ktape = nullptr;
+    void* etape = nullptr;
     int ktape_slots = 0;
-    void* pos2_b = nullptr;      // 2D table path: design positions of odd steps (int2 per column)
-    float4* pos2_sc = nullptr;   // and their sin, cos table
+    void* pos_b = nullptr;
+    void* pos_sc = nullptr;
+    int pos_slots = 0;
+    double* jpart = nullptr;
     // host state
     std::vector<double> motion;
     bool have_design = false, have_motion = false, fwd_valid = false;
@@ -97,17 +102,16 @@ struct lks_ctx {
     long long stats[5] = {0, 0, 0, 0, 0};
     const void* last = nullptr;  // buffer holding the newest forward level
     bool fused3d = false;        // FP32 3D non-periodic: one fused kernel per forward step
-    // instance table of this context (D2Q9 FP32: the table kernels of lks_fused2d.cu)
+    // instance table of this context (D2Q9: the table kernels of lks_fused2d.cu)
     bool fused2d = false;
     Motion* dmotion = nullptr;   // device motion rows
-    void** dbufs = nullptr;      // device buffer table (BUF_*)
-    std::vector<void*> hbufs;    // its host copy
-    Inst* dinst = nullptr;
+    std::vector<void*> hbufs;    // buffers by index (BUF_*)
+    void* dinst = nullptr;       // Inst<T>
     int* dpre = nullptr;         // device prefix arrays, U_COUNT x 2
-    int* nbase = nullptr;        // device step base of this context's own runs
+    int* nbase = nullptr;        // device: step base of this context's own runs, grid barrier
     Plan plan;
     int geo_gen = 0;             // bumped when the footprint box changes
-    int tile_fwd = 0, tile_adj = 0;   // tile shapes of the fused 2D kernels
+    int tile_fwd = 0, tile_adj = 0;   // strip heights of the fused 2D kernels
     bool gaxis = false;          // 3D rotation about an axis other than z
     int step3d_req = 1;          // fused 3D step variant requested (-1: time them once)
     int step3d_var = -1;         // variant in use (-1: not chosen yet)
@@ -218,6 +222,7 @@ struct Group {
     bool table = false;          // instance-table kernels
     const Plan* plan = nullptr;
     int* nbase = nullptr;
+    RunResult* result = nullptr;    // device, one per context
     int tile_fwd = 0, tile_adj = 0;
     GraphCache* graphs = nullptr;   // null: launch directly
     cudaStream_t st = nullptr;
@@ -233,7 +238,9 @@ lks_status transfer_join(lks_ctx* c);
 lks_status finish_motion(lks_ctx* c);
 lks_status design_prep(lks_ctx* c);
 const double* design_gradient(lks_ctx* c, cudaStream_t st);
-cudaError_t build_plan(const std::vector<lks_ctx*>& cs, Inst* dinst, int* dpre, int* nbase,
+lks_status own_plan(lks_ctx* c);
+template <class T>
+cudaError_t build_plan(const std::vector<lks_ctx*>& cs, void* dinst, int* dpre, int* nbase,
                        cudaStream_t st, Plan& p);
 template <class T>
 lks_status transfer_at(lks_ctx* c, int n);

@@ -1,21 +1,30 @@
-// D2Q9 FP32 kernels over instance tables (lks_table.h): every launch covers all instances of a
-// plan with a persistent grid that walks the concatenated work units.
+// D2Q9 kernels over instance tables (lks_table.h): every launch covers all instances of a plan.
 //
-//   k_t_design_pos  x_ref, y_ref of every design column (col_pos_sc), for a run's first step;
-//   k_t_transfer2d  kappa and u_S on every footprint-box node (transfer2d_node, Sec. 2.3), into
-//                   the box buffer or the transfer tape, and the next step's design positions;
-//   k_t_step2d      fused LKS step (Alg. 1; Sec. 2.2 f^eq with the viscosity term, Eqs. rho,
-//                   u, u_ex_2, bc_rho, bc_u) on TX x TY tiles: the state tile with a two-cell
-//                   halo goes to shared memory, f^eq of the tile and a one-cell rim is
-//                   evaluated once per node and direction, then gathered;
-//   k_t_objective   one block per instance inside the objective window (Sec. 2.5);
-//   k_t_adj2d       fused exact adjoint step (structure of Alg. 2, Eqs. arho, au, as): lambda
-//                   plus the transpose of the boundary copies, to mu (Brinkman transpose and
-//                   the kappa sensitivity density e), moments
-//                   of F~ on the tile and a one-cell rim, adjoint equilibrium and the full
+//   k_t_design_pos  x_ref, y_ref of every design node (Sec. 2.3) for a group of steps;
+//   k_t_transfer2d  kappa and u_S on every footprint-box node for a group of steps: the transfer
+//                   depends on the motion and the design only, so the transfers of many steps
+//                   are one launch with full grids instead of a short launch before each step;
+//   k_t_step        the LKS step (Alg. 1; Sec. 2.2 f^eq with the viscosity term, Eqs. rho, u,
+//                   u_ex_2, bc_rho, bc_u), any number of steps in one launch;
+//   k_t_adj         the exact adjoint step (structure of Alg. 2, Eqs. arho, au, as): lambda plus
+//                   the transpose of the boundary copies, to mu (Brinkman transpose and the kappa
+//                   sensitivity density e), moments of F~, adjoint equilibrium and the full
 //                   transposed velocity gradient including the one-sided boundary rows;
-//   k_t_sens        dJ/dgamma gather per design node (sens2d_node, Sec. 2.4).
+//   k_t_sens        dJ/dgamma gather per design node (Sec. 2.4) for a group of steps;
+//   k_t_objective   the objective of one level, in parts (Sec. 2.5);
+//   k_t_begin, k_t_end, k_t_result   what a run does once, over all instances.
+//
+// The two stencils march a warp up a strip of columns, lane = column.  What they need from the
+// rows below and above stays in registers, what they need from the columns beside comes by warp
+// shuffles, so a strip runs without shared memory, barriers or index arithmetic per node.  A
+// warp's 32 columns give 28 outputs (f^eq, or the adjoint's moments, need one column of halo and
+// the values they read one more).  The 32 x 8 tile kernels these replace spent 410 (step) and 418
+// (adjoint) instructions per node, over half of them on tile index arithmetic and shared-memory
+// traffic, and waited at four barriers.
 #include <cuda_runtime.h>
+
+#include <algorithm>
+#include <type_traits>
 
 #include "lks_table.h"
 #include "lks_units.cuh"
@@ -25,6 +34,101 @@ namespace lks {
 namespace {
 
 constexpr int NT = 256;
+constexpr int kSensThreads = 64;     // small blocks: a design has few nodes, each a long loop
+constexpr int kStripThreads = 256;   // at most eight strips (warps) per block
+constexpr unsigned FULL = 0xffffffffu;
+
+// Resident blocks of eight warps the strip kernels are compiled for.
+template <class T>
+constexpr int strip_minb() {
+    return sizeof(T) == 4 ? 2 : 1;
+}
+
+// Loads of a node record through L2 (another SM may have written it earlier in the same launch)
+// and through the read-only path.
+__device__ __forceinline__ V4<float> ldcg4(const V4<float>* p) {
+    const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
+    return V4<float>{v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ V4<double> ldcg4(const V4<double>* p) {
+    const double2 a = __ldcg(reinterpret_cast<const double2*>(p));
+    const double2 b = __ldcg(reinterpret_cast<const double2*>(p) + 1);
+    return V4<double>{a.x, a.y, b.x, b.y};
+}
+template <class V>
+__device__ __forceinline__ V ldcg3(const V4<float>* p) {
+    const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
+    return V{v.x, v.y, v.z};
+}
+template <class V>
+__device__ __forceinline__ V ldcg3(const V4<double>* p) {
+    const double2 a = __ldcg(reinterpret_cast<const double2*>(p));
+    return V{a.x, a.y, __ldcg(reinterpret_cast<const double*>(p) + 2)};
+}
+template <class V>
+__device__ __forceinline__ V ldg3(const V4<float>* p) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+    return V{v.x, v.y, v.z};
+}
+template <class V>
+__device__ __forceinline__ V ldg3(const V4<double>* p) {
+    const double2 a = __ldg(reinterpret_cast<const double2*>(p));
+    return V{a.x, a.y, __ldg(reinterpret_cast<const double*>(p) + 2)};
+}
+
+// A record from shared memory and to global memory as whole vectors (the pointers come from memory,
+// so the compiler does not know their space, and it would split the struct).
+__device__ __forceinline__ V4<float> lds4(const V4<float>* p) {
+    V4<float> v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.r), "=f"(v.x), "=f"(v.y), "=f"(v.z)
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+    return v;
+}
+__device__ __forceinline__ V4<double> lds4(const V4<double>* p) {
+    V4<double> v;
+    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+    asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.r), "=d"(v.x) : "r"(a));
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v.y) : "r"(a + 16));
+    v.z = 0.0;
+    return v;
+}
+__device__ __forceinline__ void stg4(V4<float>* p, const V4<float>& v) {
+    asm volatile("st.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.r), "f"(v.x),
+                 "f"(v.y), "f"(v.z)
+                 : "memory");
+}
+__device__ __forceinline__ void stg4(V4<double>* p, const V4<double>& v) {
+    asm volatile("st.global.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(v.r), "d"(v.x) : "memory");
+    asm volatile("st.global.v2.f64 [%0], {%1, %2};" ::"l"(reinterpret_cast<char*>(p) + 16),
+                 "d"(v.y), "d"(v.z)
+                 : "memory");
+}
+// One record of V4<T> from global to shared memory, asynchronously and through L2: skipped unless
+// `go`, zeros instead of the record unless `in`; and the groups such copies are counted in.
+template <class T>
+__device__ __forceinline__ void cp_record(V4<T>* dst, const V4<T>* src, bool go, bool in) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int bytes = in ? 16 : 0;
+#pragma unroll
+    for (int o = 0; o < (int)sizeof(V4<T>); o += 16)
+        asm volatile(
+            "{ .reg .pred p; setp.ne.s32 p, %3, 0;"
+            " @p cp.async.cg.shared.global [%0], [%1], 16, %2; }" ::"r"(d + o),
+            "l"(reinterpret_cast<const char*>(src) + o), "r"(bytes), "r"((int)go)
+            : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+__device__ __forceinline__ int ld_acquire(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 
 // Instance of work unit u: the last i with pre[i] <= u (pre has count + 1 entries).
 __device__ __forceinline__ int find_inst(const int* __restrict__ pre, int count, int u) {
@@ -42,93 +146,77 @@ __device__ __forceinline__ int wrap_any(int i, int n) {
     return i < 0 ? i + n : i;
 }
 
-__device__ __forceinline__ int step_of(const Plan& p, int noff) { return __ldg(p.nbase) + noff; }
-
-// Stage instance i's record in shared memory when the block moves to it: kernels then read the
-// geometry from shared memory, which their global stores cannot alias, instead of reloading it
-// from global memory after every store.  Called by all threads; ends with a barrier when it
-// copies.
-// kslot >= 0 points the staged record's kus at slot kslot of the instance's transfer tape.
-__device__ __forceinline__ void stage_inst(const Plan& p, int i, int& cur, Inst& sI,
-                                          int kslot = -1) {
-    if (i == cur) return;
-    __syncthreads();
-    const int* src = reinterpret_cast<const int*>(p.tab + i);
-    int* dst = reinterpret_cast<int*>(&sI);
-    for (int k = threadIdx.x; k < (int)(sizeof(Inst) / 4); k += blockDim.x) dst[k] = __ldg(src + k);
-    __syncthreads();
-    if (kslot >= 0) {
-        if (threadIdx.x == 0) sI.kus = sI.kus_tape + (long long)kslot * sI.g.boxN;
-        __syncthreads();
-    }
-    cur = i;
+template <class T>
+__device__ __forceinline__ const Inst<T>* table(const Plan& p) {
+    return (const Inst<T>*)p.tab;
 }
 
-// kappa, u_S records of a launch: the box buffer or slot kslot of the transfer tape (a taped
-// forward step writes its transfer there; the adjoint of that step reads it back).
-__device__ __forceinline__ V4<float>* kus_slot(const Inst& I, int kslot) {
-    return kslot < 0 ? I.kus : I.kus_tape + (long long)kslot * I.g.boxN;
+template <class T>
+__device__ __forceinline__ V4<T>* buf(const Inst<T>& I, int b) {
+    return b < BUF_POOL ? (V4<T>*)I.bufs[b]
+                        : (V4<T>*)(I.pool + (long long)(b - BUF_POOL) * I.snap);
 }
 
-// ---------------------------------------------------------------- element-wise phases
+// ---------------------------------------------------------------- transfer
 
-// Design positions of step n (unit u of the design-column units) into the set of n's parity.
-__device__ __forceinline__ void design_pos_unit(const Plan& p, int u, int n) {
+// Design positions of steps n0 .. n0 + n - 1 into position slots 0 .. n - 1.
+template <class T>
+__global__ void __launch_bounds__(NT) k_t_design_pos(Plan p, int noff, int n) {
     const int* pre = p.pre + U_DCOL * (p.count + 1);
-    const int i = find_inst(pre, p.count, u);
-    const Inst& I = p.tab[i];
-    const long long k = (long long)(u - pre[i]) * kUnitThreads + threadIdx.x;
-    if (k >= I.d.ncol) return;
-    int2 b;
-    float4 sc;
-    col_pos_sc(I.d, I.motion[n], k, b, sc);
-    I.pos_b[n & 1][k] = b;
-    I.pos_sc[n & 1][k] = sc;
+    const int n0 = __ldg(p.nbase) + noff, total = p.total[U_DCOL];
+    for (int w = blockIdx.x; w < total * n; w += gridDim.x) {
+        const int s = w / total, u = w - s * total;
+        const int i = find_inst(pre, p.count, u);
+        const Inst<T>& I = table<T>(p)[i];
+        const long long k = (long long)(u - pre[i]) * kUnitThreads + threadIdx.x;
+        if (k >= I.d.ncol) continue;
+        int2 b;
+        V4<T> sc;
+        col_pos_sc<T>(I.d, I.motion[n0 + s], k, b, sc);
+        I.pos_b[s * I.d.ncol + k] = b;
+        I.pos_sc[s * I.d.ncol + k] = sc;
+    }
 }
 
-__global__ void __launch_bounds__(NT) k_t_design_pos(Plan p, int noff) {
-    const int n = step_of(p, noff);
-    for (int u = blockIdx.x; u < p.total[U_DCOL]; u += gridDim.x) design_pos_unit(p, u, n);
-}
-
-// One 16 x 16 tile of the footprint box per work unit.  The design nodes any node of the tile can
-// reach (the tile's inverse rigid image widened by the kernel radius: at most 30 x 30 nodes) are
-// staged in shared memory with contiguous reads and binned by their integer base into a table of
-// cells; every node then visits the 4 x 4 cells whose taps cover it, so that it touches only the
-// design nodes in its support (about 16, against some 36 window candidates).  A tile whose table
-// overflows runs the candidate loop of transfer2d_node on the staged copy instead.
+// One 16 x 16 tile of the footprint box of one step per work unit.  The design nodes any node of
+// the tile can reach (the tile's inverse rigid image widened by the kernel radius: at most 30 x 30
+// nodes) are staged in shared memory with contiguous reads and binned by their integer base into a
+// table of cells; every node then visits the 4 x 4 cells whose taps cover it, so that it touches
+// only the design nodes in its support (about 16, against some 36 window candidates).  A tile whose
+// table overflows, or whose window is wider than the staging area, scans the candidate window.
 constexpr int kTrWin = 32;   // staged window side (design nodes)
 static_assert(kBoxTile * kBoxTile == NT, "one box tile per block of NT threads");
 // Cells of the tile's design-node table: the integer bases b that can reach a node of the tile
 // (b in [x - 2, x + 1] per axis), kTrCells per axis; a unit-spaced rotated lattice puts at most
-// two design nodes in one unit cell, kTrCap leaves room (a fuller cell sends the tile back to the
-// candidate loop).
+// two design nodes in one unit cell, kTrCap leaves room.
 constexpr int kTrCells = kBoxTile + 3, kTrCap = 4;
 
-// With next, the units past the box tiles form the design positions of step n + 1 (the next
-// transfer's), into the other parity's set.
-__global__ void __launch_bounds__(NT, 5) k_t_transfer2d(Plan p, int noff, int kslot, int next) {
-    __shared__ int2 sb[kTrWin * kTrWin];
-    __shared__ float4 ssc[kTrWin * kTrWin];
-    __shared__ float skr[kTrWin * kTrWin];
-    __shared__ int swin[4];
-    __shared__ int scnt[kTrCells * kTrCells];
-    __shared__ unsigned short sent[kTrCells * kTrCells * kTrCap];
-    __shared__ int sfull;
+template <class T>
+struct TrSmem {
+    V4<T> sc[kTrWin * kTrWin];
+    T kr[kTrWin * kTrWin];
+    int cnt[kTrCells * kTrCells];
+    int win[4];
+    int full;
+    unsigned short ent[kTrCells * kTrCells * kTrCap];
+};
+
+template <class T>
+__global__ void __launch_bounds__(NT) k_t_transfer2d(Plan p, int noff, int nsteps, int kslot0) {
+    extern __shared__ __align__(32) unsigned char smem_raw[];
+    TrSmem<T>& S = *reinterpret_cast<TrSmem<T>*>(smem_raw);
     const int* pre = p.pre + U_BOX * (p.count + 1);
-    const int n = step_of(p, noff);
-    const int nbox = p.total[U_BOX];
-    const int nall = nbox + (next ? p.total[U_DCOL] : 0);
-    for (int u = blockIdx.x; u < nall; u += gridDim.x) {
-        if (u >= nbox) {   // block-uniform: no barrier follows in this iteration
-            design_pos_unit(p, u - nbox, n + 1);
-            continue;
-        }
+    const int n0 = __ldg(p.nbase) + noff, nbox = p.total[U_BOX];
+    for (int w = blockIdx.x; w < nbox * nsteps; w += gridDim.x) {
+        const int step = w / nbox, u = w - step * nbox;
         const int i = find_inst(pre, p.count, u);
-        const Inst& I = p.tab[i];
+        const Inst<T>& I = table<T>(p)[i];
         const Design& d = I.d;
         const Geom& g = I.g;
-        const Motion& m = I.motion[n];
+        const Motion& m = I.motion[n0 + step];
+        const int2* __restrict__ pb = I.pos_b + (long long)step * d.ncol;
+        const V4<T>* __restrict__ psc = I.pos_sc + (long long)step * d.ncol;
+        V4<T>* kus = kslot0 < 0 ? I.kus : I.kus_tape + (long long)(kslot0 + step) * g.boxN;
         const int ntx = (g.bn[0] + kBoxTile - 1) / kBoxTile;
         const int t = u - pre[i];
         const int bx0 = (t % ntx) * kBoxTile, by0 = (t / ntx) * kBoxTile;
@@ -136,9 +224,10 @@ __global__ void __launch_bounds__(NT, 5) k_t_transfer2d(Plan p, int noff, int ks
         const int bx = bx0 + lx, by = by0 + ly;
         const bool node = bx < g.bn[0] && by < g.bn[1];
         const int x = g.blo[0] + bx, y = g.blo[1] + by;
+        // this node's candidate window, through the inverse rigid map in single precision with a
+        // margin far above its rounding (it only has to contain the support)
         const float c = m.cf, s = m.sf;
         const float R = 2.f * (fabsf(c) + fabsf(s)) + 0.01f;
-        // this node's candidate window (the same expressions as transfer2d_node)
         const float px = (float)x - m.xgf[0], py = (float)y - m.xgf[1];
         const float ic = c * px + s * py + d.xiGf[0];
         const float jc = -s * px + c * py + d.xiGf[1];
@@ -146,51 +235,66 @@ __global__ void __launch_bounds__(NT, 5) k_t_transfer2d(Plan p, int noff, int ks
         const int j0 = max(0, (int)ceilf(jc - R)), j1 = min(d.L[1] - 1, (int)floorf(jc + R));
         __syncthreads();   // the previous unit's staged window is no longer read
         if (threadIdx.x == 0) {
-            swin[0] = 1 << 30;
-            swin[1] = -(1 << 30);
-            swin[2] = 1 << 30;
-            swin[3] = -(1 << 30);
-            sfull = 0;
+            S.win[0] = 1 << 30;
+            S.win[1] = -(1 << 30);
+            S.win[2] = 1 << 30;
+            S.win[3] = -(1 << 30);
+            S.full = 0;
         }
-        for (int e = threadIdx.x; e < kTrCells * kTrCells; e += NT) scnt[e] = 0;
+        for (int e = threadIdx.x; e < kTrCells * kTrCells; e += NT) S.cnt[e] = 0;
         __syncthreads();
-        if (node && i0 <= i1 && j0 <= j1) {
-            atomicMin(&swin[0], i0);
-            atomicMax(&swin[1], i1);
-            atomicMin(&swin[2], j0);
-            atomicMax(&swin[3], j1);
+        {   // the tile's window: warp minima and maxima first, then one atomic per warp
+            const bool any = node && i0 <= i1 && j0 <= j1;
+            const int a0 = __reduce_min_sync(FULL, any ? i0 : (1 << 30));
+            const int a1 = __reduce_max_sync(FULL, any ? i1 : -(1 << 30));
+            const int b0 = __reduce_min_sync(FULL, any ? j0 : (1 << 30));
+            const int b1 = __reduce_max_sync(FULL, any ? j1 : -(1 << 30));
+            if ((threadIdx.x & 31) == 0 && a0 <= a1) {
+                atomicMin(&S.win[0], a0);
+                atomicMax(&S.win[1], a1);
+                atomicMin(&S.win[2], b0);
+                atomicMax(&S.win[3], b1);
+            }
         }
         __syncthreads();
-        const int wi0 = swin[0], wj0 = swin[2];
-        const int wni = swin[1] - wi0 + 1, wnj = swin[3] - wj0 + 1;
+        const int wi0 = S.win[0], wj0 = S.win[2];
+        const bool none = S.win[1] < wi0;
+        const int wni = S.win[1] - wi0 + 1, wnj = S.win[3] - wj0 + 1;
+        const long long bi = (long long)by * g.bn[0] + bx;
+        if (none) {   // no design node reaches the tile (block-uniform)
+            V4<T> o;
+            o.r = o.x = o.y = o.z = (T)0;
+            if (node) kus[bi] = o;
+            continue;
+        }
         const bool staged = wni <= kTrWin && wnj <= kTrWin;
         // the tile's first analysis node less 2: the lowest base whose taps reach the tile
         const int cx0 = g.blo[0] + bx0 - 2, cy0 = g.blo[1] + by0 - 2;
-        if (staged && wni > 0 && wnj > 0) {
-            const int2* base = I.pos_b[n & 1];
-            for (int e = threadIdx.x; e < wni * wnj; e += NT) {
-                const int jj = e / wni, ii = e - jj * wni;
-                const int k = (wj0 + jj) * d.L[0] + wi0 + ii;
-                const int2 bk = __ldg(base + k);
-                sb[jj * kTrWin + ii] = bk;
-                ssc[jj * kTrWin + ii] = __ldg(I.pos_sc[n & 1] + k);
-                skr[jj * kTrWin + ii] = __ldg(I.kref + k);
+        if (staged) {
+            const int li = threadIdx.x & 31;   // 32 lanes along i, 8 rows of j at a time
+            for (int jj = threadIdx.x >> 5; jj < wnj; jj += NT / 32) {
+                if (li >= wni) continue;
+                const int k = (wj0 + jj) * d.L[0] + wi0 + li, e = jj * kTrWin + li;
+                const int2 bk = __ldg(pb + k);
+                S.sc[e] = psc[k];
+                S.kr[e] = I.kref[k];
                 const int cx = bk.x - cx0, cy = bk.y - cy0;
                 if ((unsigned)cx < (unsigned)kTrCells && (unsigned)cy < (unsigned)kTrCells) {
                     const int cell = cy * kTrCells + cx;
-                    const int slot = atomicAdd(&scnt[cell], 1);
-                    if (slot < kTrCap) sent[cell * kTrCap + slot] = (unsigned short)(jj * kTrWin + ii);
-                    else sfull = 1;
+                    const int slot = atomicAdd(&S.cnt[cell], 1);
+                    if (slot < kTrCap) S.ent[cell * kTrCap + slot] = (unsigned short)e;
+                    else S.full = 1;
                 }
             }
         }
         __syncthreads();
         // each cell's design nodes in design index order (the staging order of the slots is not
         // fixed)
-        if (staged && !sfull) {
+        const bool cells = staged && !S.full;
+        if (cells) {
             for (int cell = threadIdx.x; cell < kTrCells * kTrCells; cell += NT) {
-                const int cnt = scnt[cell];
-                unsigned short* ent = sent + cell * kTrCap;
+                const int cnt = S.cnt[cell];
+                unsigned short* ent = S.ent + cell * kTrCap;
                 for (int a1 = 1; a1 < cnt; ++a1)
                     for (int a2 = a1; a2 > 0 && ent[a2 - 1] > ent[a2]; --a2) {
                         const unsigned short tmp = ent[a2];
@@ -201,15 +305,9 @@ __global__ void __launch_bounds__(NT, 5) k_t_transfer2d(Plan p, int noff, int ks
         }
         __syncthreads();
         if (!node) continue;
-        const long long bi = (long long)by * g.bn[0] + bx;
-        if (!staged) {   // a window wider than the staging area: the global-memory path
-            transfer2d_node(d, g, m, I.pos_b[n & 1], I.pos_sc[n & 1], I.kref, kus_slot(I, kslot),
-                            bi);
-            continue;
-        }
-        const float gx0 = d.xiGf[0], gy0 = d.xiGf[1];
-        float kap = 0.f, m0 = 0.f, m1x = 0.f, m1y = 0.f;
-        if (!sfull) {
+        const T gx0 = (T)d.xiG[0] - (T)wi0, gy0 = (T)d.xiG[1] - (T)wj0;
+        T kap = (T)0, m0 = (T)0, m1x = (T)0, m1y = (T)0;
+        if (cells) {
             // the design nodes whose base b reaches (x, y): b = (x, y) + 1 - (qx, qy), qx, qy in
             // 0..3, visited by tap (qy, qx) and then in design index order within a cell
             const int ccx = x - cx0 + 1, ccy = y - cy0 + 1;
@@ -218,786 +316,924 @@ __global__ void __launch_bounds__(NT, 5) k_t_transfer2d(Plan p, int noff, int ks
 #pragma unroll
                 for (int qx = 0; qx < 4; ++qx) {
                     const int cell = (ccy - qy) * kTrCells + (ccx - qx);
-                    const int cnt = scnt[cell];
+                    const int cnt = S.cnt[cell];
                     for (int a1 = 0; a1 < cnt; ++a1) {
-                        const int sk = sent[cell * kTrCap + a1];
-                        const float4 sc = ssc[sk];
-                        const float W = tap_weight(qx, sc.x, sc.y) * tap_weight(qy, sc.z, sc.w);
-                        kap += W * skr[sk];
+                        const int sk = S.ent[cell * kTrCap + a1];
+                        const V4<T> sc = S.sc[sk];
+                        const T W = tap_weight<T>(qx, sc.r, sc.x) * tap_weight<T>(qy, sc.y, sc.z);
+                        kap += W * S.kr[sk];
                         m0 += W;
-                        m1x += W * ((float)(wi0 + (sk & (kTrWin - 1))) - gx0);
-                        m1y += W * ((float)(wj0 + (sk / kTrWin)) - gy0);
+                        m1x += W * ((T)(sk & (kTrWin - 1)) - gx0);
+                        m1y += W * ((T)(sk / kTrWin) - gy0);
                     }
                 }
         } else {
             for (int j = j0; j <= j1; ++j)
                 for (int ii = i0; ii <= i1; ++ii) {
-                    const int sk = (j - wj0) * kTrWin + (ii - wi0);
-                    const int2 b = sb[sk];
+                    const int k = j * d.L[0] + ii;
+                    const int2 b = __ldg(pb + k);
                     const int qx = x - b.x + 1, qy = y - b.y + 1;
                     if ((unsigned)qx > 3u || (unsigned)qy > 3u) continue;
-                    const float4 sc = ssc[sk];
-                    const float W = tap_weight(qx, sc.x, sc.y) * tap_weight(qy, sc.z, sc.w);
-                    kap += W * skr[sk];
+                    const V4<T> sc = psc[k];
+                    const T W = tap_weight<T>(qx, sc.r, sc.x) * tap_weight<T>(qy, sc.y, sc.z);
+                    kap += W * I.kref[k];
                     m0 += W;
-                    m1x += W * ((float)ii - gx0);
-                    m1y += W * ((float)j - gy0);
+                    m1x += W * ((T)(ii - wi0) - gx0);
+                    m1y += W * ((T)(j - wj0) - gy0);
                 }
         }
-        const float om = m.omf;
-        V4<float> o;
+        const bool f32 = sizeof(T) == 4;
+        const T om = f32 ? (T)m.omf : (T)m.om, cT = f32 ? (T)m.cf : (T)m.c,
+                sT = f32 ? (T)m.sf : (T)m.s;
+        const T ug0 = f32 ? (T)m.ugf[0] : (T)m.uG[0], ug1 = f32 ? (T)m.ugf[1] : (T)m.uG[1];
+        V4<T> o;
         o.r = kap;
-        o.x = (-s * m1x - c * m1y) * om + m.ugf[0] * m0;
-        o.y = (c * m1x - s * m1y) * om + m.ugf[1] * m0;
-        o.z = 0.f;
-        kus_slot(I, kslot)[bi] = o;
+        o.x = (-sT * m1x - cT * m1y) * om + ug0 * m0;
+        o.y = (cT * m1x - sT * m1y) * om + ug1 * m0;
+        o.z = (T)0;
+        kus[bi] = o;
     }
 }
 
-__global__ void __launch_bounds__(kObjThreads) k_t_objective(Plan p, int noff, int src) {
-    const int n = step_of(p, noff);
-    for (int i = blockIdx.x; i < p.count; i += gridDim.x) {
-        const Inst& I = p.tab[i];
-        if (n < I.win_begin || n > I.win_end) continue;   // uniform over the block
-        objective_block<float>(I.g, (const V4<float>*)I.bufs[src], I.jstep + n);
-    }
-}
-
-__global__ void __launch_bounds__(NT) k_t_sens(Plan p, int noff) {
+// Sensitivity gather of steps noff + n - 1 down to noff: one thread per design node sums its
+// 4 x 4 taps of every step's e, and adds kappa' times each sum to dJ/dgamma in step order (FP64).
+template <class T>
+__global__ void __launch_bounds__(kSensThreads) k_t_sens(Plan p, int noff, int nsteps, int eslot0) {
     const int* pre = p.pre + U_DCOL * (p.count + 1);
-    const int n = step_of(p, noff);
-    for (int u = blockIdx.x; u < p.total[U_DCOL]; u += gridDim.x) {
+    const int n0 = __ldg(p.nbase) + noff;
+    constexpr int SUB = kUnitThreads / kSensThreads;
+    for (int w = blockIdx.x; w < p.total[U_DCOL] * SUB; w += gridDim.x) {
+        const int u = w / SUB;
         const int i = find_inst(pre, p.count, u);
-        const Inst& I = p.tab[i];
-        const long long k = (long long)(u - pre[i]) * kUnitThreads + threadIdx.x;
-        if (k < I.d.ncol) sens2d_node(I.d, I.g, I.motion[n], I.e, I.kprime, I.gacc, k);
+        const Inst<T>& I = table<T>(p)[i];
+        const long long k = (long long)(u - pre[i]) * kUnitThreads + (w % SUB) * kSensThreads +
+                            threadIdx.x;
+        if (k >= I.d.ncol) continue;
+        const double kp = (double)I.kprime[k];
+        double acc = I.gacc[k];
+#pragma unroll 2
+        for (int s = nsteps - 1; s >= 0; --s)
+            acc += kp * (double)sens2d_sum<T>(I.d, I.g, I.motion[n0 + s],
+                                              I.e + (long long)(eslot0 + s) * I.g.boxN, k);
+        I.gacc[k] = acc;
     }
+}
+
+// ---------------------------------------------------------------- objective (Sec. 2.5)
+
+// Partial sum `part` of the objective over the target list at one level, by one warp: FP64, fixed
+// order.
+template <class T>
+__device__ __forceinline__ void objective_part(const Inst<T>& I, const V4<T>* s, int n, int part,
+                                               int lane) {
+    const Geom& g = I.g;
+    const int tot = (int)g.ocount, np = I.jparts;
+    const int per = (tot + np - 1) / np, k1 = min(tot, (part + 1) * per);
+    double acc = 0.0;
+#pragma unroll 4
+    for (int k = part * per + lane; k < k1; k += 32) {
+        const V4<T> v = ldcg4(s + g.otarget[k]);
+        acc += g.okind == 0 ? (double)v.r : g.odir[0] * (double)v.x + g.odir[1] * (double)v.y;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+    if (lane == 0) I.jpart[(long long)n * np + part] = acc;
+}
+
+// Unit u of the objective units: instance and part, skipped outside the window.
+template <class T>
+__device__ __forceinline__ void objective_unit(const Plan& p, int u, int n, int b, int lane) {
+    const int* pre = p.pre + U_OBJ * (p.count + 1);
+    const int i = find_inst(pre, p.count, u);
+    const Inst<T>& I = table<T>(p)[i];
+    if (n < I.win_begin || n > I.win_end) return;   // uniform over the warp
+    objective_part<T>(I, buf(I, b), n, u - pre[i], lane);
+}
+
+template <class T>
+__global__ void __launch_bounds__(NT) k_t_objective(Plan p, int noff, int b) {
+    const int u = blockIdx.x * (NT / 32) + threadIdx.x / 32;
+    if (u < p.total[U_OBJ])
+        objective_unit<T>(p, u, __ldg(p.nbase) + noff, b, threadIdx.x & 31);
+}
+
+// Start of a run: the error words, and for an adjoint run lambda^N and dJ/dgamma, to zero.
+template <class T>
+__global__ void __launch_bounds__(NT) k_t_begin(Plan p, int adjoint) {
+    const Inst<T>& I = table<T>(p)[blockIdx.y];
+    const int t = blockIdx.x * NT + threadIdx.x, nt = gridDim.x * NT;
+    if (t < 4) I.flags[t] = 0;
+    if (!adjoint) return;
+    uint4* l = (uint4*)buf(I, BUF_LAM0);
+    const int n = (int)(I.g.nodes * (sizeof(V4<T>) / 16));
+    for (int k = t; k < n; k += nt) l[k] = make_uint4(0u, 0u, 0u, 0u);
+    for (long long k = t; k < I.d.nd; k += nt) I.gacc[k] = 0.0;
+}
+
+// End of a run: buffer src to dst, and on a forward run the divergence check of that state.
+template <class T>
+__global__ void __launch_bounds__(NT) k_t_end(Plan p, int dst, int src, int check) {
+    const Inst<T>& I = table<T>(p)[blockIdx.y];
+    const V4<T>* a = buf(I, src);
+    V4<T>* b = buf(I, dst);
+    const int n = (int)I.g.nodes;
+    for (int k = blockIdx.x * NT + threadIdx.x; k < n; k += gridDim.x * NT) {
+        const V4<T> v = a[k];
+        b[k] = v;
+        const T m = fabs(v.x) + fabs(v.y) + fabs(v.z);
+        if (check && (!(m < (T)0.5) || !(fabs(v.r) < (T)1e30))) atomicOr(I.flags + 2, 1);
+    }
+}
+
+// Per instance: j = -(rho0 + mean(rho - rho0))/3 (J1) or -mean(n.u) (J2) of every step of the
+// window up to n_last from the parts, J = h sum_n j_n (fixed order), and the error words.
+template <class T>
+__global__ void __launch_bounds__(NT) k_t_result(Plan p, int n_last, int adjoint, RunResult* out) {
+    const Inst<T>& I = table<T>(p)[blockIdx.x];
+    __shared__ double red[NT];
+    double acc = 0.0;
+    if (!adjoint) {
+        const int w1 = min(I.win_end, n_last);
+        const double h = 1.0 / (double)(I.win_end - I.win_begin + 1);
+        for (int n = I.win_begin + threadIdx.x; n <= w1; n += NT) {
+            double sum = 0.0;
+            for (int q = 0; q < I.jparts; ++q) sum += I.jpart[(long long)n * I.jparts + q];
+            acc += h * (I.g.okind == 0 ? -(I.g.rho0 + sum / I.g.ocount) / 3.0 : -sum / I.g.ocount);
+        }
+    }
+    red[threadIdx.x] = acc;
+    __syncthreads();
+    for (int w = NT / 2; w > 0; w >>= 1) {
+        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) out[blockIdx.x].J = red[0];
+    if (threadIdx.x < 4) out[blockIdx.x].flags[threadIdx.x] = I.flags[threadIdx.x];
 }
 
 __global__ void k_set_int(int* dst, int v) { *dst = v; }
 
-// deriv_coef in single precision (same rows: central, periodic, one-sided on boundary nodes).
-__device__ __forceinline__ float deriv_coef_f(int i, int n, int periodic, int off) {
-    if (periodic || (i > 0 && i < n - 1)) return off == 1 ? 0.5f : (off == -1 ? -0.5f : 0.f);
-    if (i == 0) return off == 0 ? -1.5f : (off == 1 ? 2.f : (off == 2 ? -0.5f : 0.f));
-    return off == 0 ? 1.5f : (off == -1 ? -2.f : (off == -2 ? 0.5f : 0.f));
+// Buffer src of every instance to its buffer dst (whole records of 16 bytes).
+template <class T>
+__global__ void __launch_bounds__(NT) k_t_copy(Plan p, int dst, int src) {
+    const Inst<T>& I = table<T>(p)[blockIdx.y];
+    const uint4* a = (const uint4*)buf(I, src);
+    uint4* b = (uint4*)buf(I, dst);
+    const int n = (int)(I.g.nodes * (sizeof(V4<T>) / 16));
+    for (int k = blockIdx.x * NT + threadIdx.x; k < n; k += gridDim.x * NT) b[k] = a[k];
 }
 
-// ---------------------------------------------------------------- fused forward step
+// ---------------------------------------------------------------- strips
 
-// Tile position of unit `local` of an instance for tiles TX x TY.
-template <int TX, int TY>
-__device__ __forceinline__ void tile_xy(const Geom& g, int local, int& x0, int& y0) {
-    const int ntx = tile_count(g.n[0], TX, g.periodic[0]);
-    const int ky = local / ntx, kx = local - ky * ntx;
-    x0 = kx * TX - tile_origin(g.n[0], TX, g.periodic[0]);
-    y0 = ky * TY - tile_origin(g.n[1], TY, g.periodic[1]);
+// All blocks of a cooperative launch meet for the `round`-th time (1, 2, ...): *bar counts arrivals
+// from zero, so that one release and the polling of one word do (an arrival count that the last
+// block turns into a generation costs a second trip to L2: 3.0 us a meeting against 2.0).  The wait
+// is bounded (about a second); a block that gives up sets the error word and returns false, and so
+// do the others after it.
+__device__ __forceinline__ bool grid_meet(const Plan& p, int nblocks, int round) {
+    __shared__ int ok;
+    __syncthreads();
+    if (nblocks == 1) return true;
+    if (threadIdx.x == 0) {
+        int good = 1;
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.bar) : "memory");
+        const int want = nblocks * round;
+        const long long t0 = clock64();
+        while (ld_acquire(p.bar) < want)
+            if (clock64() - t0 > (1LL << 31)) {
+                atomicOr(p.err, 8);
+                good = 0;
+                break;
+            }
+        ok = good;
+    }
+    __syncthreads();
+    return ok != 0;
 }
 
-// Load a (TY+4) x (TX+4) tile of float4 node records starting at (x0-2, y0-2): periodic axes
-// wrap, positions outside a non-periodic axis read as zero.
-template <int TX, int TY>
-__device__ __forceinline__ void load_tile(const Geom& g, const float4* __restrict__ src, int x0,
-                                          int y0, float4* S) {
-    constexpr int HX = TX + 4, HY = TY + 4;
+// The arithmetic below is written with explicitly rounded operations, which the compiler neither
+// contracts nor reorders: every strip height then computes bitwise the same state.
+template <class T>
+__device__ __forceinline__ T fma_(T a, T b, T c);
+template <>
+__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+template <>
+__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
+template <class T>
+__device__ __forceinline__ T mul_(T a, T b);
+template <>
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+template <>
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+template <class T>
+__device__ __forceinline__ T add_(T a, T b);
+template <>
+__device__ __forceinline__ float add_(float a, float b) { return __fadd_rn(a, b); }
+template <>
+__device__ __forceinline__ double add_(double a, double b) { return __dadd_rn(a, b); }
+template <class T>
+__device__ __forceinline__ T sub_(T a, T b);
+template <>
+__device__ __forceinline__ float sub_(float a, float b) { return __fsub_rn(a, b); }
+template <>
+__device__ __forceinline__ double sub_(double a, double b) { return __dsub_rn(a, b); }
+template <class T>
+__device__ __forceinline__ T inv_(T a);
+template <>
+__device__ __forceinline__ float inv_(float a) { return __frcp_rn(a); }
+template <>
+__device__ __forceinline__ double inv_(double a) { return __drcp_rn(a); }
+
+template <class T>
+__device__ __forceinline__ T from_left(T v) { return __shfl_up_sync(FULL, v, 1); }
+template <class T>
+__device__ __forceinline__ T from_right(T v) { return __shfl_down_sync(FULL, v, 1); }
+
+template <class T>
+struct V3 {
+    T r, x, y;
+};
+
+// Geometry of a strip as its lane sees it.
+struct Strip {
+    int x;          // this lane's column, wrapped on a periodic axis
+    int xs;         // the strip's first output column
+    int ya, yb;     // first and last row of the strip (clipped to the grid)
+    bool in;        // column inside the grid
+    bool own;       // one of the strip's output columns
+    int mode;       // kInner, kSide or kGeneral
+};
+
+// What a strip and its halo of two nodes and kReach more rows touch: no face and no node next to
+// one; only an x face of a grid without wraps and static solids; anything else.
+enum { kInner = 0, kSide = 1, kGeneral = 2 };
+
+template <class T>
+__device__ __forceinline__ Strip strip_of(const Inst<T>& I, int local, int rows, int lane) {
+    const Geom& g = I.g;
     const int n0 = g.n[0], n1 = g.n[1];
-    const bool p0 = g.periodic[0], p1 = g.periodic[1];
-    for (int k = threadIdx.x; k < HX * HY; k += NT) {
-        const int ly = k / HX, lx = k - ly * HX;
-        int gx = x0 - 2 + lx, gy = y0 - 2 + ly;
-        if (p0) gx = wrap_any(gx, n0);
-        if (p1) gy = wrap_any(gy, n1);
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (gx >= 0 && gx < n0 && gy >= 0 && gy < n1) v = __ldg(src + (long long)gy * n0 + gx);
-        S[k] = v;
-    }
+    const int ns = strip_count(n0, kStripW, g.periodic[0]);
+    const int kc = local / ns, kx = local - kc * ns;
+    Strip s;
+    s.xs = kx * kStripW - strip_origin(n0, kStripW, g.periodic[0]);
+    const int xr = s.xs - 2 + lane;
+    s.own = lane >= 2 && lane < 2 + kStripW && xr >= 0 && xr < n0;
+    s.x = g.periodic[0] ? wrap_any(xr, n0) : xr;
+    s.in = s.x >= 0 && s.x < n0;
+    s.ya = kc * rows;
+    s.yb = min(s.ya + rows, n1) - 1;
+    const bool plain = !g.periodic[0] && !g.periodic[1] && !g.ks && s.ya >= 4 && s.yb <= n1 - 5;
+    const bool xmid = s.xs >= 4 && s.xs + kStripW + 1 <= n0 - 3;
+    // (the adjoint's kSide path finds the face column in the lane beside a node next to it)
+    const bool xcut = s.xs - 2 + 31 == n0 - 2;
+    s.mode = !plain || xcut ? kGeneral : (xmid ? kInner : kSide);
+    return s;
 }
 
-// The arithmetic of the helpers below is written with explicitly rounded operations
-// (__fmaf_rn, __fmul_rn, __fadd_rn, __fsub_rn), which the compiler neither contracts nor
-// reorders: the tile and the row-marching forward kernels then compute bitwise the same state.
-#define FMA_ __fmaf_rn
-#define MUL_ __fmul_rn
-#define ADD_ __fadd_rn
-#define SUB_ __fsub_rn
-
-// First derivative of the velocity along one axis from a node's record v and its neighbours at
-// +-1 (p1, m1) and +-2 (p2, m2): central, or the second-order one-sided difference on a
-// non-periodic boundary node (side -1: low face, +1: high face).
-__device__ __forceinline__ void dvel_v(int side, const float4& v, const float4& p1,
-                                       const float4& m1, const float4& p2, const float4& m2,
-                                       float& dux, float& duy) {
-    if (side == 0) {
-        dux = FMA_(0.5f, p1.y, MUL_(-0.5f, m1.y));
-        duy = FMA_(0.5f, p1.z, MUL_(-0.5f, m1.z));
-    } else if (side < 0) {
-        dux = FMA_(-1.5f, v.y, FMA_(2.f, p1.y, MUL_(-0.5f, p2.y)));
-        duy = FMA_(-1.5f, v.z, FMA_(2.f, p1.z, MUL_(-0.5f, p2.z)));
-    } else {
-        dux = FMA_(1.5f, v.y, FMA_(-2.f, m1.y, MUL_(0.5f, m2.y)));
-        duy = FMA_(1.5f, v.z, FMA_(-2.f, m1.z, MUL_(0.5f, m2.z)));
-    }
+// The value bc_value gives a boundary node of face f from its source's value, with the face's values
+// rounded once on the host.
+template <class T>
+__device__ __forceinline__ V4<T> face_value2(const Inst<T>& I, int f, const V4<T>& o) {
+    const V4<T> p = I.bcf[f];
+    const bool keep = I.bckeep[f] != 0;
+    V4<T> b;
+    b.r = keep ? o.r : p.r;
+    b.x = keep || f >= 2 ? p.x : o.x;
+    b.y = keep || f < 2 ? p.y : o.y;
+    b.z = (T)0;
+    return b;
 }
 
-// The same at the node whose record sits at S[s] (neighbours at +-step); reads only the
-// values the side uses.
-__device__ __forceinline__ void dvel(const float4* S, int s, int step, int side, float& dux,
-                                     float& duy) {
-    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (side == 0) dvel_v(0, z, S[s + step], S[s - step], z, z, dux, duy);
-    else if (side < 0) dvel_v(-1, S[s], S[s + step], z, S[s + 2 * step], z, dux, duy);
-    else dvel_v(1, S[s], z, S[s - step], z, S[s - 2 * step], dux, duy);
-}
-
-__device__ __forceinline__ int face_side(int c, int n, int periodic) {
-    if (periodic) return 0;
-    return c == 0 ? -1 : (c == n - 1 ? 1 : 0);
-}
-
-// A tile is interior when its two-cell halo lies inside the grid at least one node away from
-// every non-periodic boundary: then no index wraps, no node of the halo is a boundary node and
-// no boundary node is sourced from the tile, and the kernels take a path without those tests.
-template <int TX, int TY>
-__device__ __forceinline__ bool interior_tile(const Geom& g, int x0, int y0) {
-    return x0 - 3 >= 0 && x0 + TX + 2 <= g.n[0] - 1 && y0 - 3 >= 0 && y0 + TY + 2 <= g.n[1] - 1;
-}
-
-// f^eq of the eight moving directions (D2Q9 order 1..8) at a node with record v and velocity
-// gradient g_ab = d u_a / d x_b: w_i (rho - rho0 - 1.5 u^2 + 4.5 (c.u)^2 + A c.S.c + 3 c.u),
-// opposite directions sharing their symmetric part.
-__device__ __forceinline__ void feq8_v(const float4& v, float A, float gxx, float gyx, float gxy,
-                                       float gyy, float f[8]) {
-    // the weight products w1, 4.5 w1, 3 w1, ... are those of Wts<float, 2>, which keep the
-    // lattice identities exact in single precision
-    using W = Wts<float, 2>;
-    const float ux = v.y, uy = v.z;
-    const float base = FMA_(-1.5f, FMA_(ux, ux, MUL_(uy, uy)), v.x);
-    const float ax = MUL_(A, MUL_(2.f, gxx)), ay = MUL_(A, MUL_(2.f, gyy));
-    const float sd = ADD_(MUL_(2.f, gxx), MUL_(2.f, gyy)), so = MUL_(2.f, ADD_(gxy, gyx));
-    const float ad = MUL_(A, ADD_(sd, so)), ae = MUL_(A, SUB_(sd, so));
-    const float cpp = ADD_(ux, uy), cmp = SUB_(uy, ux);
-    const float sx = FMA_(MUL_(W::h_1, ux), ux, MUL_(W::w1, ADD_(base, ax)));
-    const float sy = FMA_(MUL_(W::h_1, uy), uy, MUL_(W::w1, ADD_(base, ay)));
-    const float spp = FMA_(MUL_(W::h_2, cpp), cpp, MUL_(W::w2, ADD_(base, ad)));
-    const float smp = FMA_(MUL_(W::h_2, cmp), cmp, MUL_(W::w2, ADD_(base, ae)));
-    f[0] = FMA_(W::w3_1, ux, sx);
-    f[1] = FMA_(W::w3_1, uy, sy);
-    f[2] = FMA_(-W::w3_1, ux, sx);
-    f[3] = FMA_(-W::w3_1, uy, sy);
-    f[4] = FMA_(W::w3_2, cpp, spp);
-    f[5] = FMA_(W::w3_2, cmp, smp);
-    f[6] = FMA_(-W::w3_2, cpp, spp);
-    f[7] = FMA_(-W::w3_2, cmp, smp);
-}
-
-// Rest direction: f_0 = w0 (rho - rho0 - 1.5 u^2).
-__device__ __forceinline__ float feq0_v(const float4& v) {
-    return MUL_(Wts<float, 2>::w0, FMA_(-1.5f, FMA_(v.y, v.y, MUL_(v.z, v.z)), v.x));
-}
-
-// Output node from its nine gathered values: rho* = sum f_i, u* = sum c_i f_i (Eqs. rho, u),
-// the body force and the Brinkman update (Eq. u_ex_2) with kappa, u_S (ks, zero outside the
-// footprint box) and a static solid's kappa_s.
-__device__ __forceinline__ V4<float> gather_out(float f0, float f1, float f2, float f3, float f4,
-                                                float f5, float f6, float f7, float f8,
-                                                const float4& ks, float kst, float bfx,
-                                                float bfy) {
-    V4<float> o;
-    o.r = ADD_(ADD_(ADD_(ADD_(f0, f1), ADD_(f2, f3)), ADD_(ADD_(f4, f5), ADD_(f6, f7))), f8);
-    const float usx = ADD_(ADD_(ADD_(SUB_(f1, f3), SUB_(f5, f6)), SUB_(f8, f7)), bfx);
-    const float usy = ADD_(SUB_(ADD_(SUB_(f2, f4), ADD_(f5, f6)), ADD_(f7, f8)), bfy);
-    if (ks.x != 0.f || ks.y != 0.f || ks.z != 0.f) {
-        const float inv = __fdiv_rn(1.f, ADD_(ADD_(1.f, ks.x), kst));
-        o.x = MUL_(FMA_(ks.x, ks.y, usx), inv);
-        o.y = MUL_(FMA_(ks.x, ks.z, usy), inv);
-    } else if (kst != 0.f) {
-        const float inv = __fdiv_rn(1.f, ADD_(1.f, kst));
-        o.x = MUL_(usx, inv);
-        o.y = MUL_(usy, inv);
-    } else {
-        o.x = usx;
-        o.y = usy;
-    }
-    o.z = 0.f;
-    return o;
-}
-
-// Does the node rectangle [xa, xb] x [ya, yb] meet the footprint box (the target box)?  Tested
-// once per tile, so that tiles away from the moving body or the objective skip the per-node
-// tests.  Periodic wraps are not taken into account: callers pass the flag only where no node
-// of the rectangle wraps.
-__device__ __forceinline__ bool meets_box(const Geom& g, int xa, int xb, int ya, int yb) {
-    return g.boxN > 0 && xb >= g.blo[0] && xa < g.blo[0] + g.bn[0] && yb >= g.blo[1] &&
-           ya < g.blo[1] + g.bn[1];
-}
-__device__ __forceinline__ bool meets_target(const Geom& g, int xa, int xb, int ya, int yb) {
-    return xb >= g.obox[0] && xa <= g.obox[1] && yb >= g.obox[2] && ya <= g.obox[3];
-}
-
-// Boundary copies sourced by interior node (x, y) of value o (Eqs. bc_rho, bc_u): a node next to
-// one face writes that face's boundary node with the face's single-precision values (the values
-// bc_value gives); a node next to two faces (a corner's source) takes the general rule.
-__device__ __forceinline__ void write_bc2(const Inst& I, int x, int y, const V4<float>& o,
-                                          V4<float>* out) {
+// Boundary copies sourced by interior node (x, y) of value o (Eqs. bc_rho, bc_u): the node beside
+// it on an x face, on a y face, and the corner of the two with the face that wins there.  (Along
+// an axis of three nodes one node lies next to both faces: the general rule.)
+template <class T>
+__device__ __forceinline__ void write_bc2(const Inst<T>& I, int x, int y, const V4<T>& o,
+                                          V4<T>* out) {
     const Geom& g = I.g;
     const int n0 = g.n[0], n1 = g.n[1];
     const bool xl = !g.periodic[0] && x == 1, xh = !g.periodic[0] && x == n0 - 2;
     const bool yl = !g.periodic[1] && y == 1, yh = !g.periodic[1] && y == n1 - 2;
-    const int nf = (int)xl + (int)xh + (int)yl + (int)yh;
-    if (nf == 0) return;
-    if (nf > 1) {
+    if ((xl && xh) || (yl && yh)) {
         write_bc_from(g, x, y, 0, o, out);
         return;
     }
-    const int f = xl ? 0 : (xh ? 1 : (yl ? 2 : 3));
-    const int bx = xl ? 0 : (xh ? n0 - 1 : x), by = yl ? 0 : (yh ? n1 - 1 : y);
-    const float4 p = I.bcf[f];
-    V4<float> b;
-    if (I.bckeep[f]) {
-        b.r = o.r;
-        b.x = p.x;
-        b.y = p.y;
-    } else {
-        b.r = p.w;
-        b.x = f < 2 ? o.x : p.x;
-        b.y = f < 2 ? p.y : o.y;
-    }
-    b.z = 0.f;
-    out[(long long)by * n0 + bx] = b;
+    const int fx = xh ? 1 : 0, fy = yh ? 3 : 2;
+    const int bx = xl ? 0 : n0 - 1, by = yl ? 0 : n1 - 1;
+    if (xl || xh) stg4(out + (y * n0 + bx), face_value2<T>(I, fx, o));
+    if (yl || yh) stg4(out + (by * n0 + x), face_value2<T>(I, fy, o));
+    if ((xl || xh) && (yl || yh))
+        stg4(out + (by * n0 + bx), face_value2<T>(I, I.corner[fx + 2 * (fy - 2)], o));
 }
 
-// kappa, u_S at node (x, y) of the footprint box, else zero.
-__device__ __forceinline__ float4 kus_at(const Inst& I, int x, int y) {
-    long long bi;
-    return in_box(I.g, x, y, 0, bi) ? __ldg((const float4*)I.kus + bi)
-                                    : make_float4(0.f, 0.f, 0.f, 0.f);
-}
+// One strip of the forward step.  F-row f evaluates f_i^eq at the lane's node (x, f); each output
+// row collects three F-rows.  Per output node the directions are grouped by c_x: the node's own
+// column adds f0 + f2 + f4 to rho and f2 - f4 to u_y; the column to the left sends
+// P = f1 + f5 + f8 and Tp = f5 - f8, the column to the right M = f3 + f6 + f7 and Tm = f6 - f7
+// (rho takes P + M, u_x P - M, u_y Tp + Tm): four values by shuffle instead of six.
+// State rows, and kappa and u_S, pass through rings in shared memory (per lane: each lane reads
+// only the records it copied), copied kAhead rows before they are read, so that the march holds no
+// loads in flight in registers.  The mode changes which nodes are special, not the arithmetic.
+constexpr int kAhead = 4, kRing = 8;
+static_assert(kAhead + 3 <= kRing && (kRing & (kRing - 1)) == 0, "ring slots by mask");
 
-// One tile of the forward step.  EDGE: the general path (wraps, grid edges, boundary nodes).
-template <int TX, int TY, bool EDGE>
-__device__ __forceinline__ void step_tile(const Inst& I, int x0, int y0, int src, int dst,
-                                          float4* S, float* F) {
-    constexpr int HX = TX + 4, FX = TX + 2, FY = TY + 2, FN = FX * FY;
+template <class T, int MODE>
+__device__ __forceinline__ void step_strip(const Inst<T>& I, const Strip& s, const V4<T>* src,
+                                           V4<T>* out, const V4<T>* kus, V4<T>* ring) {
+    using W = Wts<T, 2>;
+    constexpr bool GEN = MODE == kGeneral, SIDE = MODE != kInner;
+    V4<T>* ringk = ring + kRing * 32;   // kappa, u_S
     const Geom& g = I.g;
     const int n0 = g.n[0], n1 = g.n[1];
-    const float4* sp = (const float4*)I.bufs[src];
-    if (EDGE) {
-        load_tile<TX, TY>(g, sp, x0, y0, S);
-    } else {
-        const float4* base = sp + (long long)(y0 - 2) * n0 + (x0 - 2);
-        for (int k = threadIdx.x; k < HX * (TY + 4); k += NT) {
-            const int ly = k / HX, lx = k - ly * HX;
-            S[k] = __ldg(base + (long long)ly * n0 + lx);
+    const bool p0 = GEN && g.periodic[0], p1 = GEN && g.periodic[1];
+    const int ya = !GEN || p1 ? s.ya : max(s.ya, 1), yb = !GEN || p1 ? s.yb : min(s.yb, n1 - 2);
+    if (ya > yb) return;   // uniform
+    const int x = s.x;
+    const bool xin = !SIDE || s.in;
+    const bool ocol = s.own && (!SIDE || p0 || (x >= 1 && x <= n0 - 2));
+    const int sx = !SIDE || p0 ? 0 : (x == 0 ? -1 : (x == n0 - 1 ? 1 : 0));
+    const bool xface = SIDE && (!GEN || __any_sync(FULL, sx != 0));
+    const bool xnear = GEN && __any_sync(FULL, ocol && !p0 && (x == 1 || x == n0 - 2));
+    // kSide: the face column a node next to it writes, and its prescribed values
+    const int wf = SIDE && !GEN && ocol ? (x == 1 ? 0 : (x == n0 - 2 ? 1 : -1)) : -1;
+    const int bx = x - g.blo[0], bn0 = g.bn[0], bn1 = g.bn[1], by0 = g.blo[1];
+    const bool bcol = g.boxN > 0 && ocol && bx >= 0 && bx < bn0;
+    const bool bany = __any_sync(FULL, bcol) && ya < by0 + bn1 && yb >= by0;
+    const T* ks_st = GEN ? (const T*)g.ks : nullptr;
+    const T A = I.A, bfx = I.bf[0], bfy = I.bf[1];
+    const V4<T>* scol = src + (xin ? x : 0);
+    const V4<T>* kcol = kus + (bcol ? bx : 0);
+    V4<T>* ocl = out + (ocol ? x : 0);
+    // a state row, and kappa, u_S two rows below it (the output row that completes when the state
+    // row is first read), as one copy group; node indices fit 32 bits (checked at create)
+    auto issue = [&](int row) {
+        int r = row;
+        bool in = xin;
+        if (GEN) {
+            if (p1) r += r < 0 ? n1 : (r >= n1 ? -n1 : 0);
+            in = xin && r >= 0 && r < n1;
+            if (!in) r = 0;
         }
-    }
-    __syncthreads();
-    const bool tbox = EDGE || meets_box(g, x0, x0 + TX - 1, y0, y0 + TY - 1);
-    const float A = I.Af, bfx = I.bf[0], bfy = I.bf[1];
-    // f^eq of every direction at the tile and its one-cell rim
-    for (int k = threadIdx.x; k < FN; k += NT) {
-        const int fy = k / FX, fx = k - fy * FX;
-        const int s = (fy + 1) * HX + fx + 1;
-        float gxx, gyx, gxy, gyy;   // g_ab = d u_a / d x_b
-        if (EDGE) {
-            int gx = x0 - 1 + fx, gy = y0 - 1 + fy;
-            if (g.periodic[0]) gx = wrap_any(gx, n0);
-            else if (gx < 0 || gx >= n0) continue;
-            if (g.periodic[1]) gy = wrap_any(gy, n1);
-            else if (gy < 0 || gy >= n1) continue;
-            dvel(S, s, 1, face_side(gx, n0, g.periodic[0]), gxx, gyx);
-            dvel(S, s, HX, face_side(gy, n1, g.periodic[1]), gxy, gyy);
-        } else {
-            dvel(S, s, 1, 0, gxx, gyx);
-            dvel(S, s, HX, 0, gxy, gyy);
+        cp_record<T>(ring + (row & (kRing - 1)) * 32, scol + r * n0, row <= yb + 2, in);
+        if (bany) {
+            const int kr = row - 2 - by0;
+            const bool kin = bcol && (unsigned)kr < (unsigned)bn1;
+            cp_record<T>(ringk + ((row - 2) & (kRing - 1)) * 32, kcol + (kin ? kr * bn0 : 0),
+                         row - 2 <= yb, kin);
         }
-        float fv[8];
-        feq8_v(S[s], A, gxx, gyx, gxy, gyy, fv);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) F[q * FN + k] = fv[q];
-    }
-    __syncthreads();
-    // gather rho* = sum f_i(x - c_i), u* = sum c_i f_i(x - c_i); Brinkman update; BCs
-    V4<float>* out = (V4<float>*)I.bufs[dst];
-    for (int k = threadIdx.x; k < TX * TY; k += NT) {
-        const int ty = k / TX, tx = k - ty * TX;
-        const int x = x0 + tx, y = y0 + ty;
-        if (EDGE && (x < 0 || x >= n0 || y < 0 || y >= n1 || is_boundary(g, x, y, 0))) continue;
-        const int f = (ty + 1) * FX + tx + 1;
-        const float f0 = feq0_v(S[(ty + 2) * HX + tx + 2]);
-        const float f1 = F[0 * FN + f - 1];        // from x - (1, 0)
-        const float f2 = F[1 * FN + f - FX];       // from x - (0, 1)
-        const float f3 = F[2 * FN + f + 1];        // from x + (1, 0)
-        const float f4 = F[3 * FN + f + FX];       // from x + (0, 1)
-        const float f5 = F[4 * FN + f - FX - 1];   // from x - (1, 1)
-        const float f6 = F[5 * FN + f - FX + 1];   // from x - (-1, 1)
-        const float f7 = F[6 * FN + f + FX + 1];   // from x + (1, 1)
-        const float f8 = F[7 * FN + f + FX - 1];   // from x - (1, -1)
-        const long long m = (long long)y * n0 + x;
-        const float kst = g.ks ? ((const float*)g.ks)[m] : 0.f;
-        const V4<float> o = gather_out(f0, f1, f2, f3, f4, f5, f6, f7, f8,
-                                       tbox ? kus_at(I, x, y) : make_float4(0.f, 0.f, 0.f, 0.f),
-                                       kst, bfx, bfy);
-        out[m] = o;
-        if (EDGE) write_bc2(I, x, y, o, out);
-    }
-    __syncthreads();
-}
-
-template <int TX, int TY>
-__global__ void __launch_bounds__(NT) k_t_step2d(Plan p, const int* __restrict__ pre, int total,
-                                                 int src, int dst, int kslot) {
-    constexpr int HX = TX + 4, HY = TY + 4;
-    extern __shared__ float4 smem[];
-    float4* S = smem;                          // HY x HX state records
-    float* F = (float*)(smem + HX * HY);       // 8 planes of FY x FX: f_1..f_8
-    __shared__ Inst sI;
-    int cur = -1;
-    for (int u = blockIdx.x; u < total; u += gridDim.x) {
-        const int i = find_inst(pre, p.count, u);
-        stage_inst(p, i, cur, sI, kslot);
-        int x0, y0;
-        tile_xy<TX, TY>(sI.g, u - pre[i], x0, y0);
-        if (interior_tile<TX, TY>(sI.g, x0, y0))
-            step_tile<TX, TY, false>(sI, x0, y0, src, dst, S, F);
-        else
-            step_tile<TX, TY, true>(sI, x0, y0, src, dst, S, F);
-    }
-}
-
-// cp.async: 16-byte copies global -> shared (src_bytes 0 fills zeros), commit, wait.
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, int src_bytes) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src),
-                 "r"(src_bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_wait1() {
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-}
-
-// ---------------------------------------------------------------- row-marching forward step
-// A block owns a strip of SW = NTH - 2 output columns and a chunk of YC output rows and marches
-// up the rows.  State rows stream through a six-row cp.async ring two rows ahead of use; per
-// F-row f every thread evaluates f^eq at column x0 - 1 + t (the strip and one rim column on
-// each side: 2 / SW extra work where a tile recomputes its whole rim), the six directions that
-// leave the column go through shared memory, and each output node collects its nine values
-// over three consecutive F-rows in registers.  With the helpers above the values are those of
-// the tile kernel, bit for bit.
-template <int NTH, int YC>
-__global__ void __launch_bounds__(NTH) k_t_step2d_rows(Plan p, const int* __restrict__ pre,
-                                                        int total, int src, int dst, int kslot) {
-    // ring of state rows: 8 slots (6 in use: two rows below the f^eq row to three above), so
-    // that the slot of a row is its index & 7, negative indices included
-    constexpr int SW = NTH - 2, RW = NTH + 2, NR = 8;
-    __shared__ float4 R[NR][RW];     // state rows, columns x0 - 2 .. x0 + SW + 1
-    __shared__ float Fs[6][NTH];     // f_1, f_3, f_5, f_6, f_7, f_8 of the current F-row
-    __shared__ Inst sI;
-    int cur = -1;
-    const int t = threadIdx.x;
-    for (int u = blockIdx.x; u < total; u += gridDim.x) {
-        const int i = find_inst(pre, p.count, u);
-        stage_inst(p, i, cur, sI, kslot);
-        const Geom& g = sI.g;
-        const int n0 = g.n[0], n1 = g.n[1], p0 = g.periodic[0], p1 = g.periodic[1];
-        const int ns = tile_count(n0, SW, p0);
-        const int loc = u - pre[i];
-        const int kc = loc / ns, kx = loc - kc * ns;
-        const int x0 = kx * SW - tile_origin(n0, SW, p0);
-        const int y0 = kc * YC - tile_origin(n1, YC, p1), y1 = y0 + YC;
-        const float4* sp = (const float4*)sI.bufs[src];
-        V4<float>* out = (V4<float>*)sI.bufs[dst];
-        const float A = sI.Af, bfx = sI.bf[0], bfy = sI.bf[1];
-        const bool tbox = p0 || p1 || meets_box(g, x0, x0 + SW, y0, y1 - 1);
-        auto slot = [](int r) { return r & (NR - 1); };
-        auto issue_row = [&](int r) {   // state row r (unwrapped index) into its ring slot
-            float4* row = R[slot(r)];
-            int gy = r;
-            bool rin = true;
-            if (p1) gy = wrap_any(gy, n1);
-            else rin = gy >= 0 && gy < n1;
-            for (int k = t; k < RW; k += NTH) {
-                int gx = x0 - 2 + k;
-                bool in = rin;
-                if (p0) gx = wrap_any(gx, n0);
-                else in = in && gx >= 0 && gx < n0;
-                cp_async16(row + k, in ? sp + (long long)gy * n0 + gx : sp, in ? 16 : 0);
+        cp_commit();
+    };
+    // sums of output row f - 1 (a) and f (b) as F-row f is reached: the directions already met
+    T a_r = (T)0, a_y = (T)0, a_P = (T)0, a_Tp = (T)0, a_M = (T)0, a_Tm = (T)0;
+    T b_2 = (T)0, b_5 = (T)0, b_6 = (T)0;
+    auto march = [&](int f, auto emit) {
+        constexpr bool EMIT = decltype(emit)::value;
+        issue(f + 1 + kAhead);
+        cp_wait<kAhead>();   // row f + 1 has landed
+        const int y = f - 1;   // output row this F-row completes
+        V4<T> v0, vp, vm, kv;
+        v0 = lds4(ring + (f & (kRing - 1)) * 32);
+        vp = lds4(ring + ((f + 1) & (kRing - 1)) * 32);
+        vm = lds4(ring + ((f - 1) & (kRing - 1)) * 32);
+        kv.r = kv.x = kv.y = (T)0;
+        if (EMIT && bany) kv = lds4(ringk + (y & (kRing - 1)) * 32);
+        T kst = (T)0;
+        if (GEN && EMIT && ks_st && ocol) kst = ks_st[y * n0 + x];
+        // twice the velocity gradient, D_ab = 2 d u_a / d x_b
+        const T l1x = from_left(v0.x), l1y = from_left(v0.y);
+        const T r1x = from_right(v0.x), r1y = from_right(v0.y);
+        T Dxx = sub_<T>(r1x, l1x), Dyx = sub_<T>(r1y, l1y);
+        T Dxy = sub_<T>(vp.x, vm.x), Dyy = sub_<T>(vp.y, vm.y);
+        if (xface) {   // one-sided along x on a boundary column
+            const T l2x = __shfl_up_sync(FULL, v0.x, 2), l2y = __shfl_up_sync(FULL, v0.y, 2);
+            const T r2x = __shfl_down_sync(FULL, v0.x, 2), r2y = __shfl_down_sync(FULL, v0.y, 2);
+            if (sx < 0) {
+                Dxx = fma_<T>((T)-3, v0.x, fma_<T>((T)4, r1x, -r2x));
+                Dyx = fma_<T>((T)-3, v0.y, fma_<T>((T)4, r1y, -r2y));
+            } else if (sx > 0) {
+                Dxx = fma_<T>((T)3, v0.x, fma_<T>((T)-4, l1x, l2x));
+                Dyx = fma_<T>((T)3, v0.y, fma_<T>((T)-4, l1y, l2y));
             }
-        };
-        __syncthreads();   // the ring and Fs of the previous unit are no longer read
-        for (int r = y0 - 3; r <= y0 + 1; ++r) issue_row(r);
-        cp_async_commit();
-        // this thread's f^eq column and, for 1 <= t <= SW, output column
-        const int xr = x0 - 1 + t;
-        int xc = xr;
-        bool cin = true;
-        if (p0) xc = wrap_any(xc, n0);
-        else cin = xc >= 0 && xc < n0;
-        const int sx = face_side(xc, n0, p0);
-        const bool ocol = t >= 1 && t <= SW &&
-                          (p0 ? (xr >= 0 && xr < n0) : (xr >= 1 && xr <= n0 - 2));
-        float a2 = 0.f, a5 = 0.f, a6 = 0.f;   // f2, f5, f6 collected for the next row
-        float b2 = 0.f, b5 = 0.f, b6 = 0.f;   // the same for the row after that
-        float c0 = 0.f, c1 = 0.f, c3 = 0.f;   // f0, f1, f3 collected for the next row
-        for (int f = y0 - 1; f <= y1; ++f) {
-            if (f + 3 <= y1 + 2) issue_row(f + 3);
-            cp_async_commit();
-            cp_async_wait1();
-            __syncthreads();
-            float fv[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            float f0 = 0.f;
-            int fy = f;
-            bool rin = true;
-            if (p1) fy = wrap_any(fy, n1);
-            else rin = fy >= 0 && fy < n1;
-            if (cin && rin) {   // f^eq at (xc, f)
-                const float4* r0 = R[slot(f)];
-                const float4* rp = R[slot(f + 1)];
-                const float4* rm = R[slot(f - 1)];
-                const int c = t + 1;
-                const float4 v = r0[c], z = make_float4(0.f, 0.f, 0.f, 0.f);
-                float gxx, gyx, gxy, gyy;
-                if (sx == 0) dvel_v(0, z, r0[c + 1], r0[c - 1], z, z, gxx, gyx);
-                else if (sx < 0) dvel_v(-1, v, r0[c + 1], z, r0[c + 2], z, gxx, gyx);
-                else dvel_v(1, v, z, r0[c - 1], z, r0[c - 2], gxx, gyx);
-                const int sy = face_side(fy, n1, p1);
-                if (sy == 0) dvel_v(0, z, rp[c], rm[c], z, z, gxy, gyy);
-                else if (sy < 0) dvel_v(-1, v, rp[c], z, R[slot(f + 2)][c], z, gxy, gyy);
-                else dvel_v(1, v, z, rm[c], z, R[slot(f - 2)][c], gxy, gyy);
-                feq8_v(v, A, gxx, gyx, gxy, gyy, fv);
-                f0 = feq0_v(v);
+        }
+        if (GEN && !p1 && (f == 0 || f == n1 - 1)) {   // one-sided along y on a boundary row
+            V3<T> far;
+            far.r = far.x = far.y = (T)0;
+            if (xin) far = ldcg3<V3<T>>(scol + (f == 0 ? 2 : n1 - 3) * n0);
+            if (f == 0) {
+                Dxy = fma_<T>((T)-3, v0.x, fma_<T>((T)4, vp.x, -far.x));
+                Dyy = fma_<T>((T)-3, v0.y, fma_<T>((T)4, vp.y, -far.y));
+            } else {
+                Dxy = fma_<T>((T)3, v0.x, fma_<T>((T)-4, vm.x, far.x));
+                Dyy = fma_<T>((T)3, v0.y, fma_<T>((T)-4, vm.y, far.y));
             }
-            Fs[0][t] = fv[0];   // f_1
-            Fs[1][t] = fv[2];   // f_3
-            Fs[2][t] = fv[4];   // f_5
-            Fs[3][t] = fv[5];   // f_6
-            Fs[4][t] = fv[6];   // f_7
-            Fs[5][t] = fv[7];   // f_8
-            __syncthreads();
-            if (t >= 1 && t <= SW) {
-                // values the nodes (x, f - 1), (x, f), (x, f + 1) receive from F-row f
-                const float g4 = fv[3], g7 = Fs[4][t + 1], g8 = Fs[5][t - 1];
-                const float g1 = Fs[0][t - 1], g3 = Fs[1][t + 1];
-                const float g2 = fv[1], g5 = Fs[2][t - 1], g6 = Fs[3][t + 1];
-                const int y = f - 1;   // output row completed by this F-row
-                bool orow = y >= y0 && y < y1;
-                orow = orow && (p1 ? (y >= 0 && y < n1) : (y >= 1 && y <= n1 - 2));
-                if (ocol && orow) {
-                    const long long m = (long long)y * n0 + xc;
-                    const float kst = g.ks ? ((const float*)g.ks)[m] : 0.f;
-                    const V4<float> o = gather_out(
-                        c0, c1, b2, c3, g4, b5, b6, g7, g8,
-                        tbox ? kus_at(sI, xc, y) : make_float4(0.f, 0.f, 0.f, 0.f), kst, bfx,
-                        bfy);
-                    out[m] = o;
-                    write_bc2(sI, xc, y, o, out);
+        }
+        // f_i^eq = w_i (rho - rho0 - 1.5 u^2 + 4.5 (c.u)^2 + A c.S.c + 3 c.u), opposite directions
+        // sharing their symmetric part; the weight products are those of Wts<T, 2>
+        const T ux = v0.x, uy = v0.y;
+        const T P = fma_<T>((T)-1.5, fma_<T>(ux, ux, mul_<T>(uy, uy)), v0.r);
+        const T sd = add_<T>(Dxx, Dyy), so = add_<T>(Dxy, Dyx);
+        const T cp = add_<T>(ux, uy), cm = sub_<T>(uy, ux);
+        const T ex = fma_<T>(mul_<T>(W::h_1, ux), ux, mul_<T>(W::w1, fma_<T>(A, Dxx, P)));
+        const T ey = fma_<T>(mul_<T>(W::h_1, uy), uy, mul_<T>(W::w1, fma_<T>(A, Dyy, P)));
+        const T ep = fma_<T>(mul_<T>(W::h_2, cp), cp,
+                             mul_<T>(W::w2, fma_<T>(A, add_<T>(sd, so), P)));
+        const T em = fma_<T>(mul_<T>(W::h_2, cm), cm,
+                             mul_<T>(W::w2, fma_<T>(A, sub_<T>(sd, so), P)));
+        const T f0 = mul_<T>(W::w0, P);
+        const T f1 = fma_<T>(W::w3_1, ux, ex), f3 = fma_<T>(-W::w3_1, ux, ex);
+        const T f2 = fma_<T>(W::w3_1, uy, ey), f4 = fma_<T>(-W::w3_1, uy, ey);
+        const T f5 = fma_<T>(W::w3_2, cp, ep), f7 = fma_<T>(-W::w3_2, cp, ep);
+        const T f6 = fma_<T>(W::w3_2, cm, em), f8 = fma_<T>(-W::w3_2, cm, em);
+        if (EMIT) {
+            const T Pl = from_left(add_<T>(a_P, f8)), Tl = from_left(sub_<T>(a_Tp, f8));
+            const T Mr = from_right(add_<T>(a_M, f7)), Tr = from_right(sub_<T>(a_Tm, f7));
+            V4<T> o;
+            o.r = add_<T>(add_<T>(a_r, f4), add_<T>(Pl, Mr));
+            o.x = add_<T>(sub_<T>(Pl, Mr), bfx);
+            o.y = add_<T>(add_<T>(sub_<T>(a_y, f4), add_<T>(Tl, Tr)), bfy);
+            o.z = (T)0;
+            if (bany || (GEN && ks_st)) {   // off the body kappa = 0: times 1, plus 0
+                T den = add_<T>((T)1, kv.r);
+                if (GEN) den = add_<T>(den, kst);
+                const T inv = inv_<T>(den);
+                o.x = mul_<T>(fma_<T>(kv.r, kv.x, o.x), inv);
+                o.y = mul_<T>(fma_<T>(kv.r, kv.y, o.y), inv);
+            }
+            if (ocol) {
+                stg4(ocl + y * n0, o);
+                if (GEN) {
+                    if (xnear || (!p1 && (y == 1 || y == n1 - 2))) write_bc2<T>(I, x, y, o, out);
+                } else if (wf >= 0) {
+                    stg4(ocl + y * n0 + (wf == 0 ? -1 : 1), face_value2<T>(I, wf, o));
                 }
-                b2 = a2;
-                b5 = a5;
-                b6 = a6;
-                a2 = g2;
-                a5 = g5;
-                a6 = g6;
-                c0 = f0;
-                c1 = g1;
-                c3 = g3;
             }
         }
+        a_r = add_<T>(b_2, f0);
+        a_y = b_2;
+        a_P = add_<T>(b_5, f1);
+        a_Tp = b_5;
+        a_M = add_<T>(b_6, f3);
+        a_Tm = b_6;
+        b_2 = f2;
+        b_5 = f5;
+        b_6 = f6;
+    };
+    for (int r = ya - 2; r < ya + kAhead; ++r) issue(r);
+    march(ya - 1, std::false_type{});
+    march(ya, std::false_type{});
+#pragma unroll 2
+    for (int f = ya + 1; f <= yb + 1; ++f) march(f, std::true_type{});
+    cp_wait<0>();
+}
+
+// The general path out of line, so that its registers do not weigh on the interior strips.
+template <class T>
+__device__ __noinline__ void step_strip_gen(const Inst<T>& I, const Strip& s, const V4<T>* src,
+                                             V4<T>* out, const V4<T>* kus, V4<T>* ring) {
+    step_strip<T, kGeneral>(I, s, src, out, kus, ring);
+}
+
+// Each warp's copy of the instance record it works on, staged when the warp moves to another
+// instance: geometry then comes from shared memory, which the stores to global memory cannot
+// alias.
+template <class T>
+__device__ __forceinline__ void stage_inst(const Plan& p, int i, int& cur, Inst<T>& sI, int lane) {
+    if (i != cur) {
+        __syncwarp();
+        const int* src = reinterpret_cast<const int*>(table<T>(p) + i);
+        int* dst = reinterpret_cast<int*>(&sI);
+        for (int k = lane; k < (int)(sizeof(Inst<T>) / 4); k += 32) dst[k] = __ldg(src + k);
+        __syncwarp();
+        cur = i;
     }
 }
 
-// ---------------------------------------------------------------- fused adjoint step
-
-// Objective source of the adjoint step in single precision, fixed per tile.
-struct ObjSrc {
-    bool on;                  // inside the objective window
-    float r, x, y;            // d j / d (rho, ux, uy) at a target node, times h_n
-    bool cyl;
+// A warp's shared memory: its rings of rows (2 x kRing rows forward, 4 x kARing in the adjoint) and
+// its instance record.
+template <class T>
+struct StripWarp {
+    V4<T> ring[16 * 32];
+    Inst<T> inst;
 };
 
-__device__ __forceinline__ ObjSrc obj_src(const Inst& I, int n) {
-    ObjSrc o;
-    o.on = n >= I.win_begin && n <= I.win_end;
-    o.r = I.src_r;
-    o.x = I.src_x;
-    o.y = I.src_y;
-    o.cyl = I.g.ocyl_r > 0.0;
-    return o;
+template <class T>
+__global__ void __launch_bounds__(kStripThreads, strip_minb<T>())
+    k_t_step(Plan p, int unit, int rows, StripRun r) {
+    extern __shared__ __align__(32) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    StripWarp<T>& sw = reinterpret_cast<StripWarp<T>*>(smem_raw)[wid];
+    Inst<T>& sI = sw.inst;
+    V4<T>* ring = sw.ring + lane;
+    const int* pre = p.pre + unit * (p.count + 1);
+    const int total = p.total[unit], warps = gridDim.x * wpb;
+    const int nb = __ldg(p.nbase);
+    int cur = -1, su = -1;
+    Strip s;
+    for (int k = r.k0; k < r.k0 + r.n; ++k) {
+        const int src = r.taped ? r.buf + k - 1 : BUF_S0 + ((r.buf + k - 1) & 1);
+        const int dst = r.taped ? r.buf + k : BUF_S0 + ((r.buf + k) & 1);
+        // the objective of the level this step reads; the last level of the launch has its own
+        const int nobj = r.obj && k > r.k0 ? p.total[U_OBJ] : 0;
+        for (int u = wid * gridDim.x + blockIdx.x; u < total + nobj; u += warps) {
+            if (u >= total) {
+                objective_unit<T>(p, u - total, nb + k - 1, src, lane);
+                continue;
+            }
+            if (u != su) {   // a warp with one strip finds it once per launch
+                const int i = find_inst(pre, p.count, u);
+                stage_inst<T>(p, i, cur, sI, lane);
+                s = strip_of<T>(sI, u - __ldg(pre + i), rows, lane);
+                su = u;
+            }
+            const Inst<T>& I = sI;
+            const V4<T>* kus = r.kslot == kBoxBuffer
+                                   ? I.kus : I.kus_tape + (long long)(r.kslot + k) * I.g.boxN;
+            if (s.mode == kInner) step_strip<T, kInner>(I, s, buf(I, src), buf(I, dst), kus, ring);
+            else if (s.mode == kSide) step_strip<T, kSide>(I, s, buf(I, src), buf(I, dst), kus, ring);
+            else step_strip_gen<T>(I, s, buf(I, src), buf(I, dst), kus, ring);
+        }
+        if (k + 1 < r.k0 + r.n && !grid_meet(p, gridDim.x, k - r.k0 + 1)) return;
+    }
 }
 
-__device__ __forceinline__ bool in_target2(const Geom& g, const ObjSrc& o, int x, int y) {
+// ---------------------------------------------------------------- adjoint strips
+
+template <class T>
+__device__ __forceinline__ bool in_target2(const Geom& g, int x, int y) {
     if (x < g.obox[0] || x > g.obox[1] || y < g.obox[2] || y > g.obox[3]) return false;
-    if (o.cyl) {   // the same FP64 test as the host's target list
+    if (g.ocyl_r > 0.0) {   // the same FP64 test as the host's target list
         const double dx = x - g.ocyl_c[0], dy = y - g.ocyl_c[1];
         if (dx * dx + dy * dy > g.ocyl_r * g.ocyl_r) return false;
     }
     return true;
 }
 
-// lambda at a node next to a face plus the transpose of the boundary copies it sources (out of
-// line: few nodes take it, and the tile loop keeps its registers).
-__device__ __noinline__ float4 bcT_fold(const Geom& g, const float4* lam, const ObjAdd<float>& h,
-                                        int x, int y, float4 lv) {
-    V4<float> acc;
-    acc.r = lv.x;
-    acc.x = lv.y;
-    acc.y = lv.z;
-    acc.z = lv.w;
-    bcT_gather<float>(g, (const V4<float>*)lam, h, x, y, 0, acc);
-    return make_float4(acc.r, acc.x, acc.y, acc.z);
+// The transpose of the boundary copies an interior node next to a face sources (Eqs. bc_rho,
+// bc_u): the copied components of those boundary nodes, with their objective source.
+template <class T>
+__device__ __noinline__ V3<T> bcT_general(const Inst<T>& I, const V4<T>* lam, bool on, int x,
+                                          int y, V3<T> v) {
+    const Geom& g = I.g;
+    for_each_sourced_boundary(g, x, y, 0, [&](int bx, int by, int, int f) {
+        V4<T> lb = ldcg4(lam + node_index(g, bx, by, 0));
+        if (on && in_target2<T>(g, bx, by)) {
+            lb.r += I.src_r;
+            lb.x += I.src_x;
+            lb.y += I.src_y;
+        }
+        if (I.bckeep[f]) v.r += lb.r;
+        else if (f < 2) v.x += lb.x;
+        else v.y += lb.y;
+    });
+    return v;
 }
 
-// The same for a node next to a single face (most of them): its one boundary node inline, with
-// the arithmetic of bcT_gather; nodes next to two faces take bcT_fold.
-__device__ __forceinline__ float4 bcT_fold2(const Inst& I, const float4* lam,
-                                            const ObjAdd<float>& h, int x, int y, float4 lv) {
+// The same for a node next to at most one face per axis: its node on the x face, on the y face,
+// and the corner of the two.
+template <class T>
+__device__ __forceinline__ V3<T> bcT_fold(const Inst<T>& I, const V4<T>* lam, bool on, int x,
+                                          int y, V3<T> v) {
     const Geom& g = I.g;
     const int n0 = g.n[0], n1 = g.n[1];
     const bool xl = !g.periodic[0] && x == 1, xh = !g.periodic[0] && x == n0 - 2;
     const bool yl = !g.periodic[1] && y == 1, yh = !g.periodic[1] && y == n1 - 2;
-    if ((int)xl + (int)xh + (int)yl + (int)yh != 1) return bcT_fold(g, lam, h, x, y, lv);
-    const int f = xl ? 0 : (xh ? 1 : (yl ? 2 : 3));
-    const int bx = xl ? 0 : (xh ? n0 - 1 : x), by = yl ? 0 : (yh ? n1 - 1 : y);
-    V4<float> lb;
-    {
-        const float4 t = lam[(long long)by * n0 + bx];
-        lb.r = t.x;
-        lb.x = t.y;
-        lb.y = t.z;
-        lb.z = t.w;
-    }
-    obj_source(g, bx, by, 0, h, lb);
-    if (I.bckeep[f]) lv.x += lb.r;
-    else if (f < 2) lv.y += lb.x;
-    else lv.z += lb.y;
-    return lv;
+    if ((xl && xh) || (yl && yh)) return bcT_general<T>(I, lam, on, x, y, v);
+    const bool ex = xl || xh, ey = yl || yh;
+    const int fx = xh ? 1 : 0, fy = yh ? 3 : 2;
+    const int bx = xl ? 0 : n0 - 1, by = yl ? 0 : n1 - 1;
+    auto fold = [&](bool go, int cx, int cy, int f) {
+        if (!go) return;
+        V4<T> lb = ldcg4(lam + (cy * n0 + cx));
+        if (on && in_target2<T>(g, cx, cy)) {
+            lb.r = add_<T>(lb.r, I.src_r);
+            lb.x = add_<T>(lb.x, I.src_x);
+            lb.y = add_<T>(lb.y, I.src_y);
+        }
+        if (I.bckeep[f]) v.r = add_<T>(v.r, lb.r);
+        else if (f < 2) v.x = add_<T>(v.x, lb.x);
+        else v.y = add_<T>(v.y, lb.y);
+    };
+    fold(ex, bx, y, fx);
+    fold(ey, x, by, fy);
+    fold(ex && ey, bx, by, I.corner[fx + 2 * (fy - 2)]);
+    return v;
 }
 
-// One tile of the adjoint step.  EDGE: the general path (wraps, grid edges, boundary nodes,
-// one-sided boundary rows of the transposed gradient).
-template <int TX, int TY, bool EDGE>
-__device__ __forceinline__ void adj_tile(const Inst& I, int x0, int y0, const ObjSrc& os,
-                                         int lam_in, int lam_out, int sn, int sp, float4* M,
-                                         float* Q) {
-    constexpr int HX = TX + 4, HY = TY + 4, FX = TX + 2, FY = TY + 2, FN = FX * FY;
-    using W = Wts<float, 2>;
+// One strip of the adjoint step.  Row m forms mu at the lane's nodes of row m + 1 and the moments
+// of F~_i(y) = mu_rho(y + c_i) + c_i . mu_u(y + c_i) at row m, then lambda^{n-1} of row m - 1.
+// Per node the directions are grouped by c_x again: the column to the right sends its axis value
+// and, over rows m - 1 and m + 1, the sum and the difference of its two diagonal values, the
+// column to the left the same.  EDGE as in the forward step.
+// lambda, kappa and u_S, u^n (for e) and u^{n-1} pass through rings as in the forward step.
+constexpr int kARing = 4, kAAhead = kARing - 1;
+
+template <class T, int MODE>
+__device__ __forceinline__ void adj_strip(const Inst<T>& I, const Strip& s, bool on,
+                                          const V4<T>* lam, V4<T>* out, const V4<T>* __restrict__ sn,
+                                          const V4<T>* __restrict__ sp,
+                                          const V4<T>* __restrict__ kus, T* __restrict__ eo,
+                                          V4<T>* ring) {
+    using W = Wts<T, 2>;
+    constexpr bool GEN = MODE == kGeneral, SIDE = MODE != kInner;
     const Geom& g = I.g;
     const int n0 = g.n[0], n1 = g.n[1];
-    const float4* lam = (const float4*)I.bufs[lam_in];
-    const V4<float>* su = (const V4<float>*)I.bufs[sn];
-    // tiles whose halo misses the footprint box (the target) skip those per-node tests
-    const bool tbox = EDGE || meets_box(g, x0 - 2, x0 + TX + 1, y0 - 2, y0 + TY + 1);
-    const bool ttgt = os.on && (EDGE || meets_target(g, x0 - 2, x0 + TX + 1, y0 - 2, y0 + TY + 1));
-    // tiles whose halo holds a node next to a face: such a node first collects the transpose of
-    // the boundary copies it sources (Eqs. bc_rho, bc_u; boundary nodes are read only)
-    const bool tbc = EDGE || x0 - 2 <= 1 || x0 + TX + 1 >= n0 - 2 || y0 - 2 <= 1 ||
-                     y0 + TY + 1 >= n1 - 2;
-    ObjAdd<float> bsrc;   // the objective source of the boundary nodes inside the target
-    bsrc.on = os.on;
-    bsrc.r = os.r;
-    bsrc.x = os.x;
-    bsrc.y = os.y;
-    bsrc.z = 0.f;
-    // 1. mu on the tile and a two-cell halo; e on the tile's own box nodes
-    for (int k = threadIdx.x; k < HX * HY; k += NT) {
-        const int ly = k / HX, lx = k - ly * HX;
-        int gx = x0 - 2 + lx, gy = y0 - 2 + ly;
-        if (EDGE) {
-            if (g.periodic[0]) gx = wrap_any(gx, n0);
-            if (g.periodic[1]) gy = wrap_any(gy, n1);
+    const bool p0 = GEN && g.periodic[0], p1 = GEN && g.periodic[1];
+    const int ya = s.ya, yb = s.yb, x = s.x;
+    if (ya > yb) return;   // uniform
+    const bool own = s.own, xin = !SIDE || s.in;
+    const bool icol = !SIDE || p0 || (x >= 1 && x <= n0 - 2);   // not on an x face, in the grid
+    const bool xface = SIDE && !p0 && (!GEN || __any_sync(FULL, x == 0 || x == n0 - 1));
+    const bool xnear = GEN && !p0 && __any_sync(FULL, x == 1 || x == n0 - 2);
+    // kSide: the face whose column a node next to it collects
+    const int wf = SIDE && !GEN ? (x == 1 ? 0 : (x == n0 - 2 ? 1 : -1)) : -1;
+    const int bx = x - g.blo[0], bn0 = g.bn[0], bn1 = g.bn[1], by0 = g.blo[1];
+    const bool bcol = g.boxN > 0 && xin && bx >= 0 && bx < bn0;
+    // (a halo row of a wrapping strip may fall in the box from the other side)
+    const bool bany = __any_sync(FULL, bcol) && (p1 || (ya - 2 < by0 + bn1 && yb + 2 >= by0));
+    const int ty0 = g.obox[2], ty1 = g.obox[3];
+    const bool tany = on && __any_sync(FULL, xin && x >= g.obox[0] && x <= g.obox[1]) &&
+                      (p1 || (ya - 2 <= ty1 && yb + 2 >= ty0));
+    const T* ks_st = GEN ? (const T*)g.ks : nullptr;
+    const T A9 = I.A9;
+    // coefficients of the face columns' 9 S~ in the x part of the transposed gradient: the
+    // one-sided stencil less the central one, for columns 0, 1, 2 and n-1, n-2, n-3
+    T cxl = (T)0, cxh = (T)0;
+    int lane_l = 0, lane_h = 0;
+    if (xface) {
+        const int dl = x, dh = n0 - 1 - x;
+        const unsigned ml = __ballot_sync(FULL, dl == 0), mh = __ballot_sync(FULL, dh == 0);
+        lane_l = ml ? __ffs(ml) - 1 : 0;
+        lane_h = mh ? __ffs(mh) - 1 : 0;
+        if (ml) cxl = dl == 0 ? (T)-3 : (dl == 1 ? (T)3 : (dl == 2 ? (T)-1 : (T)0));
+        if (mh) cxh = dh == 0 ? (T)3 : (dh == 1 ? (T)-3 : (dh == 2 ? (T)1 : (T)0));
+    }
+    // first and last moment row: the boundary rows' one-sided parts reach rows 2 and n - 3, also
+    // where the strip starts or ends there
+    const int ma = GEN && !p1 && ya == 2 ? 0 : ya - 1;
+    const int mb = GEN && !p1 && yb == n1 - 3 ? n1 - 1 : yb + 1;
+    V4<T>* ringk = ring + kARing * 32;
+    V4<T>* ringn = ring + 2 * kARing * 32;
+    V4<T>* ringp = ring + 3 * kARing * 32;
+    const V4<T>* lcol = lam + (xin ? x : 0);
+    const V4<T>* kcol = kus + (bcol ? bx : 0);
+    const V4<T>* ncol = sn + (own ? x : 0);
+    const V4<T>* pcol = sp + (own ? x : 0);
+    V4<T>* ocl = out + (own ? x : 0);
+    auto wrap = [&](int row) { return p1 ? row + (row < 0 ? n1 : (row >= n1 ? -n1 : 0)) : row; };
+    struct Q {
+        V3<T> l, k, u;   // lambda, (kappa, u_S), u^n of one row
+    };
+    auto direct = [&](int row0) -> Q {   // (u^n is for e on the strip's own rows, from the ring)
+        Q q;
+        q.l.r = q.l.x = q.l.y = q.k.r = q.k.x = q.k.y = q.u.r = q.u.x = q.u.y = (T)0;
+        const int row = wrap(row0), kr = row - by0;
+        if (xin && (!GEN || (row >= 0 && row < n1))) q.l = ldcg3<V3<T>>(lcol + row * n0);
+        if (bany && bcol && (unsigned)kr < (unsigned)bn1) q.k = ldg3<V3<T>>(kcol + kr * bn0);
+        return q;
+    };
+    // a row of lambda, kappa, u_S and u^n, and u^{n-1} two rows below it, as one copy group
+    auto issue = [&](int row0) {
+        const int slot = (row0 & (kARing - 1)) * 32;
+        const int row = wrap(row0);
+        const bool go = row0 <= mb + 1, in = xin && (!GEN || (row >= 0 && row < n1));
+        cp_record<T>(ring + slot, lcol + (GEN && !in ? 0 : row * n0), go, in);
+        if (bany) {
+            const int kr = row - by0;
+            const bool kin = bcol && (unsigned)kr < (unsigned)bn1;
+            cp_record<T>(ringk + slot, kcol + (kin ? kr * bn0 : 0), go, kin);
+            const bool nin = kin && own && row0 >= ya && row0 <= yb;
+            cp_record<T>(ringn + slot, ncol + (nin ? row * n0 : 0), go, nin);
         }
-        float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (!EDGE || (gx >= 0 && gx < n0 && gy >= 0 && gy < n1 && !is_boundary(g, gx, gy, 0))) {
-            const long long gm = (long long)gy * n0 + gx;
-            float4 lv = __ldg(lam + gm);
-            if (tbc && sources_boundary(g, gx, gy, 0)) lv = bcT_fold2(I, lam, bsrc, gx, gy, lv);
-            float lr = lv.x, lux = lv.y, luy = lv.z;
-            if (ttgt && in_target2(g, os, gx, gy)) {
-                lr += os.r;
-                lux += os.x;
-                luy += os.y;
-            }
-            long long bi;
-            const float kst = g.ks ? ((const float*)g.ks)[gm] : 0.f;
-            if (tbox && in_box(g, gx, gy, 0, bi)) {
-                const V4<float> ks = I.kus[bi];
-                const float inv = 1.f / (1.f + ks.r + kst);
-                lux *= inv;
-                luy *= inv;
-                const bool own = lx >= 2 && lx < TX + 2 && ly >= 2 && ly < TY + 2;
-                if (own) {
-                    const V4<float> un = su[gm];
-                    I.e[bi] = lux * (ks.x - un.x) + luy * (ks.y - un.y);
+        const int pr = row0 - 2;
+        cp_record<T>(ringp + (pr & (kARing - 1)) * 32, pcol + (pr >= ya && pr <= yb ? pr * n0 : 0),
+                     pr >= ya && pr <= yb, own);
+        cp_commit();
+    };
+    // mu of a row from its loaded values: 0 on boundary nodes and outside the grid; the
+    // transposed boundary copies, the objective source, the Brinkman transpose, and e on own nodes
+    auto to_mu = [&](int row0, const Q& q) -> V3<T> {
+        V3<T> v = q.l;
+        const int row = wrap(row0);
+        if (SIDE && !GEN) {   // the face column's lambda sits in the lane beside
+            V3<T> b;
+            const bool hi = wf == 1;
+            const T br = from_left(v.r), bxv = from_left(v.x);
+            const T cr = from_right(v.r), cx = from_right(v.x);
+            b.r = hi ? cr : br;
+            b.x = hi ? cx : bxv;
+            if (wf >= 0) {
+                if (on && in_target2<T>(g, hi ? n0 - 1 : 0, row)) {
+                    b.r = add_<T>(b.r, I.src_r);
+                    b.x = add_<T>(b.x, I.src_x);
                 }
-            } else if (kst != 0.f) {
-                const float inv = 1.f / (1.f + kst);
-                lux *= inv;
-                luy *= inv;
+                if (I.bckeep[wf]) v.r = add_<T>(v.r, b.r);
+                else v.x = add_<T>(v.x, b.x);
             }
-            m = make_float4(lr, lux, luy, 0.f);
         }
-        M[k] = m;
-    }
-    __syncthreads();
-    // 2. moments of F~_i(y) = mu_rho(y + c_i) + c_i . mu_u(y + c_i) on the tile and rim
-    for (int k = threadIdx.x; k < FN; k += NT) {
-        const int fy = k / FX, fx = k - fy * FX;
-        const int s = (fy + 1) * HX + fx + 1;
-        const float4 c0 = M[s];
-        const float4 xp = M[s + 1], xm = M[s - 1], yp = M[s + HX], ym = M[s - HX];
-        const float4 pp = M[s + HX + 1], mp = M[s + HX - 1], mm = M[s - HX - 1],
-                     pm = M[s - HX + 1];
-        // F~ of the eight moving directions, then R~, 3 U~ and 9 S~ with the weight products
-        // of Wts<float, 2>
-        const float fxp = xp.x + xp.y, fxm = xm.x - xm.y, fyp = yp.x + yp.z, fym = ym.x - ym.z;
-        const float fpp = pp.x + pp.y + pp.z, fmp = mp.x - mp.y + mp.z;
-        const float fmm = mm.x - mm.y - mm.z, fpm = pm.x + pm.y - pm.z;
-        const float dsum = (fpp + fmp) + (fmm + fpm);
-        Q[k] = W::w0 * c0.x + W::w1 * ((fxp + fxm) + (fyp + fym)) + W::w2 * dsum;
-        Q[FN + k] = W::w3_1 * (fxp - fxm) + W::w3_2 * ((fpp - fmp) + (fpm - fmm));
-        Q[2 * FN + k] = W::w3_1 * (fyp - fym) + W::w3_2 * ((fpp + fmp) - (fmm + fpm));
-        Q[3 * FN + k] = W::s_1 * (fxp + fxm) + W::s_2 * dsum;
-        Q[4 * FN + k] = W::s_2 * ((fpp - fmp) + (fmm - fpm));
-        Q[5 * FN + k] = W::s_1 * (fyp + fym) + W::s_2 * dsum;
-    }
-    __syncthreads();
-    // 3. lambda^{n-1} = (R~, 3 U~ - 3 R~ u + 9 S~ u + D^T (2 A S~)) on the tile; Q holds
-    //    R~, 3 U~ and 9 S~, so the transposed gradient takes 2 A / 9 times the stored values
-    const V4<float>* sprev = (const V4<float>*)I.bufs[sp];
-    V4<float>* out = (V4<float>*)I.bufs[lam_out];
-    const float twoA = (float)(2.0 * g.A / 9.0);
-    for (int k = threadIdx.x; k < TX * TY; k += NT) {
-        const int ty = k / TX, tx = k - ty * TX;
-        const int x = x0 + tx, y = y0 + ty;
-        if (EDGE && (x < 0 || x >= n0 || y < 0 || y >= n1)) continue;
-        const int q = (ty + 1) * FX + tx + 1;
-        const V4<float> v = sprev[(long long)y * n0 + x];
-        const float R = Q[q], Ux = Q[FN + q], Uy = Q[2 * FN + q];
-        const float Sxx = Q[3 * FN + q], Sxy = Q[4 * FN + q], Syy = Q[5 * FN + q];
-        const float R3 = 3.f * R;
-        float lx = Ux - R3 * v.x;
-        float ly = Uy - R3 * v.y;
-        lx += Sxx * v.x;
-        lx += Sxy * v.y;
-        ly += Sxy * v.x;
-        ly += Syy * v.y;
-        // transposed gradient: rows y' = x - kk e_b whose stencil reaches x; phi_ab = 2 A S~_ab,
-        // b = x uses (Sxx, Sxy), b = y uses (Sxy, Syy)
-        float ax = 0.f, ay = 0.f;
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const int c = b == 0 ? x : y, nn = b == 0 ? n0 : n1, per = g.periodic[b];
-            const int step = b == 0 ? 1 : FX;
-#pragma unroll
-            for (int kk = -2; kk <= 2; ++kk) {
-                float cf;
-                if (EDGE) {
-                    int yi = c - kk;
-                    if (per) yi = wrap_any(yi, nn);
-                    else if (yi < 0 || yi >= nn) continue;
-                    cf = deriv_coef_f(yi, nn, per, kk);
-                    if (cf == 0.f) continue;
-                } else {
-                    if (kk != 1 && kk != -1) continue;
-                    cf = kk == 1 ? 0.5f : -0.5f;
+        if (SIDE && !(icol && (!GEN || p1 || (row >= 1 && row <= n1 - 2)))) {
+            v.r = v.x = v.y = (T)0;
+        } else {
+            if (GEN && (xnear || (!p1 && (row == 1 || row == n1 - 2))))
+                v = bcT_fold<T>(I, lam, on, x, row, v);
+            if (tany && row >= ty0 && row <= ty1 && in_target2<T>(g, x, row)) {
+                v.r = add_<T>(v.r, I.src_r);
+                v.x = add_<T>(v.x, I.src_x);
+                v.y = add_<T>(v.y, I.src_y);
+            }
+            if (bany || (GEN && ks_st)) {
+                const T kst = GEN && ks_st ? ks_st[row * n0 + x] : (T)0;
+                const int kr = row - by0;
+                const bool box = bany && bcol && (unsigned)kr < (unsigned)bn1;
+                if (box || (GEN && kst != (T)0)) {
+                    T den = add_<T>((T)1, q.k.r);
+                    if (GEN) den = add_<T>(den, kst);
+                    const T inv = inv_<T>(den);
+                    v.x = mul_<T>(v.x, inv);
+                    v.y = mul_<T>(v.y, inv);
+                    if (box && own && row0 >= ya && row0 <= yb)
+                        eo[kr * bn0 + bx] = fma_<T>(v.x, sub_<T>(q.k.x, q.u.x),
+                                                    mul_<T>(v.y, sub_<T>(q.k.y, q.u.y)));
                 }
-                const int qq = q - kk * step;
-                // rows two nodes away are boundary rows, which the tile origin keeps inside
-                // the tile; the test only keeps a shared-memory read in bounds regardless
-                if (EDGE && (qq < 0 || qq >= FN)) continue;
-                const float pa = twoA * Q[(b == 0 ? 3 : 4) * FN + qq];
-                const float pb = twoA * Q[(b == 0 ? 4 : 5) * FN + qq];
-                ax += cf * pa;
-                ay += cf * pb;
             }
         }
-        V4<float> o;
-        o.r = R;
-        o.x = lx + ax;
-        o.y = ly + ay;
-        o.z = 0.f;
-        out[(long long)y * n0 + x] = o;
+        return v;
+    };
+    // row m - 1 (its lower diagonal and axis values), row m (its axis values)
+    T d_P, d_Q, d_y, c_r, c_a, c_b, c_P, c_Q, c_y;
+    {
+        const Q qa = direct(ma - 1), qb = direct(ma);
+        for (int i = 1; i <= kARing; ++i) issue(ma + i);
+        const V3<T> a = to_mu(ma - 1, qa), b = to_mu(ma, qb);
+        d_P = sub_<T>(add_<T>(a.r, a.x), a.y);
+        d_Q = sub_<T>(sub_<T>(a.r, a.x), a.y);
+        d_y = sub_<T>(a.r, a.y);
+        c_r = b.r;
+        c_a = add_<T>(b.r, b.x);
+        c_b = sub_<T>(b.r, b.x);
+        c_P = sub_<T>(c_a, b.y);
+        c_Q = sub_<T>(c_b, b.y);
+        c_y = sub_<T>(b.r, b.y);
     }
-    __syncthreads();
-}
-
-template <int TX, int TY>
-__global__ void __launch_bounds__(NT) k_t_adj2d(Plan p, const int* __restrict__ pre, int total,
-                                                int noff, int lam_in, int lam_out, int sn,
-                                                int sp, int kslot) {
-    constexpr int HX = TX + 4, HY = TY + 4;
-    extern __shared__ float4 smem[];
-    float4* M = smem;                          // HY x HX: mu (rho, x, y, -)
-    float* Q = (float*)(smem + HX * HY);       // 6 planes of FY x FX: R~, 3 U~, 9 S~ (xx, xy, yy)
-    const int n = step_of(p, noff);
-    __shared__ Inst sI;
-    int cur = -1;
-    ObjSrc os;
-    for (int u = blockIdx.x; u < total; u += gridDim.x) {
-        const int i = find_inst(pre, p.count, u);
-        if (i != cur) {
-            stage_inst(p, i, cur, sI, kslot);
-            os = obj_src(sI, n);
+    // moments of row m - 1, its x differences, 9 S~ of row m - 2 and of boundary row 0
+    T R = (T)0, Ux = (T)0, Uy = (T)0, Sxx = (T)0, Sxy = (T)0, Syy = (T)0, gx = (T)0, gy = (T)0;
+    T Sxy2 = (T)0, Syy2 = (T)0, S0xy = (T)0, S0yy = (T)0;
+    V4<T> o;
+    o.r = o.x = o.y = o.z = (T)0;
+    auto march = [&](int m, auto emit) {
+        constexpr bool EMIT = decltype(emit)::value;
+        const int y = m - 1;   // output row
+        cp_wait<kAAhead>();    // row m + 1 has landed
+        Q q;
+        {
+            const int slot = ((m + 1) & (kARing - 1)) * 32;
+            const V4<T> l = lds4(ring + slot);
+            q.l = V3<T>{l.r, l.x, l.y};
+            q.k.r = q.k.x = q.k.y = q.u.r = q.u.x = q.u.y = (T)0;
+            if (bany) {
+                const V4<T> k = lds4(ringk + slot), n = lds4(ringn + slot);
+                q.k = V3<T>{k.r, k.x, k.y};
+                q.u = V3<T>{n.r, n.x, n.y};
+            }
         }
-        int x0, y0;
-        tile_xy<TX, TY>(sI.g, u - pre[i], x0, y0);
-        if (interior_tile<TX, TY>(sI.g, x0, y0))
-            adj_tile<TX, TY, false>(sI, x0, y0, os, lam_in, lam_out, sn, sp, M, Q);
-        else
-            adj_tile<TX, TY, true>(sI, x0, y0, os, lam_in, lam_out, sn, sp, M, Q);
+        V4<T> u;   // u^{n-1} of the output row
+        if (EMIT) u = lds4(ringp + (y & (kARing - 1)) * 32);
+        issue(m + 1 + kARing);   // into the slots just read
+        const V3<T> v = to_mu(m + 1, q);
+        const T va = add_<T>(v.r, v.x), vb = sub_<T>(v.r, v.x);
+        const T uP = add_<T>(va, v.y), uQ = add_<T>(vb, v.y), uy = add_<T>(v.r, v.y);
+        // from the right (c_x = +1) and left (c_x = -1) columns
+        const T Ap = from_right(c_a), Am = from_left(c_b);
+        const T Dp = from_right(add_<T>(uP, d_P)), Ep = from_right(sub_<T>(uP, d_P));
+        const T Dm = from_left(add_<T>(uQ, d_Q)), Em = from_left(sub_<T>(uQ, d_Q));
+        const T ax = add_<T>(Ap, Am), ay = add_<T>(uy, d_y), ds = add_<T>(Dp, Dm);
+        const T nR = fma_<T>(W::w2, ds, fma_<T>(W::w1, add_<T>(ax, ay), mul_<T>(W::w0, c_r)));
+        const T nUx = fma_<T>(W::w3_1, sub_<T>(Ap, Am), mul_<T>(W::w3_2, sub_<T>(Dp, Dm)));
+        const T nUy = fma_<T>(W::w3_1, sub_<T>(uy, d_y), mul_<T>(W::w3_2, add_<T>(Ep, Em)));
+        T nSxx = fma_<T>(W::s_2, ds, ax), nSyy = fma_<T>(W::s_2, ds, ay);   // s_1 = 1
+        T nSxy = mul_<T>(W::s_2, sub_<T>(Ep, Em));
+        if (SIDE && (!xin || (GEN && !p1 && (m < 0 || m >= n1)))) nSxx = nSyy = nSxy = (T)0;
+        T ngx = sub_<T>(from_left(nSxx), from_right(nSxx));
+        T ngy = sub_<T>(from_left(nSxy), from_right(nSxy));
+        if (xface) {
+            const T lxx = __shfl_sync(FULL, nSxx, lane_l), lxy = __shfl_sync(FULL, nSxy, lane_l);
+            const T hxx = __shfl_sync(FULL, nSxx, lane_h), hxy = __shfl_sync(FULL, nSxy, lane_h);
+            ngx = fma_<T>(cxh, hxx, fma_<T>(cxl, lxx, ngx));
+            ngy = fma_<T>(cxh, hxy, fma_<T>(cxl, lxy, ngy));
+        }
+        if (GEN && !p1) {
+            if (m == 0) {
+                S0xy = nSxy;
+                S0yy = nSyy;
+            }
+            if (m == n1 - 1 && y - 1 >= ya && own) {
+                // the high boundary row's one-sided part reaches row n - 3, written by the
+                // previous iteration: add it now
+                o.x = fma_<T>(A9, nSxy, o.x);
+                o.y = fma_<T>(A9, nSyy, o.y);
+                stg4(ocl + (y - 1) * n0, o);
+            }
+        }
+        if (EMIT && (!GEN || y <= yb)) {   // uniform
+            T tx = add_<T>(gx, sub_<T>(Sxy2, nSxy)), ty = add_<T>(gy, sub_<T>(Syy2, nSyy));
+            if (GEN && !p1) {
+                if (y <= 2) {
+                    const T cy = y == 0 ? (T)-3 : (y == 1 ? (T)3 : (T)-1);
+                    tx = fma_<T>(cy, S0xy, tx);
+                    ty = fma_<T>(cy, S0yy, ty);
+                }
+                if (y == n1 - 1) {
+                    tx = fma_<T>((T)3, Sxy, tx);
+                    ty = fma_<T>((T)3, Syy, ty);
+                } else if (y == n1 - 2) {
+                    tx = fma_<T>((T)-3, nSxy, tx);
+                    ty = fma_<T>((T)-3, nSyy, ty);
+                }
+            }
+            const T R3 = mul_<T>((T)3, R);
+            T lx = fma_<T>(-R3, u.x, Ux), ly = fma_<T>(-R3, u.y, Uy);
+            lx = fma_<T>(Sxy, u.y, fma_<T>(Sxx, u.x, lx));
+            ly = fma_<T>(Syy, u.y, fma_<T>(Sxy, u.x, ly));
+            o.r = R;
+            o.x = fma_<T>(A9, tx, lx);
+            o.y = fma_<T>(A9, ty, ly);
+            if (own) stg4(ocl + y * n0, o);
+        }
+        Sxy2 = Sxy;
+        Syy2 = Syy;
+        R = nR;
+        Ux = nUx;
+        Uy = nUy;
+        Sxx = nSxx;
+        Sxy = nSxy;
+        Syy = nSyy;
+        gx = ngx;
+        gy = ngy;
+        d_P = c_P;
+        d_Q = c_Q;
+        d_y = c_y;
+        c_r = v.r;
+        c_a = va;
+        c_b = vb;
+        c_P = sub_<T>(va, v.y);
+        c_Q = sub_<T>(vb, v.y);
+        c_y = sub_<T>(v.r, v.y);
+    };
+    int m = ma;
+    for (; m <= ya; ++m) march(m, std::false_type{});   // two rows, three from boundary row 0
+#pragma unroll 2
+    for (; m <= mb; ++m) march(m, std::true_type{});
+    cp_wait<0>();
+}
+
+template <class T>
+__device__ __noinline__ void adj_strip_gen(const Inst<T>& I, const Strip& s, bool on,
+                                            const V4<T>* lam, V4<T>* out, const V4<T>* sn,
+                                            const V4<T>* sp, const V4<T>* kus, T* eo,
+                                            V4<T>* ring) {
+    adj_strip<T, kGeneral>(I, s, on, lam, out, sn, sp, kus, eo, ring);
+}
+
+template <class T>
+__global__ void __launch_bounds__(kStripThreads, strip_minb<T>())
+    k_t_adj(Plan p, int unit, int rows, StripRun r) {
+    extern __shared__ __align__(32) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    StripWarp<T>& sw = reinterpret_cast<StripWarp<T>*>(smem_raw)[wid];
+    Inst<T>& sI = sw.inst;
+    V4<T>* ring = sw.ring + lane;
+    const int* pre = p.pre + unit * (p.count + 1);
+    const int total = p.total[unit], warps = gridDim.x * wpb;
+    const int nb = __ldg(p.nbase);
+    int cur = -1, su = -1;
+    Strip s;
+    for (int j = 0; j < r.n; ++j) {
+        const int k = r.k0 - j, par = (r.buf + j) & 1;
+        for (int u = wid * gridDim.x + blockIdx.x; u < total; u += warps) {
+            if (u != su) {   // a warp with one strip finds it once per launch
+                const int i = find_inst(pre, p.count, u);
+                stage_inst<T>(p, i, cur, sI, lane);
+                s = strip_of<T>(sI, u - __ldg(pre + i), rows, lane);
+                su = u;
+            }
+            const Inst<T>& I = sI;
+            const long long bn = I.g.boxN;
+            const V4<T>* kus =
+                r.kslot == kBoxBuffer ? I.kus : I.kus_tape + (long long)(r.kslot + k) * bn;
+            const bool on = nb + k >= I.win_begin && nb + k <= I.win_end;
+            T* eo = I.e + (long long)(r.eslot + k) * bn;
+            const V4<T>* lam = buf(I, BUF_LAM0 + par);
+            V4<T>* lo = buf(I, BUF_LAM0 + 1 - par);
+            const V4<T>*sn = buf(I, r.tape + k), *sp = buf(I, r.tape + k - 1);
+            if (s.mode == kInner) adj_strip<T, kInner>(I, s, on, lam, lo, sn, sp, kus, eo, ring);
+            else if (s.mode == kSide) adj_strip<T, kSide>(I, s, on, lam, lo, sn, sp, kus, eo, ring);
+            else adj_strip_gen<T>(I, s, on, lam, lo, sn, sp, kus, eo, ring);
+        }
+        if (j + 1 < r.n && !grid_meet(p, gridDim.x, j + 1)) return;
     }
 }
 
-// Row-marching step configurations 5..8: threads per strip and rows per chunk.
-template <int C>
-struct RowCfg {
-    static constexpr int NTH = tile_tx(C) + 2, YC = tile_ty(C);
-};
-
-template <int C>
-int occ_rows() {
-    int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &b, k_t_step2d_rows<RowCfg<C>::NTH, RowCfg<C>::YC>, RowCfg<C>::NTH, 0);
-    return b;
-}
-
-template <int C>
-cudaError_t rows_cfg(const Plan& p, int src, int dst, int kslot, cudaStream_t st) {
-    const int unit = U_TILE0 + C;
-    if (p.total[unit] == 0) return cudaSuccess;
-    k_t_step2d_rows<RowCfg<C>::NTH, RowCfg<C>::YC><<<p.grid[unit], RowCfg<C>::NTH, 0, st>>>(
-        p, p.pre + unit * (p.count + 1), p.total[unit], src, dst, kslot);
-    return cudaGetLastError();
-}
-
-template <int C>
-struct Cfg {
-    static constexpr int TX = tile_tx(C), TY = tile_ty(C);
-    static constexpr size_t step_smem = (size_t)(TX + 4) * (TY + 4) * 16 + (size_t)8 * (TX + 2) * (TY + 2) * 4;
-    static constexpr size_t adj_smem = (size_t)(TX + 4) * (TY + 4) * 16 + (size_t)6 * (TX + 2) * (TY + 2) * 4;
-};
-
-template <int C>
-int occ_step() {
-    int b = 0;
-    cudaFuncSetAttribute(k_t_step2d<Cfg<C>::TX, Cfg<C>::TY>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<C>::step_smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_t_step2d<Cfg<C>::TX, Cfg<C>::TY>, NT,
-                                                  Cfg<C>::step_smem);
-    return b;
-}
-template <int C>
-int occ_adj() {
-    int b = 0;
-    cudaFuncSetAttribute(k_t_adj2d<Cfg<C>::TX, Cfg<C>::TY>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<C>::adj_smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_t_adj2d<Cfg<C>::TX, Cfg<C>::TY>, NT,
-                                                  Cfg<C>::adj_smem);
-    return b;
-}
+// ---------------------------------------------------------------- host side
 
 int sm_count() {
     int dev = 0, sms = 0;
@@ -1011,92 +1247,130 @@ int cap_grid(long long units, int per_sm) {
     return (int)std::max(1LL, std::min(units, g));
 }
 
-template <int C>
-cudaError_t step_cfg(const Plan& p, int src, int dst, int kslot, cudaStream_t st) {
-    const int unit = U_TILE0 + C;
-    if (p.total[unit] == 0) return cudaSuccess;
-    k_t_step2d<Cfg<C>::TX, Cfg<C>::TY><<<p.grid[unit], NT, Cfg<C>::step_smem, st>>>(
-        p, p.pre + unit * (p.count + 1), p.total[unit], src, dst, kslot);
-    return cudaGetLastError();
-}
-
-template <int C>
-cudaError_t adj_cfg(const Plan& p, int noff, int li, int lo, int sn, int sp, int kslot,
-                    cudaStream_t st) {
-    const int unit = U_TILE0 + C;
-    if (p.total[unit] == 0) return cudaSuccess;
-    k_t_adj2d<Cfg<C>::TX, Cfg<C>::TY><<<p.grid[U_COUNT + C], NT, Cfg<C>::adj_smem, st>>>(
-        p, p.pre + unit * (p.count + 1), p.total[unit], noff, li, lo, sn, sp, kslot);
-    return cudaGetLastError();
+// Blocks and warps per block of a strip kernel over `units` strips: the strips spread over all
+// SMs, eight warps to a block at most; a launch of several steps keeps every block resident and
+// loops over the rest.
+template <class K>
+cudaError_t launch_strips(K kern, size_t warp_bytes, long long units, bool meet, const Plan& p,
+                          int unit, int rows, const StripRun& r, cudaStream_t st) {
+    const int sms = sm_count();
+    const int wpb = (int)std::min<long long>(kStripThreads / 32, (units + sms - 1) / sms);
+    const int w = units <= kStripThreads / 32 ? (int)units : wpb;   // a few strips: one block
+    const size_t smem = warp_bytes * w;
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(
+            (const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    long long grid = (units + w - 1) / w;
+    if (meet && grid > sms) {
+        int per = 0;
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 32 * w, smem);
+        if (e != cudaSuccess) return e;
+        grid = std::min<long long>(grid, (long long)sms * std::max(per, 1));
+    }
+    if (!meet || grid == 1) {
+        kern<<<(unsigned)grid, 32 * w, smem, st>>>(p, unit, rows, r);
+        return cudaGetLastError();
+    }
+    cudaError_t e = cudaMemsetAsync(p.bar, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    Plan pp = p;
+    int un = unit, ro = rows;
+    StripRun rr = r;
+    void* args[] = {&pp, &un, &ro, &rr};
+    return cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)grid), dim3(32 * w), args,
+                                       smem, st);
 }
 
 }  // namespace
 
-void plan_grids(Plan& p) {
-    int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_t_transfer2d, NT, 0);
-    p.grid[U_BOX] = cap_grid(p.total[U_BOX], b);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_t_design_pos, NT, 0);
-    p.grid[U_DCOL] = cap_grid(p.total[U_DCOL], b);
-    p.grid[U_INST] = std::max(1, p.count);
-    const int os[kTileCfgs] = {occ_step<0>(), occ_step<1>(), occ_step<2>(), occ_step<3>(),
-                               occ_step<4>(), occ_rows<5>(),  occ_rows<6>(),  occ_rows<7>(),
-                               occ_rows<8>()};
-    const int oa[kAdjCfgs] = {occ_adj<0>(), occ_adj<1>(), occ_adj<2>(), occ_adj<3>(),
-                              occ_adj<4>()};
-    for (int c = 0; c < kTileCfgs; ++c) p.grid[U_TILE0 + c] = cap_grid(p.total[U_TILE0 + c], os[c]);
-    for (int c = 0; c < kAdjCfgs; ++c) p.grid[U_COUNT + c] = cap_grid(p.total[U_TILE0 + c], oa[c]);
-    cudaGetLastError();
+int default_strips(const Plan& p, int type_size) {
+    // the shortest strips that are all resident at once: a small grid's step is one march, whose
+    // length is its latency (512^2: 2, 4, 8, 16, 32 rows took 29.6, 25.0, 27.8, 36.4, 54.1 ms over
+    // 600 steps and their adjoint); but where taller ones fit one block, whose barrier is its own,
+    // those
+    const int per = kStripThreads / 32;
+    const int room = sm_count() * per * (type_size == 4 ? strip_minb<float>() : strip_minb<double>());
+    int k = 0;
+    while (k + 1 < kStripCfgs && p.total[U_STRIP0 + k] > room) ++k;
+    if (p.total[U_STRIP0 + k] > per && k + 1 < kStripCfgs && p.total[U_STRIP0 + k + 1] <= per) ++k;
+    return k;
 }
 
-cudaError_t launch_t_design_pos(const Plan& p, int noff, cudaStream_t st) {
-    if (p.total[U_DCOL] == 0) return cudaSuccess;
-    k_t_design_pos<<<p.grid[U_DCOL], NT, 0, st>>>(p, noff);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_t_transfer2d(const Plan& p, int noff, int kslot, bool next, cudaStream_t st) {
-    if (p.total[U_BOX] == 0) return cudaSuccess;
-    k_t_transfer2d<<<p.grid[U_BOX], NT, 0, st>>>(p, noff, kslot, next ? 1 : 0);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_t_step2d(const Plan& p, int cfg, int src, int dst, int kslot,
-                            cudaStream_t st) {
-    switch (cfg) {
-        case 0: return step_cfg<0>(p, src, dst, kslot, st);
-        case 1: return step_cfg<1>(p, src, dst, kslot, st);
-        case 2: return step_cfg<2>(p, src, dst, kslot, st);
-        case 3: return step_cfg<3>(p, src, dst, kslot, st);
-        case 4: return step_cfg<4>(p, src, dst, kslot, st);
-        case 5: return rows_cfg<5>(p, src, dst, kslot, st);
-        case 6: return rows_cfg<6>(p, src, dst, kslot, st);
-        case 7: return rows_cfg<7>(p, src, dst, kslot, st);
-        case 8: return rows_cfg<8>(p, src, dst, kslot, st);
-        default: return cudaErrorInvalidValue;
+template <class T>
+cudaError_t launch_t_transfer(const Plan& p, int noff, int n, int kslot0, cudaStream_t st) {
+    if (p.total[U_DCOL] == 0 || p.total[U_BOX] == 0 || n <= 0) return cudaSuccess;
+    k_t_design_pos<T><<<cap_grid((long long)p.total[U_DCOL] * n, 8), NT, 0, st>>>(p, noff, n);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    constexpr size_t smem = sizeof(TrSmem<T>);
+    static std::atomic<unsigned> attr{0};
+    if (!device_done(attr)) {
+        e = cudaFuncSetAttribute(k_t_transfer2d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem);
+        if (e != cudaSuccess) return e;
+        device_mark(attr);
     }
+    const long long units = (long long)p.total[U_BOX] * n;
+    k_t_transfer2d<T><<<cap_grid(units, sizeof(T) == 4 ? 8 : 4), NT, smem, st>>>(p, noff, n, kslot0);
+    return cudaGetLastError();
 }
 
+template <class T>
+cudaError_t launch_t_step(const Plan& p, int cfg, const StripRun& r, cudaStream_t st) {
+    if (cfg < 0 || cfg >= kStripCfgs) return cudaErrorInvalidValue;
+    const int unit = U_STRIP0 + cfg;
+    return launch_strips(k_t_step<T>, sizeof(StripWarp<T>),
+                         p.total[unit] + (r.obj && r.n > 1 ? p.total[U_OBJ] : 0), r.n > 1, p, unit,
+                         strip_rows(cfg), r, st);
+}
+
+template <class T>
+cudaError_t launch_t_adj(const Plan& p, int cfg, const StripRun& r, cudaStream_t st) {
+    if (cfg < 0 || cfg >= kStripCfgs) return cudaErrorInvalidValue;
+    const int unit = U_STRIP0 + cfg;
+    return launch_strips(k_t_adj<T>, sizeof(StripWarp<T>), p.total[unit], r.n > 1, p, unit,
+                         strip_rows(cfg), r, st);
+}
+
+template <class T>
 cudaError_t launch_t_objective(const Plan& p, int noff, int src, cudaStream_t st) {
-    k_t_objective<<<p.grid[U_INST], kObjThreads, 0, st>>>(p, noff, src);
+    const int per = NT / 32;
+    k_t_objective<T><<<(p.total[U_OBJ] + per - 1) / per, NT, 0, st>>>(p, noff, src);
     return cudaGetLastError();
 }
 
-cudaError_t launch_t_adj2d(const Plan& p, int cfg, int noff, int lam_in, int lam_out, int sn,
-                           int sp, int kslot, cudaStream_t st) {
-    switch (cfg) {
-        case 0: return adj_cfg<0>(p, noff, lam_in, lam_out, sn, sp, kslot, st);
-        case 1: return adj_cfg<1>(p, noff, lam_in, lam_out, sn, sp, kslot, st);
-        case 2: return adj_cfg<2>(p, noff, lam_in, lam_out, sn, sp, kslot, st);
-        case 3: return adj_cfg<3>(p, noff, lam_in, lam_out, sn, sp, kslot, st);
-        case 4: return adj_cfg<4>(p, noff, lam_in, lam_out, sn, sp, kslot, st);
-        default: return cudaErrorInvalidValue;
-    }
+// Blocks per instance of the element-wise kernels.
+inline int per_instance(const Plan& p) { return std::max(1, 8 * sm_count() / p.count); }
+
+template <class T>
+cudaError_t launch_t_begin(const Plan& p, bool adjoint, cudaStream_t st) {
+    k_t_begin<T><<<dim3(adjoint ? per_instance(p) : 1, p.count), NT, 0, st>>>(p, adjoint);
+    return cudaGetLastError();
 }
 
-cudaError_t launch_t_sens(const Plan& p, int noff, cudaStream_t st) {
-    if (p.total[U_DCOL] == 0) return cudaSuccess;
-    k_t_sens<<<p.grid[U_DCOL], NT, 0, st>>>(p, noff);
+template <class T>
+cudaError_t launch_t_end(const Plan& p, int dst, int src, int n_last, bool adjoint, RunResult* out,
+                         cudaStream_t st) {
+    k_t_end<T><<<dim3(per_instance(p), p.count), NT, 0, st>>>(p, dst, src, !adjoint);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_t_result<T><<<p.count, NT, 0, st>>>(p, n_last, adjoint, out);
+    return cudaGetLastError();
+}
+
+template <class T>
+cudaError_t launch_t_sens(const Plan& p, int noff, int n, int eslot0, cudaStream_t st) {
+    if (p.total[U_DCOL] == 0 || n <= 0) return cudaSuccess;
+    const long long units = (long long)p.total[U_DCOL] * (kUnitThreads / kSensThreads);
+    k_t_sens<T><<<cap_grid(units, 32), kSensThreads, 0, st>>>(p, noff, n, eslot0);
+    return cudaGetLastError();
+}
+
+template <class T>
+cudaError_t launch_t_copy(const Plan& p, int dst, int src, cudaStream_t st) {
+    k_t_copy<T><<<dim3(per_instance(p), p.count), NT, 0, st>>>(p, dst, src);
     return cudaGetLastError();
 }
 
@@ -1104,5 +1378,19 @@ cudaError_t launch_set_int(int* dst, int v, cudaStream_t st) {
     k_set_int<<<1, 1, 0, st>>>(dst, v);
     return cudaGetLastError();
 }
+
+#define LKS_INST_2D(T)                                                                      \
+    template cudaError_t launch_t_transfer<T>(const Plan&, int, int, int, cudaStream_t);    \
+    template cudaError_t launch_t_step<T>(const Plan&, int, const StripRun&, cudaStream_t); \
+    template cudaError_t launch_t_adj<T>(const Plan&, int, const StripRun&, cudaStream_t);  \
+    template cudaError_t launch_t_objective<T>(const Plan&, int, int, cudaStream_t);        \
+    template cudaError_t launch_t_begin<T>(const Plan&, bool, cudaStream_t);                \
+    template cudaError_t launch_t_end<T>(const Plan&, int, int, int, bool, RunResult*,      \
+                                         cudaStream_t);                                     \
+    template cudaError_t launch_t_sens<T>(const Plan&, int, int, int, cudaStream_t);        \
+    template cudaError_t launch_t_copy<T>(const Plan&, int, int, cudaStream_t);
+
+LKS_INST_2D(float)
+LKS_INST_2D(double)
 
 }  // namespace lks

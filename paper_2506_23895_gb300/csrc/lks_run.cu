@@ -177,8 +177,7 @@ lks_status transfer_at(lks_ctx* c, int n) {
     if (c->d.nd == 0 || c->g.boxN == 0) return LKS_OK;
     if (c->fused2d) {
         CU(launch_set_int(c->nbase, n, c->st));
-        CU(launch_t_design_pos(c->plan, 0, c->st));
-        CU(launch_t_transfer2d(c->plan, 0, -1, false, c->st));
+        CU(launch_t_transfer<T>(c->plan, 0, 1, -1, c->st));
         c->stats[4] += 3;
         return LKS_OK;
     }
@@ -389,6 +388,7 @@ Group self_group(lks_ctx*& c) {
     G.table = c->fused2d;
     G.plan = &c->plan;
     G.nbase = c->nbase;
+    G.result = (RunResult*)c->scal;
     G.tile_fwd = c->tile_fwd;
     G.tile_adj = c->tile_adj;
     G.st = c->st;
@@ -399,68 +399,46 @@ Group self_group(lks_ctx*& c) {
 bool tape_transfers(const Group& G) {
     if (!G.table) return false;
     for (int i = 0; i < G.count; ++i)
-        if (!G.cs[i]->ktape || G.cs[i]->K + 1 > G.cs[i]->ktape_slots) return false;
+        if (G.cs[i]->d.nd > 0 && G.cs[i]->K + 1 > G.cs[i]->ktape_slots) return false;
     return true;
 }
 
-// Table-path launch sequences of one forward / adjoint step at offset k from *nbase.  kslot >= 0:
-// the step's transfer goes to (forward) or comes from (adjoint) slot kslot of the transfer tape.
-// The design positions of a run's first step come from their own launch, those of the later
-// steps from the previous step's transfer (first, next).
-cudaError_t table_fwd_launches(const Group& G, int k, int src, int dst, bool with_obj, int kslot,
-                               bool first, bool next, lks_ctx* timed, int n, int& nl) {
-    cudaError_t e;
-    if (first) {
-        if ((e = launch_t_design_pos(*G.plan, k, G.st)) != cudaSuccess) return e;
-        ++nl;
-    }
-    if ((e = launch_t_transfer2d(*G.plan, k, kslot, next, G.st)) != cudaSuccess) return e;
-    const bool tm = timed && timing_begin(timed, n, 0);
-    if ((e = launch_t_step2d(*G.plan, G.tile_fwd, src, dst, kslot, G.st)) != cudaSuccess)
-        return e;
-    if (tm) timing_end(timed, 0);
-    nl += 2;
-    if (with_obj) {
-        if ((e = launch_t_objective(*G.plan, k, dst, G.st)) != cudaSuccess) return e;
-        ++nl;
-    }
-    return cudaSuccess;
+// Steps of a run handled by one launch: at most kRunSteps (which bounds a launch to some
+// milliseconds) and as many as there are transfer slots.
+constexpr int kRunSteps = 512;
+int group_chunk(const Group& G) {
+    int n = kRunSteps;
+    for (int i = 0; i < G.count; ++i)
+        if (G.cs[i]->d.nd > 0) n = std::min(n, G.cs[i]->ktape_slots);
+    return std::max(n, 1);
 }
 
-// The adjoint step gathers the transpose of the boundary copies itself, and the sensitivity
-// gather forms the design positions of its step.
-cudaError_t table_adj_launches(const Group& G, int k, int lam_in, int lam_out, int sn, int sp,
-                               int kslot, lks_ctx* timed, int n, int& nl) {
-    cudaError_t e;
-    if (kslot < 0) {
-        if ((e = launch_t_design_pos(*G.plan, k, G.st)) != cudaSuccess) return e;
-        if ((e = launch_t_transfer2d(*G.plan, k, -1, false, G.st)) != cudaSuccess) return e;
+// Transfers of steps k .. k + n - 1 (offsets from *nbase) into slots slot .. slot + n - 1.
+template <class T>
+cudaError_t table_transfers(const Group& G, int k, int n, int slot, int& nl) {
+    int pos = n;
+    for (int i = 0; i < G.count; ++i)
+        if (G.cs[i]->d.nd > 0) pos = std::min(pos, G.cs[i]->pos_slots);
+    for (int j = 0; j < n; j += pos) {
+        const cudaError_t e =
+            launch_t_transfer<T>(*G.plan, k + j, std::min(pos, n - j), slot + j, G.st);
+        if (e != cudaSuccess) return e;
         nl += 2;
     }
-    const bool tm = timed && timing_begin(timed, n, 1);
-    if ((e = launch_t_adj2d(*G.plan, G.tile_adj, k, lam_in, lam_out, sn, sp, kslot, G.st)) !=
-        cudaSuccess)
-        return e;
-    if (tm) timing_end(timed, 1);
-    if ((e = launch_t_sens(*G.plan, k, G.st)) != cudaSuccess) return e;
-    nl += 2;
     return cudaSuccess;
 }
 
-// Run `len` table-path steps from base: fn(k, nl) issues step k (1..len) and counts launches.
-// With a graph cache the sequence is captured once per key and replayed.
+// Run table-path steps from base: fn(nl, direct) issues them and counts launches.  With a graph
+// cache the sequence is captured once per key and replayed.
 template <class Fn>
-lks_status table_run(Group& G, std::tuple<int, int, int, int, int, int> key, int base, int len,
-                     Fn fn) {
+lks_status table_run(Group& G, std::tuple<int, int, int, int, int, int> key, int base, Fn fn) {
     GCU(launch_set_int(G.nbase, base, G.st));
     ++G.launches;
     if (!G.graphs) {
         int nl = 0;
-        for (int k = 1; k <= len; ++k) {
-            cudaError_t e = fn(k, nl, true);
-            if (e != cudaSuccess)
-                return gfail(G, LKS_ERR_CUDA, "table kernel launch: %s", cudaGetErrorString(e));
-        }
+        const cudaError_t e = fn(nl, true);
+        if (e != cudaSuccess)
+            return gfail(G, LKS_ERR_CUDA, "table kernel launch: %s", cudaGetErrorString(e));
         G.launches += nl;
         return LKS_OK;
     }
@@ -468,8 +446,7 @@ lks_status table_run(Group& G, std::tuple<int, int, int, int, int, int> key, int
     if (it == G.graphs->execs.end()) {
         GCU(cudaStreamBeginCapture(G.st, cudaStreamCaptureModeThreadLocal));
         int nl = 0;
-        cudaError_t e = cudaSuccess;
-        for (int k = 1; k <= len && e == cudaSuccess; ++k) e = fn(k, nl, false);
+        cudaError_t e = fn(nl, false);
         cudaGraph_t graph = nullptr;
         cudaError_t e2 = cudaStreamEndCapture(G.st, &graph);
         if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -508,24 +485,45 @@ lks_status run_steps(Group& G, int from_level, int to_level, bool with_obj, int 
         for (int i = 0; i < G.count && with_obj; ++i)
             obj = obj || (G.cs[i]->cfg.win_begin <= to_level &&
                           G.cs[i]->cfg.win_end > from_level);
-        // a taped step leaves its transfer in the transfer tape slot of its level
+        // a taped step leaves its transfer in the slot of its level, for the adjoint
         const bool kt = tape_seg >= 0 && tape_transfers(G);
-        auto fn = [&](int k, int& nl, bool direct) -> cudaError_t {
-            int src, dst;
-            if (tape_seg >= 0) {
-                src = BUF_POOL + toff + k - 1;
-                dst = BUF_POOL + toff + k;
-            } else {
-                const int w = (w0 + k - 1) & 1;
-                src = BUF_S0 + w;
-                dst = BUF_S0 + 1 - w;
+        auto fn = [&](int& nl, bool direct) -> cudaError_t {
+            lks_ctx* timed = direct && G.count == 1 && c0->timing_stride > 0 ? c0 : nullptr;
+            const int chunk = kt ? kRunSteps : group_chunk(G);
+            for (int k0 = 1; k0 <= len; k0 += chunk) {
+                const int n = std::min(chunk, len - k0 + 1);
+                const int slot = kt ? toff + k0 : 0;
+                cudaError_t e = table_transfers<T>(G, k0, n, slot, nl);
+                if (e != cudaSuccess) return e;
+                StripRun r;
+                r.taped = tape_seg >= 0;
+                r.buf = tape_seg >= 0 ? BUF_POOL + toff : w0;
+                r.tape = 0;
+                r.kslot = slot - k0;
+                r.eslot = 0;
+                r.obj = obj;
+                // one launch for the chunk; with timing on, one per step with events around it
+                for (int k = k0; k < k0 + n; k += r.n) {
+                    r.k0 = k;
+                    r.n = timed ? 1 : n;
+                    const bool tm = timed && timing_begin(timed, from_level + k, 0);
+                    if ((e = launch_t_step<T>(*G.plan, G.tile_fwd, r, G.st)) != cudaSuccess)
+                        return e;
+                    if (tm) timing_end(timed, 0);
+                    ++nl;
+                    if (!obj) continue;
+                    const int kl = k + r.n - 1;
+                    const int last = tape_seg >= 0 ? BUF_POOL + toff + kl : BUF_S0 + ((w0 + kl) & 1);
+                    if ((e = launch_t_objective<T>(*G.plan, kl, last, G.st)) != cudaSuccess)
+                        return e;
+                    ++nl;
+                }
             }
-            return table_fwd_launches(G, k, src, dst, obj, kt ? toff + k : -1, k == 1, k < len,
-                                      (direct && G.count == 1) ? c0 : nullptr, from_level + k, nl);
+            return cudaSuccess;
         };
         const auto key = std::make_tuple(tape_seg >= 0 ? 1 : 0, obj ? 1 : 0, len,
                                          tape_seg >= 0 ? toff : w0, G.tile_fwd, kt ? 1 : 0);
-        lks_status s = table_run(G, key, from_level, len, fn);
+        lks_status s = table_run(G, key, from_level, fn);
         if (s != LKS_OK) return s;
         for (int i = 0; i < G.count; ++i) {
             lks_ctx* c = G.cs[i];
@@ -566,17 +564,30 @@ lks_status run_steps(Group& G, int from_level, int to_level, bool with_obj, int 
     return LKS_OK;
 }
 
-lks_status restore_level(Group& G, int seg) {
-    for (int i = 0; i < G.count; ++i) {
-        lks_ctx* c = G.cs[i];
-        const int lev = seg_start(c, seg);
-        if (c->work_level == lev) continue;
-        if (seg != 0 && c->slot_of[seg] < 0) return fail(c, LKS_ERR_ARG, "schedule: no snapshot");
-        const void* src = (seg == 0) ? c->s0 : (const void*)slot_ptr(c, c->slot_of[seg]);
-        lks_status s = copy_state(c, c->s[c->work], src, G.st);
-        if (s != LKS_OK) return s;
-        c->work_level = lev;
+// Copy a state of every context of the group: one launch over the instances on the table path
+// (buffers by index, equal in every context), a memory copy otherwise.
+template <class T>
+lks_status group_copy(Group& G, int dst, int src) {
+    if (G.table) {
+        GCU(launch_t_copy<T>(*G.plan, dst, src, G.st));
+        ++G.launches;
+        return LKS_OK;
     }
+    lks_ctx* c = G.cs[0];
+    return copy_state(c, c->hbufs[dst], c->hbufs[src], G.st);
+}
+
+template <class T>
+lks_status restore_level(Group& G, int seg) {
+    // the contexts of a group follow one schedule: equal slots and levels
+    lks_ctx* c0 = G.cs[0];
+    const int lev = seg_start(c0, seg);
+    if (c0->work_level == lev) return LKS_OK;
+    if (seg != 0 && c0->slot_of[seg] < 0) return gfail(G, LKS_ERR_ARG, "schedule: no snapshot");
+    const int src = seg == 0 ? (int)BUF_INIT : BUF_POOL + c0->slot_of[seg];
+    lks_status s = group_copy<T>(G, BUF_S0 + c0->work, src);
+    if (s != LKS_OK) return s;
+    for (int i = 0; i < G.count; ++i) G.cs[i]->work_level = lev;
     return LKS_OK;
 }
 
@@ -585,20 +596,17 @@ lks_status exec_forward_action(Group& G, const Act& a, bool with_obj) {
     lks_ctx* c0 = G.cs[0];
     switch (a.kind) {
         case A_RESTORE:
-            return restore_level(G, a.a);
+            return restore_level<T>(G, a.a);
         case A_ADVANCE:
             return run_steps<T>(G, seg_start(c0, a.a), seg_start(c0, a.b), with_obj, -1);
         case A_STORE:
             for (int i = 0; i < G.count; ++i) {
                 lks_ctx* c = G.cs[i];
                 if (c->free_slots.empty()) return fail(c, LKS_ERR_NOMEM, "schedule: out of slots");
-                const int sl = c->free_slots.back();
+                c->slot_of[a.a] = c->free_slots.back();
                 c->free_slots.pop_back();
-                c->slot_of[a.a] = sl;
-                lks_status s = copy_state(c, slot_ptr(c, sl), c->s[c->work], G.st);
-                if (s != LKS_OK) return s;
             }
-            return LKS_OK;
+            return group_copy<T>(G, BUF_POOL + c0->slot_of[a.a], BUF_S0 + c0->work);
         case A_FREE:
             for (int i = 0; i < G.count; ++i) {
                 lks_ctx* c = G.cs[i];
@@ -606,13 +614,11 @@ lks_status exec_forward_action(Group& G, const Act& a, bool with_obj) {
                 c->slot_of[a.a] = -1;
             }
             return LKS_OK;
-        case A_TAPE:
-            for (int i = 0; i < G.count; ++i) {
-                lks_ctx* c = G.cs[i];
-                lks_status s = copy_state(c, slot_ptr(c, 0), c->s[c->work], G.st);
-                if (s != LKS_OK) return s;
-            }
+        case A_TAPE: {
+            lks_status s = group_copy<T>(G, BUF_POOL, BUF_S0 + c0->work);
+            if (s != LKS_OK) return s;
             return run_steps<T>(G, seg_start(c0, a.a), seg_end(c0, a.a), with_obj, a.a);
+        }
         default:
             return gfail(G, LKS_ERR_ARG, "schedule: unexpected action");
     }
@@ -631,19 +637,49 @@ lks_status exec_adj(Group& G, int seg) {
         return LKS_OK;
     }
     const int par0 = c0->lam_par;
-    // the tape of this segment (levels 0..len) holds the transfer of step a + kk in slot kk
+    // the tape of this segment (levels 0..len) holds the transfer of step a + k in slot k, or the
+    // transfers are formed again
     const bool kt = tape_transfers(G);
-    auto fn = [&](int k, int& nl, bool direct) -> cudaError_t {
-        const int kk = len - k + 1;                 // step n = a + kk, from b down to a + 1
-        const int par = par0 ^ ((k - 1) & 1);
-        return table_adj_launches(G, kk, BUF_LAM0 + par, BUF_LAM0 + 1 - par, BUF_POOL + kk,
-                                  BUF_POOL + kk - 1, kt ? kk : -1,
-                                  (direct && G.count == 1) ? c0 : nullptr, a + kk, nl);
+    auto fn = [&](int& nl, bool direct) -> cudaError_t {
+        lks_ctx* timed = direct && G.count == 1 && c0->timing_stride > 0 ? c0 : nullptr;
+        const int chunk = group_chunk(G);
+        for (int k1 = len; k1 >= 1; k1 -= chunk) {   // steps a + k1 down to a + k0
+            const int n = std::min(chunk, k1), k0 = k1 - n + 1;
+            cudaError_t e = cudaSuccess;
+            if (!kt && (e = table_transfers<T>(G, k0, n, 0, nl)) != cudaSuccess) return e;
+            StripRun r;
+            r.taped = 1;
+            r.tape = BUF_POOL;
+            r.kslot = kt ? 0 : -k0;
+            r.eslot = -k0;
+            r.obj = 0;
+            for (int k = k1; k >= k0; k -= r.n) {
+                r.k0 = k;
+                r.n = timed ? 1 : n;
+                r.buf = par0 ^ ((len - k) & 1);
+                const bool tm = timed && timing_begin(timed, a + k, 1);
+                if ((e = launch_t_adj<T>(*G.plan, G.tile_adj, r, G.st)) != cudaSuccess) return e;
+                if (tm) timing_end(timed, 1);
+                ++nl;
+            }
+            if ((e = launch_t_sens<T>(*G.plan, k0, n, 0, G.st)) != cudaSuccess) return e;
+            ++nl;
+        }
+        return cudaSuccess;
     };
     const auto key = std::make_tuple(2, kt ? 1 : 0, len, par0, 0, G.tile_adj);
-    lks_status s = table_run(G, key, a, len, fn);
+    lks_status s = table_run(G, key, a, fn);
     if (s != LKS_OK) return s;
     for (int i = 0; i < G.count; ++i) G.cs[i]->lam_par = par0 ^ (len & 1);
+    return LKS_OK;
+}
+
+// The status a run's error words stand for.
+lks_status run_status(lks_ctx* c, const int* f) {
+    if (f[1]) return fail(c, LKS_ERR_ARG, "transfer tap list overflow");
+    if (f[3] & 8) return fail(c, LKS_ERR_TIMEOUT, "a bounded wait ran out in a fused kernel");
+    if (f[3]) return fail(c, LKS_ERR_CUDA, "fused step reported error %d", f[3]);
+    if (f[2]) return fail(c, LKS_ERR_DIVERGED, "state diverged (non-finite or |u| >= 0.5)");
     return LKS_OK;
 }
 
@@ -666,6 +702,7 @@ lks_status do_forward(Group& G, int N) {
         c->work_level = -1;
         c->last = nullptr;
         c->fwd_valid = false;
+        if (G.table) continue;
         {
             lks_status s = transfer_join(c);
             if (s != LKS_OK) return s;
@@ -673,12 +710,41 @@ lks_status do_forward(Group& G, int N) {
         CU(cudaMemsetAsync(c->jstep, 0, (size_t)(c->cfg.max_steps + 2) * 8, G.st));
         CU(cudaMemsetAsync(c->flags, 0, 64, G.st));
     }
+    if (G.table) {
+        GCU(launch_t_begin<T>(*G.plan, false, G.st));
+        ++G.launches;
+    }
     const std::vector<Act>& acts = G.cs[0]->acts;
     size_t i = 0;
     for (; i < acts.size(); ++i) {
         lks_status s = exec_forward_action<T>(G, acts[i], true);
         if (s != LKS_OK) return s;
         if (acts[i].kind == A_TAPE) break;
+    }
+    if (G.table) {
+        std::vector<RunResult> res(G.count);
+        lks_ctx* c0 = G.cs[0];
+        int last = 0;
+        while (c0->hbufs[last] != c0->last) ++last;
+        GCU(launch_t_end<T>(*G.plan, BUF_SEND, last, N, false, G.result, G.st));
+        G.launches += 2;
+        GCU(cudaMemcpyAsync(res.data(), G.result, sizeof(RunResult) * G.count,
+                            cudaMemcpyDeviceToHost, G.st));
+        GCU(cudaStreamSynchronize(G.st));
+        lks_status worst = LKS_OK;
+        for (int k = 0; k < G.count; ++k) {
+            lks_ctx* c = G.cs[k];
+            c->adj_begin = i + 1;
+            const lks_status s = run_status(c, res[k].flags);
+            if (s != LKS_OK) {
+                if (worst == LKS_OK) worst = s;
+                continue;
+            }
+            c->have_end = true;
+            c->J = res[k].J;
+            c->fwd_valid = true;
+        }
+        return worst;
     }
     std::vector<std::vector<double>> js(G.count);
     std::vector<int> fl(4 * (size_t)G.count);
@@ -698,12 +764,7 @@ lks_status do_forward(Group& G, int N) {
     lks_status worst = LKS_OK;
     for (int k = 0; k < G.count; ++k) {
         lks_ctx* c = G.cs[k];
-        const int* f = fl.data() + 4 * k;
-        lks_status s = LKS_OK;
-        if (f[1]) s = fail(c, LKS_ERR_ARG, "transfer tap list overflow");
-        else if (f[3] & 8) s = fail(c, LKS_ERR_TIMEOUT, "a tensor-copy wait timed out in the fused step");
-        else if (f[3]) s = fail(c, LKS_ERR_CUDA, "fused step reported error %d", f[3]);
-        else if (f[2]) s = fail(c, LKS_ERR_DIVERGED, "state diverged (non-finite or |u| >= 0.5)");
+        const lks_status s = run_status(c, fl.data() + 4 * k);
         if (s != LKS_OK) {
             if (worst == LKS_OK) worst = s;
             continue;
@@ -724,6 +785,7 @@ lks_status do_adjoint(Group& G) {
     for (int i = 0; i < G.count; ++i) {
         lks_ctx* c = G.cs[i];
         c->lam_par = 0;
+        if (G.table) continue;
         CU(cudaMemsetAsync(c->flags, 0, 64, G.st));
         if (c->adj_warm && c->have_lend)   // warm start: lambda^N from the last lambda^0
             CU(cudaMemcpyAsync(c->lam[0], c->l_end, c->snap_bytes, cudaMemcpyDeviceToDevice, G.st));
@@ -731,6 +793,16 @@ lks_status do_adjoint(Group& G) {
             CU(cudaMemsetAsync(c->lam[0], 0, c->snap_bytes, G.st));
         if (c->u3) CU(cudaMemsetAsync(c->u3, 0, c->snap_bytes, G.st));
         if (c->d.nd > 0) CU(cudaMemsetAsync(c->gacc, 0, (size_t)c->d.nd * 8, G.st));
+    }
+    if (G.table) {
+        GCU(launch_t_begin<T>(*G.plan, true, G.st));
+        ++G.launches;
+        for (int i = 0; i < G.count; ++i) {   // warm starts: lambda^N from the last lambda^0
+            lks_ctx* c = G.cs[i];
+            if (c->adj_warm && c->have_lend)
+                CU(cudaMemcpyAsync(c->lam[0], c->l_end, c->snap_bytes, cudaMemcpyDeviceToDevice,
+                                   G.st));
+        }
     }
     lks_ctx* c0 = G.cs[0];
     for (size_t i = c0->adj_begin - 1; i < c0->acts.size(); ++i) {
@@ -740,6 +812,24 @@ lks_status do_adjoint(Group& G) {
         if (s != LKS_OK) return s;
     }
     // the tape of the last segment has been overwritten: a second adjoint needs a new forward
+    if (G.table) {
+        std::vector<RunResult> res(G.count);
+        GCU(launch_t_end<T>(*G.plan, BUF_LEND, BUF_LAM0 + c0->lam_par, 0, true, G.result, G.st));
+        G.launches += 2;
+        GCU(cudaMemcpyAsync(res.data(), G.result, sizeof(RunResult) * G.count,
+                            cudaMemcpyDeviceToHost, G.st));
+        for (int k = 0; k < G.count; ++k) {
+            G.cs[k]->fwd_valid = false;
+            G.cs[k]->have_lend = true;
+        }
+        GCU(cudaStreamSynchronize(G.st));
+        lks_status worst = LKS_OK;
+        for (int k = 0; k < G.count; ++k) {
+            const lks_status s = run_status(G.cs[k], res[k].flags);
+            if (s != LKS_OK && worst == LKS_OK) worst = s;
+        }
+        return worst;
+    }
     std::vector<int> fl(4 * (size_t)G.count);
     for (int k = 0; k < G.count; ++k) {
         lks_ctx* c = G.cs[k];
@@ -757,11 +847,7 @@ lks_status do_adjoint(Group& G) {
     lks_status worst = LKS_OK;
     for (int k = 0; k < G.count; ++k) {
         lks_ctx* c = G.cs[k];
-        const int* f = fl.data() + 4 * k;
-        lks_status s = LKS_OK;
-        if (f[1]) s = fail(c, LKS_ERR_ARG, "transfer tap list overflow");
-        else if (f[3] & 8) s = fail(c, LKS_ERR_TIMEOUT, "a tensor-copy wait timed out in the fused step");
-        else if (f[3]) s = fail(c, LKS_ERR_CUDA, "fused step reported error %d", f[3]);
+        const lks_status s = run_status(c, fl.data() + 4 * k);
         if (s != LKS_OK && worst == LKS_OK) worst = s;
     }
     return worst;
@@ -777,40 +863,50 @@ lks_status reset_initial(lks_ctx* c) {
 }
 
 // Host record of a context's instance-table entry (valid once design and motion are set).
-Inst make_inst(const lks_ctx* c) {
-    Inst I;
+template <class T>
+Inst<T> make_inst(const lks_ctx* c) {
+    Inst<T> I;
     std::memset(&I, 0, sizeof(I));
     I.g = c->g;
     I.d = c->d;
-    I.pos_b[0] = reinterpret_cast<int2*>(c->ts.col_base);
-    I.pos_sc[0] = c->ts.col_sc;
-    I.pos_b[1] = reinterpret_cast<int2*>(c->pos2_b);
-    I.pos_sc[1] = c->pos2_sc;
+    I.pos_b = (int2*)c->pos_b;
+    I.pos_sc = (V4<T>*)c->pos_sc;
     I.motion = c->dmotion;
-    I.bufs = c->dbufs;
-    I.kref = (const float*)c->kref;
-    I.kprime = (const float*)c->kprime;
-    I.kus = (V4<float>*)c->kus;
-    I.kus_tape = (V4<float>*)c->ktape;
-    I.e = (float*)c->e;
+    for (int b = 0; b < BUF_POOL; ++b) I.bufs[b] = c->hbufs[b];
+    I.pool = c->pool;
+    I.snap = (long long)c->snap_bytes;
+    I.kref = (const T*)c->kref;
+    I.kprime = (const T*)c->kprime;
+    I.kus = (V4<T>*)c->kus;
+    I.kus_tape = (V4<T>*)c->ktape;
+    I.e = (T*)c->etape;
     I.gacc = c->gacc;
-    I.jstep = c->jstep;
+    I.flags = c->flags;
+    I.jpart = c->jpart;
+    I.jparts = obj_parts(c->g.ocount);
     I.win_begin = c->cfg.win_begin;
     I.win_end = c->cfg.win_end;
     // the same FP64 expressions as the per-node source of the plain kernels, rounded once
     const double h = 1.0 / (double)(c->cfg.win_end - c->cfg.win_begin + 1);
     const Geom& g = c->g;
-    I.hwin = h;
-    I.Af = (float)g.A;
-    I.bf[0] = (float)g.body[0];
-    I.bf[1] = (float)g.body[1];
-    I.src_r = g.okind == 0 ? (float)(-h / (3.0 * g.ocount)) : 0.f;
-    I.src_x = g.okind == 0 ? 0.f : (float)(-h * g.odir[0] / g.ocount);
-    I.src_y = g.okind == 0 ? 0.f : (float)(-h * g.odir[1] / g.ocount);
+    I.A = (T)g.A;
+    I.A9 = (T)(g.A / 9.0);
+    I.bf[0] = (T)g.body[0];
+    I.bf[1] = (T)g.body[1];
+    I.src_r = g.okind == 0 ? (T)(-h / (3.0 * g.ocount)) : (T)0;
+    I.src_x = g.okind == 0 ? (T)0 : (T)(-h * g.odir[0] / g.ocount);
+    I.src_y = g.okind == 0 ? (T)0 : (T)(-h * g.odir[1] / g.ocount);
     for (int f = 0; f < 4; ++f) {
-        I.bcf[f] = make_float4((float)g.bcv[f][0], (float)g.bcv[f][1], 0.f,
-                               (float)(g.bcv[f][3] - g.rho0));
+        I.bcf[f].r = (T)(g.bcv[f][3] - g.rho0);
+        I.bcf[f].x = (T)g.bcv[f][0];
+        I.bcf[f].y = (T)g.bcv[f][1];
+        I.bcf[f].z = (T)0;
         I.bckeep[f] = g.bc[f] == BC_WALL || g.bc[f] == BC_INLET;
+    }
+    for (int q = 0; q < 4; ++q) {   // WALL > INLET > OUTLET, ties to the lower face
+        auto prec = [&](int f) { return g.bc[f] == BC_WALL ? 3 : (g.bc[f] == BC_INLET ? 2 : 1); };
+        const int fx = q & 1, fy = 2 + (q >> 1);
+        I.corner[q] = prec(fy) > prec(fx) ? fy : fx;
     }
     return I;
 }
@@ -824,29 +920,33 @@ void inst_units(const lks_ctx* c, int out[U_COUNT]) {
     // nodes a tile reads in shared memory)
     out[U_BOX] = body ? ((g.bn[0] + kBoxTile - 1) / kBoxTile) * ((g.bn[1] + kBoxTile - 1) / kBoxTile)
                       : 0;
-    out[U_INST] = 1;
-    for (int k = 0; k < kTileCfgs; ++k)
-        out[U_TILE0 + k] = tile_count(g.n[0], tile_tx(k), g.periodic[0]) *
-                           tile_count(g.n[1], tile_ty(k), g.periodic[1]);
+    out[U_OBJ] = obj_parts(g.ocount);
+    for (int k = 0; k < kStripCfgs; ++k)
+        out[U_STRIP0 + k] = strip_count(g.n[0], kStripW, g.periodic[0]) *
+                            ((g.n[1] + strip_rows(k) - 1) / strip_rows(k));
 }
 
 // Build a plan over contexts: the table and prefix arrays go to dinst / dpre (device, with
-// room for cs.size() entries), the host plan gets the totals and the persistent grids.
-cudaError_t build_plan(const std::vector<lks_ctx*>& cs, Inst* dinst, int* dpre, int* nbase,
+// room for cs.size() entries), the host plan gets the totals.  nbase: device words of the plan's
+// owner: the step base, then the grid barrier's count.
+template <class T>
+cudaError_t build_plan(const std::vector<lks_ctx*>& cs, void* dinst, int* dpre, int* nbase,
                        cudaStream_t st, Plan& p) {
     const int B = (int)cs.size();
-    std::vector<Inst> tab(B);
+    std::vector<Inst<T>> tab(B);
     std::vector<int> pre((size_t)U_COUNT * (B + 1), 0);
     for (int i = 0; i < B; ++i) {
-        tab[i] = make_inst(cs[i]);
+        tab[i] = make_inst<T>(cs[i]);
         int u[U_COUNT];
         inst_units(cs[i], u);
         for (int k = 0; k < U_COUNT; ++k)
             pre[(size_t)k * (B + 1) + i + 1] = pre[(size_t)k * (B + 1) + i] + u[k];
     }
-    cudaError_t e = cudaMemcpyAsync(dinst, tab.data(), sizeof(Inst) * B, cudaMemcpyHostToDevice, st);
+    cudaError_t e =
+        cudaMemcpyAsync(dinst, tab.data(), sizeof(Inst<T>) * B, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(dpre, pre.data(), pre.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(nbase, 0, 2 * sizeof(int), st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // host vectors go out of scope
     if (e != cudaSuccess) return e;
     std::memset(&p, 0, sizeof(p));
@@ -854,9 +954,21 @@ cudaError_t build_plan(const std::vector<lks_ctx*>& cs, Inst* dinst, int* dpre, 
     p.pre = dpre;
     p.count = B;
     p.nbase = nbase;
+    p.bar = nbase + 1;
+    p.err = cs[0]->flags + 3;
     for (int k = 0; k < U_COUNT; ++k) p.total[k] = pre[(size_t)k * (B + 1) + B];
-    plan_grids(p);
     return cudaGetLastError();
+}
+
+// The one-entry plan of a table context, and its strip height.
+lks_status own_plan(lks_ctx* c) {
+    std::vector<lks_ctx*> one(1, c);
+    if (c->prec == LKS_FP64)
+        CU(build_plan<double>(one, c->dinst, c->dpre, c->nbase, c->st, c->plan));
+    else
+        CU(build_plan<float>(one, c->dinst, c->dpre, c->nbase, c->st, c->plan));
+    c->tile_fwd = c->tile_adj = default_strips(c->plan, (int)c->tsz);
+    return LKS_OK;
 }
 
 // kappa_ref and kappa' from the stored gamma, through the filter chain when it is on (the
@@ -896,13 +1008,15 @@ lks_status finish_motion(lks_ctx* c) {
     CU(cudaStreamSynchronize(c->st));
     ++c->geo_gen;
     if (c->fused2d) {
-        std::vector<lks_ctx*> one(1, c);
-        CU(build_plan(one, c->dinst, c->dpre, c->nbase, c->st, c->plan));
+        const lks_status s = own_plan(c);
+        if (s != LKS_OK) return s;
     }
     c->have_motion = true;
     return LKS_OK;
 }
 
+template cudaError_t build_plan<float>(const std::vector<lks_ctx*>&, void*, int*, int*,
+                                      cudaStream_t, Plan&);
 template lks_status transfer_at<float>(lks_ctx*, int);
 template lks_status transfer_at<double>(lks_ctx*, int);
 template lks_status reset_initial<float>(lks_ctx*);

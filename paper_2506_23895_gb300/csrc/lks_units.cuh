@@ -25,8 +25,8 @@ __device__ __forceinline__ void design_col_pos(const Design& d, const Motion& m,
 }
 
 // ---------------------------------------------------------------- 2D transfer (table path)
-// Design column k for the D2Q9 instance-table kernels: integer base of x_ref, y_ref (FP64, as
-// design_col_pos) and, per axis, S = sin(pi f/2), C = cos(pi f/2) of the fraction f.  The four
+// Design column k for the D2Q9 instance-table kernels: integer base of x_ref, y_ref and, per axis,
+// S = sin(pi f/2), C = cos(pi f/2) of the fraction f.  The four
 // taps of the cosine kernel then follow without further trigonometry: for an analysis node at
 // base + q, q = -1, 0, 1, 2, w = (1 - S)/4, (1 + C)/4, (1 + S)/4, (1 - C)/4 (w(r) =
 // (1 + cos(pi r/2))/4 at r = q - f).
@@ -56,91 +56,64 @@ __device__ __forceinline__ int ref_coord(float ah, float al, float da, float bh,
     return gi + (int)fl;
 }
 
+template <class T>
 __device__ __forceinline__ void col_pos_sc(const Design& d, const Motion& m, long long k, int2& b,
-                                           float4& sc) {
+                                           V4<T>& sc);
+
+template <>
+__device__ __forceinline__ void col_pos_sc<float>(const Design& d, const Motion& m, long long k,
+                                                  int2& b, V4<float>& sc) {
     const int i = (int)((unsigned)k % (unsigned)d.L[0]), j = (int)((unsigned)k / (unsigned)d.L[0]);
     const float dx = (float)i - d.xiGf[0], dy = (float)j - d.xiGf[1];
     float fx, fy;   // Eq. rigid_body_position: x_ref = c dx - s dy + x_G, y_ref = s dx + c dy + y_G
     b.x = ref_coord(m.ch, m.cl, dx, m.sh, m.sl, dy, m.xgi[0], m.xgh[0], m.xgl[0], fx);
     b.y = ref_coord(m.sh, m.sl, dx, -m.ch, -m.cl, dy, m.xgi[1], m.xgh[1], m.xgl[1], fy);
-    sincospif(0.5f * fx, &sc.x, &sc.y);
-    sincospif(0.5f * fy, &sc.z, &sc.w);
+    sincospif(0.5f * fx, &sc.r, &sc.x);
+    sincospif(0.5f * fy, &sc.y, &sc.z);
 }
 
-
-__device__ __forceinline__ float tap_weight(int q1, float S, float C) {
-    // q1 = q + 1 in 0..3
-    const float t = q1 == 0 ? -S : (q1 == 1 ? C : (q1 == 2 ? S : -C));
-    return 0.25f * (1.f + t);
+template <>
+__device__ __forceinline__ void col_pos_sc<double>(const Design& d, const Motion& m, long long k,
+                                                   int2& b, V4<double>& sc) {
+    const int i = (int)((unsigned)k % (unsigned)d.L[0]), j = (int)((unsigned)k / (unsigned)d.L[0]);
+    const double dx = i - d.xiG[0], dy = j - d.xiG[1];
+    const double xr = m.c * dx - m.s * dy + m.xG[0], yr = m.s * dx + m.c * dy + m.xG[1];
+    const double bx = floor(xr), by = floor(yr);
+    b = make_int2((int)bx, (int)by);
+    sincospi(0.5 * (xr - bx), &sc.r, &sc.x);
+    sincospi(0.5 * (yr - by), &sc.y, &sc.z);
 }
 
-// kappa(x) = sum_xi W(x - x_ref(xi)) kappa_ref(xi) and u_S = omega R'(theta) m1 + u_G m0 with
-// m0 = sum W, m1 = sum W (xi - xi_G) at box node bi (Eqs. brinkman_ref, velocity_ref; u_ref is
-// affine in xi).  The design nodes whose taps cover x are found through the inverse rigid map
-// (a window widened against rounding) and summed in design index order.
-__device__ __forceinline__ void transfer2d_node(const Design& d, const Geom& g, const Motion& m,
-                                                const int2* __restrict__ pb,
-                                                const float4* __restrict__ psc,
-                                                const float* __restrict__ kref,
-                                                V4<float>* kus, long long bi) {
-    const int x = g.blo[0] + (int)((unsigned)bi % (unsigned)g.bn[0]);
-    const int y = g.blo[1] + (int)((unsigned)bi / (unsigned)g.bn[0]);
-    const float c = m.cf, s = m.sf;
-    const float px = (float)x - m.xgf[0], py = (float)y - m.xgf[1];
-    const float ic = c * px + s * py + d.xiGf[0];
-    const float jc = -s * px + c * py + d.xiGf[1];
-    const float R = 2.f * (fabsf(c) + fabsf(s)) + 0.01f;
-    const int i0 = max(0, (int)ceilf(ic - R)), i1 = min(d.L[0] - 1, (int)floorf(ic + R));
-    const int j0 = max(0, (int)ceilf(jc - R)), j1 = min(d.L[1] - 1, (int)floorf(jc + R));
-    const float gx0 = d.xiGf[0], gy0 = d.xiGf[1];
-    float kap = 0.f, m0 = 0.f, m1x = 0.f, m1y = 0.f;
-    for (int j = j0; j <= j1; ++j)
-        for (int i = i0; i <= i1; ++i) {
-            const int k = j * d.L[0] + i;
-            const int2 b = __ldg(pb + k);
-            const int qx = x - b.x + 1, qy = y - b.y + 1;
-            if ((unsigned)qx > 3u || (unsigned)qy > 3u) continue;
-            const float4 sc = __ldg(psc + k);
-            const float W = tap_weight(qx, sc.x, sc.y) * tap_weight(qy, sc.z, sc.w);
-            kap += W * __ldg(kref + k);
-            m0 += W;
-            m1x += W * ((float)i - gx0);
-            m1y += W * ((float)j - gy0);
-        }
-    const float om = m.omf;
-    V4<float> o;
-    o.r = kap;
-    o.x = (-s * m1x - c * m1y) * om + m.ugf[0] * m0;
-    o.y = (c * m1x - s * m1y) * om + m.ugf[1] * m0;
-    o.z = 0.f;
-    kus[bi] = o;
+// Weight of tap q1 - 1 = -1, 0, 1, 2 from S = sin(pi f/2), C = cos(pi f/2) of the fraction f.
+template <class T>
+__device__ __forceinline__ T tap_weight(int q1, T S, T C) {
+    const T t = q1 == 0 ? -S : (q1 == 1 ? C : (q1 == 2 ? S : -C));
+    return (T)0.25 * ((T)1 + t);
 }
 
-// Sensitivity gather for design node k on the table path: sum over its 4 x 4 taps of
-// W e(x) with the same tap weights as transfer2d_node (the node's position at the step formed
-// here, by the same function), times kappa', added to dJ/dgamma (FP64).
-__device__ __forceinline__ void sens2d_node(const Design& d, const Geom& g, const Motion& m,
-                                            const float* __restrict__ e,
-                                            const float* __restrict__ kprime,
-                                            double* __restrict__ gacc, long long k) {
+// sum of W e(x) over the 4 x 4 taps of design node k (the transpose of the kappa transfer) with
+// the tap weights of the transfer, the node's position at the step formed here.
+template <class T>
+__device__ __forceinline__ T sens2d_sum(const Design& d, const Geom& g, const Motion& m,
+                                        const T* __restrict__ e, long long k) {
     int2 b;
-    float4 sc;
-    col_pos_sc(d, m, k, b, sc);
+    V4<T> sc;
+    col_pos_sc<T>(d, m, k, b, sc);
     const int ex0 = b.x - 1 - g.blo[0], ey0 = b.y - 1 - g.blo[1];
-    float acc = 0.f;
+    T acc = (T)0;
 #pragma unroll
     for (int ty = 0; ty < 4; ++ty) {
         const int ey = ey0 + ty;
         if (ey < 0 || ey >= g.bn[1]) continue;
-        const float wy = tap_weight(ty, sc.z, sc.w);
+        const T wy = tap_weight<T>(ty, sc.y, sc.z);
 #pragma unroll
         for (int tx = 0; tx < 4; ++tx) {
             const int ex = ex0 + tx;
             if (ex < 0 || ex >= g.bn[0]) continue;
-            acc += (tap_weight(tx, sc.x, sc.y) * wy) * e[(long long)ey * g.bn[0] + ex];
+            acc += (tap_weight<T>(tx, sc.r, sc.x) * wy) * e[(long long)ey * g.bn[0] + ex];
         }
     }
-    gacc[k] += (double)kprime[k] * (double)acc;
+    return acc;
 }
 
 // ---------------------------------------------------------------- sensitivity gather (Sec. 2.4)
