@@ -166,12 +166,12 @@ struct Layout {
 
 enum {
     L_S0, L_S1, L_SINIT, L_L0, L_L1, L_F, L_MU, L_PHI, L_KUS, L_E, L_GAMMA, L_KREF, L_KPRIME,
-    L_GACC, L_JSTEP, L_CBASE, L_CFRAC, L_ZTI, L_ZTW, L_TCNT, L_TIDX, L_TW, L_CM, L_DZB, L_DZF,
+    L_GACC, L_JSTEP, L_CBASE, L_ZTI, L_ZTW, L_TIDX, L_TW, L_CM, L_DZB, L_DZF,
     L_FLAGS, L_KREFT, L_K2, L_FACE, L_TGT, L_U3, L_MOTION, L_INST, L_PRE, L_GBAR,
-    L_HP, L_FWS, L_GOUT, L_GTMP, L_SCAL, L_CSC, L_KS, L_SEND, L_LEND, L_GBASE, L_GFRAC,
+    L_HP, L_FWS, L_GOUT, L_GTMP, L_FQ, L_SCAL, L_CSC, L_KS, L_SEND, L_LEND, L_GBASE, L_GFRAC,
     L_GCNT, L_GIDX,
     // the second transfer buffer set (3D): same sizes as L_KUS, L_K2, L_CBASE, ...
-    L_KUS2, L_K22, L_CBASE2, L_CFRAC2, L_CSC2, L_ZTI2, L_ZTW2, L_TCNT2, L_TIDX2, L_TW2, L_CM2,
+    L_KUS2, L_K22, L_CBASE2, L_CSC2, L_ZTI2, L_ZTW2, L_TIDX2, L_TW2, L_CM2,
     L_DZB2, L_DZF2, L_GBASE2, L_GFRAC2, L_GCNT2, L_GIDX2, L_E2,
     L_KTAPE, L_ETAPE, L_PB, L_PSC, L_JPART, L_POOL,
     L_COUNT
@@ -201,15 +201,13 @@ Layout make_layout(const lks_config* cfg) {
     sz[L_GACC] = (size_t)std::max(nd, 1LL) * 8;
     sz[L_JSTEP] = (size_t)(cfg->max_steps + 2) * 8;
     sz[L_CBASE] = (size_t)std::max(ncol, 1LL) * 2 * 4;
-    sz[L_CFRAC] = (size_t)std::max(ncol, 1LL) * 2 * T;
     sz[L_ZTI] = (size_t)nzb * 4 * 4;
     sz[L_ZTW] = (size_t)nzb * 4 * T;
-    sz[L_TCNT] = nd ? (size_t)cols * 4 : 0;
     sz[L_TIDX] = nd ? (size_t)cols * kMaxTaps * 4 : 0;
     sz[L_TW] = nd ? (size_t)cols * kMaxTaps * T : 0;
     sz[L_CM] = nd ? (size_t)cols * 3 * T : 0;
     sz[L_DZB] = (size_t)std::max(cfg->lz, 1) * 4;
-    sz[L_DZF] = (size_t)std::max(cfg->lz, 1) * T;
+    sz[L_DZF] = 2 * T;
     // snapshot pool
     const long long N = cfg->max_steps;
     long long P;
@@ -230,15 +228,15 @@ Layout make_layout(const lks_config* cfg) {
     sz[L_MOTION] = (size_t)(cfg->max_steps + 1) * sizeof(Motion);
     sz[L_INST] = std::max(sizeof(Inst<float>), sizeof(Inst<double>));
     sz[L_PRE] = (size_t)U_COUNT * 2 * sizeof(int);
-    sz[L_GBAR] = sz[L_HP] = sz[L_FWS] = sz[L_GOUT] = sz[L_GTMP] = (size_t)std::max(nd, 1LL) * 8;
+    sz[L_GBAR] = sz[L_HP] = sz[L_FWS] = sz[L_GOUT] = sz[L_GTMP] = sz[L_FQ] = (size_t)std::max(nd, 1LL) * 8;
     sz[L_SCAL] = 64;
-    sz[L_CSC] = (size_t)std::max(ncol, 1LL) * 16;
+    sz[L_CSC] = (size_t)std::max(ncol, 1LL) * 4 * T;
     sz[L_KS] = (size_t)nodes * T;
     sz[L_SEND] = sz[L_LEND] = state;
     {   // general-axis transfer: per design node and per box cell (worst case: every node)
         const bool ga = general_axis(cfg) && nd > 0;
         sz[L_GBASE] = ga ? (size_t)nd * 16 : 0;
-        sz[L_GFRAC] = ga ? (size_t)nd * 4 * T : 0;
+        sz[L_GFRAC] = ga ? (size_t)nd * 12 * T : 0;
         sz[L_GCNT] = ga ? (size_t)nodes * 4 : 0;
         sz[L_GIDX] = ga ? (size_t)nodes * kCellMax * 4 : 0;
     }
@@ -252,9 +250,9 @@ Layout make_layout(const lks_config* cfg) {
     }
     {   // second transfer set for the prefetch of the next step's transfer (3D only)
         const bool two = dim == 3 && nd > 0;
-        const int first[17] = {L_KUS, L_K2, L_CBASE, L_CFRAC, L_CSC, L_ZTI, L_ZTW, L_TCNT,
+        const int first[15] = {L_KUS, L_K2, L_CBASE, L_CSC, L_ZTI, L_ZTW,
                                L_TIDX, L_TW, L_CM, L_DZB, L_DZF, L_GBASE, L_GFRAC, L_GCNT, L_GIDX};
-        for (int i = 0; i < 17; ++i) sz[L_KUS2 + i] = two ? sz[first[i]] : 0;
+        for (int i = 0; i < 15; ++i) sz[L_KUS2 + i] = two ? sz[first[i]] : 0;
         sz[L_E2] = two ? sz[L_E] : 0;
     }
     // 2D contexts on the table kernels form the transfers (kappa, u_S on the footprint box) of many
@@ -390,16 +388,14 @@ lks_status lks_create(const lks_config* cfg, void* workspace, size_t ws_bytes, l
     c->gacc = (double*)(w + L.off[L_GACC]);
     c->jstep = (double*)(w + L.off[L_JSTEP]);
     c->ts.col_base = (int*)(w + L.off[L_CBASE]);
-    c->ts.col_frac = w + L.off[L_CFRAC];
-    c->ts.col_sc = (float4*)(w + L.off[L_CSC]);
+    c->ts.col_sc = w + L.off[L_CSC];
     c->ts.zt_idx = (int*)(w + L.off[L_ZTI]);
     c->ts.zt_w = w + L.off[L_ZTW];
-    c->ts.tap_cnt = (int*)(w + L.off[L_TCNT]);
     c->ts.tap_idx = (int*)(w + L.off[L_TIDX]);
     c->ts.tap_w = w + L.off[L_TW];
     c->ts.col_m = w + L.off[L_CM];
     c->ts.dz_base = (int*)(w + L.off[L_DZB]);
-    c->ts.dz_frac = w + L.off[L_DZF];
+    c->ts.dz_sc = w + L.off[L_DZF];
     c->flags = (int*)(w + L.off[L_FLAGS]);
     {
         const std::vector<int> tl = target_list(cfg);
@@ -436,13 +432,14 @@ lks_status lks_create(const lks_config* cfg, void* workspace, size_t ws_bytes, l
     c->fws = (double*)(w + L.off[L_FWS]);
     c->gout = (double*)(w + L.off[L_GOUT]);
     c->gtmp = (double*)(w + L.off[L_GTMP]);
+    c->fq = (double*)(w + L.off[L_FQ]);
     c->scal = (double*)(w + L.off[L_SCAL]);
     c->ks = w + L.off[L_KS];
     c->gaxis = general_axis(cfg) && c->d.nd > 0;
     if (general_axis(cfg))
         for (int a = 0; a < 3; ++a) c->axis[a] = cfg->rot_axis[a];
     c->as.base = (int4*)(w + L.off[L_GBASE]);
-    c->as.frac = w + L.off[L_GFRAC];
+    c->as.rec = w + L.off[L_GFRAC];
     c->as.cnt = (int*)(w + L.off[L_GCNT]);
     c->as.idx = (int*)(w + L.off[L_GIDX]);
     {   // the two transfer sets
@@ -456,18 +453,16 @@ lks_status lks_create(const lks_config* cfg, void* workspace, size_t ws_bytes, l
         b.k2 = w + L.off[L_K22];
         b.ts = c->ts;
         b.ts.col_base = (int*)(w + L.off[L_CBASE2]);
-        b.ts.col_frac = w + L.off[L_CFRAC2];
-        b.ts.col_sc = (float4*)(w + L.off[L_CSC2]);
+        b.ts.col_sc = w + L.off[L_CSC2];
         b.ts.zt_idx = (int*)(w + L.off[L_ZTI2]);
         b.ts.zt_w = w + L.off[L_ZTW2];
-        b.ts.tap_cnt = (int*)(w + L.off[L_TCNT2]);
         b.ts.tap_idx = (int*)(w + L.off[L_TIDX2]);
         b.ts.tap_w = w + L.off[L_TW2];
         b.ts.col_m = w + L.off[L_CM2];
         b.ts.dz_base = (int*)(w + L.off[L_DZB2]);
-        b.ts.dz_frac = w + L.off[L_DZF2];
+        b.ts.dz_sc = w + L.off[L_DZF2];
         b.as.base = (int4*)(w + L.off[L_GBASE2]);
-        b.as.frac = w + L.off[L_GFRAC2];
+        b.as.rec = w + L.off[L_GFRAC2];
         b.as.cnt = (int*)(w + L.off[L_GCNT2]);
         b.as.idx = (int*)(w + L.off[L_GIDX2]);
         c->pf_on = cfg->dim == 3 && c->d.nd > 0;
@@ -555,7 +550,7 @@ lks_status lks_volume(lks_ctx* c, double vmax, double* G_out, double* dGdgamma, 
         LAUNCHED();
         const double* src = c->gtmp;
         if (c->fR > 0.0) {
-            launch_filter_T(c->d, c->fR, c->gtmp, c->hp, c->fws, c->gout, c->st);
+            launch_filter_T(c->d, c->fR, c->gtmp, c->hp, c->fws, c->fq, c->gout, c->st);
             LAUNCHED();
             src = c->gout;
         }

@@ -152,6 +152,7 @@ struct lks_ctx {
     double* fws = nullptr;       // filter normaliser per design node
     double* gout = nullptr;      // dJ/dgamma through the chain
     double* gtmp = nullptr;      // design-grid scratch
+    double* fq = nullptr;        // the transposed chain's scaled input
     double* scal = nullptr;      // device scalars
     // static solids and warm starts
     void* ks = nullptr;          // static Brinkman field storage (g.ks points here when set)

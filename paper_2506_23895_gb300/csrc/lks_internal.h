@@ -68,29 +68,27 @@ struct Motion {
 // the fill and the sensitivity gather.
 struct TransferScratch {
     int* col_base;       // [ncol][2] floor of x_ref, y_ref per design column
-    void* col_frac;      // [ncol][2] T: fractional part in [0,1)
-    float4* col_sc;      // [ncol] sin, cos of (pi f / 2) for f = x and y fractions (2D table path)
+    void* col_sc;        // [ncol] V4<T>: sin, cos of (pi f / 2), f the x and y fractions in [0,1)
     int* zt_idx;         // [bn_z][4] design z index per analysis z of the box (-1: none)
     void* zt_w;          // [bn_z][4] T: kernel weight
-    int* tap_cnt;        // [box columns]
-    int* tap_idx;        // [box columns][kMaxTaps] design column index
+    int* tap_idx;        // [box columns][kMaxTaps] design column index (one thread per column)
     void* tap_w;         // [box columns][kMaxTaps] T
     void* col_m;         // [box columns][3] T: m0, m1x, m1y
     int* dz_base;        // [lz] floor of the moved z of each design plane
-    void* dz_frac;       // [lz] T: its fractional part
+    void* dz_sc;         // [2] T: sin, cos of (pi f / 2), f its fraction (equal in all planes)
     int* err;            // device error word (bit 0: tap overflow)
 };
 
 constexpr int kMaxTaps = 32;
 
-// Scratch of the general-axis transfer: per design node the integer base of x_ref (int4) and
-// its fraction (V4<T>); per footprint-box cell the design nodes whose base is that cell.
+// Scratch of the general-axis transfer: per design node the integer base of x_ref (int4) and a
+// record of three V4<T>; per footprint-box cell the design nodes whose base is that cell.
 constexpr int kCellMax = 8;   // a unit cube holds at most 8 points at mutual distance >= 1
 struct AxisScratch {
     int4* base;
-    void* frac;
+    void* rec;
     int* cnt;    // [box cells]
-    int* idx;    // [box cells][kCellMax], ascending design index
+    int* idx;    // [box cells][kCellMax], in no fixed order
 };
 
 // Per-device once-only host state (kernel attributes are per device): bit d of `mask` records
@@ -166,11 +164,11 @@ template <class T>
 void launch_sens(const Design& d, const Geom& g, TransferScratch ts, const T* e,
                  const T* kprime, double* gacc, cudaStream_t st);
 // Design chain (FP64): gb = H(F gamma), hp = H'(F gamma), wsum = filter normaliser; the
-// transposed chain out = F^T (hp * g) (hp = nullptr: F^T g); a fixed-order sum.
+// transposed chain out = F^T (hp * g) (hp = nullptr: F^T g; q: scratch); a fixed-order sum.
 void launch_filter(const Design& d, double R, double beta, double eta, const double* gamma,
                    double* gb, double* hp, double* wsum, cudaStream_t st);
 void launch_filter_T(const Design& d, double R, const double* g, const double* hp,
-                     const double* wsum, double* out, cudaStream_t st);
+                     const double* wsum, double* q, double* out, cudaStream_t st);
 void launch_design_sum(long long nd, const double* a, double* out, cudaStream_t st);
 void launch_fill_f64(double* a, long long n, double v, cudaStream_t st);
 // General-axis transfer (kappa, u_S on the box) and its sensitivity gather.

@@ -993,8 +993,8 @@ lks_status design_prep(lks_ctx* c) {
 // dJ/dgamma of the last adjoint: the accumulator, or its pull-back through the filter chain.
 const double* design_gradient(lks_ctx* c, cudaStream_t st) {
     if (c->fR <= 0.0) return c->gacc;
-    launch_filter_T(c->d, c->fR, c->gacc, c->hp, c->fws, c->gout, st);
-    ++c->stats[4];
+    launch_filter_T(c->d, c->fR, c->gacc, c->hp, c->fws, c->fq, c->gout, st);
+    c->stats[4] += 2;
     return c->gout;
 }
 

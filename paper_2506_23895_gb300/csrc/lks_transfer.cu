@@ -24,7 +24,9 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kSmallThreads = 64;
-inline unsigned grid_for(long long n) { return (unsigned)((n + kThreads - 1) / kThreads); }
+constexpr int kFiltThreads = 128;
+inline unsigned grid_of(long long n, int t) { return (unsigned)((n + t - 1) / t); }
+inline unsigned grid_for(long long n) { return grid_of(n, kThreads); }
 
 __global__ void k_design_prep_check(long long nd, const double* gamma, int* bad) {
     long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -58,15 +60,16 @@ __global__ void k_design_pos(Design d, Geom g, Motion m, TransferScratch ts) {
     k -= d.ncol;
     const int lz = d.L[2];
     if (k < lz) {  // moved z of design plane k (3D: pure shift; 2D: the single plane at 0)
-        T* dzf = (T*)ts.dz_frac;
         if (g.dim == 3) {
             const double zr = (double)k - d.xiG[2] + m.xG[2];
             const double bz = floor(zr);
             ts.dz_base[k] = (int)bz;
-            dzf[k] = (T)(zr - bz);
+            if (k == 0) {
+                T* z = (T*)ts.dz_sc;
+                sincospi_half<T>((T)(zr - bz), z[0], z[1]);
+            }
         } else {
             ts.dz_base[k] = 0;
-            dzf[k] = (T)0;
         }
         return;
     }
@@ -105,8 +108,8 @@ __global__ void k_design_pos(Design d, Geom g, Motion m, TransferScratch ts) {
 
 // One warp per box column.  The lanes test the candidate design columns of a window around the
 // inverse rigid map (j outer, i inner, 32 at a time); a ballot keeps the accepted ones in that
-// order, and every lane sums the moments over them in the same order, so the lists and sums are
-// those of a sequential scan.  The window is found in single precision with a margin far above
+// order, and the moments are summed over them in the same order, so the lists and sums are those
+// of a sequential scan.  The window is found in single precision with a margin far above
 // its rounding: it only has to contain the support, each candidate is tested exactly.  The warp
 // then forms K2[col][zeta] = sum over the taps of W_xy kappa_ref(zeta, tap), the x-y transfer of
 // every design plane, lanes running along zeta (coalesced in kref_t), taps in list order.
@@ -118,6 +121,7 @@ __global__ void __launch_bounds__(kThreads)
                 T* __restrict__ k2) {
     __shared__ T s_w[kTapWarps][kMaxTaps];
     __shared__ int s_k[kTapWarps][kMaxTaps];
+    __shared__ T s_d[kTapWarps][2][kMaxTaps];   // xi - xi_G of each tap
     const long long ncols = (long long)g.bn[0] * g.bn[1];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long col = (long long)blockIdx.x * kTapWarps + wid;
@@ -136,12 +140,9 @@ __global__ void __launch_bounds__(kThreads)
     // xi - xi_G in T: from the single-precision centre where that is exact
     const bool fxi = sizeof(T) == 4 && (double)d.xiGf[0] == d.xiG[0] &&
                      (double)d.xiGf[1] == d.xiG[1];
-    const T* frac = (const T*)ts.col_frac;
-    int* tidx = ts.tap_idx + col * kMaxTaps;
-    T* tw = (T*)ts.tap_w + col * kMaxTaps;
+    const V4<T>* sc = (const V4<T>*)ts.col_sc;
     int cnt = 0;
     bool over = false;
-    T m0 = (T)0, m1x = (T)0, m1y = (T)0;
     for (int b = 0; b < nc && !over; b += 32) {
         const int c = b + lane;
         int k = 0;
@@ -149,42 +150,38 @@ __global__ void __launch_bounds__(kThreads)
         if (c < nc) {
             const int j = j0 + c / wi, i = i0 + c % wi;
             k = j * d.L[0] + i;
-            const T rx = (T)(x - ts.col_base[2 * k]) - frac[2 * k];
-            const T ry = (T)(y - ts.col_base[2 * k + 1]) - frac[2 * k + 1];
-            if (fabs(rx) < (T)2 && fabs(ry) < (T)2) W = peskin(rx) * peskin(ry);   // exact in T
-            di = fxi ? (T)((float)i - d.xiGf[0]) : (T)(i - d.xiG[0]);
-            dj = fxi ? (T)((float)j - d.xiGf[1]) : (T)(j - d.xiG[1]);
+            const int qx = x - ts.col_base[2 * k] + 1, qy = y - ts.col_base[2 * k + 1] + 1;
+            if ((unsigned)qx <= 3u && (unsigned)qy <= 3u) {
+                const V4<T> t = sc[k];
+                W = tap_weight<T>(qx, t.r, t.x) * tap_weight<T>(qy, t.y, t.z);
+                di = fxi ? (T)((float)i - d.xiGf[0]) : (T)(i - d.xiG[0]);
+                dj = fxi ? (T)((float)j - d.xiGf[1]) : (T)(j - d.xiG[1]);
+            }
         }
         const unsigned acc = __ballot_sync(0xffffffffu, W != (T)0);
         const int pos = cnt + __popc(acc & ((1u << lane) - 1u));
         if (W != (T)0 && pos < kMaxTaps) {
-            tidx[pos] = k;
-            tw[pos] = W;
             s_k[wid][pos] = k;
             s_w[wid][pos] = W;
+            s_d[wid][0][pos] = di;
+            s_d[wid][1][pos] = dj;
         }
-        for (unsigned r = acc; r != 0u; r &= r - 1u) {   // warp-uniform: taps in window order
-            if (cnt == kMaxTaps) {
-                over = true;
-                break;
-            }
-            const int src = __ffs(r) - 1;
-            const T Ws = __shfl_sync(0xffffffffu, W, src);
-            m0 += Ws;
-            m1x += Ws * __shfl_sync(0xffffffffu, di, src);
-            m1y += Ws * __shfl_sync(0xffffffffu, dj, src);
-            ++cnt;
+        cnt += __popc(acc);
+        if (cnt > kMaxTaps) {
+            over = true;
+            cnt = kMaxTaps;
         }
-    }
-    if (lane == 0) {
-        if (over) atomicOr(ts.err, 1);
-        ts.tap_cnt[col] = cnt;
-        T* cm = (T*)ts.col_m + 3 * col;
-        cm[0] = m0;
-        cm[1] = m1x;
-        cm[2] = m1y;
     }
     __syncwarp();
+    // m0, m1x, m1y on lanes 0, 1, 2, each over the taps in list order (every lane summing all three
+    // from shuffles took 80 of the 130 FP64 instructions of a column)
+    if (lane < 3) {
+        T a = (T)0;
+        for (int e = 0; e < cnt; ++e)
+            a += s_w[wid][e] * (lane == 0 ? (T)1 : s_d[wid][lane - 1][e]);
+        ((T*)ts.col_m)[3 * col + lane] = a;
+    }
+    if (lane == 0 && over) atomicOr(ts.err, 1);
     const int lz = d.L[2];
     const T* sw = s_w[wid];
     const int* sk = s_k[wid];
@@ -214,7 +211,7 @@ __global__ void __launch_bounds__(kThreads)
     const float R = 2.f * (fabsf(m.cf) + fabsf(m.sf)) + 0.01f;
     const int i0 = max(0, (int)ceilf(ic - R)), i1 = min(d.L[0] - 1, (int)floorf(ic + R));
     const int j0 = max(0, (int)ceilf(jc - R)), j1 = min(d.L[1] - 1, (int)floorf(jc + R));
-    const T* frac = (const T*)ts.col_frac;
+    const V4<T>* sc = (const V4<T>*)ts.col_sc;
     int* tidx = ts.tap_idx + col * kMaxTaps;
     T* tw = (T*)ts.tap_w + col * kMaxTaps;
     int cnt = 0;
@@ -222,10 +219,10 @@ __global__ void __launch_bounds__(kThreads)
     for (int j = j0; j <= j1; ++j)
         for (int i = i0; i <= i1; ++i) {
             const int k = j * d.L[0] + i;
-            const T rx = (T)(x - ts.col_base[2 * k]) - frac[2 * k];
-            const T ry = (T)(y - ts.col_base[2 * k + 1]) - frac[2 * k + 1];
-            if (!(fabs(rx) < (T)2 && fabs(ry) < (T)2)) continue;   // exact in T
-            const T W = peskin(rx) * peskin(ry);
+            const int qx = x - ts.col_base[2 * k] + 1, qy = y - ts.col_base[2 * k + 1] + 1;
+            if ((unsigned)qx > 3u || (unsigned)qy > 3u) continue;
+            const V4<T> t = sc[k];
+            const T W = tap_weight<T>(qx, t.r, t.x) * tap_weight<T>(qy, t.y, t.z);
             if (W == (T)0) continue;
             if (cnt == kMaxTaps) {
                 atomicOr(ts.err, 1);
@@ -240,7 +237,6 @@ __global__ void __launch_bounds__(kThreads)
             m1x += W * (T)(i - d.xiG[0]);
             m1y += W * (T)(j - d.xiG[1]);
         }
-    ts.tap_cnt[col] = cnt;
     T* cm = (T*)ts.col_m + 3 * col;
     cm[0] = m0;
     cm[1] = m1x;
@@ -353,54 +349,113 @@ __global__ void k_box_to_grid(Geom g, const V4<T>* __restrict__ kus, double* kap
 // Density filter with linear weights w = max(0, R - |xi_i - xi_j|) over the design grid and the
 // tanh Heaviside projection (the projection filter the paper cites, Secs. 1 and 3.1), in FP64:
 // gb = H(F gamma), hp = H'(F gamma), wsum = sum_j w_ij.  One thread per design node, offsets
-// visited in (z, y, x) order.
-__global__ void k_filter(Design d, double R, int rr, double beta, double eta,
-                         const double* __restrict__ gamma, double* __restrict__ gb,
-                         double* __restrict__ hp, double* __restrict__ wsum) {
-    const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (k >= d.nd) return;
+// visited in (z, y, x) order.  The offsets of non-zero weight are the same for every node, so each
+// block lists them once (57 of 343 at R = 2.4): a square root and a branch at every offset of every
+// node took 294 us, and a division in the transpose 369 us, on a 33 x 41 x 27 design.
+constexpr int kFiltMax = 1024;   // listed offsets; a wider filter forms its weights as it goes
+
+struct FiltList {
+    double w[kFiltMax];
+    int off[kFiltMax];   // dx + 512, dy + 512, dz + 512 in ten bits each
+    int n;               // -1: more than kFiltMax
+};
+
+__device__ __forceinline__ void filter_list(FiltList& f, double R, int rr, int rz) {
+    if (threadIdx.x < 32) {
+        const int side = 2 * rr + 1, lane = threadIdx.x;
+        const long long all = (long long)side * side * (2 * rz + 1);
+        int n = 0;
+        for (long long t0 = 0; t0 < all && n >= 0; t0 += 32) {
+            const long long t = t0 + lane;
+            double w = 0.0;
+            int dx = 0, dy = 0, dz = 0;
+            if (t < all) {
+                const unsigned u = (unsigned)t;
+                dx = (int)(u % side) - rr;
+                dy = (int)(u / side % side) - rr;
+                dz = (int)(u / side / side) - rz;
+                w = R - sqrt((double)(dx * dx + dy * dy + dz * dz));
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, w > 0.0);
+            if (n + __popc(m) > kFiltMax) n = -1;
+            else {
+                const int at = n + __popc(m & ((1u << lane) - 1u));
+                if (w > 0.0) {
+                    f.w[at] = w;
+                    f.off[at] = (dx + 512) | (dy + 512) << 10 | (dz + 512) << 20;
+                }
+                n += __popc(m);
+            }
+        }
+        if (lane == 0) f.n = n;
+    }
+    __syncthreads();
+}
+
+// sum over the offsets of w a[neighbour] (acc) and of w (W) at design node k.
+__device__ __forceinline__ void filter_sum(const Design& d, const FiltList& f, double R, int rr,
+                                           int rz, const double* __restrict__ a, long long k,
+                                           double& acc, double& W) {
     const int x = (int)(k % d.L[0]), y = (int)((k / d.L[0]) % d.L[1]), z = (int)(k / d.ncol);
-    const int rz = d.L[2] > 1 ? rr : 0;
-    double acc = 0.0, W = 0.0;
+    auto add = [&](int dx, int dy, int dz, double w) {
+        const int xx = x + dx, yy = y + dy, zz = z + dz;
+        if ((unsigned)xx >= (unsigned)d.L[0] || (unsigned)yy >= (unsigned)d.L[1] ||
+            (unsigned)zz >= (unsigned)d.L[2])
+            return;
+        acc += w * a[((long long)zz * d.L[1] + yy) * d.L[0] + xx];
+        W += w;
+    };
+    acc = W = 0.0;
+    if (f.n >= 0) {
+        for (int t = 0; t < f.n; ++t) {
+            const int o = f.off[t];
+            add((o & 1023) - 512, (o >> 10 & 1023) - 512, (o >> 20 & 1023) - 512, f.w[t]);
+        }
+        return;
+    }
     for (int dz = -rz; dz <= rz; ++dz)
         for (int dy = -rr; dy <= rr; ++dy)
             for (int dx = -rr; dx <= rr; ++dx) {
                 const double w = R - sqrt((double)(dx * dx + dy * dy + dz * dz));
-                if (!(w > 0.0)) continue;
-                const int xx = x + dx, yy = y + dy, zz = z + dz;
-                if (xx < 0 || yy < 0 || zz < 0 || xx >= d.L[0] || yy >= d.L[1] || zz >= d.L[2])
-                    continue;
-                acc += w * gamma[((long long)zz * d.L[1] + yy) * d.L[0] + xx];
-                W += w;
+                if (w > 0.0) add(dx, dy, dz, w);
             }
-    const double gt = acc / W;
-    const double den = tanh(beta * eta) + tanh(beta * (1.0 - eta));
-    const double t = tanh(beta * (gt - eta));
-    gb[k] = (tanh(beta * eta) + t) / den;
+}
+
+// tb = tanh(beta eta), den = tb + tanh(beta (1 - eta)).
+__global__ void __launch_bounds__(kFiltThreads)
+    k_filter(Design d, double R, int rr, double beta, double eta, double tb, double den,
+             const double* __restrict__ gamma, double* __restrict__ gb, double* __restrict__ hp,
+             double* __restrict__ wsum) {
+    __shared__ FiltList f;
+    const int rz = d.L[2] > 1 ? rr : 0;
+    filter_list(f, R, rr, rz);
+    const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (k >= d.nd) return;
+    double acc, W;
+    filter_sum(d, f, R, rr, rz, gamma, k, acc, W);
+    const double t = tanh(beta * (acc / W - eta));
+    gb[k] = (tb + t) / den;
     hp[k] = beta * (1.0 - t * t) / den;
     wsum[k] = W;
 }
 
-// Transposed chain: out_j = sum_i w_ij hp_i g_i / wsum_i (a gather over the same offsets).
-__global__ void k_filter_T(Design d, double R, int rr, const double* __restrict__ g,
+// Transposed chain: out_j = sum_i w_ij q_i (a gather over the same offsets), q_i = hp_i g_i / wsum_i.
+__global__ void k_filter_q(long long nd, const double* __restrict__ g,
                            const double* __restrict__ hp, const double* __restrict__ wsum,
-                           double* __restrict__ out) {
+                           double* __restrict__ q) {
+    const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (k < nd) q[k] = (hp ? hp[k] * g[k] : g[k]) / wsum[k];
+}
+
+__global__ void __launch_bounds__(kFiltThreads)
+    k_filter_T(Design d, double R, int rr, const double* __restrict__ q, double* __restrict__ out) {
+    __shared__ FiltList f;
+    const int rz = d.L[2] > 1 ? rr : 0;
+    filter_list(f, R, rr, rz);
     const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (k >= d.nd) return;
-    const int x = (int)(k % d.L[0]), y = (int)((k / d.L[0]) % d.L[1]), z = (int)(k / d.ncol);
-    const int rz = d.L[2] > 1 ? rr : 0;
-    double acc = 0.0;
-    for (int dz = -rz; dz <= rz; ++dz)
-        for (int dy = -rr; dy <= rr; ++dy)
-            for (int dx = -rr; dx <= rr; ++dx) {
-                const double w = R - sqrt((double)(dx * dx + dy * dy + dz * dz));
-                if (!(w > 0.0)) continue;
-                const int xx = x + dx, yy = y + dy, zz = z + dz;
-                if (xx < 0 || yy < 0 || zz < 0 || xx >= d.L[0] || yy >= d.L[1] || zz >= d.L[2])
-                    continue;
-                const long long i = ((long long)zz * d.L[1] + yy) * d.L[0] + xx;
-                acc += w * (hp ? hp[i] * g[i] : g[i]) / wsum[i];
-            }
+    double acc, W;
+    filter_sum(d, f, R, rr, rz, q, k, acc, W);
     out[k] = acc;
 }
 
@@ -432,14 +487,16 @@ void launch_fill_f64(double* a, long long n, double v, cudaStream_t st) {
 void launch_filter(const Design& d, double R, double beta, double eta, const double* gamma,
                    double* gb, double* hp, double* wsum, cudaStream_t st) {
     if (d.nd == 0) return;
-    k_filter<<<grid_for(d.nd), kThreads, 0, st>>>(d, R, (int)ceil(R), beta, eta, gamma, gb, hp,
-                                                  wsum);
+    const double tb = tanh(beta * eta), den = tb + tanh(beta * (1.0 - eta));
+    k_filter<<<grid_of(d.nd, kFiltThreads), kFiltThreads, 0, st>>>(d, R, (int)ceil(R), beta, eta,
+                                                                  tb, den, gamma, gb, hp, wsum);
 }
 
 void launch_filter_T(const Design& d, double R, const double* g, const double* hp,
-                     const double* wsum, double* out, cudaStream_t st) {
+                     const double* wsum, double* q, double* out, cudaStream_t st) {
     if (d.nd == 0) return;
-    k_filter_T<<<grid_for(d.nd), kThreads, 0, st>>>(d, R, (int)ceil(R), g, hp, wsum, out);
+    k_filter_q<<<grid_for(d.nd), kThreads, 0, st>>>(d.nd, g, hp, wsum, q);
+    k_filter_T<<<grid_of(d.nd, kFiltThreads), kFiltThreads, 0, st>>>(d, R, (int)ceil(R), q, out);
 }
 
 void launch_design_sum(long long nd, const double* a, double* out, cudaStream_t st) {

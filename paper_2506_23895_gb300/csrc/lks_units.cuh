@@ -7,23 +7,6 @@
 
 namespace lks {
 
-// ---------------------------------------------------------------- design positions (Sec. 2.3)
-// x_ref, y_ref of design column k (FP64) as integer base + fraction in [0,1).
-template <class T>
-__device__ __forceinline__ void design_col_pos(const Design& d, const Motion& m,
-                                               const TransferScratch& ts, long long k) {
-    T* frac = (T*)ts.col_frac;
-    const int i = (int)((unsigned)k % (unsigned)d.L[0]), j = (int)((unsigned)k / (unsigned)d.L[0]);
-    const double dx = i - d.xiG[0], dy = j - d.xiG[1];
-    const double xr = m.c * dx - m.s * dy + m.xG[0];   // Eq. rigid_body_position
-    const double yr = m.s * dx + m.c * dy + m.xG[1];
-    const double bx = floor(xr), by = floor(yr);
-    ts.col_base[2 * k] = (int)bx;
-    ts.col_base[2 * k + 1] = (int)by;
-    frac[2 * k] = (T)(xr - bx);
-    frac[2 * k + 1] = (T)(yr - by);
-}
-
 // ---------------------------------------------------------------- 2D transfer (table path)
 // Design column k for the D2Q9 instance-table kernels: integer base of x_ref, y_ref and, per axis,
 // S = sin(pi f/2), C = cos(pi f/2) of the fraction f.  The four
@@ -56,6 +39,18 @@ __device__ __forceinline__ int ref_coord(float ah, float al, float da, float bh,
     return gi + (int)fl;
 }
 
+// sin and cos of pi f / 2.
+template <class T>
+__device__ __forceinline__ void sincospi_half(T f, T& s, T& c);
+template <>
+__device__ __forceinline__ void sincospi_half<float>(float f, float& s, float& c) {
+    sincospif(0.5f * f, &s, &c);
+}
+template <>
+__device__ __forceinline__ void sincospi_half<double>(double f, double& s, double& c) {
+    sincospi(0.5 * f, &s, &c);
+}
+
 template <class T>
 __device__ __forceinline__ void col_pos_sc(const Design& d, const Motion& m, long long k, int2& b,
                                            V4<T>& sc);
@@ -68,8 +63,8 @@ __device__ __forceinline__ void col_pos_sc<float>(const Design& d, const Motion&
     float fx, fy;   // Eq. rigid_body_position: x_ref = c dx - s dy + x_G, y_ref = s dx + c dy + y_G
     b.x = ref_coord(m.ch, m.cl, dx, m.sh, m.sl, dy, m.xgi[0], m.xgh[0], m.xgl[0], fx);
     b.y = ref_coord(m.sh, m.sl, dx, -m.ch, -m.cl, dy, m.xgi[1], m.xgh[1], m.xgl[1], fy);
-    sincospif(0.5f * fx, &sc.r, &sc.x);
-    sincospif(0.5f * fy, &sc.y, &sc.z);
+    sincospi_half<float>(fx, sc.r, sc.x);
+    sincospi_half<float>(fy, sc.y, sc.z);
 }
 
 template <>
@@ -80,8 +75,8 @@ __device__ __forceinline__ void col_pos_sc<double>(const Design& d, const Motion
     const double xr = m.c * dx - m.s * dy + m.xG[0], yr = m.s * dx + m.c * dy + m.xG[1];
     const double bx = floor(xr), by = floor(yr);
     b = make_int2((int)bx, (int)by);
-    sincospi(0.5 * (xr - bx), &sc.r, &sc.x);
-    sincospi(0.5 * (yr - by), &sc.y, &sc.z);
+    sincospi_half<double>(xr - bx, sc.r, sc.x);
+    sincospi_half<double>(yr - by, sc.y, sc.z);
 }
 
 // Weight of tap q1 - 1 = -1, 0, 1, 2 from S = sin(pi f/2), C = cos(pi f/2) of the fraction f.
@@ -89,6 +84,26 @@ template <class T>
 __device__ __forceinline__ T tap_weight(int q1, T S, T C) {
     const T t = q1 == 0 ? -S : (q1 == 1 ? C : (q1 == 2 ? S : -C));
     return (T)0.25 * ((T)1 + t);
+}
+
+// ---------------------------------------------------------------- design positions (Sec. 2.3)
+// x_ref, y_ref of design column k (FP64) as integer base, and sin, cos of (pi f / 2) of the fractions
+// f in [0,1): every tap weight then takes one multiply-add, where evaluating the kernel takes a
+// cosine at each (analysis column, design column) pair.
+template <class T>
+__device__ __forceinline__ void design_col_pos(const Design& d, const Motion& m,
+                                               const TransferScratch& ts, long long k) {
+    const int i = (int)((unsigned)k % (unsigned)d.L[0]), j = (int)((unsigned)k / (unsigned)d.L[0]);
+    const double dx = i - d.xiG[0], dy = j - d.xiG[1];
+    const double xr = m.c * dx - m.s * dy + m.xG[0];   // Eq. rigid_body_position
+    const double yr = m.s * dx + m.c * dy + m.xG[1];
+    const double bx = floor(xr), by = floor(yr);
+    ts.col_base[2 * k] = (int)bx;
+    ts.col_base[2 * k + 1] = (int)by;
+    V4<T> sc;
+    sincospi_half<T>((T)(xr - bx), sc.r, sc.x);
+    sincospi_half<T>((T)(yr - by), sc.y, sc.z);
+    ((V4<T>*)ts.col_sc)[k] = sc;
 }
 
 // sum of W e(x) over the 4 x 4 taps of design node k (the transpose of the kappa transfer) with
@@ -130,16 +145,15 @@ __device__ __forceinline__ void sens_run(const Design& d, const Geom& g, const T
     const unsigned k = (unsigned)t % (unsigned)d.ncol;   // design column
     const int z0 = (int)((unsigned)t / (unsigned)d.ncol) * kSensRun;
     const int z1 = min(d.L[2], z0 + kSensRun);
-    const T* frac = (const T*)ts.col_frac;
     const int bx = ts.col_base[2 * k], by = ts.col_base[2 * k + 1];
-    const T fx = frac[2 * k], fy = frac[2 * k + 1];
+    const V4<T> sc = ((const V4<T>*)ts.col_sc)[k];
+    const T zs = ((const T*)ts.dz_sc)[0], zc = ((const T*)ts.dz_sc)[1];
     T wx[4], wy[4], wz[4];
-    const T fz = ((const T*)ts.dz_frac)[0];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        wx[q] = peskin((T)(q - 1) - fx);
-        wy[q] = peskin((T)(q - 1) - fy);
-        wz[q] = (g.dim == 3) ? peskin((T)(q - 1) - fz) : (q == 1 ? (T)1 : (T)0);
+        wx[q] = tap_weight<T>(q, sc.r, sc.x);
+        wy[q] = tap_weight<T>(q, sc.y, sc.z);
+        wz[q] = (g.dim == 3) ? tap_weight<T>(q, zs, zc) : (q == 1 ? (T)1 : (T)0);
     }
     const int ex0 = bx - 1 - g.blo[0], ey0 = by - 1 - g.blo[1];
     // x-y tap sum of analysis plane z (0 outside the box, where W vanishes)
