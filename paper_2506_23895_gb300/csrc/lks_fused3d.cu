@@ -19,6 +19,7 @@
 #include <type_traits>
 
 #include "lks_device.cuh"
+#include "lks_march3d.h"
 #include "lks_tma.cuh"
 
 namespace lks {
@@ -897,445 +898,6 @@ __global__ void __launch_bounds__(ZCfg<TY_>::NTHR, ZCfg<TY_>::MINB)
         zbody<TY_, false>(tmap, a, smem, hfx, hfy, q0, q1, nplanes);
 }
 
-// ---------------------------------------------------------------- plane-pair z-march variant
-// The same step with two planes per iteration and packed single-precision arithmetic:
-//   * a thread owns one column of a 32 x 8 tile and evaluates f^eq at two consecutive planes
-//     (a, a + 1) per iteration, with the two planes' values held as float2 pairs, so the f^eq
-//     core, the gather sums and the z-accumulation run on paired FP32 instructions
-//     (__ffma2_rn, __fadd2_rn, __fmul2_rn: two operations per instruction issue);
-//   * the 12 values that leave the column travel through shared memory as (plane a, plane a+1)
-//     pairs: an in-plane shift keeps the pairing, so every exchange is one 8-byte store and one
-//     8-byte load for two nodes; the exchange buffers alternate, one block barrier per pair;
-//   * raw planes arrive through the same TMA boxes into a six-slot ring, two new planes per
-//     iteration, every thread waiting on the mbarriers of the planes it reads (bounded waits);
-//   * an iteration completes the outputs of planes a - 1 and a: plane a - 1 from the carried
-//     cz = 0 and cz = +1 sums of plane a - 1 and a - 2 plus the cz = -1 sums of plane a, plane
-//     a from its own cz = 0 sums, the carried cz = +1 sums of plane a - 1 and the cz = -1 sums
-//     of plane a + 1.
-// Derivatives are formed per plane in single precision as in feq_node; the arithmetic of f^eq,
-// the gather and the Brinkman update is that of the other variants, with the sums in a
-// different order (results agree to rounding).
-struct PCfg {
-    static constexpr int TX = 32, TY = 8;
-    static constexpr int HX = TX + 5, HY = TY + 4, FW = TX + 2, FX = FW + 1, FY = TY + 2;
-    static constexpr int NTHR = TX * TY, NHALO = FW * FY - TX * TY, FS = FX * FY;
-    static constexpr int NSLOT = 6;
-    static constexpr int MINB = 2;     // resident blocks per SM
-    static constexpr unsigned PLANE_BYTES = HX * HY * 16;
-    static constexpr int SLOT = (PLANE_BYTES + 127) / 128 * 128 / 16;   // float4 per ring slot
-    static constexpr size_t OFF_F = (size_t)NSLOT * SLOT * 16;
-    static constexpr size_t OFF_BAR = OFF_F + (size_t)2 * NCROSS * FS * 8;
-    static constexpr size_t SMEM = OFF_BAR + NSLOT * 8;
-};
-
-// Packed constants of the pair kernel (both lanes equal).
-struct PairK {
-    float2 A, hA, m15, w0, w1, w13, nw13, h1, w2, w23, nw23, h2, w2x2, nw2x2, mone;
-};
-
-__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-// a - b: b * (-1) is exact, so this rounds once like a subtraction
-__device__ __forceinline__ float2 psub(float2 a, float2 b, float2 mone) {
-    return __ffma2_rn(b, mone, a);
-}
-
-// Dab = 2 d u_a / d x_b of one plane at one column (naming as in feq_node): c0 points at the
-// node in its ring plane, c is the node, um / up the velocity one plane below / above.
-struct D9 {
-    float xx, yx, zx, xy, yy, zy, xz, yz, zz;
-};
-
-template <bool EDGE>
-__device__ __forceinline__ void deriv_plane(const float4* __restrict__ c0, const float4& c,
-                                            const float3& um, const float3& up, int xm, int ym,
-                                            int zm, const float4& zfar, D9& d) {
-    constexpr int HXs = PCfg::HX;
-    if (EDGE) {
-        const float4 cm4 = make_float4(0.f, um.x, um.y, um.z);
-        const float4 cp4 = make_float4(0.f, up.x, up.y, up.z);
-        deriv2(xm, c, c0[-1], c0[1], xm == 2 ? c0[-2] : c, xm == 1 ? c0[2] : c, d.xx, d.yx, d.zx);
-        deriv2(ym, c, c0[-HXs], c0[HXs], ym == 2 ? c0[-2 * HXs] : c, ym == 1 ? c0[2 * HXs] : c,
-               d.xy, d.yy, d.zy);
-        deriv2(zm, c, cm4, cp4, zfar, zfar, d.xz, d.yz, d.zz);
-    } else {
-        const float4 e = c0[1], w = c0[-1], n = c0[HXs], s = c0[-HXs];
-        d.xx = e.y - w.y;
-        d.yx = e.z - w.z;
-        d.zx = e.w - w.w;
-        d.xy = n.y - s.y;
-        d.yy = n.z - s.z;
-        d.zy = n.w - s.w;
-        d.xz = up.x - um.x;
-        d.yz = up.y - um.y;
-        d.zz = up.z - um.z;
-    }
-}
-
-// f^eq of one column at two planes (lanes: plane a, plane a + 1) from the node values c* and
-// the derivatives of each plane: stores the 12 values that leave the column into the pair
-// planes at sFn (FS pairs apart) and returns rest, +z and -z.  The operations are those of
-// feq_node on pairs.
-__device__ __forceinline__ void feq_pair(const PairK& k, const float4& ca, const float4& cb,
-                                         const D9& da, const D9& db, float2* __restrict__ sFn,
-                                         float2& f_rest, float2& f_pz, float2& f_mz) {
-    constexpr int FS = PCfg::FS;
-    const float2 r = make_float2(ca.x, cb.x), ux = make_float2(ca.y, cb.y);
-    const float2 uy = make_float2(ca.z, cb.z), uz = make_float2(ca.w, cb.w);
-    const float2 ASxx = pmul(k.A, make_float2(da.xx, db.xx));
-    const float2 ASyy = pmul(k.A, make_float2(da.yy, db.yy));
-    const float2 ASzz = pmul(k.A, make_float2(da.zz, db.zz));
-    const float2 ASxy = pmul(k.hA, padd(make_float2(da.xy, db.xy), make_float2(da.yx, db.yx)));
-    const float2 ASxz = pmul(k.hA, padd(make_float2(da.xz, db.xz), make_float2(da.zx, db.zx)));
-    const float2 ASyz = pmul(k.hA, padd(make_float2(da.yz, db.yz), make_float2(da.zy, db.zy)));
-    const float2 uu = pfma(uz, uz, pfma(uy, uy, pmul(ux, ux)));
-    const float2 P = pfma(k.m15, uu, r);
-    f_rest = pmul(k.w0, P);
-    const float2 Px = padd(P, ASxx);
-    {
-        const float2 b = pfma(pmul(k.h1, ux), ux, pmul(k.w1, Px));
-        sFn[0 * FS] = pfma(k.w13, ux, b);
-        sFn[1 * FS] = pfma(k.nw13, ux, b);
-    }
-    {
-        const float2 b = pfma(pmul(k.h1, uy), uy, pmul(k.w1, padd(P, ASyy)));
-        sFn[2 * FS] = pfma(k.w13, uy, b);
-        sFn[3 * FS] = pfma(k.nw13, uy, b);
-    }
-    {
-        const float2 b = pfma(pmul(k.h1, uz), uz, pmul(k.w1, padd(P, ASzz)));
-        f_pz = pfma(k.w13, uz, b);
-        f_mz = pfma(k.nw13, uz, b);
-    }
-    const float2 T0 = pmul(k.w2, padd(padd(Px, ASyy), ASzz));
-    const float2 s1 = padd(ux, uy), d1 = psub(ux, uy, k.mone);
-    const float2 q1 = padd(ASxz, ASyz), q2 = psub(ASyz, ASxz, k.mone);
-    {   // (+,+,+) / (-,-,-)
-        const float2 cu = padd(s1, uz);
-        const float2 sym = pfma(pmul(k.h2, cu), cu, pfma(k.w2x2, padd(ASxy, q1), T0));
-        sFn[4 * FS] = pfma(k.w23, cu, sym);
-        sFn[11 * FS] = pfma(k.nw23, cu, sym);
-    }
-    {   // (-,+,+) / (+,-,-)
-        const float2 cu = psub(uz, d1, k.mone);
-        const float2 sym = pfma(pmul(k.h2, cu), cu, pfma(k.w2x2, psub(q2, ASxy, k.mone), T0));
-        sFn[5 * FS] = pfma(k.w23, cu, sym);
-        sFn[10 * FS] = pfma(k.nw23, cu, sym);
-    }
-    {   // (+,-,+) / (-,+,-)
-        const float2 cu = padd(uz, d1);
-        const float2 sym = pfma(pmul(k.h2, cu), cu, pfma(k.nw2x2, padd(ASxy, q2), T0));
-        sFn[6 * FS] = pfma(k.w23, cu, sym);
-        sFn[9 * FS] = pfma(k.nw23, cu, sym);
-    }
-    {   // (-,-,+) / (+,+,-)
-        const float2 cu = psub(uz, s1, k.mone);
-        const float2 sym = pfma(pmul(k.h2, cu), cu, pfma(k.w2x2, psub(ASxy, q1, k.mone), T0));
-        sFn[7 * FS] = pfma(k.w23, cu, sym);
-        sFn[8 * FS] = pfma(k.nw23, cu, sym);
-    }
-}
-
-struct PairArgs {
-    FusedArgs f;
-    PairK k;
-    float2 bf2[3];   // body force, both lanes
-    int has_bf;
-};
-
-// Write one output node (Brinkman update, store, boundary copies it sources).
-__device__ __forceinline__ void pair_out(const Geom& g, const PairArgs& a, int gx, int gy,
-                                         int qz, float r, float ux, float uy, float uz,
-                                         bool box_col, const float4* kus_col,
-                                         long long box_plane, float4* out_col_ptr,
-                                         long long zstride, bool bc_col) {
-    float4 o;
-    o.x = r;
-    const int bz = qz - g.blo[2];
-    if (box_col && bz >= 0 && bz < g.bn[2]) {
-        const float4 ks = kus_col[(long long)qz * box_plane];
-        const float inv = 1.f / (1.f + ks.x);
-        o.y = fmaf(ks.x, ks.y, ux) * inv;
-        o.z = fmaf(ks.x, ks.z, uy) * inv;
-        o.w = fmaf(ks.x, ks.w, uz) * inv;
-    } else {
-        o.y = ux;
-        o.z = uy;
-        o.w = uz;
-    }
-    out_col_ptr[(long long)qz * zstride] = o;
-    if (bc_col || qz == 1 || qz == g.n[2] - 2) write_bc_f(g, gx, gy, qz, o, a.f.out);
-}
-
-// The z derivative at a z-face plane is the one-sided difference; with a ghost value
-// g = 3 u(0) - 3 u(1) + u(2) below plane 0 (or 3 u(n-1) - 3 u(n-2) + u(n-3) above plane n-1) the
-// central difference u(1) - g (g - u(n-2)) equals it, so the pair path keeps one formula.
-__device__ __forceinline__ float3 zghost(const float3& f, const float3& s, const float3& t) {
-    return make_float3(fmaf(3.f, f.x - s.x, t.x), fmaf(3.f, f.y - s.y, t.y),
-                       fmaf(3.f, f.z - s.z, t.z));
-}
-
-__device__ __forceinline__ float3 u3(const float4& v) { return make_float3(v.y, v.z, v.w); }
-
-// z derivatives (2 d u / d z) of the pair's planes a0 (da) and a0 + 1 (db) at a z face, from
-// the ghost value: um, ua, ub, uc are u at a0 - 1 .. a0 + 2; col points at the column in the
-// source state (for u(2) or u(nz - 3) when the pair does not hold it).
-__device__ __forceinline__ void zface_fix(int a0, int nz, const float3& um, const float3& ua,
-                                       const float3& ub, const float3& uc,
-                                       const float4* __restrict__ col, long long zstride,
-                                       D9& da, D9& db) {
-    if (a0 == 0) {   // plane 0 first: ghost below it
-        const float3 gh = zghost(ua, ub, uc);
-        da.xz = ub.x - gh.x;
-        da.yz = ub.y - gh.y;
-        da.zz = ub.z - gh.z;
-    }
-    if (a0 == -1) {  // plane 0 second
-        const float3 gh = zghost(ub, uc, u3(col[2 * zstride]));
-        db.xz = uc.x - gh.x;
-        db.yz = uc.y - gh.y;
-        db.zz = uc.z - gh.z;
-    }
-    if (a0 + 1 == nz - 1) {   // plane nz-1 second: ghost above it
-        const float3 gh = zghost(ub, ua, um);
-        db.xz = gh.x - ua.x;
-        db.yz = gh.y - ua.y;
-        db.zz = gh.z - ua.z;
-    }
-    if (a0 == nz - 1) {   // plane nz-1 first
-        const float3 gh = zghost(ua, um, u3(col[(long long)(nz - 3) * zstride]));
-        da.xz = gh.x - um.x;
-        da.yz = gh.y - um.y;
-        da.zz = gh.z - um.z;
-    }
-}
-
-// The plane-pair march of one interior tile (its raw halo inside the grid, no x or y face
-// within two nodes): no face tests in x and y; z-face planes through ghost values.
-__device__ __forceinline__ void pbody(const CUtensorMap& tmap, const PairArgs& a,
-                                      unsigned char* smem, int hfx, int hfy, int q0, int q1) {
-    using C = PCfg;
-    constexpr int TX = C::TX, HX = C::HX, FX = C::FX;
-    constexpr int FS = C::FS, NSLOT = C::NSLOT;
-    float4* raw = reinterpret_cast<float4*>(smem);
-    float2* sFbase = reinterpret_cast<float2*>(smem + C::OFF_F);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR);
-    const Geom& g = a.f.g;
-    const PairK& k = a.k;
-    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const int tid = threadIdx.x;
-    const int tx = tid % TX, ty = tid / TX;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * C::TY;
-    const int gx = x0 + tx, gy = y0 + ty;
-    const int hgx = x0 - 1 + hfx, hgy = y0 - 1 + hfy;
-    const int hp = (ty + 2) * HX + (tx + 2);
-    const int hr = (hfy + 1) * HX + (hfx + 1);
-    const int fop = (ty + 1) * FX + (tx + 1);
-    const int forr = hfy * FX + hfx;
-    constexpr int RIMW = (C::NHALO + 31) / 32 * 32;
-    const bool has_rim = tid < RIMW;
-    const bool bc_col = false;
-    const int bxx = gx - g.blo[0], byy = gy - g.blo[1];
-    const bool box_col = g.boxN > 0 && bxx >= 0 && byy >= 0 && bxx < g.bn[0] && byy < g.bn[1];
-    const long long box_plane = (long long)g.bn[0] * g.bn[1];
-    const float4* kus_col =
-        a.f.kus + ((long long)byy * g.bn[0] + bxx) - (long long)g.blo[2] * box_plane;
-    const long long zstride = (long long)nx * ny;
-    float4* out_col_ptr = a.f.out + ((long long)gy * nx + gx);
-    const float4* src_col = a.f.src + ((long long)gy * nx + gx);
-    const float4* src_rim = a.f.src + ((long long)hgy * nx + hgx);
-    const int zlo = max(q0, 1), zhi = min(q1 - 1, nz - 2);
-    const int npairs = ((q1 - q0 + 1) >> 1) + 1;
-    const int nplanes = 2 * npairs + 2;
-
-    bool ok = true;
-    float3 um, rum;
-    float4 ca, rca;
-    {
-        bool good = true;
-        for (int j = 0; j < 4; ++j) good = mbar_wait_once(smem_addr(&bars[j]), 0) && good;
-        um = u3(raw[hp]);
-        ca = raw[(size_t)C::SLOT + hp];
-        rum = u3(raw[hr]);
-        rca = raw[(size_t)C::SLOT + hr];
-        ok = !__syncthreads_or(!good);
-    }
-    float pend_r = 0.f, pend_x = 0.f, pend_y = 0.f, pend_z = 0.f;
-    float pc_r = 0.f, pc_x = 0.f, pc_y = 0.f, pc_z = 0.f;
-    int ik = NSLOT;
-    // ring slots and phase parities of the loads of planes a0, a0 + 1, a0 + 2
-    int sa = 1, sb = 2, sc = 3, pb = 0, pcp = 0;
-    for (int it = 0; ok && it < npairs; ++it) {
-        const int a0 = q0 - 1 + 2 * it;
-        bool good = true;
-        if (it > 0) good = mbar_wait_once(smem_addr(&bars[sb]), pb);
-        good = mbar_wait_once(smem_addr(&bars[sc]), pcp) && good;
-        const float4* ra = raw + (size_t)sa * C::SLOT;
-        const float4* rb = raw + (size_t)sb * C::SLOT;
-        const float4* rc = raw + (size_t)sc * C::SLOT;
-        float2* sF = sFbase + (size_t)(it & 1) * NCROSS * FS;
-        const float4 cb = rb[hp], cc = rc[hp];
-        const float3 ub = u3(cb), uc = u3(cc), ua = u3(ca);
-        const bool zface = a0 <= 0 || a0 + 1 >= nz - 1;
-        float2 f_rest, f_pz, f_mz;
-        {
-            D9 da, db;
-            const float4 z0 = make_float4(0.f, 0.f, 0.f, 0.f);
-            deriv_plane<false>(ra + hp, ca, um, ub, 0, 0, 0, z0, da);
-            deriv_plane<false>(rb + hp, cb, ua, uc, 0, 0, 0, z0, db);
-            if (zface) zface_fix(a0, nz, um, ua, ub, uc, src_col, zstride, da, db);
-            feq_pair(k, ca, cb, da, db, sF + fop, f_rest, f_pz, f_mz);
-            if (has_rim) {
-                const float4 rcb = rb[hr], rcc = rc[hr];
-                const float3 rua = u3(rca), rub = u3(rcb), ruc = u3(rcc);
-                deriv_plane<false>(ra + hr, rca, rum, rub, 0, 0, 0, z0, da);
-                deriv_plane<false>(rb + hr, rcb, rua, ruc, 0, 0, 0, z0, db);
-                if (zface) zface_fix(a0, nz, rum, rua, rub, ruc, src_rim, zstride, da, db);
-                float2 d0, d1, d2;
-                feq_pair(k, rca, rcb, da, db, sF + forr, d0, d1, d2);
-                rum = rub;
-                rca = rcc;
-            }
-        }
-        um = ub;
-        ca = cc;
-        if (__syncthreads_or(!good)) {
-            ok = false;
-            break;
-        }
-        if (tid == 0) {
-            const int jmax = min(2 * it + 9, nplanes);
-            if (ik < jmax) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            for (; ik < jmax; ++ik)
-                tma_load_box(smem_addr(raw + (size_t)(ik % NSLOT) * C::SLOT), &tmap, x0 - 2,
-                             y0 - 2, q0 - 2 + ik, smem_addr(&bars[ik % NSLOT]), C::PLANE_BYTES);
-        }
-        // advance the slots by two planes
-        sa = sc;
-        sb += 2;
-        if (sb >= NSLOT) {
-            sb -= NSLOT;
-            pb ^= 1;
-        }
-        sc += 2;
-        if (sc >= NSLOT) {
-            sc -= NSLOT;
-            pcp ^= 1;
-        }
-        const float2* sFp = sF + fop;
-        const float2 fpx = sFp[0 * FS - 1], fmx = sFp[1 * FS + 1];
-        const float2 fpy = sFp[2 * FS - FX], fmy = sFp[3 * FS + FX];
-        const float2 cpp_p = sFp[4 * FS - 1 - FX], cmp_p = sFp[5 * FS + 1 - FX];
-        const float2 cpm_p = sFp[6 * FS - 1 + FX], cmm_p = sFp[7 * FS + 1 + FX];
-        const float2 cpp_m = sFp[8 * FS - 1 - FX], cmp_m = sFp[9 * FS + 1 - FX];
-        const float2 cpm_m = sFp[10 * FS - 1 + FX], cmm_m = sFp[11 * FS + 1 + FX];
-        float2 Mr, Mx, My;
-        {
-            const float2 sxp = padd(cpp_m, cpm_m), sxm = padd(cmp_m, cmm_m);
-            const float2 syp = padd(cpp_m, cmp_m), sym = padd(cpm_m, cmm_m);
-            Mr = padd(padd(sxp, sxm), f_mz);
-            Mx = psub(sxp, sxm, k.mone);
-            My = psub(syp, sym, k.mone);
-        }
-        const float2 Zr = padd(padd(padd(f_rest, fpx), padd(fmx, fpy)), fmy);
-        const float2 Zx = psub(fpx, fmx, k.mone), Zy = psub(fpy, fmy, k.mone);
-        float2 Pr, Px, Py;
-        {
-            const float2 sxp = padd(cpp_p, cpm_p), sxm = padd(cmp_p, cmm_p);
-            const float2 syp = padd(cpp_p, cmp_p), sym = padd(cpm_p, cmm_p);
-            Pr = padd(padd(sxp, sxm), f_pz);
-            Px = psub(sxp, sxm, k.mone);
-            Py = psub(syp, sym, k.mone);
-        }
-        float2 orr = padd(make_float2(pend_r, Zr.x + pc_r), Mr);
-        float2 oxx = padd(make_float2(pend_x, Zx.x + pc_x), Mx);
-        float2 oyy = padd(make_float2(pend_y, Zy.x + pc_y), My);
-        float2 ozz = psub(make_float2(pend_z, pc_z), Mr, k.mone);
-        if (a.has_bf) {
-            oxx = padd(oxx, a.bf2[0]);
-            oyy = padd(oyy, a.bf2[1]);
-            ozz = padd(ozz, a.bf2[2]);
-        }
-        pend_r = Zr.y + Pr.x;
-        pend_x = Zx.y + Px.x;
-        pend_y = Zy.y + Py.x;
-        pend_z = Pr.x;
-        pc_r = Pr.y;
-        pc_x = Px.y;
-        pc_y = Py.y;
-        pc_z = Pr.y;
-        if (a0 - 1 >= zlo && a0 - 1 <= zhi)
-            pair_out(g, a, gx, gy, a0 - 1, orr.x, oxx.x, oyy.x, ozz.x, box_col, kus_col,
-                     box_plane, out_col_ptr, zstride, bc_col);
-        if (a0 >= zlo && a0 <= zhi)
-            pair_out(g, a, gx, gy, a0, orr.y, oxx.y, oyy.y, ozz.y, box_col, kus_col, box_plane,
-                     out_col_ptr, zstride, bc_col);
-    }
-    if (!ok) {
-        if (tid == 0) {
-            atomicOr(a.f.err, 8);
-            const long long t0 = clock64();
-            while (clock64() - t0 < (1LL << 28)) {
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// Interior tiles march plane pairs; tiles near an x or y face take the register z-march of
-// variant 1 (zbody, its own five-slot ring inside the same shared memory) for their face rules.
-__global__ void __launch_bounds__(PCfg::NTHR, PCfg::MINB)
-    k_zpair3d(const __grid_constant__ CUtensorMap tmap, const PairArgs a) {
-    using C = PCfg;
-    using Z = ZCfg<8>;
-    static_assert(C::TX == Z::TX && C::TY == Z::TY && C::SLOT == Z::SLOT && C::HX == Z::HX &&
-                      C::HY == Z::HY && Z::SMEM <= C::SMEM,
-                  "edge tiles reuse the register z-march in the same shared memory");
-    constexpr int TX = C::TX, TY = C::TY;
-    extern __shared__ __align__(128) unsigned char smem[];
-    float4* raw = reinterpret_cast<float4*>(smem);
-    const Geom& g = a.f.g;
-    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const int tid = threadIdx.x;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    const int q0 = blockIdx.z * a.f.zchunk;
-    const int q1 = min(nz, q0 + a.f.zchunk);
-    int hfx, hfy;
-    rim_node<TX, TY, C::NHALO>(tid, x0, nx, hfx, hfy);
-    if ((smem_addr(smem) & 127u) != 0u) {
-        if (tid == 0) atomicOr(a.f.err, 16);
-        return;
-    }
-    const bool interior = x0 >= 3 && x0 + TX + 2 <= nx - 1 && y0 >= 3 && y0 + TY + 2 <= ny - 1;
-    if (interior) {
-        const int npairs = ((q1 - q0 + 1) >> 1) + 1;
-        const int nplanes = 2 * npairs + 2;
-        uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR);
-        if (tid == 0) {
-            for (int s = 0; s < C::NSLOT; ++s) mbar_init(smem_addr(&bars[s]));
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            for (int j = 0; j < C::NSLOT && j < nplanes; ++j)
-                tma_load_box(smem_addr(raw + (size_t)j * C::SLOT), &tmap, x0 - 2, y0 - 2,
-                             q0 - 2 + j, smem_addr(&bars[j]), C::PLANE_BYTES);
-        }
-        __syncthreads();
-        pbody(tmap, a, smem, hfx, hfy, q0, q1);
-    } else {
-        const int nplanes = q1 - q0 + 4;
-        uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Z::OFF_BAR);
-        if (tid == 0) {
-            for (int s = 0; s < Z::NSLOT; ++s) mbar_init(smem_addr(&bars[s]));
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            for (int j = 0; j < Z::NSLOT && j < nplanes; ++j)
-                tma_load_box(smem_addr(raw + (size_t)j * Z::SLOT), &tmap, x0 - 2, y0 - 2,
-                             q0 - 2 + j, smem_addr(&bars[j]), Z::PLANE_BYTES);
-        }
-        __syncthreads();
-        zbody<8, false>(tmap, a.f, smem, hfx, hfy, q0, q1, nplanes);
-    }
-}
-
 PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
     if (!fn) {
@@ -1417,47 +979,12 @@ cudaError_t launch_zstep(const Geom& g, const CUtensorMap& map, const FusedArgs&
     return cudaGetLastError();
 }
 
-cudaError_t launch_zpair(const Geom& g, const CUtensorMap& map, const FusedArgs& f0,
-                         cudaStream_t st) {
-    using C = PCfg;
-    static std::atomic<unsigned> attr{0};   // devices whose shared-memory limit is raised
-    if (!device_done(attr)) {
-        cudaError_t e = cudaFuncSetAttribute(k_zpair3d, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)C::SMEM);
-        if (e != cudaSuccess) return e;
-        device_mark(attr);
-    }
-    PairArgs a;
-    a.f = f0;
-    const auto two = [](float v) { return make_float2(v, v); };
-    a.k.A = two(f0.A);
-    a.k.hA = two(0.5f * f0.A);
-    a.k.m15 = two(-1.5f);
-    using Wf = Wts<float, 3>;
-    a.k.w0 = two(Wf::w0);
-    a.k.w1 = two(Wf::w1);
-    a.k.w13 = two(Wf::w3_1);
-    a.k.nw13 = two(-Wf::w3_1);
-    a.k.h1 = two(Wf::h_1);
-    a.k.w2 = two(Wf::w2);
-    a.k.w23 = two(Wf::w3_2);
-    a.k.nw23 = two(-Wf::w3_2);
-    a.k.h2 = two(Wf::h_2);
-    a.k.w2x2 = two(2.f * Wf::w2);
-    a.k.nw2x2 = two(-2.f * Wf::w2);
-    a.k.mone = two(-1.f);
-    for (int d = 0; d < 3; ++d) a.bf2[d] = two(f0.bf[d]);
-    a.has_bf = (f0.bf[0] != 0.f || f0.bf[1] != 0.f || f0.bf[2] != 0.f) ? 1 : 0;
-    const int tiles_x = (g.n[0] + C::TX - 1) / C::TX, tiles_y = (g.n[1] + C::TY - 1) / C::TY;
-    a.f.zchunk = fused_zchunk_waves(g, (long long)tiles_x * tiles_y, C::MINB);
-    const int chunks = (g.n[2] + a.f.zchunk - 1) / a.f.zchunk;
-    k_zpair3d<<<dim3(tiles_x, tiles_y, chunks), C::NTHR, C::SMEM, st>>>(map, a);
-    return cudaGetLastError();
-}
-
-// One fused forward step src -> dst in variant v (0: shared-memory z-march with two barriers
-// per plane, 1: register z-march, 2: plane-pair z-march with packed arithmetic), all on
-// 32 x 8 tiles.  Returns a CUDA error code.
+// One fused forward step src -> dst in variant v (0: shared-memory z-march with two barriers per
+// plane, 1: z-march by size, 2: the row march of lks_march3d.cu).  The row march does a fifth less
+// work per node, but its blocks are larger and take longer to start, so it needs enough of them:
+// per step 96 x 90 x 101 37.9 us against 34.4 on 32 x 8 tiles, 151 x 83 x 117 36.1 against 38.6,
+// 128^3 48.5 against 51.2, 256^3 198 against 216 (with k_bc_shell3d).  The line lies between the
+// first two.  Returns a CUDA error code.
 cudaError_t launch_fused_step3d(const Geom& g, const V4<float>* src, const V4<float>* kus,
                                 V4<float>* dst, int* err, cudaStream_t st, int v) {
     FusedArgs a;
@@ -1473,10 +1000,10 @@ cudaError_t launch_fused_step3d(const Geom& g, const V4<float>* src, const V4<fl
     for (int k = 0; k < 3; ++k) a.bf[k] = (float)g.body[k];
     CUtensorMap map;
     if (v == 1 || v == 2) {
+        const long long inner = (g.n[0] - 2LL) * (g.n[1] - 2) * (g.n[2] - 2);
         cudaError_t e;
-        if (v == 2) {
-            if (!encode_state_map(&map, src, g, PCfg::HX, PCfg::HY)) return cudaErrorInvalidValue;
-            e = launch_zpair(g, map, a, st);
+        if (v == 2 || inner >= 1200000) {
+            e = launch_step_march(g, src, kus, dst, err, st, 0);
         } else {
             if (!encode_state_map(&map, src, g, ZCfg<8>::HX, ZCfg<8>::HY))
                 return cudaErrorInvalidValue;

@@ -144,9 +144,10 @@ cudaError_t launch_fused_step3d(const Geom& g, const V4<float>* src, const V4<fl
                                 V4<float>* dst, int* err, cudaStream_t st, int variant);
 // Offsets of the six face arrays (3 floats per face node) and their total length.
 void face_offsets(const Geom& g, FaceOffsets& fo, long long& total);
-// variant 0: two block barriers per plane; 1: one barrier per plane (conversion one plane ahead)
+// lam_in is read and modified (the adjoint of a step's last part is applied in place).  variant 0:
+// blocks of three warps; 1: the block height chosen by the grid.
 constexpr int kAdj3dVariants = 2;
-cudaError_t launch_fused_adj3d(const Geom& g, const V4<float>* lam_in, V4<float>* lam_out,
+cudaError_t launch_fused_adj3d(const Geom& g, V4<float>* lam_in, V4<float>* lam_out,
                                const V4<float>* kus, const V4<float>* sn, const V4<float>* sp,
                                float* e, float* face, double h, int* err, cudaStream_t st,
                                int variant);

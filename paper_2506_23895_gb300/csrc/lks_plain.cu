@@ -227,44 +227,7 @@ __global__ void k_objective(Geom g, const V4<T>* __restrict__ s, double* jstep) 
     objective_block<T>(g, s, jstep);
 }
 
-// Transpose of the boundary copies: each interior node adjacent to the boundary collects the
-// copied components of the boundary nodes it sources (WALL/INLET copy rho, OUTLET copies the
-// normal velocity).  Boundary nodes are read only; later kernels treat them as zero.
-// Shell enumeration: slab s (0..5) is the interior layer next to face s (axis s/2, low or
-// high side); a node next to several faces is handled by the first slab that contains it.
-__device__ __forceinline__ bool shell_node(const Geom& g, long long t, int& x, int& y, int& z) {
-    const unsigned per0 = (unsigned)g.n[1] * g.n[2], per1 = (unsigned)g.n[0] * g.n[2],
-                   per2 = (unsigned)g.n[0] * g.n[1];
-    unsigned r = (unsigned)t;
-    int slab = 0;
-    while (slab < 6) {
-        const unsigned pa = slab < 2 ? per0 : (slab < 4 ? per1 : per2);
-        if (r < pa) break;
-        r -= pa;
-        ++slab;
-    }
-    t = r;
-    if (slab >= 6) return false;
-    const int a = slab / 2;
-    if (a >= g.dim || g.periodic[a]) return false;
-    const int fixed = (slab & 1) ? g.n[a] - 2 : 1;
-    int c[3];
-    const int b0 = (a == 0) ? 1 : 0, b1 = (a == 2) ? 1 : 2;
-    c[a] = fixed;
-    c[b0] = (int)((unsigned)t % (unsigned)g.n[b0]);
-    c[b1] = (int)((unsigned)t / (unsigned)g.n[b0]);
-    // owned by an earlier slab?
-    for (int e = 0; e < slab; ++e) {
-        const int ae = e / 2;
-        if (ae >= g.dim || g.periodic[ae]) continue;
-        if (c[ae] == ((e & 1) ? g.n[ae] - 2 : 1)) return false;
-    }
-    x = c[0];
-    y = c[1];
-    z = c[2];
-    return !is_boundary(g, x, y, z);
-}
-
+// Transpose of the boundary copies on the interior nodes next to a face.
 template <class T>
 __global__ void k_adj_bcT(Geom g, V4<T>* lam, ObjAdd<T> h) {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;

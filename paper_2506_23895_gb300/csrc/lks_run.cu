@@ -311,16 +311,16 @@ lks_status adjoint_step(lks_ctx* c, int n, const void* sn, const void* sp) {
         CU(cudaStreamWaitEvent(c->st, c->ev_sens[c->epar], 0));
     }
     const bool tm = timing_begin(c, n, 1);
-    launch_adj_bcT<T>(c->g, lc, hn, c->st);
-    LAUNCHED();
     if (sizeof(T) == 4 && c->fused3d && !c->g.ks) {
-        cudaError_t e = launch_fused_adj3d(c->g, (const V4<float>*)lc, (V4<float>*)ln,
+        cudaError_t e = launch_fused_adj3d(c->g, (V4<float>*)lc, (V4<float>*)ln,
                                            (const V4<float>*)c->kus, (const V4<float>*)sn,
                                            (const V4<float>*)sp, (float*)c->e, c->face, hn,
                                            c->flags + 3, c->st, c->adj3d_var);
         if (e != cudaSuccess) return fail(c, LKS_ERR_CUDA, "fused adjoint: %s", cudaGetErrorString(e));
-        c->stats[4] += 2;
+        c->stats[4] += 3;
     } else {
+        launch_adj_bcT<T>(c->g, lc, hn, c->st);
+        LAUNCHED();
         launch_adj_mu<T>(c->g, lc, (const V4<T>*)c->kus, (const V4<T>*)sn, st4<T>(c->mu),
                          (T*)c->e, hn, c->st, (const V4<T>*)c->u3);
         LAUNCHED();
