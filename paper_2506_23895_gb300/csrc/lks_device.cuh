@@ -237,17 +237,7 @@ __device__ __forceinline__ void write_bc_from(const Geom& g, int x, int y, int z
     });
 }
 
-// ------------------------------------------------------------------ gradient stencil
-// First derivative along an axis: central difference, periodic wrap, and the second-order
-// one-sided difference on a non-periodic boundary node (the reading taken for the velocity
-// gradient of f^eq).  coef(i, off): weight of row i's stencil at offset off (0 if none).
-__device__ __forceinline__ double deriv_coef(int i, int n, int periodic, int off) {
-    if (periodic) return off == 1 ? 0.5 : (off == -1 ? -0.5 : 0.0);
-    if (i == 0) return off == 0 ? -1.5 : (off == 1 ? 2.0 : (off == 2 ? -0.5 : 0.0));
-    if (i == n - 1) return off == 0 ? 1.5 : (off == -1 ? -2.0 : (off == -2 ? 0.5 : 0.0));
-    return off == 1 ? 0.5 : (off == -1 ? -0.5 : 0.0);
-}
-
+// ------------------------------------------------------------------ transfer kernel
 // Peskin four-point cosine kernel w(r) = (1 + cos(pi r / 2)) / 4 for |r| < 2 (Sec. 2.3).
 __device__ __forceinline__ double peskin(double r) {
     return fabs(r) < 2.0 ? 0.25 * (1.0 + cospi(0.5 * r)) : 0.0;

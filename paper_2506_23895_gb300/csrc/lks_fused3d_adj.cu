@@ -1,6 +1,6 @@
 // What the fused D3Q15 adjoint step does beside its z-march (lks_march3d_adj.cu) on non-periodic grids:
-//   k_adj_prep   before it, in place on lambda^n: the transpose of the boundary copies, the
-//                objective source and, in the footprint box, the Brinkman transpose with e;
+//   k_adj_prep   (lks_plain.cu) before it, in place on lambda^n: the transpose of the boundary
+//                copies, the objective source and, in the footprint box, the Brinkman transpose with e;
 //   k_adj_bcorr  after it: the one-sided rows of the transposed velocity gradient.
 #include <algorithm>
 
@@ -10,55 +10,6 @@
 namespace lks {
 
 namespace {
-
-// Nodes of lambda^n that differ from mu: the nodes of the footprint box, then the nodes next to a
-// face, then the objective's target nodes, each by the first range that holds it.  A box node's
-// (1 + kappa)^-1 and e = mu_u . (u_S - u^n) need two more records; inside the march they were two
-// dependent loads that every plane waited for (128^3: 70 us a step with the march's own arithmetic
-// at 30), here they are one pass over the box.
-__global__ void __launch_bounds__(256)
-    k_adj_prep(Geom g, float4* __restrict__ lam, ObjAdd<float> h, const float4* __restrict__ kus,
-               const float4* __restrict__ sn, float* __restrict__ e, unsigned shell) {
-    unsigned t = blockIdx.x * 256u + threadIdx.x;
-    const unsigned boxN = (unsigned)g.boxN;
-    int x, y, z;
-    long long bi = -1;
-    if (t < boxN) {
-        const unsigned r = t / (unsigned)g.bn[0];
-        x = g.blo[0] + (int)(t - r * (unsigned)g.bn[0]);
-        y = g.blo[1] + (int)(r % (unsigned)g.bn[1]);
-        z = g.blo[2] + (int)(r / (unsigned)g.bn[1]);
-        bi = t;
-    } else if ((t -= boxN) < shell) {
-        if (!shell_node(g, t, x, y, z) || in_box(g, x, y, z, bi)) return;
-        bi = -1;
-    } else if ((t -= shell) < (unsigned)g.ocount && h.on) {
-        const unsigned m = (unsigned)g.otarget[t], r = m / (unsigned)g.n[0];
-        x = (int)(m - r * (unsigned)g.n[0]);
-        y = (int)(r % (unsigned)g.n[1]);
-        z = (int)(r / (unsigned)g.n[1]);
-        if (is_boundary(g, x, y, z) || sources_boundary(g, x, y, z) || in_box(g, x, y, z, bi))
-            return;
-        bi = -1;
-    } else {
-        return;
-    }
-    const long long m = node_index(g, x, y, z);
-    const float4 l = lam[m];
-    V4<float> v{l.x, l.y, l.z, l.w};
-    if (sources_boundary(g, x, y, z))
-        bcT_gather<float>(g, reinterpret_cast<const V4<float>*>(lam), h, x, y, z, v);
-    obj_source(g, x, y, z, h, v);
-    if (bi >= 0) {
-        const float4 ks = kus[bi], un = sn[m];
-        const float inv = __frcp_rn(1.f + ks.x);
-        v.x *= inv;
-        v.y *= inv;
-        v.z *= inv;
-        e[bi] = v.x * (ks.y - un.y) + v.y * (ks.z - un.z) + v.z * (ks.w - un.w);
-    }
-    lam[m] = make_float4(v.r, v.x, v.y, v.z);
-}
 
 // One-sided parts of the transposed gradient on non-periodic axes: node z within two rows of
 // a face gets delta * (2 A S~_{.beta}) of the face node it projects to, with delta = -3/2,
@@ -129,13 +80,7 @@ cudaError_t launch_fused_adj3d(const Geom& g, V4<float>* lam_in, V4<float>* lam_
                                const V4<float>* kus, const V4<float>* sn, const V4<float>* sp,
                                float* e, float* face, double h, int* err, cudaStream_t st,
                                int variant) {
-    const unsigned near = 2u * ((unsigned)g.n[1] * g.n[2] + (unsigned)g.n[0] * g.n[2] +
-                                (unsigned)g.n[0] * g.n[1]);
-    const ObjAdd<float> o = obj_add<float>(g, h);
-    const long long prep = g.boxN + near + (o.on ? (long long)g.ocount : 0);
-    k_adj_prep<<<(unsigned)((prep + 255) / 256), 256, 0, st>>>(
-        g, reinterpret_cast<float4*>(lam_in), o, reinterpret_cast<const float4*>(kus),
-        reinterpret_cast<const float4*>(sn), e, near);
+    launch_adj_prep<float>(g, lam_in, kus, sn, e, h, st);
     cudaError_t r = cudaGetLastError();
     if (r != cudaSuccess) return r;
     r = launch_adj_march(g, lam_in, lam_out, sp, face, err, st, variant == 0 ? 3 : 0);

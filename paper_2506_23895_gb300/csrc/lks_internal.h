@@ -121,6 +121,10 @@ template <class T>
 void launch_objective(const Geom& g, const V4<T>* s, double* jstep, cudaStream_t st);
 template <class T>
 void launch_adj_bcT(const Geom& g, V4<T>* lam, double h, cudaStream_t st);
+// lambda^n to mu in place but for the boundary nodes, which the moments take as 0 (no static solids).
+template <class T>
+void launch_adj_prep(const Geom& g, V4<T>* lam, const V4<T>* kus, const V4<T>* sn, T* e, double h,
+                     cudaStream_t st);
 // u3 (optional): 3 U~ of the last moments, for the printed-ALKS variant (else nullptr).
 template <class T>
 void launch_adj_mu(const Geom& g, const V4<T>* lam, const V4<T>* kus, const V4<T>* sn,

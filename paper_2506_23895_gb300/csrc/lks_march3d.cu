@@ -25,9 +25,9 @@
 
 #include <algorithm>
 
-#include "lks_device.cuh"
 #include "lks_march3d.h"
 #include "lks_tma.cuh"
+#include "lks_units.cuh"
 
 namespace lks {
 
@@ -68,69 +68,6 @@ __device__ __forceinline__ void st_if(float4* p, const float4& v, bool go) {
         " @p st.global.v4.f32 [%4], {%0, %1, %2, %3}; }" ::"f"(v.x),
         "f"(v.y), "f"(v.z), "f"(v.w), "l"(p), "r"((int)go)
         : "memory");
-}
-
-// The 15 values of f^eq at a node: rest and axes, and the corners [s_x > 0 ? 0 : 1] for s_y = +1 (u)
-// and -1 (d), s_z = +1 (p) and -1 (m).
-struct Feq {
-    float f0, xp, xm, yp, ym, zp, zm;
-    float up[2], um[2], dp[2], dm[2];
-};
-
-// f^eq (Sec. 2.2) from the node c and D_ab = 2 d u_a / d x_b.
-__device__ __forceinline__ void feq(const float4& c, float A, float Dxx, float Dyx, float Dzx,
-                                    float Dxy, float Dyy, float Dzy, float Dxz, float Dyz,
-                                    float Dzz, Feq& f) {
-    using W = Wts<float, 3>;
-    const float hA = 0.5f * A;
-    const float ASxx = A * Dxx, ASyy = A * Dyy, ASzz = A * Dzz;
-    const float ASxy = hA * (Dxy + Dyx), ASxz = hA * (Dxz + Dzx), ASyz = hA * (Dyz + Dzy);
-    const float ux = c.y, uy = c.z, uz = c.w;
-    const float P = c.x - 1.5f * (ux * ux + uy * uy + uz * uz);
-    f.f0 = W::w0 * P;
-    const float bx = fmaf(W::h_1 * ux, ux, W::w1 * (P + ASxx));
-    f.xp = fmaf(W::w3_1, ux, bx);
-    f.xm = fmaf(-W::w3_1, ux, bx);
-    const float by = fmaf(W::h_1 * uy, uy, W::w1 * (P + ASyy));
-    f.yp = fmaf(W::w3_1, uy, by);
-    f.ym = fmaf(-W::w3_1, uy, by);
-    const float bz = fmaf(W::h_1 * uz, uz, W::w1 * (P + ASzz));
-    f.zp = fmaf(W::w3_1, uz, bz);
-    f.zm = fmaf(-W::w3_1, uz, bz);
-    const float T0 = W::w2 * (P + ASxx + ASyy + ASzz);
-    const float s1 = ux + uy, d1 = ux - uy, w2x2 = 2.f * W::w2;
-    const float q1 = ASxz + ASyz, q2 = ASyz - ASxz;
-    {   // (+,+,+) and (-,-,-)
-        const float cu = s1 + uz;
-        const float s = fmaf(W::h_2 * cu, cu, fmaf(w2x2, ASxy + q1, T0));
-        f.up[0] = fmaf(W::w3_2, cu, s);
-        f.dm[1] = fmaf(-W::w3_2, cu, s);
-    }
-    {   // (-,+,+) and (+,-,-)
-        const float cu = uz - d1;
-        const float s = fmaf(W::h_2 * cu, cu, fmaf(w2x2, q2 - ASxy, T0));
-        f.up[1] = fmaf(W::w3_2, cu, s);
-        f.dm[0] = fmaf(-W::w3_2, cu, s);
-    }
-    {   // (+,-,+) and (-,+,-)
-        const float cu = uz + d1;
-        const float s = fmaf(W::h_2 * cu, cu, fmaf(-w2x2, ASxy + q2, T0));
-        f.dp[0] = fmaf(W::w3_2, cu, s);
-        f.um[1] = fmaf(-W::w3_2, cu, s);
-    }
-    {   // (-,-,+) and (+,+,-)
-        const float cu = uz - s1;
-        const float s = fmaf(W::h_2 * cu, cu, fmaf(w2x2, ASxy - q1, T0));
-        f.dp[1] = fmaf(W::w3_2, cu, s);
-        f.um[0] = fmaf(-W::w3_2, cu, s);
-    }
-}
-
-// Second-order one-sided 2 d/dx at a low (hi = false) or high boundary node from it and its
-// neighbours one and two nodes inward.
-__device__ __forceinline__ float onesided(bool hi, float c, float n1, float n2) {
-    const float d = fmaf(-3.f, c, fmaf(4.f, n1, -n2));
-    return hi ? -d : d;
 }
 
 __global__ void __launch_bounds__(32 * kMaxWarps, 2)
@@ -244,7 +181,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 2)
         if (box) good = mbar_wait_once(smem_addr(&kbars[ks]), kpar) && good;
         const unsigned kaddr = kown + ks * kbytes;
         float* sb = seams + ((p & 1) * nw + wid) * seam_warp + lane;
-        Feq f;
+        Feq<float> f;
         float upP[2], upM[2], upY;   // what row r - 1 sends up, to row r
         float md[5];                 // row r - 1: f0, xp, xm, zp, zm
         float lowP[2], lowM[2], lowY;   // what row r - 2 sent up, to row r - 1
@@ -289,7 +226,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 2)
                     Dyz = onesided(h, cc.z, h ? um[r].y : n.z, t.z);
                     Dzz = onesided(h, cc.w, h ? um[r].z : n.w, t.w);
                 }
-                feq(cc, A, Dxx, Dyx, Dzx, Dxy, Dyy, Dzy, Dxz, Dyz, Dzz, f);
+                feq<float>(cc.x, cc.y, cc.z, cc.w, A, Dxx, Dyx, Dzx, Dxy, Dyy, Dzy, Dxz, Dyz, Dzz, f);
                 um[r] = make_float3(cc.y, cc.z, cc.w);
                 c[r] = n;
                 if (r == 0) {   // what row 0 sends down, x-combined, to the warp below

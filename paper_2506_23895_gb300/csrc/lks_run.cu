@@ -319,12 +319,18 @@ lks_status adjoint_step(lks_ctx* c, int n, const void* sn, const void* sp) {
         if (e != cudaSuccess) return fail(c, LKS_ERR_CUDA, "fused adjoint: %s", cudaGetErrorString(e));
         c->stats[4] += 3;
     } else {
-        launch_adj_bcT<T>(c->g, lc, hn, c->st);
+        const V4<T>* mu = lc;
+        if (c->g.ks || c->u3) {
+            launch_adj_bcT<T>(c->g, lc, hn, c->st);
+            LAUNCHED();
+            launch_adj_mu<T>(c->g, lc, (const V4<T>*)c->kus, (const V4<T>*)sn, st4<T>(c->mu),
+                             (T*)c->e, hn, c->st, (const V4<T>*)c->u3);
+            mu = st4<T>(c->mu);
+        } else {
+            launch_adj_prep<T>(c->g, lc, (const V4<T>*)c->kus, (const V4<T>*)sn, (T*)c->e, hn, c->st);
+        }
         LAUNCHED();
-        launch_adj_mu<T>(c->g, lc, (const V4<T>*)c->kus, (const V4<T>*)sn, st4<T>(c->mu),
-                         (T*)c->e, hn, c->st, (const V4<T>*)c->u3);
-        LAUNCHED();
-        launch_adj_moments<T>(c->g, st4<T>(c->mu), (const V4<T>*)sp, ln, (T*)c->phi, c->st,
+        launch_adj_moments<T>(c->g, mu, (const V4<T>*)sp, ln, (T*)c->phi, c->st,
                               (V4<T>*)c->u3);
         LAUNCHED();
         launch_adj_divT<T>(c->g, (const T*)c->phi, ln, c->st);

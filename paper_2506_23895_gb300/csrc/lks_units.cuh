@@ -7,6 +7,75 @@
 
 namespace lks {
 
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+
+// ---------------------------------------------------------------- equilibrium (Sec. 2.2)
+// The 15 values of f^eq at a node: rest and axes, and the corners [s_x > 0 ? 0 : 1] for s_y = +1 (u)
+// and -1 (d), s_z = +1 (p) and -1 (m).
+template <class T>
+struct Feq {
+    T f0, xp, xm, yp, ym, zp, zm;
+    T up[2], um[2], dp[2], dm[2];
+};
+
+// f^eq (Sec. 2.2) from rho - rho0, u and D_ab = 2 d u_a / d x_b: the symmetric part of each pair of
+// opposite directions is formed once, 68 operations in all.
+template <class T>
+__device__ __forceinline__ void feq(T r, T ux, T uy, T uz, T A, T Dxx, T Dyx, T Dzx, T Dxy, T Dyy,
+                                    T Dzy, T Dxz, T Dyz, T Dzz, Feq<T>& f) {
+    using W = Wts<T, 3>;
+    const T hA = (T)0.5 * A;
+    const T ASxx = A * Dxx, ASyy = A * Dyy, ASzz = A * Dzz;
+    const T ASxy = hA * (Dxy + Dyx), ASxz = hA * (Dxz + Dzx), ASyz = hA * (Dyz + Dzy);
+    const T P = r - (T)1.5 * (ux * ux + uy * uy + uz * uz);
+    f.f0 = W::w0 * P;
+    const T bx = fma_(W::h_1 * ux, ux, W::w1 * (P + ASxx));
+    f.xp = fma_(W::w3_1, ux, bx);
+    f.xm = fma_(-W::w3_1, ux, bx);
+    const T by = fma_(W::h_1 * uy, uy, W::w1 * (P + ASyy));
+    f.yp = fma_(W::w3_1, uy, by);
+    f.ym = fma_(-W::w3_1, uy, by);
+    const T bz = fma_(W::h_1 * uz, uz, W::w1 * (P + ASzz));
+    f.zp = fma_(W::w3_1, uz, bz);
+    f.zm = fma_(-W::w3_1, uz, bz);
+    const T T0 = W::w2 * (P + ASxx + ASyy + ASzz);
+    const T s1 = ux + uy, d1 = ux - uy, w2x2 = (T)2 * W::w2;
+    const T q1 = ASxz + ASyz, q2 = ASyz - ASxz;
+    {   // (+,+,+) and (-,-,-)
+        const T cu = s1 + uz;
+        const T s = fma_(W::h_2 * cu, cu, fma_(w2x2, ASxy + q1, T0));
+        f.up[0] = fma_(W::w3_2, cu, s);
+        f.dm[1] = fma_(-W::w3_2, cu, s);
+    }
+    {   // (-,+,+) and (+,-,-)
+        const T cu = uz - d1;
+        const T s = fma_(W::h_2 * cu, cu, fma_(w2x2, q2 - ASxy, T0));
+        f.up[1] = fma_(W::w3_2, cu, s);
+        f.dm[0] = fma_(-W::w3_2, cu, s);
+    }
+    {   // (+,-,+) and (-,+,-)
+        const T cu = uz + d1;
+        const T s = fma_(W::h_2 * cu, cu, fma_(-w2x2, ASxy + q2, T0));
+        f.dp[0] = fma_(W::w3_2, cu, s);
+        f.um[1] = fma_(-W::w3_2, cu, s);
+    }
+    {   // (-,-,+) and (+,+,-)
+        const T cu = uz - s1;
+        const T s = fma_(W::h_2 * cu, cu, fma_(w2x2, ASxy - q1, T0));
+        f.dp[1] = fma_(W::w3_2, cu, s);
+        f.um[0] = fma_(-W::w3_2, cu, s);
+    }
+}
+
+// Second-order one-sided 2 d/dx at a low (hi = false) or high boundary node from it and its
+// neighbours one and two nodes inward.
+template <class T>
+__device__ __forceinline__ T onesided(bool hi, T c, T n1, T n2) {
+    const T d = fma_((T)-3, c, fma_((T)4, n1, -n2));
+    return hi ? -d : d;
+}
+
 // ---------------------------------------------------------------- 2D transfer (table path)
 // Design column k for the D2Q9 instance-table kernels: integer base of x_ref, y_ref and, per axis,
 // S = sin(pi f/2), C = cos(pi f/2) of the fraction f.  The four
