@@ -178,35 +178,46 @@ __global__ void __launch_bounds__(NT) k_t_design_pos(Plan p, int noff, int n) {
     }
 }
 
-// One 16 x 16 tile of the footprint box of one step per work unit.  The design nodes any node of
-// the tile can reach (the tile's inverse rigid image widened by the kernel radius: at most 30 x 30
-// nodes) are staged in shared memory with contiguous reads and binned by their integer base into a
-// table of cells; every node then visits the 4 x 4 cells whose taps cover it, so that it touches
-// only the design nodes in its support (about 16, against some 36 window candidates).  A tile whose
-// table overflows, or whose window is wider than the staging area, scans the candidate window.
-constexpr int kTrWin = 32;   // staged window side (design nodes)
-static_assert(kBoxTile * kBoxTile == NT, "one box tile per block of NT threads");
-// Cells of the tile's design-node table: the integer bases b that can reach a node of the tile
-// (b in [x - 2, x + 1] per axis), kTrCells per axis; a unit-spaced rotated lattice puts at most
-// two design nodes in one unit cell, kTrCap leaves room.
-constexpr int kTrCells = kBoxTile + 3, kTrCap = 4;
+// One 32 x 16 tile of the footprint box of one step per work unit.  The design nodes whose taps reach
+// the tile (integer base in the 35 x 19 cells from two below it to one above) go to shared memory
+// ordered by cell (x fastest) and then by design index.  A thread gathers a run of kTrRun nodes of one
+// column: a design node serves up to four of them, and the four cells of a row of its support are one
+// range of the list.  A tile with more design nodes than the lists hold scans the candidates of each
+// node.  Bound by instruction issue; 64 channels of side 128 to 512, per step: 55 us (one thread a
+// node, 16 cells each with a list of its own: 98 us).
+constexpr int kTrRun = 4;
+constexpr int kTrThreads = kBoxTileX * kBoxTileY / kTrRun;
+constexpr int kTrCX = kBoxTileX + 3, kTrCY = kBoxTileY + 3, kTrCells = kTrCX * kTrCY;
+constexpr int kTrPer = (kTrCells + kTrThreads - 1) / kTrThreads;   // cells a thread lists
+// a unit-spaced rotated lattice puts at most two nodes in one cell, and about one
+constexpr int kTrCap = 4, kTrList = 768;
+constexpr int kTrRow = 64;   // a window row's nodes: at most 34.4 + 2 (4 / sqrt 2) + 1 of them
 
 template <class T>
 struct TrSmem {
-    V4<T> sc[kTrWin * kTrWin];
-    T kr[kTrWin * kTrWin];
-    int cnt[kTrCells * kTrCells];
-    int win[4];
+    union {
+        V4<T> sc[kTrList];   // sin, cos of the fractions
+        struct {             // before these: the cells' unordered lists
+            int cnt[kTrCells];
+            unsigned short ent[kTrCells * kTrCap];
+        };
+    };
+    V4<T> kx[kTrList];    // kappa_ref, xi - xi_G, the cell's x
+    int warp[kTrThreads / 32];
     int full;
-    unsigned short ent[kTrCells * kTrCells * kTrCap];
+    unsigned short start[kTrCells + 1];
+    unsigned short key[kTrList];   // window row and place of a listed node
 };
 
 template <class T>
-__global__ void __launch_bounds__(NT) k_t_transfer2d(Plan p, int noff, int nsteps, int kslot0) {
+__global__ void __launch_bounds__(kTrThreads, sizeof(T) == 4 ? 8 : 4)
+    k_t_transfer2d(Plan p, int noff, int nsteps, int kslot0) {
     extern __shared__ __align__(32) unsigned char smem_raw[];
     TrSmem<T>& S = *reinterpret_cast<TrSmem<T>*>(smem_raw);
     const int* pre = p.pre + U_BOX * (p.count + 1);
     const int n0 = __ldg(p.nbase) + noff, nbox = p.total[U_BOX];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    constexpr int NW = kTrThreads / 32;
     for (int w = blockIdx.x; w < nbox * nsteps; w += gridDim.x) {
         const int step = w / nbox, u = w - step * nbox;
         const int i = find_inst(pre, p.count, u);
@@ -216,142 +227,193 @@ __global__ void __launch_bounds__(NT) k_t_transfer2d(Plan p, int noff, int nstep
         const Motion& m = I.motion[n0 + step];
         const int2* __restrict__ pb = I.pos_b + (long long)step * d.ncol;
         const V4<T>* __restrict__ psc = I.pos_sc + (long long)step * d.ncol;
+        const T* __restrict__ kref = I.kref;
         V4<T>* kus = kslot0 < 0 ? I.kus : I.kus_tape + (long long)(kslot0 + step) * g.boxN;
-        const int ntx = (g.bn[0] + kBoxTile - 1) / kBoxTile;
+        const int ntx = (g.bn[0] + kBoxTileX - 1) / kBoxTileX;
         const int t = u - pre[i];
-        const int bx0 = (t % ntx) * kBoxTile, by0 = (t / ntx) * kBoxTile;
-        const int lx = threadIdx.x % kBoxTile, ly = threadIdx.x / kBoxTile;
-        const int bx = bx0 + lx, by = by0 + ly;
-        const bool node = bx < g.bn[0] && by < g.bn[1];
-        const int x = g.blo[0] + bx, y = g.blo[1] + by;
-        // this node's candidate window, through the inverse rigid map in single precision with a
+        const int bx0 = (t % ntx) * kBoxTileX, by0 = (t / ntx) * kBoxTileY;
+        const int lx = tid % kBoxTileX, ly = tid / kBoxTileX * kTrRun;
+        // the tile's window of candidates through the inverse rigid map, in single precision with a
         // margin far above its rounding (it only has to contain the support)
-        const float c = m.cf, s = m.sf;
-        const float R = 2.f * (fabsf(c) + fabsf(s)) + 0.01f;
-        const float px = (float)x - m.xgf[0], py = (float)y - m.xgf[1];
-        const float ic = c * px + s * py + d.xiGf[0];
-        const float jc = -s * px + c * py + d.xiGf[1];
-        const int i0 = max(0, (int)ceilf(ic - R)), i1 = min(d.L[0] - 1, (int)floorf(ic + R));
-        const int j0 = max(0, (int)ceilf(jc - R)), j1 = min(d.L[1] - 1, (int)floorf(jc + R));
-        __syncthreads();   // the previous unit's staged window is no longer read
-        if (threadIdx.x == 0) {
-            S.win[0] = 1 << 30;
-            S.win[1] = -(1 << 30);
-            S.win[2] = 1 << 30;
-            S.win[3] = -(1 << 30);
-            S.full = 0;
-        }
-        for (int e = threadIdx.x; e < kTrCells * kTrCells; e += NT) S.cnt[e] = 0;
-        __syncthreads();
-        {   // the tile's window: warp minima and maxima first, then one atomic per warp
-            const bool any = node && i0 <= i1 && j0 <= j1;
-            const int a0 = __reduce_min_sync(FULL, any ? i0 : (1 << 30));
-            const int a1 = __reduce_max_sync(FULL, any ? i1 : -(1 << 30));
-            const int b0 = __reduce_min_sync(FULL, any ? j0 : (1 << 30));
-            const int b1 = __reduce_max_sync(FULL, any ? j1 : -(1 << 30));
-            if ((threadIdx.x & 31) == 0 && a0 <= a1) {
-                atomicMin(&S.win[0], a0);
-                atomicMax(&S.win[1], a1);
-                atomicMin(&S.win[2], b0);
-                atomicMax(&S.win[3], b1);
-            }
-        }
-        __syncthreads();
-        const int wi0 = S.win[0], wj0 = S.win[2];
-        const bool none = S.win[1] < wi0;
-        const int wni = S.win[1] - wi0 + 1, wnj = S.win[3] - wj0 + 1;
-        const long long bi = (long long)by * g.bn[0] + bx;
-        if (none) {   // no design node reaches the tile (block-uniform)
-            V4<T> o;
-            o.r = o.x = o.y = o.z = (T)0;
-            if (node) kus[bi] = o;
-            continue;
-        }
-        const bool staged = wni <= kTrWin && wnj <= kTrWin;
-        // the tile's first analysis node less 2: the lowest base whose taps reach the tile
-        const int cx0 = g.blo[0] + bx0 - 2, cy0 = g.blo[1] + by0 - 2;
-        if (staged) {
-            const int li = threadIdx.x & 31;   // 32 lanes along i, 8 rows of j at a time
-            for (int jj = threadIdx.x >> 5; jj < wnj; jj += NT / 32) {
-                if (li >= wni) continue;
-                const int k = (wj0 + jj) * d.L[0] + wi0 + li, e = jj * kTrWin + li;
-                const int2 bk = __ldg(pb + k);
-                S.sc[e] = psc[k];
-                S.kr[e] = I.kref[k];
+        const float c = m.cf, s = m.sf, ac = fabsf(c), as = fabsf(s);
+        const float hx = 0.5f * (kBoxTileX - 1), hy = 0.5f * (kBoxTileY - 1);
+        const float px = (float)(g.blo[0] + bx0) + hx - m.xgf[0];
+        const float py = (float)(g.blo[1] + by0) + hy - m.xgf[1];
+        const float ic = c * px + s * py + d.xiGf[0], jc = -s * px + c * py + d.xiGf[1];
+        const float ri = ac * (hx + 2.f) + as * (hy + 2.f) + 0.05f;
+        const float rj = as * (hx + 2.f) + ac * (hy + 2.f) + 0.05f;
+        const int wi0 = max(0, (int)ceilf(ic - ri)), wi1 = min(d.L[0] - 1, (int)floorf(ic + ri));
+        const int wj0 = max(0, (int)ceilf(jc - rj)), wj1 = min(d.L[1] - 1, (int)floorf(jc + rj));
+        T kap[kTrRun], m0[kTrRun], m1x[kTrRun], m1y[kTrRun];
+#pragma unroll
+        for (int j = 0; j < kTrRun; ++j) kap[j] = m0[j] = m1x[j] = m1y[j] = (T)0;
+        if (wi0 <= wi1 && wj0 <= wj1) {   // uniform over the block
+            const int cx0 = g.blo[0] + bx0 - 2, cy0 = g.blo[1] + by0 - 2;   // first cell
+            __syncthreads();   // the previous unit's lists are no longer read
+            if (tid == 0) S.full = 0;
+            for (int e = tid; e < kTrCells; e += kTrThreads) S.cnt[e] = 0;
+            __syncthreads();
+            // count the listed nodes of each cell, a warp per window row, over the part of the row
+            // that can lie in the cells
+            const float ox = m.xgf[0] - c * d.xiGf[0] - (float)cx0;
+            const float oy = m.xgf[1] - s * d.xiGf[0] - (float)cy0;
+            const float rc = __fdividef(1.f, c), rs = __fdividef(1.f, s);   // used where not near 0
+            auto span = [&](int j, int& i0, int& i1) {
+                const float dj = (float)j - d.xiGf[1];
+                const float xj = ox - s * dj, yj = oy + c * dj;   // of node i = 0, from the first cell
+                float lo = (float)wi0, hi = (float)wi1;
+                if (ac > 0.2f) {
+                    const float e0 = -xj * rc, e1 = ((float)kTrCX - xj) * rc;
+                    lo = fmaxf(lo, fminf(e0, e1) - 0.1f);
+                    hi = fminf(hi, fmaxf(e0, e1) + 0.1f);
+                }
+                if (as > 0.2f) {
+                    const float e0 = -yj * rs, e1 = ((float)kTrCY - yj) * rs;
+                    lo = fmaxf(lo, fminf(e0, e1) - 0.1f);
+                    hi = fminf(hi, fmaxf(e0, e1) + 0.1f);
+                }
+                i0 = (int)ceilf(lo) + lane;
+                i1 = j <= wj1 ? (int)floorf(hi) : -1;
+            };
+            auto put = [&](int j, int ii, const int2& bk) {
                 const int cx = bk.x - cx0, cy = bk.y - cy0;
-                if ((unsigned)cx < (unsigned)kTrCells && (unsigned)cy < (unsigned)kTrCells) {
-                    const int cell = cy * kTrCells + cx;
-                    const int slot = atomicAdd(&S.cnt[cell], 1);
-                    if (slot < kTrCap) S.ent[cell * kTrCap + slot] = (unsigned short)e;
-                    else S.full = 1;
+                if ((unsigned)cx >= (unsigned)kTrCX || (unsigned)cy >= (unsigned)kTrCY) return;
+                const int cell = cy * kTrCX + cx;
+                const int slot = atomicAdd(&S.cnt[cell], 1);
+                if (slot < kTrCap)
+                    S.ent[cell * kTrCap + slot] = (unsigned short)((j - wj0) * kTrRow + (ii - wi0));
+                else S.full = 1;
+            };
+            constexpr int RB = 3;   // rows whose loads are in flight together
+            for (int j = wj0 + wid; j <= wj1; j += RB * NW) {
+                int i0[RB], i1[RB];
+                int2 bk[RB];
+#pragma unroll
+                for (int r = 0; r < RB; ++r) {
+                    span(j + r * NW, i0[r], i1[r]);
+                    if (i0[r] <= i1[r]) bk[r] = __ldg(pb + (j + r * NW) * d.L[0] + i0[r]);
+                }
+#pragma unroll
+                for (int r = 0; r < RB; ++r) {
+                    if (i0[r] <= i1[r]) put(j + r * NW, i0[r], bk[r]);
+                    for (int ii = i0[r] + 32; ii <= i1[r]; ii += 32)
+                        put(j + r * NW, ii, __ldg(pb + (j + r * NW) * d.L[0] + ii));
                 }
             }
-        }
-        __syncthreads();
-        // each cell's design nodes in design index order (the staging order of the slots is not
-        // fixed)
-        const bool cells = staged && !S.full;
-        if (cells) {
-            for (int cell = threadIdx.x; cell < kTrCells * kTrCells; cell += NT) {
-                const int cnt = S.cnt[cell];
-                unsigned short* ent = S.ent + cell * kTrCap;
-                for (int a1 = 1; a1 < cnt; ++a1)
-                    for (int a2 = a1; a2 > 0 && ent[a2 - 1] > ent[a2]; --a2) {
-                        const unsigned short tmp = ent[a2];
-                        ent[a2] = ent[a2 - 1];
-                        ent[a2 - 1] = tmp;
-                    }
+            __syncthreads();
+            // list offsets: kTrPer consecutive cells per thread, summed over the block
+            int nc[kTrPer], sum = 0;
+#pragma unroll
+            for (int e = 0; e < kTrPer; ++e) {
+                const int cell = tid * kTrPer + e;
+                nc[e] = cell < kTrCells ? S.cnt[cell] : 0;
+                sum += nc[e];
             }
-        }
-        __syncthreads();
-        if (!node) continue;
-        const T gx0 = (T)d.xiG[0] - (T)wi0, gy0 = (T)d.xiG[1] - (T)wj0;
-        T kap = (T)0, m0 = (T)0, m1x = (T)0, m1y = (T)0;
-        if (cells) {
-            // the design nodes whose base b reaches (x, y): b = (x, y) + 1 - (qx, qy), qx, qy in
-            // 0..3, visited by tap (qy, qx) and then in design index order within a cell
-            const int ccx = x - cx0 + 1, ccy = y - cy0 + 1;
+            int at = sum;
 #pragma unroll
-            for (int qy = 0; qy < 4; ++qy)
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(FULL, at, o);
+                if (lane >= o) at += v;
+            }
+            if (lane == 31) S.warp[wid] = at;
+            __syncthreads();
+            int total = 0;
 #pragma unroll
-                for (int qx = 0; qx < 4; ++qx) {
-                    const int cell = (ccy - qy) * kTrCells + (ccx - qx);
-                    const int cnt = S.cnt[cell];
-                    for (int a1 = 0; a1 < cnt; ++a1) {
-                        const int sk = S.ent[cell * kTrCap + a1];
-                        const V4<T> sc = S.sc[sk];
-                        const T W = tap_weight<T>(qx, sc.r, sc.x) * tap_weight<T>(qy, sc.y, sc.z);
-                        kap += W * S.kr[sk];
-                        m0 += W;
-                        m1x += W * ((T)(sk & (kTrWin - 1)) - gx0);
-                        m1y += W * ((T)(sk / kTrWin) - gy0);
+            for (int k = 0; k < NW; ++k) {
+                if (k < wid) at += S.warp[k];
+                total += S.warp[k];
+            }
+            at -= sum;
+            if (!S.full && total <= kTrList) {
+#pragma unroll
+                for (int e = 0; e < kTrPer; ++e) {
+                    const int cell = tid * kTrPer + e;
+                    if (cell >= kTrCells) break;
+                    S.start[cell] = (unsigned short)at;
+                    if (nc[e] == 0) continue;
+                    // in design index order (the order of the slots is not fixed)
+                    unsigned short* ent = S.ent + cell * kTrCap;
+                    for (int a1 = 1; a1 < nc[e]; ++a1)
+                        for (int a2 = a1; a2 > 0 && ent[a2 - 1] > ent[a2]; --a2) {
+                            const unsigned short tmp = ent[a2];
+                            ent[a2] = ent[a2 - 1];
+                            ent[a2 - 1] = tmp;
+                        }
+                    for (int a1 = 0; a1 < nc[e]; ++a1) {
+                        S.key[at + a1] = ent[a1];
+                        S.kx[at + a1].z = (T)(cell % kTrCX);
                     }
+                    at += nc[e];
                 }
-        } else {
-            for (int j = j0; j <= j1; ++j)
-                for (int ii = i0; ii <= i1; ++ii) {
+                if (tid == 0) S.start[kTrCells] = (unsigned short)total;
+                __syncthreads();
+#pragma unroll 3
+                for (int e = tid; e < total; e += kTrThreads) {
+                    const int key = S.key[e], ii = wi0 + key % kTrRow, j = wj0 + key / kTrRow;
                     const int k = j * d.L[0] + ii;
-                    const int2 b = __ldg(pb + k);
-                    const int qx = x - b.x + 1, qy = y - b.y + 1;
-                    if ((unsigned)qx > 3u || (unsigned)qy > 3u) continue;
-                    const V4<T> sc = psc[k];
-                    const T W = tap_weight<T>(qx, sc.r, sc.x) * tap_weight<T>(qy, sc.y, sc.z);
-                    kap += W * I.kref[k];
-                    m0 += W;
-                    m1x += W * ((T)(ii - wi0) - gx0);
-                    m1y += W * ((T)(j - wj0) - gy0);
+                    S.sc[e] = psc[k];
+                    S.kx[e].r = kref[k];
+                    S.kx[e].x = (T)ii - (T)d.xiG[0];
+                    S.kx[e].y = (T)j - (T)d.xiG[1];
                 }
+                __syncthreads();
+#pragma unroll
+                for (int dy = -2; dy <= kTrRun; ++dy) {   // cell row against the run's first node
+                    const int c0 = (ly + dy + 2) * kTrCX + lx;
+                    const int e1 = S.start[c0 + 4];
+#pragma unroll 1
+                    for (int e = S.start[c0]; e < e1; ++e) {
+                        const V4<T> A = S.sc[e], B = S.kx[e];
+                        const T wx = tap_weight<T>(lx + 3 - (int)B.z, A.r, A.x);
+#pragma unroll
+                        for (int j = 0; j < kTrRun; ++j) {
+                            const int qy = j + 1 - dy;
+                            if (qy < 0 || qy > 3) continue;
+                            const T W = wx * tap_weight<T>(qy, A.y, A.z);
+                            kap[j] += W * B.r;
+                            m0[j] += W;
+                            m1x[j] += W * B.x;
+                            m1y[j] += W * B.y;
+                        }
+                    }
+                }
+            } else {
+                const int x = g.blo[0] + bx0 + lx, y0 = g.blo[1] + by0 + ly;
+                for (int j = wj0; j <= wj1; ++j)
+                    for (int ii = wi0; ii <= wi1; ++ii) {
+                        const int k = j * d.L[0] + ii;
+                        const int2 b = __ldg(pb + k);
+                        const int qx = x - b.x + 1, q0 = y0 - b.y + 1;
+                        if ((unsigned)qx > 3u || q0 > 3 || q0 + kTrRun - 1 < 0) continue;
+                        const V4<T> A = psc[k];
+                        const T wx = tap_weight<T>(qx, A.r, A.x);
+#pragma unroll
+                        for (int r = 0; r < kTrRun; ++r) {
+                            if ((unsigned)(q0 + r) > 3u) continue;
+                            const T W = wx * tap_weight<T>(q0 + r, A.y, A.z);
+                            kap[r] += W * kref[k];
+                            m0[r] += W;
+                            m1x[r] += W * ((T)ii - (T)d.xiG[0]);
+                            m1y[r] += W * ((T)j - (T)d.xiG[1]);
+                        }
+                    }
+            }
         }
         const bool f32 = sizeof(T) == 4;
         const T om = f32 ? (T)m.omf : (T)m.om, cT = f32 ? (T)m.cf : (T)m.c,
                 sT = f32 ? (T)m.sf : (T)m.s;
         const T ug0 = f32 ? (T)m.ugf[0] : (T)m.uG[0], ug1 = f32 ? (T)m.ugf[1] : (T)m.uG[1];
-        V4<T> o;
-        o.r = kap;
-        o.x = (-sT * m1x - cT * m1y) * om + ug0 * m0;
-        o.y = (cT * m1x - sT * m1y) * om + ug1 * m0;
-        o.z = (T)0;
-        kus[bi] = o;
+        if (bx0 + lx >= g.bn[0]) continue;
+#pragma unroll
+        for (int j = 0; j < kTrRun; ++j) {
+            if (by0 + ly + j >= g.bn[1]) break;
+            V4<T> o;
+            o.r = kap[j];
+            o.x = (-sT * m1x[j] - cT * m1y[j]) * om + ug0 * m0[j];
+            o.y = (cT * m1x[j] - sT * m1y[j]) * om + ug1 * m0[j];
+            o.z = (T)0;
+            kus[(long long)(by0 + ly + j) * g.bn[0] + bx0 + lx] = o;
+        }
     }
 }
 
@@ -1313,7 +1375,7 @@ cudaError_t launch_t_transfer(const Plan& p, int noff, int n, int kslot0, cudaSt
         device_mark(attr);
     }
     const long long units = (long long)p.total[U_BOX] * n;
-    k_t_transfer2d<T><<<cap_grid(units, sizeof(T) == 4 ? 8 : 4), NT, smem, st>>>(p, noff, n, kslot0);
+    k_t_transfer2d<T><<<cap_grid(units, sizeof(T) == 4 ? 8 : 4), kTrThreads, smem, st>>>(p, noff, n, kslot0);
     return cudaGetLastError();
 }
 

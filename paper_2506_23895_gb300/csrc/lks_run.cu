@@ -922,9 +922,10 @@ void inst_units(const lks_ctx* c, int out[U_COUNT]) {
     const Geom& g = c->g;
     const bool body = c->d.nd > 0 && g.boxN > 0;
     out[U_DCOL] = body ? (int)((c->d.ncol + kUnitThreads - 1) / kUnitThreads) : 0;
-    // footprint box in tiles of kBoxTile x kBoxTile nodes (the 2D transfer stages the design
+    // footprint box in tiles of kBoxTileX x kBoxTileY nodes (the 2D transfer stages the design
     // nodes a tile reads in shared memory)
-    out[U_BOX] = body ? ((g.bn[0] + kBoxTile - 1) / kBoxTile) * ((g.bn[1] + kBoxTile - 1) / kBoxTile)
+    out[U_BOX] = body ? ((g.bn[0] + kBoxTileX - 1) / kBoxTileX) *
+                            ((g.bn[1] + kBoxTileY - 1) / kBoxTileY)
                       : 0;
     out[U_OBJ] = obj_parts(g.ocount);
     for (int k = 0; k < kStripCfgs; ++k)

@@ -53,7 +53,7 @@ __host__ __device__ constexpr int strip_rows(int k) { return 2 << k; }   // 2, 4
 // Work-unit kinds: design columns in blocks of kUnitThreads, footprint-box tiles, objective parts,
 // strips of each row count.
 constexpr int kUnitThreads = 256;
-constexpr int kBoxTile = 16;   // box tiles of the 2D transfer: kBoxTile^2 = kUnitThreads nodes
+constexpr int kBoxTileX = 32, kBoxTileY = 16;   // box tiles of the 2D transfer
 enum { U_DCOL = 0, U_BOX, U_OBJ, U_STRIP0, U_COUNT = U_STRIP0 + kStripCfgs };
 
 // Parts the objective's target list is summed in, one warp each: about eight values per lane.
