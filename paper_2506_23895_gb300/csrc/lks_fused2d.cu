@@ -24,7 +24,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <type_traits>
 
 #include "lks_table.h"
 #include "lks_units.cuh"
@@ -749,8 +748,7 @@ __device__ __forceinline__ void step_strip(const Inst<T>& I, const Strip& s, con
     // sums of output row f - 1 (a) and f (b) as F-row f is reached: the directions already met
     T a_r = (T)0, a_y = (T)0, a_P = (T)0, a_Tp = (T)0, a_M = (T)0, a_Tm = (T)0;
     T b_2 = (T)0, b_5 = (T)0, b_6 = (T)0;
-    auto march = [&](int f, auto emit) {
-        constexpr bool EMIT = decltype(emit)::value;
+    auto march = [&](int f, bool emit) {   // emit: uniform, the row completes an output row
         issue(f + 1 + kAhead);
         cp_wait<kAhead>();   // row f + 1 has landed
         const int y = f - 1;   // output row this F-row completes
@@ -759,9 +757,9 @@ __device__ __forceinline__ void step_strip(const Inst<T>& I, const Strip& s, con
         vp = lds4(ring + ((f + 1) & (kRing - 1)) * 32);
         vm = lds4(ring + ((f - 1) & (kRing - 1)) * 32);
         kv.r = kv.x = kv.y = (T)0;
-        if (EMIT && bany) kv = lds4(ringk + (y & (kRing - 1)) * 32);
+        if (emit && bany) kv = lds4(ringk + (y & (kRing - 1)) * 32);
         T kst = (T)0;
-        if (GEN && EMIT && ks_st && ocol) kst = ks_st[y * n0 + x];
+        if (GEN && emit && ks_st && ocol) kst = ks_st[y * n0 + x];
         // twice the velocity gradient, D_ab = 2 d u_a / d x_b
         const T l1x = from_left(v0.x), l1y = from_left(v0.y);
         const T r1x = from_right(v0.x), r1y = from_right(v0.y);
@@ -807,7 +805,7 @@ __device__ __forceinline__ void step_strip(const Inst<T>& I, const Strip& s, con
         const T f2 = fma_<T>(W::w3_1, uy, ey), f4 = fma_<T>(-W::w3_1, uy, ey);
         const T f5 = fma_<T>(W::w3_2, cp, ep), f7 = fma_<T>(-W::w3_2, cp, ep);
         const T f6 = fma_<T>(W::w3_2, cm, em), f8 = fma_<T>(-W::w3_2, cm, em);
-        if (EMIT) {
+        if (emit) {
             const T Pl = from_left(add_<T>(a_P, f8)), Tl = from_left(sub_<T>(a_Tp, f8));
             const T Mr = from_right(add_<T>(a_M, f7)), Tr = from_right(sub_<T>(a_Tm, f7));
             V4<T> o;
@@ -842,10 +840,11 @@ __device__ __forceinline__ void step_strip(const Inst<T>& I, const Strip& s, con
         b_6 = f6;
     };
     for (int r = ya - 2; r < ya + kAhead; ++r) issue(r);
-    march(ya - 1, std::false_type{});
-    march(ya, std::false_type{});
-#pragma unroll 2
-    for (int f = ya + 1; f <= yb + 1; ++f) march(f, std::true_type{});
+    // one copy of the body: with the two rows before the first output apart and the loop unrolled by
+    // two, warps in three modes ran out of the instruction cache (64 channels of side 128 to 512:
+    // gradient 59.4 ms so, 51.6 ms with one)
+#pragma unroll 1
+    for (int f = ya - 1; f <= yb + 1; ++f) march(f, f > ya);
     cp_wait<0>();
 }
 
@@ -1126,7 +1125,12 @@ __device__ __forceinline__ void adj_strip(const Inst<T>& I, const Strip& s, bool
     {
         const Q qa = direct(ma - 1), qb = direct(ma);
         for (int i = 1; i <= kARing; ++i) issue(ma + i);
-        const V3<T> a = to_mu(ma - 1, qa), b = to_mu(ma, qb);
+        V3<T> a, b = qa.l;
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) {   // one copy of to_mu
+            a = b;
+            b = to_mu(ma - 1 + i, i == 0 ? qa : qb);
+        }
         d_P = sub_<T>(add_<T>(a.r, a.x), a.y);
         d_Q = sub_<T>(sub_<T>(a.r, a.x), a.y);
         d_y = sub_<T>(a.r, a.y);
@@ -1142,8 +1146,7 @@ __device__ __forceinline__ void adj_strip(const Inst<T>& I, const Strip& s, bool
     T Sxy2 = (T)0, Syy2 = (T)0, S0xy = (T)0, S0yy = (T)0;
     V4<T> o;
     o.r = o.x = o.y = o.z = (T)0;
-    auto march = [&](int m, auto emit) {
-        constexpr bool EMIT = decltype(emit)::value;
+    auto march = [&](int m, bool emit) {   // emit: uniform, row m - 1 is an output row
         const int y = m - 1;   // output row
         cp_wait<kAAhead>();    // row m + 1 has landed
         Q q;
@@ -1159,7 +1162,8 @@ __device__ __forceinline__ void adj_strip(const Inst<T>& I, const Strip& s, bool
             }
         }
         V4<T> u;   // u^{n-1} of the output row
-        if (EMIT) u = lds4(ringp + (y & (kARing - 1)) * 32);
+        u.r = u.x = u.y = u.z = (T)0;
+        if (emit) u = lds4(ringp + (y & (kARing - 1)) * 32);
         issue(m + 1 + kARing);   // into the slots just read
         const V3<T> v = to_mu(m + 1, q);
         const T va = add_<T>(v.r, v.x), vb = sub_<T>(v.r, v.x);
@@ -1196,7 +1200,7 @@ __device__ __forceinline__ void adj_strip(const Inst<T>& I, const Strip& s, bool
                 stg4(ocl + (y - 1) * n0, o);
             }
         }
-        if (EMIT && (!GEN || y <= yb)) {   // uniform
+        if (emit && (!GEN || y <= yb)) {   // uniform
             T tx = add_<T>(gx, sub_<T>(Sxy2, nSxy)), ty = add_<T>(gy, sub_<T>(Syy2, nSyy));
             if (GEN && !p1) {
                 if (y <= 2) {
@@ -1241,10 +1245,9 @@ __device__ __forceinline__ void adj_strip(const Inst<T>& I, const Strip& s, bool
         c_Q = sub_<T>(vb, v.y);
         c_y = sub_<T>(v.r, v.y);
     };
-    int m = ma;
-    for (; m <= ya; ++m) march(m, std::false_type{});   // two rows, three from boundary row 0
-#pragma unroll 2
-    for (; m <= mb; ++m) march(m, std::true_type{});
+    // (two rows before the first output, three from boundary row 0; one copy of the body as above)
+#pragma unroll 1
+    for (int m = ma; m <= mb; ++m) march(m, m > ya);
     cp_wait<0>();
 }
 
