@@ -111,8 +111,10 @@ def peaks():
 # Source files each timed stencil step is built from; committed ncu counters count only
 # while these files are unchanged.
 STEP_SOURCES = {
-    "forward_step": ("lks_fused3d.cu", "lks_device.cuh", "lks_tma.cuh", "lks_internal.h"),
-    "adjoint_step": ("lks_fused3d_adj.cu", "lks_plain.cu", "lks_units.cuh", "lks_device.cuh",
+    "forward_step": ("lks_fused3d.cu", "lks_march3d.cu", "lks_march3d.h", "lks_units.cuh",
+                     "lks_device.cuh", "lks_tma.cuh", "lks_internal.h"),
+    "adjoint_step": ("lks_fused3d_adj.cu", "lks_march3d_adj.cu", "lks_march3d.h", "lks_march3d.cu",
+                     "lks_plain.cu", "lks_units.cuh", "lks_device.cuh",
                      "lks_tma.cuh", "lks_internal.h"),
 }
 
@@ -407,8 +409,8 @@ def run_batch_line(args, lks, W, ws, rank, local, dev):
 
 
 # kernel of each fused 3D forward-step variant (lks_step_variant)
-STEP3D_KERNELS = {0: "k_fused_step3d", 1: "k_zstep3d<8> + k_bc_shell3d",
-                  2: "k_zpair3d + k_bc_shell3d"}
+STEP3D_KERNELS = {0: "k_fused_step3d", 1: "k_step_march + k_bc_shell3d",
+                  2: "k_step_march + k_bc_shell3d"}
 
 
 def run_ours(args):
@@ -524,7 +526,7 @@ def run_ours(args):
           "avg_launch_ms": fwd_step_ms, "samples": tm["fwd_n"]}
     ra = {"bound": "hbm", "achieved": ach_adj, "peak": peak, "unit": "GB/s",
           "frac": ach_adj / peak, "traffic": ncu_traffic("adjoint_step"),
-          "kernel": "adjoint stencil step: k_adj_bcT + k_fused_adj3d + k_adj_bcorr",
+          "kernel": "adjoint stencil step: k_adj_prep + k_adj_march + k_adj_bcorr",
           "share_of_pass": share_adj, "launches_per_pass": H,
           "concurrent": "the next step's transfer and the sensitivity gather run beside it on a "
                         "side stream",

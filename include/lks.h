@@ -281,8 +281,8 @@ int lks_inject_alloc_failure(int nth);
 /* ---- batches: many problems in lock step (designs, finite-difference perturbations, grids of
  * different sizes).  The paper solves one problem at a time; a batch runs the same Algorithm 1
  * and adjoint sweep for every member context, with each phase of a step one persistent kernel
- * launch over all members, runs of steps captured into CUDA graphs and replayed, and the tile
- * shape of the fused step and adjoint kernels chosen by timing every candidate on the batch.
+ * launch over all members, runs of steps captured into CUDA graphs and replayed, and the
+ * strip height of the step and adjoint kernels chosen by timing every candidate on the batch.
  * Each member keeps its own design, motion, objective, state and gradient: results are bitwise
  * those of the member run alone with lks_forward / lks_adjoint. */
 typedef struct lks_batch lks_batch;
@@ -295,10 +295,10 @@ typedef struct lks_batch lks_batch;
  * at every call.  LKS_ERR_NOMEM if that fails. */
 lks_status lks_batch_create(lks_ctx* const* ctxs, int n, lks_batch** out);
 
-/* use_graphs: 1 (default) capture and replay runs of steps, 0 launch directly.  tile_fwd:
- * configuration of the fused step kernel (0..4 tiles, 5..8 row-marching strips; see
- * lks_batch_tile_shapes); tile_adj: configuration of the fused adjoint kernel (0..4 tiles);
- * -1 (default) autotunes at the next forward.  LKS_ERR_ARG on an index out of range. */
+/* use_graphs: 1 (default) capture and replay runs of steps, 0 launch directly.  tile_fwd,
+ * tile_adj: strip height of the step and the adjoint kernel as an index into
+ * lks_batch_tile_shapes; -1 (default) autotunes at the next forward.  LKS_ERR_ARG on an index out
+ * of range. */
 lks_status lks_batch_set_options(lks_batch* b, int use_graphs, int tile_fwd, int tile_adj);
 
 /* lks_forward for every member: J_out (host, n doubles, may be NULL) receives each member's
@@ -311,8 +311,8 @@ lks_status lks_batch_forward(lks_batch* b, int n_steps, double* J_out);
  * forward on every member. */
 lks_status lks_batch_adjoint(lks_batch* b, double* const* dJdgamma, int on_device);
 
-/* The work-unit extent (tx, ty) of every step configuration (the adjoint uses the first
- * five); returns their number (writes <= cap pairs) or -1 on bad arguments.  Host only. */
+/* The output columns and rows (tx, ty) of every strip configuration; returns their number
+ * (writes <= cap pairs) or -1 on bad arguments.  Host only. */
 int lks_batch_tile_shapes(int* txty, int cap);
 
 /* chosen2: configuration indices in use for [step, adjoint] (-1 before the first forward);

@@ -4,9 +4,10 @@
 // equilibrium with the viscosity term) into a Q-plane scratch, k_gather sums f_i^eq(x - c_i)
 // into rho*, u* (Eqs. rho, u), applies the Brinkman update u = (u* + kappa u_S)/(1 + kappa)
 // (Eq. u_ex_2) and writes the boundary nodes sourced from each interior node (Eqs. bc_rho,
-// bc_u).  Adjoint step (Alg. 2 structure, exact transpose of the above): k_adj_bcT pushes
-// boundary adjoints onto their copy sources, k_adj_mu divides by (1 + kappa) and forms the
-// kappa sensitivity density e, k_adj_moments gathers F~_i(y) = mu_rho(y+c_i) + c_i.mu_u(y+c_i)
+// bc_u).  Adjoint step (Alg. 2 structure, exact transpose of the above): k_adj_prep adds the
+// boundary adjoints to their copy sources, divides by (1 + kappa) and forms the kappa sensitivity
+// density e, in place (k_adj_bcT and k_adj_mu where a static solid is set, and for the printed
+// variant), k_adj_moments gathers F~_i(y) = mu_rho(y+c_i) + c_i.mu_u(y+c_i)
 // into the moments of Eqs. arho, au, as and the adjoint equilibrium, k_adj_divT adds the
 // transposed velocity-gradient term.  These kernels are templated on the scalar type; the
 // double instantiation is the plain FP64 path.

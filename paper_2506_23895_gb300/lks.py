@@ -392,7 +392,7 @@ def state_bytes(problem, precision: int = FP32) -> int:
 
 
 def tile_shapes():
-    """Candidate (tx, ty) tile shapes of the fused 2D kernels."""
+    """Candidate (columns, rows) strips of the 2D kernels."""
     lib = load()
     n = lib.lks_batch_tile_shapes(None, 0)
     a = (ctypes.c_int * (2 * n))()
@@ -402,7 +402,7 @@ def tile_shapes():
 
 class Batch:
     """Many D2Q9 FP32 problems advanced in lock step (lks_batch_*): one launch per phase over
-    all members, runs of steps replayed from CUDA graphs, autotuned tile shapes.
+    all members, runs of steps replayed from CUDA graphs, autotuned strip heights.
 
     The members are Solvers built with equal max_steps and `slots` snapshot slots each."""
 
