@@ -626,8 +626,8 @@ struct Strip {
     int mode;       // kInner, kSide or kGeneral
 };
 
-// What a strip and its halo of two nodes and kReach more rows touch: no face and no node next to
-// one; only an x face of a grid without wraps and static solids; anything else.
+// What a strip and its halo of two nodes and two more rows touch: no face and no node next to one;
+// only x faces of a grid without wraps and static solids, no node next to both; anything else.
 enum { kInner = 0, kSide = 1, kGeneral = 2 };
 
 template <class T>
@@ -644,7 +644,10 @@ __device__ __forceinline__ Strip strip_of(const Inst<T>& I, int local, int rows,
     s.in = s.x >= 0 && s.x < n0;
     s.ya = kc * rows;
     s.yb = min(s.ya + rows, n1) - 1;
-    const bool plain = !g.periodic[0] && !g.periodic[1] && !g.ks && s.ya >= 4 && s.yb <= n1 - 5;
+    // (along an x axis of three nodes the inner column lies next to both faces, where a kSide lane
+    // serves one)
+    const bool plain = n0 > 3 && !g.periodic[0] && !g.periodic[1] && !g.ks && s.ya >= 4 &&
+                       s.yb <= n1 - 5;
     const bool xmid = s.xs >= 4 && s.xs + kStripW + 1 <= n0 - 3;
     // (the adjoint's kSide path finds the face column in the lane beside a node next to it)
     const bool xcut = s.xs - 2 + 31 == n0 - 2;
