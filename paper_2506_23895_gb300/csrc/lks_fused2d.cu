@@ -1315,6 +1315,23 @@ int cap_grid(long long units, int per_sm) {
     return (int)std::max(1LL, std::min(units, g));
 }
 
+// The shared-memory limit of the strip kernels, raised once per device to what eight warps take: the
+// limit belongs to the kernel, not to a context, so a launch must not set it to its own size while
+// another thread's context is about to launch a larger one.
+template <class T>
+cudaError_t raise_strip_limits() {
+    static std::atomic<unsigned> attr{0};
+    if (device_done(attr)) return cudaSuccess;
+    constexpr int most = (int)sizeof(StripWarp<T>) * (kStripThreads / 32);
+    for (const void* kern : {(const void*)k_t_step<T>, (const void*)k_t_adj<T>}) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e != cudaSuccess) return e;
+    }
+    device_mark(attr);
+    return cudaSuccess;
+}
+
 // Blocks and warps per block of a strip kernel over `units` strips: the strips spread over all
 // SMs, eight warps to a block at most; a launch of several steps keeps every block resident and
 // loops over the rest.
@@ -1325,11 +1342,6 @@ cudaError_t launch_strips(K kern, size_t warp_bytes, long long units, bool meet,
     const int wpb = (int)std::min<long long>(kStripThreads / 32, (units + sms - 1) / sms);
     const int w = units <= kStripThreads / 32 ? (int)units : wpb;   // a few strips: one block
     const size_t smem = warp_bytes * w;
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(
-            (const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
     long long grid = (units + w - 1) / w;
     if (meet && grid > sms) {
         int per = 0;
@@ -1388,6 +1400,8 @@ cudaError_t launch_t_transfer(const Plan& p, int noff, int n, int kslot0, cudaSt
 template <class T>
 cudaError_t launch_t_step(const Plan& p, int cfg, const StripRun& r, cudaStream_t st) {
     if (cfg < 0 || cfg >= kStripCfgs) return cudaErrorInvalidValue;
+    const cudaError_t e = raise_strip_limits<T>();
+    if (e != cudaSuccess) return e;
     const int unit = U_STRIP0 + cfg;
     return launch_strips(k_t_step<T>, sizeof(StripWarp<T>),
                          p.total[unit] + (r.obj && r.n > 1 ? p.total[U_OBJ] : 0), r.n > 1, p, unit,
@@ -1397,6 +1411,8 @@ cudaError_t launch_t_step(const Plan& p, int cfg, const StripRun& r, cudaStream_
 template <class T>
 cudaError_t launch_t_adj(const Plan& p, int cfg, const StripRun& r, cudaStream_t st) {
     if (cfg < 0 || cfg >= kStripCfgs) return cudaErrorInvalidValue;
+    const cudaError_t e = raise_strip_limits<T>();
+    if (e != cudaSuccess) return e;
     const int unit = U_STRIP0 + cfg;
     return launch_strips(k_t_adj<T>, sizeof(StripWarp<T>), p.total[unit], r.n > 1, p, unit,
                          strip_rows(cfg), r, st);
