@@ -44,7 +44,7 @@ typedef enum {
     LKS_ERR_NOMEM = 3,    /* workspace too small or device allocation failed */
     LKS_ERR_CUDA = 4,     /* a CUDA runtime call failed */
     LKS_ERR_DIVERGED = 5, /* non-finite or |u| > 0.5 state after a forward run */
-    LKS_ERR_TIMEOUT = 6   /* reserved for bounded device waits */
+    LKS_ERR_TIMEOUT = 6   /* a bounded wait ran out inside a kernel; the run's results are void */
 } lks_status;
 
 /* Face boundary types; faces are ordered x-, x+, y-, y+, z-, z+ (Eqs. bc_rho, bc_u).
@@ -323,6 +323,13 @@ lks_status lks_batch_tuning(const lks_batch* b, int* chosen2, float* ms);
 /* [0] kernels launched by the last forward or adjoint call (graph nodes included), [1] graphs
  * held, [2] kernel nodes in them. */
 lks_status lks_batch_stats(const lks_batch* b, long long* stats3);
+
+/* The status each of n members ends a lock-step run with, from the four error words a run leaves per
+ * member ([1] transfer lists overfull, [2] diverged, [3] kernel errors, bit 3 a bounded wait that ran
+ * out).  A wait that ran out stops the launch over all members and is recorded with the first only: it
+ * ends the run of every member with LKS_ERR_TIMEOUT.  status: n lks_status values.  Returns n, or -1
+ * on bad arguments.  For inspection; host only, needs no device. */
+int lks_batch_statuses(const int* words, int n, int* status);
 
 const char* lks_batch_last_error(const lks_batch* b);
 void lks_batch_destroy(lks_batch* b);

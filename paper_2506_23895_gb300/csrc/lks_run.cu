@@ -680,13 +680,42 @@ lks_status exec_adj(Group& G, int seg) {
     return LKS_OK;
 }
 
-// The status a run's error words stand for.
+// The status a run's four error words stand for.
+lks_status word_status(const int* f) {
+    if (f[1]) return LKS_ERR_ARG;
+    if (f[3] & 8) return LKS_ERR_TIMEOUT;
+    if (f[3]) return LKS_ERR_CUDA;
+    return f[2] ? LKS_ERR_DIVERGED : LKS_OK;
+}
+
 lks_status run_status(lks_ctx* c, const int* f) {
-    if (f[1]) return fail(c, LKS_ERR_ARG, "transfer tap list overflow");
-    if (f[3] & 8) return fail(c, LKS_ERR_TIMEOUT, "a bounded wait ran out in a fused kernel");
-    if (f[3]) return fail(c, LKS_ERR_CUDA, "fused step reported error %d", f[3]);
-    if (f[2]) return fail(c, LKS_ERR_DIVERGED, "state diverged (non-finite or |u| >= 0.5)");
-    return LKS_OK;
+    const lks_status s = word_status(f);
+    switch (s) {
+        case LKS_ERR_ARG: return fail(c, s, "transfer tap list overflow");
+        case LKS_ERR_TIMEOUT: return fail(c, s, "a bounded wait ran out in a fused kernel");
+        case LKS_ERR_CUDA: return fail(c, s, "fused step reported error %d", f[3]);
+        case LKS_ERR_DIVERGED:
+            return fail(c, s, "state diverged (non-finite or |u| >= 0.5)");
+        default: return s;
+    }
+}
+
+// A bounded wait that ran out in a launch over a group is recorded with the group's first context
+// (Plan::err), but the run stopped half way for all of them: the record counts for each.  words: four
+// error words per context.  True if there was one.
+bool share_waits(int* words, int n) {
+    int waited = 0;
+    for (int k = 0; k < n; ++k) waited |= words[4 * k + 3] & 8;
+    for (int k = 0; k < n; ++k) words[4 * k + 3] |= waited;
+    return waited != 0;
+}
+
+// The error words of a group's finished run on the table kernels.
+std::vector<int> result_words(const std::vector<RunResult>& res, bool& waited) {
+    std::vector<int> w;
+    for (const RunResult& r : res) w.insert(w.end(), r.flags, r.flags + 4);
+    waited = share_waits(w.data(), (int)res.size());
+    return w;
 }
 
 template <class T>
@@ -737,12 +766,15 @@ lks_status do_forward(Group& G, int N) {
         GCU(cudaMemcpyAsync(res.data(), G.result, sizeof(RunResult) * G.count,
                             cudaMemcpyDeviceToHost, G.st));
         GCU(cudaStreamSynchronize(G.st));
+        bool waited;
+        const std::vector<int> words = result_words(res, waited);
         lks_status worst = LKS_OK;
         for (int k = 0; k < G.count; ++k) {
             lks_ctx* c = G.cs[k];
             c->adj_begin = i + 1;
-            const lks_status s = run_status(c, res[k].flags);
+            const lks_status s = run_status(c, &words[4 * k]);
             if (s != LKS_OK) {
+                if (waited) c->have_end = false;   // no end state: the run stopped half way
                 if (worst == LKS_OK) worst = s;
                 continue;
             }
@@ -829,9 +861,12 @@ lks_status do_adjoint(Group& G) {
             G.cs[k]->have_lend = true;
         }
         GCU(cudaStreamSynchronize(G.st));
+        bool waited;
+        const std::vector<int> words = result_words(res, waited);
         lks_status worst = LKS_OK;
         for (int k = 0; k < G.count; ++k) {
-            const lks_status s = run_status(G.cs[k], res[k].flags);
+            if (waited) G.cs[k]->have_lend = false;   // the sweep stopped half way
+            const lks_status s = run_status(G.cs[k], &words[4 * k]);
             if (s != LKS_OK && worst == LKS_OK) worst = s;
         }
         return worst;
@@ -1035,3 +1070,11 @@ template lks_status do_adjoint<double>(Group&);
 
 }  // namespace eng
 }  // namespace lks
+
+extern "C" int lks_batch_statuses(const int* words, int n, int* status) {
+    if (n < 1 || !words || !status) return -1;
+    std::vector<int> w(words, words + 4 * (size_t)n);
+    lks::eng::share_waits(w.data(), n);
+    for (int k = 0; k < n; ++k) status[k] = (int)lks::eng::word_status(&w[4 * (size_t)k]);
+    return n;
+}

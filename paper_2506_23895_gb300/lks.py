@@ -28,7 +28,7 @@ EXPORTS = ("lks_workspace_bytes", "lks_create", "lks_set_design", "lks_set_motio
            "lks_batch_tile_shapes", "lks_batch_tuning", "lks_batch_stats",
            "lks_batch_last_error", "lks_batch_destroy", "lks_set_filter", "lks_volume",
            "lks_set_static", "lks_warm_start", "lks_set_adjoint_start", "lks_get_adjoint_state",
-           "lks_inject_alloc_failure", "lks_fma_rate", "lks_adjoint_variant")
+           "lks_inject_alloc_failure", "lks_fma_rate", "lks_adjoint_variant", "lks_batch_statuses")
 
 
 class LksError(RuntimeError):
@@ -130,6 +130,9 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.lks_batch_tuning.argtypes = [P, ctypes.POINTER(ctypes.c_int),
                                      ctypes.POINTER(ctypes.c_float)]
     lib.lks_batch_stats.argtypes = [P, ctypes.POINTER(ctypes.c_longlong)]
+    lib.lks_batch_statuses.argtypes = [ctypes.POINTER(ctypes.c_int), ctypes.c_int,
+                                       ctypes.POINTER(ctypes.c_int)]
+    lib.lks_batch_statuses.restype = ctypes.c_int
     lib.lks_batch_last_error.argtypes = [P]
     lib.lks_batch_last_error.restype = ctypes.c_char_p
     lib.lks_batch_destroy.argtypes = [P]
