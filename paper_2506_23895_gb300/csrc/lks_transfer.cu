@@ -61,9 +61,11 @@ __global__ void k_design_pos(Design d, Geom g, Motion m, TransferScratch ts) {
     const int lz = d.L[2];
     if (k < lz) {  // moved z of design plane k (3D: pure shift; 2D: the single plane at 0)
         if (g.dim == 3) {
-            const double zr = (double)k - d.xiG[2] + m.xG[2];
+            // plane 0's base and fraction serve every plane: rounded per plane, the bases of far planes
+            // step up where the shift lies a few roundings below an integer, and the fraction does not
+            const double zr = m.xG[2] - d.xiG[2];
             const double bz = floor(zr);
-            ts.dz_base[k] = (int)bz;
+            ts.dz_base[k] = (int)bz + (int)k;
             if (k == 0) {
                 T* z = (T*)ts.dz_sc;
                 sincospi_half<T>((T)(zr - bz), z[0], z[1]);
