@@ -168,7 +168,8 @@ lks_status lks_get_adjoint_state(const lks_ctx* ctx, double* lambda_out);
 
 /* Set the motion schedule; needs n_rows >= max_steps + 1.  The transfer footprint (every
  * analysis node within two cells of a moved design node) must stay inside the grid and off
- * boundary nodes for every step, else LKS_ERR_ARG.  Invalidates any forward run. */
+ * boundary nodes for every step, else LKS_ERR_ARG, and the motion set before stays.  Invalidates
+ * any forward run. */
 lks_status lks_set_motion(lks_ctx* ctx, const lks_motion* motion);
 
 /* Replace the initial state (rho, ux, uy, uz planes of nodes doubles each, host).  NULL

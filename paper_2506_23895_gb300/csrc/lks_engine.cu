@@ -629,17 +629,18 @@ lks_status lks_set_motion(lks_ctx* c, const lks_motion* m) {
     if (m->n_rows < c->cfg.max_steps + 1)
         return fail(c, LKS_ERR_ARG, "motion has %d rows, need max_steps + 1 = %d", m->n_rows,
                     c->cfg.max_steps + 1);
-    c->motion.assign(m->rows, m->rows + 8 * (size_t)m->n_rows);
-    Geom& g = c->g;
+    std::vector<double> rows(m->rows, m->rows + 8 * (size_t)m->n_rows);
+    Geom g = c->g;   // (a refused motion leaves the context's own as it was)
     if (c->d.nd == 0) {
-        g.boxN = 0;
+        c->motion.swap(rows);
+        c->g.boxN = 0;
         return finish_motion(c);
     }
     // union over steps of the analysis nodes strictly within two cells of a moved design node
     double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
     const double cx[2] = {0.0, (double)(c->d.L[0] - 1)}, cy[2] = {0.0, (double)(c->d.L[1] - 1)};
     for (int n = 1; n <= c->cfg.max_steps; ++n) {
-        const Motion mo = motion_row(c, n);
+        const Motion mo = motion_row(c, &rows[8 * (size_t)n]);
         if (c->gaxis) {   // images of the design box's eight corners bound its image
             for (int cidx = 0; cidx < 8; ++cidx) {
                 double dv[3];
@@ -689,6 +690,8 @@ lks_status lks_set_motion(lks_ctx* c, const lks_motion* m) {
         g.bn[a] = h - l + 1;
     }
     g.boxN = (long long)g.bn[0] * g.bn[1] * g.bn[2];
+    c->motion.swap(rows);
+    c->g = g;
     return finish_motion(c);
 }
 

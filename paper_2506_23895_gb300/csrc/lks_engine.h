@@ -232,7 +232,7 @@ struct Group {
 
 Group self_group(lks_ctx*& c);
 char* slot_ptr(lks_ctx* c, int slot);
-Motion motion_row(const lks_ctx* c, int n);
+Motion motion_row(const lks_ctx* c, const double* row);
 lks_status run_fork(lks_ctx* c);
 lks_status run_join(lks_ctx* c, lks_status s);
 lks_status transfer_join(lks_ctx* c);

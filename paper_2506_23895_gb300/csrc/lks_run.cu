@@ -30,8 +30,7 @@ void timing_end(lks_ctx* c, int which) {
     c->tused[which] += 2;
 }
 
-Motion motion_row(const lks_ctx* c, int n) {
-    const double* r = c->motion.data() + 8 * (size_t)n;
+Motion motion_row(const lks_ctx* c, const double* r) {
     Motion m;
     m.c = std::cos(r[0]);
     m.s = std::sin(r[0]);
@@ -84,7 +83,7 @@ Motion motion_row(const lks_ctx* c, int n) {
 // The transfer of step n into buffer set x on stream st (3D and plain 2D paths).
 template <class T>
 lks_status transfer_into(lks_ctx* c, int n, const lks_ctx::XSlot& x, cudaStream_t st) {
-    const Motion m = motion_row(c, n);
+    const Motion m = motion_row(c, &c->motion[8 * (size_t)n]);
     if (c->gaxis) {
         launch_transfer_axis<T>(c->d, c->g, m, x.as, (const T*)c->kref, st4<T>(x.kus), st);
         LAUNCHED();
@@ -1045,7 +1044,7 @@ const double* design_gradient(lks_ctx* c, cudaStream_t st) {
 lks_status finish_motion(lks_ctx* c) {
     const int rows = c->cfg.max_steps + 1;
     std::vector<Motion> mr(rows);
-    for (int n = 0; n < rows; ++n) mr[n] = motion_row(c, n);
+    for (int n = 0; n < rows; ++n) mr[n] = motion_row(c, &c->motion[8 * (size_t)n]);
     CU(cudaMemcpyAsync(c->dmotion, mr.data(), sizeof(Motion) * rows, cudaMemcpyHostToDevice, c->st));
     CU(cudaStreamSynchronize(c->st));
     ++c->geo_gen;
