@@ -158,8 +158,7 @@ double count_target(const lks_config* c) {
 struct Layout {
     size_t off[96];
     size_t total;
-    int ktape_slots;   // slots of the transfer tape (0: none)
-    int pos_slots;     // steps of design positions
+    TapePlan tape;     // 2D table kernels: memory for the transfers, e and positions of several steps
     int pool_slots;
     size_t snap;
 };
@@ -173,7 +172,7 @@ enum {
     // the second transfer buffer set (3D): same sizes as L_KUS, L_K2, L_CBASE, ...
     L_KUS2, L_K22, L_CBASE2, L_CSC2, L_ZTI2, L_ZTW2, L_TIDX2, L_TW2, L_CM2,
     L_DZB2, L_DZF2, L_GBASE2, L_GFRAC2, L_GCNT2, L_GIDX2, L_E2,
-    L_KTAPE, L_ETAPE, L_PB, L_PSC, L_JPART, L_POOL,
+    L_TAPE, L_JPART, L_POOL,
     L_COUNT
 };
 static_assert(L_COUNT <= 96, "Layout::off holds 96 regions");
@@ -189,7 +188,7 @@ Layout make_layout(const lks_config* cfg) {
     const long long cols = (long long)cfg->nx * cfg->ny;   // box columns, worst case
     const int nzb = dim == 3 ? cfg->nz : 1;
     const size_t state = align256((size_t)nodes * 4 * T);
-    size_t sz[L_COUNT];
+    size_t sz[L_COUNT] = {};
     sz[L_S0] = sz[L_S1] = sz[L_SINIT] = sz[L_L0] = sz[L_L1] = state;
     sz[L_F] = (size_t)Q * nodes * T;
     sz[L_MU] = state;
@@ -256,22 +255,39 @@ Layout make_layout(const lks_config* cfg) {
         sz[L_E2] = two ? sz[L_E] : 0;
     }
     // 2D contexts on the table kernels form the transfers (kappa, u_S on the footprint box) of many
-    // steps in one launch and keep those of a taped segment for its adjoint: a tape of up to
-    // max(ceil(sqrt(N)) + 2, 64) steps (the checkpointed schedules' tape length, and short
-    // full-history runs), at least 16 where the pool is smaller, each slot sized for the whole grid
-    // (the box is known only once the motion is set); e of the same steps for the sensitivity
-    // gather, and the design positions of up to 32 steps
+    // steps in one launch, keep those of a taped segment for its adjoint where they fit, and keep e of
+    // many steps for the sensitivity gather.  Their memory is that of the plain kernels' scratch, which
+    // no table kernel uses, half of what the snapshots take but at most 256 MB, and in FP32 (16 bytes a
+    // node) a slot for each snapshot slot up to max(ceil(sqrt(N)) + 2, 64), a segment of the
+    // checkpointed schedules.  So ckpt_bytes bounds the whole; with fewer slots launches are shorter
+    // and a segment's transfers may be formed twice (512^2 FP64, 60 steps: 10.5 ms a gradient with 42
+    // of 61 slots, 8.4 with all).
     {
+        L.tape = TapePlan{};
         const bool table = dim == 2 && !(cfg->flags & (LKS_FLAG_PLAIN_KERNELS | LKS_FLAG_PAPER_ALKS));
-        const bool t2d = table && nd > 0;
-        const long long kt = std::max((long long)std::ceil(std::sqrt((double)N)) + 2, 64LL);
-        L.ktape_slots = t2d ? (int)std::min(N + 1, std::max(std::min(P, kt), 16LL)) : 0;
-        sz[L_KTAPE] = (size_t)L.ktape_slots * state;
-        sz[L_ETAPE] = (size_t)L.ktape_slots * (size_t)nodes * T;
-        L.pos_slots = std::min(L.ktape_slots, 32);
-        sz[L_PB] = (size_t)L.pos_slots * (size_t)ncol * 8;
-        sz[L_PSC] = (size_t)L.pos_slots * (size_t)ncol * 4 * T;
-        sz[L_JPART] = table ? (size_t)(cfg->max_steps + 2) * obj_parts(count_target(cfg)) * 8 : 0;
+        if (table) {
+            size_t spare = 0;
+            for (int r : {L_F, L_PHI, L_E, L_JSTEP, L_CBASE, L_CSC, L_ZTI, L_ZTW, L_TIDX, L_TW, L_CM,
+                          L_DZB, L_DZF, L_K2, L_FACE}) {
+                spare += sz[r];
+                sz[r] = 0;
+            }
+            sz[L_JPART] = (size_t)(cfg->max_steps + 2) * obj_parts(count_target(cfg)) * 8;
+            if (nd > 0) {
+                const long long kt = std::max((long long)std::ceil(std::sqrt((double)N)) + 2, 64LL);
+                L.tape.want = (int)std::min(N + 1, std::max(std::min(P, kt), 16LL));
+                L.tape.least = T == 4 ? (int)std::min(P, kt) : 1;
+                const TapeSlots all{L.tape.want, std::min(L.tape.want, kMaxESlots),
+                                    std::min(L.tape.want, kMaxPosSlots)};
+                spare -= std::min(spare, sz[L_JPART] + sz[L_FQ]);
+                L.tape.bytes = std::max(
+                    tape_bytes({L.tape.least, 1, 1}, nodes, ncol, T),
+                    std::min(tape_bytes(all, nodes, ncol, T),
+                             spare + std::min((size_t)P * state / 2, (size_t)256 << 20) +
+                                 (T == 4 ? (size_t)L.tape.least * state : 0)));
+                sz[L_TAPE] = L.tape.bytes;
+            }
+        }
     }
     sz[L_POOL] = (size_t)P * state;
     size_t off = 0;
@@ -417,12 +433,8 @@ lks_status lks_create(const lks_config* cfg, void* workspace, size_t ws_bytes, l
     c->pool_slots = L.pool_slots;
     c->snap_bytes = L.snap;
     c->fused2d = g.dim == 2 && !(cfg->flags & (LKS_FLAG_PLAIN_KERNELS | LKS_FLAG_PAPER_ALKS));
-    c->ktape_slots = c->fused2d ? L.ktape_slots : 0;
-    c->ktape = c->ktape_slots > 0 ? (void*)(w + L.off[L_KTAPE]) : nullptr;
-    c->etape = w + L.off[L_ETAPE];
-    c->pos_b = w + L.off[L_PB];
-    c->pos_sc = w + L.off[L_PSC];
-    c->pos_slots = L.pos_slots;
+    c->tape = L.tape;
+    c->tape_mem = w + L.off[L_TAPE];
     c->jpart = (double*)(w + L.off[L_JPART]);
     c->dmotion = (Motion*)(w + L.off[L_MOTION]);
     c->dinst = w + L.off[L_INST];

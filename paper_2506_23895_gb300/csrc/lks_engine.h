@@ -38,6 +38,18 @@ void plan_tape(int N, int P, int& K, int& M, int& S);
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Steps a 2D context on the table kernels keeps transfers (k), e and design positions of.
+struct TapeSlots {
+    int k = 0, e = 0, pos = 0;
+};
+// The memory it has for them: `bytes`, for `want` transfers if they fit and `least` in any case.
+struct TapePlan {
+    size_t bytes = 0;
+    int want = 0, least = 0;
+};
+// e and positions of so many steps fill a launch; more would only take memory from the transfers.
+constexpr int kMaxESlots = 64, kMaxPosSlots = 32;
+
 }  // namespace eng
 }  // namespace lks
 
@@ -78,14 +90,15 @@ struct lks_ctx {
     char* pool;
     int pool_slots;
     size_t snap_bytes;
-    // 2D table path: kappa, u_S on the footprint box and e for ktape_slots steps, design
-    // positions (base, sin/cos table) for pos_slots steps, partial objective sums
+    // 2D table path: kappa, u_S and e on the footprint box and design positions (base, sin/cos table)
+    // of several steps, placed once the box is known; partial objective sums
+    lks::eng::TapePlan tape;
+    char* tape_mem = nullptr;
+    lks::eng::TapeSlots slots;
     void* ktape = nullptr;
     void* etape = nullptr;
-    int ktape_slots = 0;
     void* pos_b = nullptr;
     void* pos_sc = nullptr;
-    int pos_slots = 0;
     double* jpart = nullptr;
     // host state
     std::vector<double> motion;
@@ -240,6 +253,8 @@ lks_status finish_motion(lks_ctx* c);
 lks_status design_prep(lks_ctx* c);
 const double* design_gradient(lks_ctx* c, cudaStream_t st);
 lks_status own_plan(lks_ctx* c);
+size_t tape_bytes(const TapeSlots& t, long long boxN, long long ncol, size_t T);
+TapeSlots tape_slots(const TapePlan& p, long long boxN, long long ncol, size_t T);
 template <class T>
 cudaError_t build_plan(const std::vector<lks_ctx*>& cs, void* dinst, int* dpre, int* nbase,
                        cudaStream_t st, Plan& p);

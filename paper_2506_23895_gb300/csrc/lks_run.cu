@@ -404,17 +404,21 @@ Group self_group(lks_ctx*& c) {
 bool tape_transfers(const Group& G) {
     if (!G.table) return false;
     for (int i = 0; i < G.count; ++i)
-        if (G.cs[i]->d.nd > 0 && G.cs[i]->K + 1 > G.cs[i]->ktape_slots) return false;
+        if (G.cs[i]->d.nd > 0 && G.cs[i]->K + 1 > G.cs[i]->slots.k) return false;
     return true;
 }
 
 // Steps of a run handled by one launch: at most kRunSteps (which bounds a launch to some
-// milliseconds) and as many as there are transfer slots.
+// milliseconds) and as many as there are slots for their transfers (unless those are kept: kt) and, in
+// the adjoint, for their e.
 constexpr int kRunSteps = 512;
-int group_chunk(const Group& G) {
+int group_chunk(const Group& G, bool kt, bool adjoint) {
     int n = kRunSteps;
-    for (int i = 0; i < G.count; ++i)
-        if (G.cs[i]->d.nd > 0) n = std::min(n, G.cs[i]->ktape_slots);
+    for (int i = 0; i < G.count; ++i) {
+        if (G.cs[i]->d.nd == 0) continue;
+        if (!kt) n = std::min(n, G.cs[i]->slots.k);
+        if (adjoint) n = std::min(n, G.cs[i]->slots.e);
+    }
     return std::max(n, 1);
 }
 
@@ -423,7 +427,7 @@ template <class T>
 cudaError_t table_transfers(const Group& G, int k, int n, int slot, int& nl) {
     int pos = n;
     for (int i = 0; i < G.count; ++i)
-        if (G.cs[i]->d.nd > 0) pos = std::min(pos, G.cs[i]->pos_slots);
+        if (G.cs[i]->d.nd > 0) pos = std::min(pos, G.cs[i]->slots.pos);
     for (int j = 0; j < n; j += pos) {
         const cudaError_t e =
             launch_t_transfer<T>(*G.plan, k + j, std::min(pos, n - j), slot + j, G.st);
@@ -494,7 +498,7 @@ lks_status run_steps(Group& G, int from_level, int to_level, bool with_obj, int 
         const bool kt = tape_seg >= 0 && tape_transfers(G);
         auto fn = [&](int& nl, bool direct) -> cudaError_t {
             lks_ctx* timed = direct && G.count == 1 && c0->timing_stride > 0 ? c0 : nullptr;
-            const int chunk = kt ? kRunSteps : group_chunk(G);
+            const int chunk = group_chunk(G, kt, false);
             for (int k0 = 1; k0 <= len; k0 += chunk) {
                 const int n = std::min(chunk, len - k0 + 1);
                 const int slot = kt ? toff + k0 : 0;
@@ -647,7 +651,7 @@ lks_status exec_adj(Group& G, int seg) {
     const bool kt = tape_transfers(G);
     auto fn = [&](int& nl, bool direct) -> cudaError_t {
         lks_ctx* timed = direct && G.count == 1 && c0->timing_stride > 0 ? c0 : nullptr;
-        const int chunk = group_chunk(G);
+        const int chunk = group_chunk(G, kt, true);
         for (int k1 = len; k1 >= 1; k1 -= chunk) {   // steps a + k1 down to a + k0
             const int n = std::min(chunk, k1), k0 = k1 - n + 1;
             cudaError_t e = cudaSuccess;
@@ -1039,6 +1043,39 @@ const double* design_gradient(lks_ctx* c, cudaStream_t st) {
     return c->gout;
 }
 
+// Bytes of so many slots for a box of boxN nodes and ncol design columns, T bytes a number.
+size_t tape_bytes(const TapeSlots& t, long long boxN, long long ncol, size_t T) {
+    return align256((size_t)t.k * boxN * 4 * T) + align256((size_t)t.e * boxN * T) +
+           align256((size_t)t.pos * ncol * 8) + align256((size_t)t.pos * ncol * 4 * T);
+}
+
+// The slots that fit p.bytes once the box is known (most boxes are a fraction of the grid, and the more
+// slots): the least transfers, positions from a quarter of the rest, then e for those transfers, both for
+// more steps, and transfers alone where e has all it can use.
+TapeSlots tape_slots(const TapePlan& p, long long boxN, long long ncol, size_t T) {
+    TapeSlots t;
+    t.k = p.least;
+    t.e = t.pos = 1;
+    const long long slack = 4 * 256, kb = boxN * 4 * (long long)T, eb = boxN * (long long)T,
+                    pb = ncol * (8 + 4 * (long long)T);
+    long long left = (long long)p.bytes - (t.k * kb + t.e * eb + t.pos * pb) - slack;
+    auto take = [&](int now, int most, long long each, long long room) -> int {
+        const long long n = std::max(0LL, std::min((long long)(most - now), room / each));
+        left -= n * each;
+        return (int)n;
+    };
+    t.pos += take(t.pos, std::min(p.want, kMaxPosSlots), pb, left / 4);
+    const int e = std::min(p.want, kMaxESlots);
+    t.e += take(t.e, std::min(e, t.k), eb, left);
+    if (t.e == t.k) {
+        const int n = take(t.k, e, kb + eb, left);
+        t.k += n;
+        t.e += n;
+    }
+    t.k += take(t.k, p.want, kb, left);
+    return t;
+}
+
 // After a new motion table: rows with cos/sin evaluated on the host go to the device (the
 // instance-table kernels read them there), and a table context rebuilds its one-entry plan.
 lks_status finish_motion(lks_ctx* c) {
@@ -1049,6 +1086,14 @@ lks_status finish_motion(lks_ctx* c) {
     CU(cudaStreamSynchronize(c->st));
     ++c->geo_gen;
     if (c->fused2d) {
+        if (c->d.nd > 0) {
+            const size_t T = c->tsz, box = (size_t)c->g.boxN, col = (size_t)c->d.ncol;
+            c->slots = tape_slots(c->tape, c->g.boxN, c->d.ncol, T);
+            c->ktape = c->tape_mem;
+            c->etape = c->tape_mem + align256(c->slots.k * box * 4 * T);
+            c->pos_b = (char*)c->etape + align256(c->slots.e * box * T);
+            c->pos_sc = (char*)c->pos_b + align256(c->slots.pos * col * 8);
+        }
         const lks_status s = own_plan(c);
         if (s != LKS_OK) return s;
     }

@@ -20,7 +20,7 @@ template <class T>
 struct Inst {
     Geom g;
     Design d;
-    int2* pos_b;              // design positions of up to pos_slots steps: integer base of
+    int2* pos_b;              // design positions of several steps: integer base of
     V4<T>* pos_sc;            // x_ref, y_ref and sin, cos of (pi f / 2) of their fractions
     const Motion* motion;     // rows 0..max_steps with cos/sin already evaluated (device)
     void* bufs[BUF_POOL];     // the buffers before the pool
