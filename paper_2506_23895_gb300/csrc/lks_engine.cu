@@ -164,7 +164,7 @@ struct Layout {
 };
 
 enum {
-    L_S0, L_S1, L_SINIT, L_L0, L_L1, L_F, L_MU, L_PHI, L_KUS, L_E, L_GAMMA, L_KREF, L_KPRIME,
+    L_S0, L_S1, L_SINIT, L_L0, L_L1, L_F, L_PHI, L_KUS, L_E, L_GAMMA, L_KREF, L_KPRIME,
     L_GACC, L_JSTEP, L_CBASE, L_ZTI, L_ZTW, L_TIDX, L_TW, L_CM, L_DZB, L_DZF,
     L_FLAGS, L_KREFT, L_K2, L_FACE, L_TGT, L_U3, L_MOTION, L_INST, L_PRE, L_GBAR,
     L_HP, L_FWS, L_GOUT, L_GTMP, L_FQ, L_SCAL, L_CSC, L_KS, L_SEND, L_LEND, L_GBASE, L_GFRAC,
@@ -190,8 +190,9 @@ Layout make_layout(const lks_config* cfg) {
     const size_t state = align256((size_t)nodes * 4 * T);
     size_t sz[L_COUNT] = {};
     sz[L_S0] = sz[L_S1] = sz[L_SINIT] = sz[L_L0] = sz[L_L1] = state;
-    sz[L_F] = (size_t)Q * nodes * T;
-    sz[L_MU] = state;
+    // f^eq of a forward step; mu of an adjoint step and the filter chain's scaled input live there too,
+    // each written and read within one step or call
+    sz[L_F] = std::max((size_t)(Q * nodes) * T, (size_t)nd * 8);
     sz[L_PHI] = (size_t)6 * nodes * T;
     sz[L_KUS] = nd ? state : 0;
     sz[L_E] = nd ? (size_t)nodes * T : 0;
@@ -227,7 +228,7 @@ Layout make_layout(const lks_config* cfg) {
     sz[L_MOTION] = (size_t)(cfg->max_steps + 1) * sizeof(Motion);
     sz[L_INST] = std::max(sizeof(Inst<float>), sizeof(Inst<double>));
     sz[L_PRE] = (size_t)U_COUNT * 2 * sizeof(int);
-    sz[L_GBAR] = sz[L_HP] = sz[L_FWS] = sz[L_GOUT] = sz[L_GTMP] = sz[L_FQ] = (size_t)std::max(nd, 1LL) * 8;
+    sz[L_GBAR] = sz[L_HP] = sz[L_FWS] = sz[L_GOUT] = sz[L_GTMP] = (size_t)std::max(nd, 1LL) * 8;
     sz[L_SCAL] = 64;
     sz[L_CSC] = (size_t)std::max(ncol, 1LL) * 4 * T;
     sz[L_KS] = (size_t)nodes * T;
@@ -272,6 +273,7 @@ Layout make_layout(const lks_config* cfg) {
                 spare += sz[r];
                 sz[r] = 0;
             }
+            sz[L_FQ] = (size_t)std::max(nd, 1LL) * 8;
             sz[L_JPART] = (size_t)(cfg->max_steps + 2) * obj_parts(count_target(cfg)) * 8;
             if (nd > 0) {
                 const long long kt = std::max((long long)std::ceil(std::sqrt((double)N)) + 2, 64LL);
@@ -390,7 +392,7 @@ lks_status lks_create(const lks_config* cfg, void* workspace, size_t ws_bytes, l
     c->lam[0] = w + L.off[L_L0];
     c->lam[1] = w + L.off[L_L1];
     c->F = w + L.off[L_F];
-    c->mu = w + L.off[L_MU];
+    c->mu = c->F;
     c->phi = w + L.off[L_PHI];
     c->kus = w + L.off[L_KUS];
     c->e = w + L.off[L_E];
@@ -444,7 +446,7 @@ lks_status lks_create(const lks_config* cfg, void* workspace, size_t ws_bytes, l
     c->fws = (double*)(w + L.off[L_FWS]);
     c->gout = (double*)(w + L.off[L_GOUT]);
     c->gtmp = (double*)(w + L.off[L_GTMP]);
-    c->fq = (double*)(w + L.off[L_FQ]);
+    c->fq = (double*)(c->fused2d ? w + L.off[L_FQ] : (char*)c->F);
     c->scal = (double*)(w + L.off[L_SCAL]);
     c->ks = w + L.off[L_KS];
     c->gaxis = general_axis(cfg) && c->d.nd > 0;

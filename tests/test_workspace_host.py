@@ -41,3 +41,17 @@ def test_2d_contexts_stay_within_their_snapshot_budget(lib, prec, n, steps, frac
         table = workspace(lib, p, prec, slots, 0)
         half = min(P * state // 2, 256 << 20)
         assert table <= plain + half + (1 + kept) * state + (64 << 10)
+
+
+@pytest.mark.parametrize("prec", [lks.FP32, lks.FP64])
+@pytest.mark.parametrize("n", [48, 96, 256])
+def test_3d_contexts_share_scratch_between_forward_and_adjoint(lib, prec, n):
+    """Seven states, the snapshots, f^eq of 15 directions, six components of S~ and the static field;
+    the adjoint's mu lives where f^eq does.  What is smaller than one number a node is left room for."""
+    p = W.small_duct3d(n_steps=20).problem
+    p.n = (n, n, n)
+    p.L = (0, 0, 0)
+    T = 8 if prec == lks.FP64 else 4
+    state = lks.state_bytes(p, prec)
+    for flags in (0, lks.FLAG_PLAIN_KERNELS):
+        assert workspace(lib, p, prec, 3, flags) <= (7 + 3) * state + (15 + 6 + 1 + 1) * n ** 3 * T
