@@ -86,10 +86,10 @@ typedef struct {
     size_t ckpt_bytes;       /* device bytes for adjoint snapshots; 0 = full history if it
                                 fits in 8 GB, else the minimum of a two-level scheme.  A 2D
                                 context with a design also keeps the transfers of many steps:
-                                in the room the plain kernels' scratch takes in other contexts,
-                                in half as much as the snapshots take but at most 256 MB, and in
-                                FP32 in a state per snapshot slot, up to
-                                max(ceil(sqrt(max_steps)) + 2, 64) */
+                                in the room the plain kernels' scratch takes in other contexts
+                                and, in FP32, a state per snapshot slot up to
+                                max(ceil(sqrt(max_steps)) + 2, 64), in FP64 half of what the
+                                snapshots take but at most 256 MB */
     void* stream;            /* cudaStream_t the work is ordered on; NULL = legacy default
                                 stream.  A 3D forward or adjoint run starts after the work
                                 already on it and is complete on it when the call returns: the

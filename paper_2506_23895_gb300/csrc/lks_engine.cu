@@ -258,11 +258,11 @@ Layout make_layout(const lks_config* cfg) {
     // 2D contexts on the table kernels form the transfers (kappa, u_S on the footprint box) of many
     // steps in one launch, keep those of a taped segment for its adjoint where they fit, and keep e of
     // many steps for the sensitivity gather.  Their memory is that of the plain kernels' scratch, which
-    // no table kernel uses, half of what the snapshots take but at most 256 MB, and in FP32 (16 bytes a
-    // node) a slot for each snapshot slot up to max(ceil(sqrt(N)) + 2, 64), a segment of the
-    // checkpointed schedules.  So ckpt_bytes bounds the whole; with fewer slots launches are shorter
-    // and a segment's transfers may be formed twice (512^2 FP64, 60 steps: 10.5 ms a gradient with 42
-    // of 61 slots, 8.4 with all).
+    // no table kernel uses, and beside it in FP32 (16 bytes a node) a slot for each snapshot slot up to
+    // max(ceil(sqrt(N)) + 2, 64), a segment of the checkpointed schedules, in FP64 half of what the
+    // snapshots take but at most 256 MB.  So ckpt_bytes bounds the whole; with fewer slots launches
+    // are shorter and a segment's transfers may be formed twice (512^2 FP64, 60 steps: 10.5 ms a
+    // gradient with 42 of 61 slots, 8.4 with all).
     {
         L.tape = TapePlan{};
         const bool table = dim == 2 && !(cfg->flags & (LKS_FLAG_PLAIN_KERNELS | LKS_FLAG_PAPER_ALKS));
@@ -282,11 +282,10 @@ Layout make_layout(const lks_config* cfg) {
                 const TapeSlots all{L.tape.want, std::min(L.tape.want, kMaxESlots),
                                     std::min(L.tape.want, kMaxPosSlots)};
                 spare -= std::min(spare, sz[L_JPART] + sz[L_FQ]);
-                L.tape.bytes = std::max(
-                    tape_bytes({L.tape.least, 1, 1}, nodes, ncol, T),
-                    std::min(tape_bytes(all, nodes, ncol, T),
-                             spare + std::min((size_t)P * state / 2, (size_t)256 << 20) +
-                                 (T == 4 ? (size_t)L.tape.least * state : 0)));
+                const size_t more = T == 4 ? (size_t)L.tape.least * state
+                                           : std::min((size_t)P * state / 2, (size_t)256 << 20);
+                L.tape.bytes = std::max(tape_bytes({L.tape.least, 1, 1}, nodes, ncol, T),
+                                        std::min(tape_bytes(all, nodes, ncol, T), spare + more));
                 sz[L_TAPE] = L.tape.bytes;
             }
         }
