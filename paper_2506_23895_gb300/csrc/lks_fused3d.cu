@@ -937,10 +937,7 @@ bool encode_state_map(CUtensorMap* map, const void* base, const Geom& g, int bx,
 // blocks per SM, weighing each chunk's three warm-up planes: the chunk count with the best
 // product of wave fill and useful-plane fraction, chunks of at least 8 planes (small grids need
 // many chunks to fill the SMs at all).
-int fused_zchunk_waves(const Geom& g, long long tiles, int per_sm) {
-    int dev = 0, nsm = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+int fused_zchunk_waves(const Geom& g, long long tiles, int per_sm, int nsm) {
     const long long slots = (long long)nsm * per_sm;
     const int maxc = std::max(1, g.n[2] / 8);
     int best = 1;
@@ -959,6 +956,34 @@ int fused_zchunk_waves(const Geom& g, long long tiles, int per_sm) {
     return (g.n[2] + best - 1) / best;
 }
 
+int device_sms() {
+    int dev = 0, nsm = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    return nsm;
+}
+
+// Is a forward step shorter as a row march (its tiles then in t) than as a z-march of 32 x 8 tiles?
+// The row march does a fifth less work per node, but its tiles are larger: it needs enough of them,
+// and loses where a part of the last ones lies outside the grid.  Both sides as fits to the step's time
+// in us on 60 grids of 0.03 to 19 M inner nodes (with k_bc_shell3d; residual 6 % and 5 %): the row march
+// by its cost, the z-march by its full waves, the blocks per SM of the last and one block's planes.
+// Measured, z-march and row march: 64 x 64 x 1000 67.9 and 87.2 us, 64 x 64 x 400 39.1 and 44.1, 160^3
+// 67.4 and 72.6, 151 x 83 x 117 37.4 and 33.8, 192^3 101 and 102, 256^3 201 and 178, 300 x 300 x 24 49.7
+// and 39.3.  Below 1.2 M inner nodes they differ by less than the fits' residual, either way.
+bool row_march_pays(const Geom& g, March3d& t) {
+    if ((g.n[0] - 2LL) * (g.n[1] - 2) * (g.n[2] - 2) < 1200000) return false;
+    t = step_march_tiles(g);
+    using C = ZCfg<8>;
+    const int nsm = device_sms();
+    const long long tiles = (long long)((g.n[0] + C::TX - 1) / C::TX) * ((g.n[1] + C::TY - 1) / C::TY);
+    const int zc = fused_zchunk_waves(g, tiles, C::MINB, nsm);
+    const long long blocks = tiles * ((g.n[2] + zc - 1) / zc), slots = (long long)nsm * C::MINB;
+    const double last = (double)((blocks % slots + nsm - 1) / nsm);
+    const double z = 15.6 + (1.09 * (double)(blocks / slots) + 0.318 * last + 0.307) * (zc + 3);
+    return 0.0382 * t.cost - 2.2 < z;
+}
+
 template <int TY_>
 cudaError_t launch_zstep(const Geom& g, const CUtensorMap& map, const FusedArgs& a0,
                          cudaStream_t st) {
@@ -973,18 +998,15 @@ cudaError_t launch_zstep(const Geom& g, const CUtensorMap& map, const FusedArgs&
     }
     FusedArgs a = a0;
     const int tiles_x = (g.n[0] + C::TX - 1) / C::TX, tiles_y = (g.n[1] + C::TY - 1) / C::TY;
-    a.zchunk = fused_zchunk_waves(g, (long long)tiles_x * tiles_y, C::MINB);
+    a.zchunk = fused_zchunk_waves(g, (long long)tiles_x * tiles_y, C::MINB, device_sms());
     const int chunks = (g.n[2] + a.zchunk - 1) / a.zchunk;
     k_zstep3d<TY_><<<dim3(tiles_x, tiles_y, chunks), C::NTHR, C::SMEM, st>>>(map, a);
     return cudaGetLastError();
 }
 
 // One fused forward step src -> dst in variant v (0: shared-memory z-march with two barriers per
-// plane, 1: z-march by size, 2: the row march of lks_march3d.cu).  The row march does a fifth less
-// work per node, but its blocks are larger and take longer to start, so it needs enough of them:
-// per step 96 x 90 x 101 37.9 us against 34.4 on 32 x 8 tiles, 151 x 83 x 117 36.1 against 38.6,
-// 128^3 48.5 against 51.2, 256^3 198 against 216 (with k_bc_shell3d).  The line lies between the
-// first two.  Returns a CUDA error code.
+// plane, 1: the row march of lks_march3d.cu or the z-march, by the grid's tiles, 2: the row march).
+// Returns a CUDA error code.
 cudaError_t launch_fused_step3d(const Geom& g, const V4<float>* src, const V4<float>* kus,
                                 V4<float>* dst, int* err, cudaStream_t st, int v) {
     FusedArgs a;
@@ -1000,10 +1022,11 @@ cudaError_t launch_fused_step3d(const Geom& g, const V4<float>* src, const V4<fl
     for (int k = 0; k < 3; ++k) a.bf[k] = (float)g.body[k];
     CUtensorMap map;
     if (v == 1 || v == 2) {
-        const long long inner = (g.n[0] - 2LL) * (g.n[1] - 2) * (g.n[2] - 2);
+        March3d t;
+        if (v == 2) t = step_march_tiles(g);
         cudaError_t e;
-        if (v == 2 || inner >= 1200000) {
-            e = launch_step_march(g, src, kus, dst, err, st, 0);
+        if (v == 2 || row_march_pays(g, t)) {
+            e = launch_step_march(g, src, kus, dst, err, st, t);
         } else {
             if (!encode_state_map(&map, src, g, ZCfg<8>::HX, ZCfg<8>::HY))
                 return cudaErrorInvalidValue;
@@ -1031,7 +1054,7 @@ cudaError_t launch_fused_step3d(const Geom& g, const V4<float>* src, const V4<fl
         device_mark(attr);
     }
     const int tiles_x = (g.n[0] + TX - 1) / TX, tiles_y = (g.n[1] + TY - 1) / TY;
-    a.zchunk = fused_zchunk_waves(g, (long long)tiles_x * tiles_y, 4);
+    a.zchunk = fused_zchunk_waves(g, (long long)tiles_x * tiles_y, 4, device_sms());
     const int chunks = (g.n[2] + a.zchunk - 1) / a.zchunk;
     dim3 grid(tiles_x, tiles_y, chunks);
     k_fused_step3d<<<grid, NTHR, SMEM_BYTES, st>>>(map, a);

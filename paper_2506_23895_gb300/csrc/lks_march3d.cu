@@ -378,15 +378,20 @@ March3d march_tiles(const MarchCost& m, int out_x, int out_y, int nz, int warps)
                                 (zc + m.start + 8.0 / per_sm);
             if (cost < best_cost * (1.0 - 1e-9)) {
                 best_cost = cost;
-                best = March3d{w, (int)tx, (int)ty, zc, (int)chunks};
+                best = March3d{w, (int)tx, (int)ty, zc, (int)chunks, cost};
             }
         }
     }
     return best;
 }
 
+March3d step_march_tiles(const Geom& g) {
+    return march_tiles(MarchCost{kOutX, R, 2, kMaxWarps, 2 * kMaxWarps, 27.0, 33.0, 1.0}, g.n[0] - 2,
+                       g.n[1] - 2, g.n[2] - 2, 0);
+}
+
 cudaError_t launch_step_march(const Geom& g, const V4<float>* src, const V4<float>* kus,
-                              V4<float>* dst, int* err, cudaStream_t st, int warps) {
+                              V4<float>* dst, int* err, cudaStream_t st, const March3d& t) {
     Args a;
     for (int k = 0; k < 3; ++k) {
         a.n[k] = g.n[k];
@@ -399,8 +404,6 @@ cudaError_t launch_step_march(const Geom& g, const V4<float>* src, const V4<floa
     a.out = reinterpret_cast<float4*>(dst);
     a.err = err;
     a.A = (float)g.A;
-    const March3d t = march_tiles(MarchCost{kOutX, R, 2, kMaxWarps, 2 * kMaxWarps, 27.0, 33.0, 1.0},
-                                  g.n[0] - 2, g.n[1] - 2, g.n[2] - 2, warps);
     a.zchunk = t.zchunk;
     auto smem_of = [](int w) {
         const size_t plane = ((size_t)(R * w + 2) * RX * 16 + 127) / 128 * 128;

@@ -9,6 +9,7 @@ struct March3d {
     int warps;                // per block, R rows each
     int tiles_x, tiles_y;
     int zchunk, chunks;
+    double cost;              // in the units of MarchCost: comparable for one kernel
 };
 
 // What a kernel's tiles look like and what its blocks cost.
@@ -29,9 +30,10 @@ struct MarchCost {
 // differ by up to a third).
 March3d march_tiles(const MarchCost& m, int out_x, int out_y, int nz, int warps);
 
-// The interior nodes of one forward step; warps > 0 fixes the block height.
+// Tiles of the forward march, and the interior nodes of one forward step on them.
+March3d step_march_tiles(const Geom& g);
 cudaError_t launch_step_march(const Geom& g, const V4<float>* src, const V4<float>* kus,
-                              V4<float>* dst, int* err, cudaStream_t st, int warps);
+                              V4<float>* dst, int* err, cudaStream_t st, const March3d& t);
 // lambda^{n-1} from lambda^n (after k_adj_prep) but for the one-sided boundary rows, whose 2 A S~ go
 // to face; warps > 0 fixes the block height.
 cudaError_t launch_adj_march(const Geom& g, const V4<float>* lam_in, V4<float>* lam_out,
