@@ -14,8 +14,9 @@ namespace {
 // One-sided parts of the transposed gradient on non-periodic axes: node z within two rows of
 // a face gets delta * (2 A S~_{.beta}) of the face node it projects to, with delta = -3/2,
 // +3/2, -1/2 at rows 0, 1, 2 (low face) and +3/2, -3/2, +1/2 at rows n-1, n-2, n-3 (high face):
-// the exact one-sided stencil minus the central one the fused kernel applied.
-__global__ void k_adj_bcorr(Geom g, const float* __restrict__ face, FaceOffsets fo,
+// the exact one-sided stencil minus the central one the fused kernel applied.  On the low x face, and
+// on the high one if hi_own, that kernel took the face's own value for the one beyond it, 1/2 of it.
+__global__ void k_adj_bcorr(Geom g, const float* __restrict__ face, FaceOffsets fo, bool hi_own,
                             float4* __restrict__ lam) {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     // enumerate slabs of thickness 3 next to each face; a node near several faces is owned by
@@ -48,7 +49,9 @@ __global__ void k_adj_bcorr(Geom g, const float* __restrict__ face, FaceOffsets 
         const int d = (f & 1) ? g.n[a] - 1 - c[a] : c[a];
         if (d > 2) continue;
         const float lo[3] = {-1.5f, 1.5f, -0.5f};
-        const float delta = (f & 1) ? -lo[d] : lo[d];
+        float delta = (f & 1) ? -lo[d] : lo[d];
+        if (f == 0 && d == 0) delta -= 0.5f;
+        if (f == 1 && d == 0 && hi_own) delta += 0.5f;
         const int e0 = (a == 0) ? 1 : 0, e1 = (a == 2) ? 1 : 2;
         const float* fp = face + fo.off[f] + 3 * ((long long)c[e1] * g.n[e0] + c[e0]);
         sx += delta * fp[0];
@@ -90,8 +93,8 @@ cudaError_t launch_fused_adj3d(const Geom& g, V4<float>* lam_in, V4<float>* lam_
     face_offsets(g, fo, tot);
     const long long shell = 6LL * ((long long)g.n[1] * g.n[2] + (long long)g.n[0] * g.n[2] +
                                    (long long)g.n[0] * g.n[1]);
-    k_adj_bcorr<<<(unsigned)((shell + 255) / 256), 256, 0, st>>>(g, face, fo,
-                                                                reinterpret_cast<float4*>(lam_out));
+    k_adj_bcorr<<<(unsigned)((shell + 255) / 256), 256, 0, st>>>(
+        g, face, fo, adj_face_in_last_lane(g), reinterpret_cast<float4*>(lam_out));
     return cudaGetLastError();
 }
 

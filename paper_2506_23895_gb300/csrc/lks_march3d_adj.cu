@@ -44,7 +44,6 @@ constexpr int NSLOT = 3;          // lambda planes in the ring
 constexpr int NUSLOT = 2;         // planes of u^{n-1}
 constexpr int kSeam = 8;          // values a column publishes at a seam: 5 of F~, 3 of S~
 constexpr int kMaxWarps = 7;      // two such blocks per SM at 128 registers
-constexpr int kOutX = 28;         // output columns of a tile
 
 struct Args {
     int n[3];
@@ -106,7 +105,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 2)
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)(NSLOT + NUSLOT) * plane_bytes +
                                                  (size_t)2 * seam_buf * 4);
     uint64_t* ubars = bars + NSLOT;
-    const int x0 = blockIdx.x * kOutX, y0 = blockIdx.y * (rows - 4);
+    const int x0 = blockIdx.x * kAdjTileX + 2, y0 = blockIdx.y * (rows - 4);
     const int q0 = blockIdx.z * a.zchunk, q1 = min(nz, q0 + a.zchunk);
     const int nplanes = q1 - q0 + 4;   // lambda planes q0 - 2 .. q1 + 1
     const bool leader = lane == 0 && wid == 0;
@@ -127,7 +126,12 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 2)
     __syncthreads();
 
     const int x = x0 - 2 + lane, yr = y0 - 2 + R * wid;   // column, first row
-    const bool xown = lane >= 2 && lane < 2 + kOutX && x < nx;
+    // The first and the last tile also own the halo columns on their face's side: nothing comes in from
+    // beyond a face, where a shuffle returns the lane's own value, which is zero for mu on a face.  (A
+    // face column in lane 0 or 31 also takes its own 9 S~ for its neighbour's; k_adj_bcorr's one-sided
+    // part takes it out.)
+    const bool xown = x < nx && (lane >= 2 || blockIdx.x == 0) &&
+                      (lane < 30 || blockIdx.x == gridDim.x - 1);
     int fl = 0;   // bits r: interior in x and y, OWN + r: an output row
     constexpr int OWN = 4;
 #pragma unroll
@@ -413,8 +417,8 @@ cudaError_t launch_adj_march(const Geom& g, const V4<float>* lam_in, V4<float>* 
     for (int f = 0; f < 6; ++f) a.face_off[f] = fo.off[f];
     a.err = err;
     a.A9 = (float)(g.A / 9.0);
-    const March3d t = march_tiles(MarchCost{kOutX, R, 4, kMaxWarps, 2 * kMaxWarps, 11.0, 50.0, 13.0},
-                                  g.n[0], g.n[1], g.n[2], warps);
+    const March3d t = march_tiles(MarchCost{kAdjTileX, R, 4, kMaxWarps, 2 * kMaxWarps, 11.0, 50.0, 13.0},
+                                  std::max(g.n[0] - 4, 1), g.n[1], g.n[2], warps);
     a.zchunk = t.zchunk;
     const size_t per_warp = (NSLOT + NUSLOT) * 512 * R + 2 * 2 * kSeam * 32 * 4;
     const size_t bars = (NSLOT + NUSLOT) * 8, smem = per_warp * t.warps + bars;
