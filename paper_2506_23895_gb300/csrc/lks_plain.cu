@@ -10,7 +10,7 @@
 // variant), k_adj_moments gathers F~_i(y) = mu_rho(y+c_i) + c_i.mu_u(y+c_i)
 // into the moments of Eqs. arho, au, as and the adjoint equilibrium, k_adj_divT adds the
 // transposed velocity-gradient term.  These kernels are templated on the scalar type; the
-// double instantiation is the plain FP64 path.
+// double instantiation is the 3D FP64 path.
 #include "lks_units.cuh"
 
 namespace lks {

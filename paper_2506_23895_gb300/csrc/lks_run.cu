@@ -365,7 +365,7 @@ int seg_end(const lks_ctx* c, int a) { return std::min((a + 1) * c->K, c->n_fwd)
 // ---------------------------------------------------------------- groups of contexts
 // A group runs one checkpoint schedule for contexts of identical step count and snapshot pool:
 // the single-context calls use a group of one, lks_batch_* a group over all its contexts.  On
-// the instance-table path (D2Q9 FP32) every phase of a step is one launch over the whole group,
+// the instance-table path (D2Q9) every phase of a step is one launch over the whole group,
 // and a run of steps can be captured once into a CUDA graph and replayed.
 
 

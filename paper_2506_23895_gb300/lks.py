@@ -345,7 +345,8 @@ class Solver:
 
     @property
     def kernels(self) -> str:
-        """'fused3d', 'fused2d' or 'plain': which kernels run this context's steps."""
+        """'fused3d' or 'fused2d' for the FP32 kernels, else 'plain': the per-node kernels, or in 2D
+        FP64 the strip kernels of 'fused2d' in double."""
         return {1: "fused3d", 2: "fused2d"}.get(self.lib.lks_uses_fused(self.ctx), "plain")
 
     def step_variant(self, request: int = -2) -> int:
@@ -362,6 +363,7 @@ class Solver:
         return v.value
 
     def set_timing(self, stride: int) -> None:
+        """Time every stride-th step (0: off); a 2D run then launches each step by itself."""
         self._check(self.lib.lks_set_timing(self.ctx, stride))
 
     def read_timing(self):

@@ -1,7 +1,7 @@
-"""The 3D FP32 row marches at the widths where their tiles change: 28 columns and the halo at the
-faces in the adjoint (32 | 33, 60 | 61, 88 | 89 nodes), 30 inner columns in the forward step, against the 64-bit oracle; and grids on
-which the default forward step takes one march or the other, against the row march.  Nine FP32 steps of
-about 30 roundings of 6e-8 stay below 2e-5 of the largest state, four times that on the gradient."""
+"""The 3D FP32 row marches at the widths where their tiles change: 28 columns and the halo at the faces in
+the adjoint (32 | 33, 60 | 61, 88 | 89 nodes), 30 inner columns in the forward step, against the 64-bit
+oracle.  Nine FP32 steps of about 30 roundings of 6e-8 stay below 2e-5 of the largest state, four times
+that on the gradient."""
 import numpy as np
 import pytest
 
