@@ -430,6 +430,7 @@ lks_status lks_create(const lks_config* cfg, void* workspace, size_t ws_bytes, l
     c->fused3d = (c->prec == LKS_FP32) &&
                  !(cfg->flags & (LKS_FLAG_PLAIN_KERNELS | LKS_FLAG_PAPER_ALKS)) &&
                  fused3d_eligible(g);
+    if (c->fused3d) c->plan3d = plan_step3d(g);
     c->pool = w + L.off[L_POOL];
     c->pool_slots = L.pool_slots;
     c->snap_bytes = L.snap;

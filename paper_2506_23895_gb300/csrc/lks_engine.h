@@ -115,6 +115,7 @@ struct lks_ctx {
     long long stats[5] = {0, 0, 0, 0, 0};
     const void* last = nullptr;  // buffer holding the newest forward level
     bool fused3d = false;        // FP32 3D non-periodic: one fused kernel per forward step
+    Step3dPlan plan3d{};
     // instance table of this context (D2Q9: the table kernels of lks_fused2d.cu)
     bool fused2d = false;
     Motion* dmotion = nullptr;   // device motion rows

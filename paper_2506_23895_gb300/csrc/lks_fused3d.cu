@@ -963,7 +963,7 @@ int device_sms() {
     return nsm;
 }
 
-// Is a forward step shorter as a row march (its tiles then in t) than as a z-march of 32 x 8 tiles?
+// Is a forward step shorter as a row march (rows) than as a z-march of 32 x 8 tiles?
 // The row march does a fifth less work per node, but its tiles are larger: it needs enough of them,
 // and loses where a part of the last ones lies outside the grid.  Both sides as fits to the step's time
 // in us on 60 grids of 0.03 to 19 M inner nodes (with k_bc_shell3d; residual 6 % and 5 %): the row march
@@ -971,21 +971,25 @@ int device_sms() {
 // Measured, z-march and row march: 64 x 64 x 1000 67.9 and 87.2 us, 64 x 64 x 400 39.1 and 44.1, 160^3
 // 67.4 and 72.6, 151 x 83 x 117 37.4 and 33.8, 192^3 101 and 102, 256^3 201 and 178, 300 x 300 x 24 49.7
 // and 39.3.  Below 1.2 M inner nodes they differ by less than the fits' residual, either way.
-bool row_march_pays(const Geom& g, March3d& t) {
-    if ((g.n[0] - 2LL) * (g.n[1] - 2) * (g.n[2] - 2) < 1200000) return false;
-    t = step_march_tiles(g);
+Step3dPlan plan_step3d(const Geom& g) {
+    Step3dPlan p;
     using C = ZCfg<8>;
     const int nsm = device_sms();
     const long long tiles = (long long)((g.n[0] + C::TX - 1) / C::TX) * ((g.n[1] + C::TY - 1) / C::TY);
-    const int zc = fused_zchunk_waves(g, tiles, C::MINB, nsm);
-    const long long blocks = tiles * ((g.n[2] + zc - 1) / zc), slots = (long long)nsm * C::MINB;
+    p.zchunk = fused_zchunk_waves(g, tiles, C::MINB, nsm);
+    p.tiles = step_march_tiles(g);
+    const long long blocks = tiles * ((g.n[2] + p.zchunk - 1) / p.zchunk);
+    const long long slots = (long long)nsm * C::MINB;
     const double last = (double)((blocks % slots + nsm - 1) / nsm);
-    const double z = 15.6 + (1.09 * (double)(blocks / slots) + 0.318 * last + 0.307) * (zc + 3);
-    return 0.0382 * t.cost - 2.2 < z;
+    const double z =
+        15.6 + (1.09 * (double)(blocks / slots) + 0.318 * last + 0.307) * (p.zchunk + 3);
+    p.rows = (g.n[0] - 2LL) * (g.n[1] - 2) * (g.n[2] - 2) >= 1200000 &&
+             0.0382 * p.tiles.cost - 2.2 < z;
+    return p;
 }
 
 template <int TY_>
-cudaError_t launch_zstep(const Geom& g, const CUtensorMap& map, const FusedArgs& a0,
+cudaError_t launch_zstep(const Geom& g, const CUtensorMap& map, const FusedArgs& a0, int zchunk,
                          cudaStream_t st) {
     using C = ZCfg<TY_>;
     static std::atomic<unsigned> attr{0};   // devices whose shared-memory limit is raised
@@ -998,7 +1002,7 @@ cudaError_t launch_zstep(const Geom& g, const CUtensorMap& map, const FusedArgs&
     }
     FusedArgs a = a0;
     const int tiles_x = (g.n[0] + C::TX - 1) / C::TX, tiles_y = (g.n[1] + C::TY - 1) / C::TY;
-    a.zchunk = fused_zchunk_waves(g, (long long)tiles_x * tiles_y, C::MINB, device_sms());
+    a.zchunk = zchunk;
     const int chunks = (g.n[2] + a.zchunk - 1) / a.zchunk;
     k_zstep3d<TY_><<<dim3(tiles_x, tiles_y, chunks), C::NTHR, C::SMEM, st>>>(map, a);
     return cudaGetLastError();
@@ -1007,8 +1011,9 @@ cudaError_t launch_zstep(const Geom& g, const CUtensorMap& map, const FusedArgs&
 // One fused forward step src -> dst in variant v (0: shared-memory z-march with two barriers per
 // plane, 1: the row march of lks_march3d.cu or the z-march, by the grid's tiles, 2: the row march).
 // Returns a CUDA error code.
-cudaError_t launch_fused_step3d(const Geom& g, const V4<float>* src, const V4<float>* kus,
-                                V4<float>* dst, int* err, cudaStream_t st, int v) {
+cudaError_t launch_fused_step3d(const Geom& g, const Step3dPlan& plan, const V4<float>* src,
+                                const V4<float>* kus, V4<float>* dst, int* err, cudaStream_t st,
+                                int v) {
     FusedArgs a;
     a.g = g;
     a.out = reinterpret_cast<float4*>(dst);
@@ -1022,15 +1027,13 @@ cudaError_t launch_fused_step3d(const Geom& g, const V4<float>* src, const V4<fl
     for (int k = 0; k < 3; ++k) a.bf[k] = (float)g.body[k];
     CUtensorMap map;
     if (v == 1 || v == 2) {
-        March3d t;
-        if (v == 2) t = step_march_tiles(g);
         cudaError_t e;
-        if (v == 2 || row_march_pays(g, t)) {
-            e = launch_step_march(g, src, kus, dst, err, st, t);
+        if (v == 2 || plan.rows) {
+            e = launch_step_march(g, src, kus, dst, err, st, plan.tiles);
         } else {
             if (!encode_state_map(&map, src, g, ZCfg<8>::HX, ZCfg<8>::HY))
                 return cudaErrorInvalidValue;
-            e = launch_zstep<8>(g, map, a, st);
+            e = launch_zstep<8>(g, map, a, plan.zchunk, st);
         }
         if (e != cudaSuccess) return e;
         ShellFaces F;

@@ -142,10 +142,25 @@ struct FaceOffsets {
     long long off[6];
 };
 bool fused3d_eligible(const Geom& g);
-int fused_zchunk_waves(const Geom& g, long long tiles, int per_sm);
+// Tiling of a row march (lks_march3d.h).
+struct March3d {
+    int warps;                // per block, R rows each
+    int tiles_x, tiles_y;
+    int zchunk, chunks;
+    double cost;              // in the units of MarchCost: comparable for one kernel
+};
+// How a grid's forward steps run: the row march's tiles, and does variant 1 take it (else the z-march,
+// in chunks of zchunk planes)?  Fixed by the grid and the device: formed once per context.
+struct Step3dPlan {
+    March3d tiles;
+    int zchunk;
+    bool rows;
+};
+Step3dPlan plan_step3d(const Geom& g);
 constexpr int kStep3dVariants = 3;
-cudaError_t launch_fused_step3d(const Geom& g, const V4<float>* src, const V4<float>* kus,
-                                V4<float>* dst, int* err, cudaStream_t st, int variant);
+cudaError_t launch_fused_step3d(const Geom& g, const Step3dPlan& plan, const V4<float>* src,
+                                const V4<float>* kus, V4<float>* dst, int* err, cudaStream_t st,
+                                int variant);
 // Offsets of the six face arrays (3 floats per face node) and their total length.
 void face_offsets(const Geom& g, FaceOffsets& fo, long long& total);
 // lam_in is read and modified (the adjoint of a step's last part is applied in place).  variant 0:

@@ -5,13 +5,6 @@
 
 namespace lks {
 
-struct March3d {
-    int warps;                // per block, R rows each
-    int tiles_x, tiles_y;
-    int zchunk, chunks;
-    double cost;              // in the units of MarchCost: comparable for one kernel
-};
-
 // What a kernel's tiles look like and what its blocks cost.
 struct MarchCost {
     int tile_x;               // output columns of a tile

@@ -243,8 +243,9 @@ lks_status choose_step3d(lks_ctx* c, const void* src, void* dst) {
         for (int r = 0; r < 4 && err == cudaSuccess; ++r) {
             if (r == 1) err = cudaEventRecord(e0, c->st);
             if (err == cudaSuccess)
-                err = launch_fused_step3d(c->g, (const V4<float>*)src, (const V4<float>*)c->kus,
-                                          (V4<float>*)dst, c->flags + 3, c->st, v);
+                err = launch_fused_step3d(c->g, c->plan3d, (const V4<float>*)src,
+                                          (const V4<float>*)c->kus, (V4<float>*)dst, c->flags + 3,
+                                          c->st, v);
         }
         if (err == cudaSuccess) err = cudaEventRecord(e1, c->st);
         if (err == cudaSuccess) err = cudaEventSynchronize(e1);
@@ -274,8 +275,9 @@ lks_status forward_step(lks_ctx* c, int n, const void* src, void* dst) {
             s = choose_step3d(c, src, dst);
             if (s != LKS_OK) return s;
         }
-        cudaError_t e = launch_fused_step3d(c->g, (const V4<float>*)src, (const V4<float>*)c->kus,
-                                            (V4<float>*)dst, c->flags + 3, c->st, c->step3d_var);
+        cudaError_t e = launch_fused_step3d(c->g, c->plan3d, (const V4<float>*)src,
+                                            (const V4<float>*)c->kus, (V4<float>*)dst,
+                                            c->flags + 3, c->st, c->step3d_var);
         if (e != cudaSuccess) return fail(c, LKS_ERR_CUDA, "fused step: %s", cudaGetErrorString(e));
         ++c->stats[4];
     } else {
