@@ -15,9 +15,10 @@ namespace {
 // a face gets delta * (2 A S~_{.beta}) of the face node it projects to, with delta = -3/2,
 // +3/2, -1/2 at rows 0, 1, 2 (low face) and +3/2, -3/2, +1/2 at rows n-1, n-2, n-3 (high face):
 // the exact one-sided stencil minus the central one the fused kernel applied.  On the low x face, and
-// on the high one if hi_own, that kernel took the face's own value for the one beyond it, 1/2 of it.
-__global__ void k_adj_bcorr(Geom g, const float* __restrict__ face, FaceOffsets fo, bool hi_own,
-                            float4* __restrict__ lam) {
+// on the high one where the last tile's last lane holds it, that kernel took the face's own value for the
+// one beyond it, 1/2 of it: x_lo, x_hi are delta at row 0 of the x faces.
+__global__ void k_adj_bcorr(Geom g, const float* __restrict__ face, FaceOffsets fo, float x_lo,
+                            float x_hi, float4* __restrict__ lam) {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     // enumerate slabs of thickness 3 next to each face; a node near several faces is owned by
     // the first slab containing it
@@ -48,10 +49,9 @@ __global__ void k_adj_bcorr(Geom g, const float* __restrict__ face, FaceOffsets 
         const int a = f / 2;
         const int d = (f & 1) ? g.n[a] - 1 - c[a] : c[a];
         if (d > 2) continue;
-        const float lo[3] = {-1.5f, 1.5f, -0.5f};
-        float delta = (f & 1) ? -lo[d] : lo[d];
-        if (f == 0 && d == 0) delta -= 0.5f;
-        if (f == 1 && d == 0 && hi_own) delta += 0.5f;
+        const float row0 = f == 0 ? x_lo : (f == 1 ? x_hi : ((f & 1) ? 1.5f : -1.5f));
+        const float s = (f & 1) ? -1.f : 1.f;
+        const float delta = d == 0 ? row0 : (d == 1 ? 1.5f * s : -0.5f * s);
         const int e0 = (a == 0) ? 1 : 0, e1 = (a == 2) ? 1 : 2;
         const float* fp = face + fo.off[f] + 3 * ((long long)c[e1] * g.n[e0] + c[e0]);
         sx += delta * fp[0];
@@ -94,7 +94,7 @@ cudaError_t launch_fused_adj3d(const Geom& g, V4<float>* lam_in, V4<float>* lam_
     const long long shell = 6LL * ((long long)g.n[1] * g.n[2] + (long long)g.n[0] * g.n[2] +
                                    (long long)g.n[0] * g.n[1]);
     k_adj_bcorr<<<(unsigned)((shell + 255) / 256), 256, 0, st>>>(
-        g, face, fo, adj_face_in_last_lane(g), reinterpret_cast<float4*>(lam_out));
+        g, face, fo, -2.f, adj_face_in_last_lane(g) ? 2.f : 1.5f, reinterpret_cast<float4*>(lam_out));
     return cudaGetLastError();
 }
 
