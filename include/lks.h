@@ -90,7 +90,7 @@ typedef struct {
                                 in the room the plain kernels' scratch takes in other contexts
                                 and, in FP32, a state per snapshot slot up to
                                 max(ceil(sqrt(max_steps)) + 2, 64), in FP64 half of what the
-                                snapshots take but at most 256 MB */
+                                snapshots take but at most 512 MB */
     void* stream;            /* cudaStream_t the work is ordered on; NULL = legacy default
                                 stream.  A 3D forward or adjoint run starts after the work
                                 already on it and is complete on it when the call returns: the

@@ -260,9 +260,10 @@ Layout make_layout(const lks_config* cfg) {
     // many steps for the sensitivity gather.  Their memory is that of the plain kernels' scratch, which
     // no table kernel uses, and beside it in FP32 (16 bytes a node) a slot for each snapshot slot up to
     // max(ceil(sqrt(N)) + 2, 64), a segment of the checkpointed schedules, in FP64 half of what the
-    // snapshots take but at most 256 MB.  So ckpt_bytes bounds the whole; with fewer slots launches
-    // are shorter and a segment's transfers may be formed twice (512^2 FP64, 60 steps: 10.5 ms a
-    // gradient with 42 of 61 slots, 8.4 with all).
+    // snapshots take but at most 512 MB (512^2 over 20,000 steps takes 400).  So ckpt_bytes bounds the
+    // whole; with fewer slots launches are shorter and a segment's transfers may be formed twice (512^2
+    // FP64: 60 steps 10.5 ms a gradient with 42 of 61 slots, 8.4 with all; 20,000 steps 4.43 s with 109
+    // of 144 and 3.92).
     {
         L.tape = TapePlan{};
         const bool table = dim == 2 && !(cfg->flags & (LKS_FLAG_PLAIN_KERNELS | LKS_FLAG_PAPER_ALKS));
@@ -279,11 +280,10 @@ Layout make_layout(const lks_config* cfg) {
                 const long long kt = std::max((long long)std::ceil(std::sqrt((double)N)) + 2, 64LL);
                 L.tape.want = (int)std::min(N + 1, std::max(std::min(P, kt), 16LL));
                 L.tape.least = T == 4 ? (int)std::min(P, kt) : 1;
-                const TapeSlots all{L.tape.want, std::min(L.tape.want, kMaxESlots),
-                                    std::min(L.tape.want, kMaxPosSlots)};
+                const TapeSlots all{L.tape.want, L.tape.want, std::min(L.tape.want, kMaxPosSlots)};
                 spare -= std::min(spare, sz[L_JPART] + sz[L_FQ]);
                 const size_t more = T == 4 ? (size_t)L.tape.least * state
-                                           : std::min((size_t)P * state / 2, (size_t)256 << 20);
+                                           : std::min((size_t)P * state / 2, (size_t)512 << 20);
                 L.tape.bytes = std::max(tape_bytes({L.tape.least, 1, 1}, nodes, ncol, T),
                                         std::min(tape_bytes(all, nodes, ncol, T), spare + more));
                 sz[L_TAPE] = L.tape.bytes;

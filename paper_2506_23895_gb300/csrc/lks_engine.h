@@ -47,8 +47,8 @@ struct TapePlan {
     size_t bytes = 0;
     int want = 0, least = 0;
 };
-// e and positions of so many steps fill a launch; more would only take memory from the transfers.
-constexpr int kMaxESlots = 64, kMaxPosSlots = 32;
+// Positions of so many steps fill a launch; more would only take memory from the transfers.
+constexpr int kMaxPosSlots = 32;
 
 }  // namespace eng
 }  // namespace lks

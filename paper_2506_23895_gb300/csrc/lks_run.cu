@@ -1052,8 +1052,8 @@ size_t tape_bytes(const TapeSlots& t, long long boxN, long long ncol, size_t T) 
 }
 
 // The slots that fit p.bytes once the box is known (most boxes are a fraction of the grid, and the more
-// slots): the least transfers, positions from a quarter of the rest, then e for those transfers, both for
-// more steps, and transfers alone where e has all it can use.
+// slots): the least transfers, positions from a quarter of the rest, then e for those transfers, and both
+// for more steps.
 TapeSlots tape_slots(const TapePlan& p, long long boxN, long long ncol, size_t T) {
     TapeSlots t;
     t.k = p.least;
@@ -1067,14 +1067,10 @@ TapeSlots tape_slots(const TapePlan& p, long long boxN, long long ncol, size_t T
         return (int)n;
     };
     t.pos += take(t.pos, std::min(p.want, kMaxPosSlots), pb, left / 4);
-    const int e = std::min(p.want, kMaxESlots);
-    t.e += take(t.e, std::min(e, t.k), eb, left);
-    if (t.e == t.k) {
-        const int n = take(t.k, e, kb + eb, left);
-        t.k += n;
-        t.e += n;
-    }
-    t.k += take(t.k, p.want, kb, left);
+    t.e += take(t.e, t.k, eb, left);
+    const int n = take(t.k, p.want, kb + eb, left);
+    t.k += n;
+    t.e += n;
     return t;
 }
 

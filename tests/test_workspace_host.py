@@ -1,6 +1,6 @@
 """Device memory of 2D contexts (host only, no GPU): a context on the table kernels takes no more than one
 on the plain kernels with the same snapshots, but for a state and, in FP32, a transfer slot for each
-snapshot slot up to max(ceil(sqrt(N)) + 2, 64), in FP64 half of what the snapshots take (256 MB at most);
+snapshot slot up to max(ceil(sqrt(N)) + 2, 64), in FP64 half of what the snapshots take (512 MB at most);
 so ckpt_bytes bounds the whole."""
 import ctypes
 import math
@@ -39,7 +39,7 @@ def test_2d_contexts_stay_within_their_snapshot_budget(lib, prec, n, steps, frac
         kept = min(P, max(math.ceil(math.sqrt(steps)) + 2, 64)) if prec == lks.FP32 else 0
         plain = workspace(lib, p, prec, slots, lks.FLAG_PLAIN_KERNELS)
         table = workspace(lib, p, prec, slots, 0)
-        half = min(P * state // 2, 256 << 20) if prec == lks.FP64 else 0
+        half = min(P * state // 2, 512 << 20) if prec == lks.FP64 else 0
         assert table <= plain + half + (1 + kept) * state + (64 << 10)
 
 
