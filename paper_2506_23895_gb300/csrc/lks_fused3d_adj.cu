@@ -14,9 +14,9 @@ namespace {
 // One-sided parts of the transposed gradient on non-periodic axes: node z within two rows of
 // a face gets delta * (2 A S~_{.beta}) of the face node it projects to, with delta = -3/2,
 // +3/2, -1/2 at rows 0, 1, 2 (low face) and +3/2, -3/2, +1/2 at rows n-1, n-2, n-3 (high face):
-// the exact one-sided stencil minus the central one the fused kernel applied.  On the low x face, and
-// on the high one where the last tile's last lane holds it, that kernel took the face's own value for the
-// one beyond it, 1/2 of it: x_lo, x_hi are delta at row 0 of the x faces.
+// the exact one-sided stencil minus the central one the fused kernel applied.  Where the march took
+// an x face's own value for the one beyond it (its lane 0 or 31), 1/2 of it comes out too: x_lo and x_hi are
+// delta at row 0 of those faces.
 __global__ void k_adj_bcorr(Geom g, const float* __restrict__ face, FaceOffsets fo, float x_lo,
                             float x_hi, float4* __restrict__ lam) {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -79,22 +79,24 @@ void face_offsets(const Geom& g, FaceOffsets& fo, long long& total) {
     total = off;
 }
 
-cudaError_t launch_fused_adj3d(const Geom& g, V4<float>* lam_in, V4<float>* lam_out,
+cudaError_t launch_fused_adj3d(const Geom& g, const Step3dPlan& plan, V4<float>* lam_in,
+                               V4<float>* lam_out,
                                const V4<float>* kus, const V4<float>* sn, const V4<float>* sp,
                                float* e, float* face, double h, int* err, cudaStream_t st,
                                int variant) {
     launch_adj_prep<float>(g, lam_in, kus, sn, e, h, st);
     cudaError_t r = cudaGetLastError();
     if (r != cudaSuccess) return r;
-    r = launch_adj_march(g, lam_in, lam_out, sp, face, err, st, variant == 0 ? 3 : 0);
+    r = launch_adj_march(g, lam_in, lam_out, sp, face, err, st, plan.adj[variant], plan.adj_org);
     if (r != cudaSuccess) return r;
     FaceOffsets fo;
     long long tot;
     face_offsets(g, fo, tot);
     const long long shell = 6LL * ((long long)g.n[1] * g.n[2] + (long long)g.n[0] * g.n[2] +
                                    (long long)g.n[0] * g.n[1]);
+    const bool lo_own = plan.adj_org == 0, hi_own = lo_own && g.n[0] > 4 && (g.n[0] - 4) % kAdjTileX == 0;
     k_adj_bcorr<<<(unsigned)((shell + 255) / 256), 256, 0, st>>>(
-        g, face, fo, -2.f, adj_face_in_last_lane(g) ? 2.f : 1.5f, reinterpret_cast<float4*>(lam_out));
+        g, face, fo, lo_own ? -2.f : -1.5f, hi_own ? 2.f : 1.5f, reinterpret_cast<float4*>(lam_out));
     return cudaGetLastError();
 }
 

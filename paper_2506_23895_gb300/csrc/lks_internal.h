@@ -149,12 +149,15 @@ struct March3d {
     int zchunk, chunks;
     double cost;              // in the units of MarchCost: comparable for one kernel
 };
-// How a grid's forward steps run: the row march's tiles, and does variant 1 take it (else the z-march,
-// in chunks of zchunk planes)?  Fixed by the grid and the device: formed once per context.
+// How a grid's steps run, fixed by the grid and the device and formed once per context.  Forward: the row
+// march's tiles, and does variant 1 take it (else the z-march, in chunks of zchunk planes)?  Adjoint: the
+// tiles of each variant and the column they start from.
 struct Step3dPlan {
     March3d tiles;
     int zchunk;
     bool rows;
+    March3d adj[2];
+    int adj_org;
 };
 Step3dPlan plan_step3d(const Geom& g);
 constexpr int kStep3dVariants = 3;
@@ -166,7 +169,8 @@ void face_offsets(const Geom& g, FaceOffsets& fo, long long& total);
 // lam_in is read and modified (the adjoint of a step's last part is applied in place).  variant 0:
 // blocks of three warps; 1: the block height chosen by the grid.
 constexpr int kAdj3dVariants = 2;
-cudaError_t launch_fused_adj3d(const Geom& g, V4<float>* lam_in, V4<float>* lam_out,
+cudaError_t launch_fused_adj3d(const Geom& g, const Step3dPlan& plan, V4<float>* lam_in,
+                               V4<float>* lam_out,
                                const V4<float>* kus, const V4<float>* sn, const V4<float>* sp,
                                float* e, float* face, double h, int* err, cudaStream_t st,
                                int variant);

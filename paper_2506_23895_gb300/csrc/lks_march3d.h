@@ -27,17 +27,15 @@ March3d march_tiles(const MarchCost& m, int out_x, int out_y, int nz, int warps)
 March3d step_march_tiles(const Geom& g);
 cudaError_t launch_step_march(const Geom& g, const V4<float>* src, const V4<float>* kus,
                               V4<float>* dst, int* err, cudaStream_t st, const March3d& t);
-// Columns from one adjoint tile to the next: a tile of 32 columns less two of halo on each side, where
-// the first and last tile's columns at the faces are no halo (a grid of 28 t + 4 columns takes t tiles).
+// Tiles of the adjoint march in blocks of `warps` warps (0: by cost), the first of 32 columns from column
+// org, -2 or 0, the next 28 on.  A tile's first and last two columns are halo, but with org 0 those at the
+// faces: a grid of 28 t + 4 columns then takes t tiles, and 28 t with org -2.
 constexpr int kAdjTileX = 28;
-// Does the last tile's last lane hold the high face column?
-inline bool adj_face_in_last_lane(const Geom& g) {
-    return g.n[0] > 4 && (g.n[0] - 4) % kAdjTileX == 0;
-}
+March3d adj_march_tiles(const Geom& g, int org, int warps);
 // lambda^{n-1} from lambda^n (after k_adj_prep) but for the one-sided boundary rows, whose 2 A S~ go
-// to face; warps > 0 fixes the block height.
+// to face.
 cudaError_t launch_adj_march(const Geom& g, const V4<float>* lam_in, V4<float>* lam_out,
                              const V4<float>* sp, float* face, int* err, cudaStream_t st,
-                             int warps);
+                             const March3d& t, int org);
 
 }  // namespace lks

@@ -91,6 +91,10 @@ __device__ __forceinline__ RowZ row_z(const float4& n, const float3& m1, const f
     return z;
 }
 
+// FACE: the tiles start at the low x face (org 0 in adj_march_tiles), else two columns before it.  Two
+// instances: with the choice at run time the other grids' march took 4 % longer (64^3 33.7 us a step
+// against 32.2).
+template <bool FACE>
 __global__ void __launch_bounds__(32 * kMaxWarps, 2)
     k_adj_march(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap umap,
                 const __grid_constant__ Args a) {
@@ -106,7 +110,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 2)
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)(NSLOT + NUSLOT) * plane_bytes +
                                                  (size_t)2 * seam_buf * 4);
     uint64_t* ubars = bars + NSLOT;
-    const int x0 = blockIdx.x * kAdjTileX + 2, y0 = blockIdx.y * (rows - 4);
+    const int x0 = blockIdx.x * kAdjTileX + (FACE ? 2 : 0), y0 = blockIdx.y * (rows - 4);
     const int q0 = blockIdx.z * a.zchunk, q1 = min(nz, q0 + a.zchunk);
     const int nplanes = q1 - q0 + 4;   // lambda planes q0 - 2 .. q1 + 1
     const bool leader = lane == 0 && wid == 0;
@@ -127,12 +131,14 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 2)
     __syncthreads();
 
     const int x = x0 - 2 + lane, yr = y0 - 2 + R * wid;   // column, first row
-    // The first and the last tile also own the halo columns on their face's side: nothing comes in from
-    // beyond a face, where a shuffle returns the lane's own value, which is zero for mu on a face.  (A
-    // face column in lane 0 or 31 also takes its own 9 S~ for its neighbour's; k_adj_bcorr's one-sided
+    // With FACE the first and the last tile also own the halo columns on their face's side: nothing comes
+    // in from beyond a face, where a shuffle returns the lane's own value, which is zero for mu on a face.
+    // (A face column in lane 0 or 31 also takes its own 9 S~ for its neighbour's; k_adj_bcorr's one-sided
     // part takes it out.)
-    const bool xown = x < nx && (lane >= 2 || blockIdx.x == 0) &&
-                      (lane < 30 || blockIdx.x == gridDim.x - 1);
+    bool xown = lane >= 2 && lane < 2 + kAdjTileX && x < nx;
+    if (FACE)
+        xown = x < nx && (lane >= 2 || blockIdx.x == 0) &&
+               (lane < 30 || blockIdx.x == gridDim.x - 1);
     int fl = 0;   // bits r: interior in x and y, OWN + r: an output row
     constexpr int OWN = 4;
 #pragma unroll
@@ -405,9 +411,14 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 2)
 
 }  // namespace
 
+March3d adj_march_tiles(const Geom& g, int org, int warps) {
+    return march_tiles(MarchCost{kAdjTileX, R, 4, kMaxWarps, 2 * kMaxWarps, 11.0, 50.0, 13.0},
+                       std::max(org == 0 ? g.n[0] - 4 : g.n[0], 1), g.n[1], g.n[2], warps);
+}
+
 cudaError_t launch_adj_march(const Geom& g, const V4<float>* lam_in, V4<float>* lam_out,
                              const V4<float>* sp, float* face, int* err, cudaStream_t st,
-                             int warps) {
+                             const March3d& t, int org) {
     Args a;
     for (int k = 0; k < 3; ++k) a.n[k] = g.n[k];
     a.lam_out = reinterpret_cast<float4*>(lam_out);
@@ -418,24 +429,26 @@ cudaError_t launch_adj_march(const Geom& g, const V4<float>* lam_in, V4<float>* 
     for (int f = 0; f < 6; ++f) a.face_off[f] = fo.off[f];
     a.err = err;
     a.A9 = (float)(g.A / 9.0);
-    const March3d t = march_tiles(MarchCost{kAdjTileX, R, 4, kMaxWarps, 2 * kMaxWarps, 11.0, 50.0, 13.0},
-                                  std::max(g.n[0] - 4, 1), g.n[1], g.n[2], warps);
     a.zchunk = t.zchunk;
     const size_t per_warp = (NSLOT + NUSLOT) * 512 * R + 2 * 2 * kSeam * 32 * 4;
     const size_t bars = (NSLOT + NUSLOT) * 8, smem = per_warp * t.warps + bars;
     static std::atomic<unsigned> attr{0};   // devices whose shared-memory limit is raised
     if (!device_done(attr)) {
-        const cudaError_t r = cudaFuncSetAttribute(
-            k_adj_march, cudaFuncAttributeMaxDynamicSharedMemorySize,
-            (int)(per_warp * kMaxWarps + bars));
-        if (r != cudaSuccess) return r;
+        for (const void* k : {(const void*)k_adj_march<false>, (const void*)k_adj_march<true>}) {
+            const cudaError_t r =
+                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(per_warp * kMaxWarps + bars));
+            if (r != cudaSuccess) return r;
+        }
         device_mark(attr);
     }
     CUtensorMap map, umap;
     if (!encode_state_map(&map, lam_in, g, 32, R * t.warps) ||
         !encode_state_map(&umap, sp, g, 32, R * t.warps))
         return cudaErrorInvalidValue;
-    k_adj_march<<<dim3(t.tiles_x, t.tiles_y, t.chunks), dim3(32, t.warps), smem, st>>>(map, umap, a);
+    const dim3 grid(t.tiles_x, t.tiles_y, t.chunks), block(32, t.warps);
+    if (org == 0) k_adj_march<true><<<grid, block, smem, st>>>(map, umap, a);
+    else k_adj_march<false><<<grid, block, smem, st>>>(map, umap, a);
     return cudaGetLastError();
 }
 

@@ -313,7 +313,7 @@ lks_status adjoint_step(lks_ctx* c, int n, const void* sn, const void* sp) {
     }
     const bool tm = timing_begin(c, n, 1);
     if (sizeof(T) == 4 && c->fused3d && !c->g.ks) {
-        cudaError_t e = launch_fused_adj3d(c->g, (V4<float>*)lc, (V4<float>*)ln,
+        cudaError_t e = launch_fused_adj3d(c->g, c->plan3d, (V4<float>*)lc, (V4<float>*)ln,
                                            (const V4<float>*)c->kus, (const V4<float>*)sn,
                                            (const V4<float>*)sp, (float*)c->e, c->face, hn,
                                            c->flags + 3, c->st, c->adj3d_var);
