@@ -1052,8 +1052,8 @@ size_t tape_bytes(const TapeSlots& t, long long boxN, long long ncol, size_t T) 
 }
 
 // The slots that fit p.bytes once the box is known (most boxes are a fraction of the grid, and the more
-// slots): the least transfers, positions from a quarter of the rest, then e for those transfers, and both
-// for more steps.
+// slots): the least transfers, positions from a quarter of the rest, then e for those transfers, both for
+// more steps, and positions from what is left.
 TapeSlots tape_slots(const TapePlan& p, long long boxN, long long ncol, size_t T) {
     TapeSlots t;
     t.k = p.least;
@@ -1071,6 +1071,7 @@ TapeSlots tape_slots(const TapePlan& p, long long boxN, long long ncol, size_t T
     const int n = take(t.k, p.want, kb + eb, left);
     t.k += n;
     t.e += n;
+    t.pos += take(t.pos, std::min(p.want, kMaxPosSlots), pb, left);
     return t;
 }
 
